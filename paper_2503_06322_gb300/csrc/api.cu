@@ -999,7 +999,7 @@ void batch_field_jobs(const BatchPlan *bp, const hpdr_field *f, int i, unsigned 
         SymIn none;
         memset(&none, 0, sizeof(none));
         size_t sm = 0;
-        coarse.push_back(coarse_args<T>(P, geo, ls, vtop, nullptr, qo, nullptr, none, nullptr, &sm));
+        coarse.push_back(coarse_args<T>(0, P, geo, ls, vtop, nullptr, qo, nullptr, none, nullptr, &sm));
         smem = std::max(smem, sm);
     }
     cb.hist = w.hist;
@@ -1095,8 +1095,8 @@ hpdr_status enqueue_batch(hpdr_ctx *ctx, BatchRes *r, BatchPlan *bp, const hpdr_
         }
     if (!join()) return HPDR_ERR_CUDA;
     // (B)
-    CK(launch_coarse_batch<float>(0, bp->coarse32, bp->n32, bp->sm32, r->origin));
-    CK(launch_coarse_batch<double>(0, bp->coarse64, bp->n64, bp->sm64, r->origin));
+    CK(launch_coarse_batch<float>(bp->coarse32, bp->n32, bp->sm32, r->origin));
+    CK(launch_coarse_batch<double>(bp->coarse64, bp->n64, bp->sm64, r->origin));
     if (codebook_fused(D)) {
         CK(launch_codebook_batch(bp->codebooks, bp->nfields, r->origin));
     } else {

@@ -375,16 +375,32 @@ __global__ void bins_kernel(BinArgs ba, const double *partials, int nparts, Scal
 // working arrays fit in shared memory) and level 0 run in a single 1024-thread
 // block out of shared memory, instead of four or five launches per level.  A
 // level of compression (Alg. 1) here:
-//   1. v_c = the kept nodes of v, compacted; w = v - P v_c on the new nodes
-//      (0 on kept ones), quantized or written to the stream;
+//   1. w = v - P v_c on the new nodes (0 on kept ones; v_c are the kept nodes
+//      of v), quantized or written to the stream;
 //   2. b = (x)_k P^T M_l w, dimension 2, then 1, then 0 (5 taps each);
 //   3. z = (x)_k M_{l-1}^{-1} b, Thomas sweeps along dimension 0, 1, then 2;
-//   4. v_{l-1} = v_c + z.
+//      the last sweep writes v_{l-1} = v_c + z.
 // Recomposition runs the levels upwards: w from the stream, b and z as above,
-// v_c = v_{l-1} - z, then v = P v_c + w.  P v_c is the multilinear
-// interpolant, taken along dimension 2, then 1, then 0.
-constexpr int kCoarseThreads = 1024;
-
+// the last sweep writing v_c = v_{l-1} - z, then v = P v_c + w.  P v_c is the
+// multilinear interpolant, taken along dimension 2, then 1, then 0.
+//
+// One block on one SM: the time is the chain of phases and the latency inside
+// each, not throughput.  So
+//   - everything a phase reads is put in shared memory once, by copies that
+//     overlap each other: the level tables, the top grid or the stream prefix
+//     [0, N_ls) of levels 0..ls (dequantized on the way), the bins;
+//   - a thread owns a coarse cell: it loads the cell's eight corners and forms
+//     the interpolant of its up to seven new nodes from them, where a thread
+//     per node met every combination of new and kept dimensions as its own
+//     branch and loaded 27 corners for 8 nodes;
+//   - binary32 coefficients are quantized in binary32 (quant_exact): the
+//     binary64 decision ran at two lanes per cycle and was half of the kernel;
+//   - lines are swept in batches loaded ahead of the recurrence, and indices
+//     are split by a multiply-high with precomputed factors.
+// Levels 4..1 and 0 of a 513^3 FP32 field: 58 -> 24 us down, 60 -> 26 us up; of
+// 129^2: 67 -> 27 and 69 -> 26 us (64 bit index divisions, tables read in global
+// memory on every use and the binary64 quantizer before).
+constexpr int kCoarseThreads = 512;
 
 // element counts of the shared arrays for top level ls (host and device)
 template <typename T>
@@ -399,225 +415,412 @@ __host__ __device__ inline void coarse_sizes(const LevelGeom<T> &g, long long &n
     r1 = m0 * c1 * c2;
 }
 
-// multilinear interpolant of the compact coarse array X at fine node (p0, p1, p2)
-template <typename T>
-__device__ __forceinline__ T coarse_interp(const LevelGeom<T> &g, const T *X, int p0, int p1, int p2)
+// i / d by a multiply-high: exact for i and d below 2^16 (the block's arrays
+// hold at most kCoarseSmem / 2 / sizeof(float) = 25600 nodes); mul = 0 for d = 1
+__device__ __forceinline__ unsigned small_div_mul(int d) { return 0xFFFFFFFFu / (unsigned)d + 1u; }
+__device__ __forceinline__ int small_div(int i, unsigned mul)
 {
-    const int c1 = g.dim[1].mc, c2 = g.dim[2].mc;
-    int a[3], b[3];
-    bool nw[3];
-    const int p[3] = {p0, p1, p2};
+    return mul == 0u ? i : (int)__umulhi((unsigned)i, mul);
+}
+
+// One dimension of one level.  Tables: wl[m], wr[m], tap[5 mc], sub[mc],
+// cp[mc], inv[mc], in this order when they are staged.
+template <typename T>
+struct CoarseDim {
+    const T *wl, *wr, *tap, *sub, *cp, *inv;
+    int m, mc;
+    unsigned mmul, cmul;   // small_div factors of m and mc
+};
+struct CoarseExt {
+    int m, mc, off;
+    unsigned mmul, cmul;
+};
+__host__ __device__ inline int coarse_tab_elems(int m, int mc) { return 2 * m + 8 * mc; }
+
+// dimension k of level l; STG: the tables sit at `extra` + their offset
+template <typename T, bool STG>
+__device__ __forceinline__ CoarseDim<T> coarse_dim(const CoarseArgs<T> &a, const CoarseExt &e, const T *extra, int l,
+                                                   int k)
+{
+    CoarseDim<T> c;
+    c.m = e.m; c.mc = e.mc; c.mmul = e.mmul; c.cmul = e.cmul;
+    if (STG) {
+        const T *t = extra + e.off;
+        c.wl = t; c.wr = t + e.m; c.tap = t + 2 * e.m;
+        c.sub = t + 2 * e.m + 5 * e.mc; c.cp = t + 2 * e.m + 6 * e.mc; c.inv = t + 2 * e.m + 7 * e.mc;
+    } else {
+        const DimTables<T> &g = a.g[l].dim[k];
+        c.wl = g.wl; c.wr = g.wr; c.tap = g.tap; c.sub = g.sub; c.cp = g.cp; c.inv = g.inv_den;
+    }
+    return c;
+}
+
+// the coarse cell at (j0, j1, j2): whether a new node follows along each
+// dimension, and the weights of that node
+template <typename T>
+struct CoarseCell {
+    int p[3];
+    bool h[3];
+    T wl[3], wr[3];
+};
+template <typename T>
+__device__ __forceinline__ CoarseCell<T> coarse_cell(const CoarseDim<T> *d, const int j[3])
+{
+    CoarseCell<T> c;
 #pragma unroll
     for (int k = 0; k < 3; k++) {
-        const int m = g.dim[k].m, mc = g.dim[k].mc;
-        nw[k] = !kept_pos(m, p[k]);
-        if (nw[k]) { a[k] = cidx_of(m, mc, p[k] - 1); b[k] = cidx_of(m, mc, p[k] + 1); }
-        else { a[k] = b[k] = cidx_of(m, mc, p[k]); }
+        c.p[k] = cpos_of(d[k].m, d[k].mc, j[k]);
+        c.h[k] = j[k] + 1 < d[k].mc && c.p[k] + 2 == cpos_of(d[k].m, d[k].mc, j[k] + 1);
+        c.wl[k] = c.h[k] ? d[k].wl[c.p[k] + 1] : (T)0;
+        c.wr[k] = c.h[k] ? d[k].wr[c.p[k] + 1] : (T)0;
     }
-    auto along2 = [&](int i0, int i1) -> T {
-        const T *row = X + ((long long)i0 * c1 + i1) * c2;
-        if (!nw[2]) return row[a[2]];
-        return fma_rn(g.dim[2].wr[p2], row[b[2]], mul_rn(g.dim[2].wl[p2], row[a[2]]));
-    };
-    auto along1 = [&](int i0) -> T {
-        if (!nw[1]) return along2(i0, a[1]);
-        return fma_rn(g.dim[1].wr[p1], along2(i0, b[1]), mul_rn(g.dim[1].wl[p1], along2(i0, a[1])));
-    };
-    if (!nw[0]) return along1(a[0]);
-    return fma_rn(g.dim[0].wr[p0], along1(b[0]), mul_rn(g.dim[0].wl[p0], along1(a[0])));
+    return c;
+}
+
+// multilinear interpolant at the cell's nodes (index 4 q0 + 2 q1 + q2; q = 1:
+// the new node of that dimension) from its corners X[o0][o1][o2] around X[0],
+// the other corner of dimension k at offset s[k] (0 without a new node);
+// dimension 2, then 1, then 0
+template <typename T>
+__device__ __forceinline__ void coarse_interp(const CoarseCell<T> &c, const T *X, const int s[3], T r[8])
+{
+    auto lerp = [&](int k, T x, T y) { return fma_rn(c.wr[k], y, mul_rn(c.wl[k], x)); };
+    T v[2][2][2];   // [side of dimension 0][side of dimension 1][kept, new column]
+#pragma unroll
+    for (int a = 0; a < 2; a++)
+#pragma unroll
+        for (int b = 0; b < 2; b++) {
+            const T *x = X + a * s[0] + b * s[1];
+            const T x0 = x[0], x1 = x[s[2]];
+            v[a][b][0] = x0;
+            v[a][b][1] = lerp(2, x0, x1);
+        }
+#pragma unroll
+    for (int q2 = 0; q2 < 2; q2++) {
+        const T y0 = lerp(1, v[0][0][q2], v[0][1][q2]), y1 = lerp(1, v[1][0][q2], v[1][1][q2]);
+        r[q2] = v[0][0][q2];
+        r[2 + q2] = y0;
+        r[4 + q2] = lerp(0, v[0][0][q2], v[1][0][q2]);
+        r[6 + q2] = lerp(0, y0, y1);
+    }
+}
+
+// f(q, p-offset, stream offset) for every new node of the cell: q as in
+// coarse_interp, the node's flat index relative to the cell's kept node, and
+// its index in the level's section of the stream
+template <typename T, typename F>
+__device__ __forceinline__ void coarse_new_nodes(const CoarseCell<T> &c, const int j[3], int m1, int m2, int c1, int c2,
+                                                 F f)
+{
+    const int base = (c.p[0] * m1 + c.p[1]) * m2 + c.p[2];
+#pragma unroll
+    for (int q = 1; q < 8; q++) {
+        const int q0 = q >> 2, q1 = (q >> 1) & 1, q2 = q & 1;
+        if ((q0 && !c.h[0]) || (q1 && !c.h[1]) || (q2 && !c.h[2])) continue;
+        const int off = (q0 * m1 + q1) * m2 + q2;
+        // kept nodes before it: whole planes, then rows, then columns
+        int cr = (j[0] + q0) * c1 * c2;
+        if (!q0) cr += (j[1] + q1) * c2;
+        if (!q0 && !q1) cr += j[2] + 1;
+        f(q, off, base + off - cr);
+    }
 }
 
 // out = in restricted along dimension k with the 5 taps of P^T M_l; in has
-// extents n[3] (n[k] = m), out the same with n[k] = mc
-template <typename T>
-__device__ void coarse_restrict(const DimTables<T> &d, int k, const int n[3], const T *in, T *out)
+// extents n0 x n1 x n2 (extent k = m), out the same with extent k = mc;
+// mul2, mul1: small_div factors of out's extents 2 and 1
+template <typename T, int k>
+__device__ __forceinline__ void coarse_restrict(const CoarseDim<T> &d, int n0, int n1, int n2, unsigned mul2,
+                                                unsigned mul1, const T *in, T *out)
 {
-    int o[3] = {n[0], n[1], n[2]};
-    o[k] = d.mc;
-    const long long tot = (long long)o[0] * o[1] * o[2];
-    const long long is[3] = {(long long)n[1] * n[2], n[2], 1};
-    for (long long idx = threadIdx.x; idx < tot; idx += blockDim.x) {
-        const int j2 = (int)(idx % o[2]);
-        const long long r = idx / o[2];
-        const int j1 = (int)(r % o[1]), j0 = (int)(r / o[1]);
-        const int jj[3] = {j0, j1, j2};
-        if (d.m <= 1) { out[idx] = in[j0 * is[0] + j1 * is[1] + j2]; continue; }
-        const int jk = jj[k];
-        const int c = cpos_of(d.m, d.mc, jk);
-        long long base = 0;
+    const int m = d.m, mc = d.mc;
+    const int o0 = k == 0 ? mc : n0, o1 = k == 1 ? mc : n1, o2 = k == 2 ? mc : n2;
+    const int is = k == 0 ? n1 * n2 : k == 1 ? n2 : 1;
+    const int tot = o0 * o1 * o2;
+    const T *tap = d.tap;
+    for (int idx = threadIdx.x; idx < tot; idx += blockDim.x) {
+        const int r = small_div(idx, mul2), j2 = idx - r * o2, j0 = small_div(r, mul1), j1 = r - j0 * o1;
+        const int jk = k == 0 ? j0 : k == 1 ? j1 : j2;
+        const int c = cpos_of(m, mc, jk);
+        const T *x = in + ((k == 0 ? c : j0) * n1 + (k == 1 ? c : j1)) * n2 + (k == 2 ? c : j2);
+        T t[5], y[5];
 #pragma unroll
-        for (int q = 0; q < 3; q++) if (q != k) base += jj[q] * is[q];
+        for (int o = -2; o <= 2; o++) {
+            const bool inside = (unsigned)(c + o) < (unsigned)m;
+            t[o + 2] = tap[jk * 5 + o + 2];
+            y[o + 2] = x[inside ? o * is : 0];
+        }
         T acc = (T)0;
 #pragma unroll
-        for (int t = 0; t < 5; t++) {
-            const int pos = c - 2 + t;
-            if (pos < 0 || pos >= d.m) continue;
-            acc = fma_rn(d.tap[jk * 5 + t], in[base + pos * is[k]], acc);
+        for (int o = -2; o <= 2; o++) {
+            const T z = fma_rn(t[o + 2], y[o + 2], acc);
+            acc = (unsigned)(c + o) < (unsigned)m ? z : acc;
         }
         out[idx] = acc;
     }
+    __syncthreads();
 }
 
-// Thomas sweeps of (x)_k M_{l-1} on the compact coarse array B (extents c[3]), in place
-template <typename T>
-__device__ void coarse_solves(const LevelGeom<T> &g, const int c[3], T *B)
+// Thomas sweeps of one line p[0], p[st], ...; fin(t, x) takes the solution
+template <typename T, typename Fin>
+__device__ __forceinline__ void coarse_line(const CoarseDim<T> &d, T *p, int st, Fin fin)
 {
-    for (int k = 0; k < 3; k++) {
-        const DimTables<T> &d = g.dim[k];
-        if (!(d.m > 1)) continue;
-        const long long st = k == 0 ? (long long)c[1] * c[2] : k == 1 ? c[2] : 1;
-        const int oa = k == 0 ? c[1] : c[0], ob = k == 2 ? c[1] : c[2];
-        for (int line = threadIdx.x; line < oa * ob; line += blockDim.x) {
-            const int u = line / ob, v = line - u * ob;
-            long long base;
-            if (k == 0) base = (long long)u * c[2] + v;
-            else if (k == 1) base = (long long)u * c[1] * c[2] + v;
-            else base = ((long long)u * c[1] + v) * c[2];
-            T *p = B + base;
-            const int n = d.mc;
-            T y = (T)0;
-            for (int t = 0; t < n; t++) { y = mul_rn(fma_rn(-d.sub[t], y, p[t * st]), d.inv_den[t]); p[t * st] = y; }
-            T x = (T)0;
-            for (int t = n - 1; t >= 0; t--) { x = fma_rn(-d.cp[t], x, p[t * st]); p[t * st] = x; }
+    constexpr int U = sizeof(T) == 4 ? 8 : 4;
+    const int n = d.mc;
+    const T *sub = d.sub, *inv = d.inv, *cp = d.cp;
+    T y = (T)0;
+#pragma unroll 1
+    for (int t0 = 0; t0 < n; t0 += U) {
+        T v[U], f[U], g[U];
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            const int t = min(t0 + u, n - 1);
+            v[u] = p[t * st]; f[u] = sub[t]; g[u] = inv[t];
         }
-        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < U; u++)
+            if (t0 + u < n) { y = mul_rn(fma_rn(-f[u], y, v[u]), g[u]); p[(t0 + u) * st] = y; }
+    }
+    T x = (T)0;
+#pragma unroll 1
+    for (int t0 = n - 1; t0 >= 0; t0 -= U) {
+        T v[U], f[U];
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            const int t = max(t0 - u, 0);
+            v[u] = p[t * st]; f[u] = cp[t];
+        }
+#pragma unroll
+        for (int u = 0; u < U; u++)
+            if (t0 - u >= 0) { x = fma_rn(-f[u], x, v[u]); fin(t0 - u, x); }
     }
 }
 
-// b = (x)_k P^T M_l W into B (R2, R1 scratch)
-template <typename T>
-__device__ void coarse_rhs(const LevelGeom<T> &g, const T *W, T *R2, T *R1, T *B)
+// b = (x)_k P^T M_l W, then z = (x)_k M_{l-1}^{-1} b in place (R2, R1, B
+// scratch); fin(j, j0, j1, t, z) takes z at the coarse node (j0, j1, t) of flat
+// index j (the dimension-2 sweep always runs: a field's last dimension is active)
+template <typename T, typename Fin>
+__device__ __forceinline__ void coarse_correct(const CoarseDim<T> *d, const T *W, T *R2, T *R1, T *B, Fin fin)
 {
-    const int m[3] = {g.dim[0].m, g.dim[1].m, g.dim[2].m};
-    const int n2[3] = {m[0], m[1], m[2]};
-    coarse_restrict<T>(g.dim[2], 2, n2, W, R2);
-    __syncthreads();
-    const int n1[3] = {m[0], m[1], g.dim[2].mc};
-    coarse_restrict<T>(g.dim[1], 1, n1, R2, R1);
-    __syncthreads();
-    const int n0[3] = {m[0], g.dim[1].mc, g.dim[2].mc};
-    coarse_restrict<T>(g.dim[0], 0, n0, R1, B);
+    const int c0 = d[0].mc, c1 = d[1].mc, c2 = d[2].mc, m0 = d[0].m, m1 = d[1].m;
+    // an inactive dimension (one node) keeps its values: no pass
+    T *const rhs = m0 > 1 ? B : m1 > 1 ? R1 : R2;
+    coarse_restrict<T, 2>(d[2], m0, m1, d[2].m, d[2].cmul, d[1].mmul, W, R2);
+    if (m1 > 1) coarse_restrict<T, 1>(d[1], m0, m1, c2, d[2].cmul, d[1].cmul, R2, R1);
+    if (m0 > 1) coarse_restrict<T, 0>(d[0], m0, c1, c2, d[2].cmul, d[1].cmul, m1 > 1 ? R1 : R2, B);
+    if (m0 > 1) {
+        const int pl = c1 * c2;
+        for (int i = threadIdx.x; i < pl; i += blockDim.x) {
+            T *p = rhs + i;
+            coarse_line<T>(d[0], p, pl, [&](int t, T x) { p[t * pl] = x; });
+        }
+        __syncthreads();
+    }
+    if (m1 > 1) {
+        for (int i = threadIdx.x; i < c0 * c2; i += blockDim.x) {
+            const int j0 = small_div(i, d[2].cmul);
+            T *p = rhs + j0 * c1 * c2 + (i - j0 * c2);
+            coarse_line<T>(d[1], p, c2, [&](int t, T x) { p[t * c2] = x; });
+        }
+        __syncthreads();
+    }
+    for (int i = threadIdx.x; i < c0 * c1; i += blockDim.x) {
+        const int j0 = small_div(i, d[1].cmul), j1 = i - j0 * c1;
+        coarse_line<T>(d[2], rhs + i * c2, 1, [&](int t, T x) { fin(i * c2 + t, j0, j1, t, x); });
+    }
     __syncthreads();
 }
 
 // MODE 0: compression (quantize), 1: decomposition (coefficient stream),
 // 2: decompression (symbols), 3: recomposition (coefficient stream)
-template <typename T, int MODE>
+template <typename T, int MODE, bool STG>
 __device__ __forceinline__ void coarse_body(const CoarseArgs<T> &a)
 {
     extern __shared__ __align__(16) unsigned char coarse_smem[];
-    long long nl, nc, r2, r1;
-    coarse_sizes<T>(a.g[a.ls], nl, nc, r2, r1);
+    __shared__ CoarseExt sext[kCoarseMaxLevels + 1][3];
+    __shared__ int snprev[kCoarseMaxLevels + 1];    // first stream index of every level
+    __shared__ T sq[kCoarseMaxLevels + 1];          // MODE 2: q of every level
+    const int ls = a.ls, tid = threadIdx.x, nt = blockDim.x, N0 = (int)a.N0;
+    long long nl_, nc_, r2_, r1_;
+    coarse_sizes<T>(a.g[ls], nl_, nc_, r2_, r1_);
+    const int nl = (int)nl_, nc = (int)nc_;
     T *VA = reinterpret_cast<T *>(coarse_smem);   // [nl]
     T *VB = VA + nl;                                // [nc]
     T *W = VB + nc;                                 // [nl]
     T *R2 = W + nl;                                 // [r2]
-    T *R1 = R2 + r2;                                // [r1]
-    T *B = R1 + r1;                                 // [nc]
+    T *R1 = R2 + (int)r2_;                          // [r1]
+    T *B = R1 + (int)r1_;                           // [nc]
     T *VK = B + nc;                                 // [nc]
-    const int tid = threadIdx.x;
-    if (MODE <= 1) {
-        for (long long i = tid; i < nl; i += blockDim.x) VA[i] = a.v_in[i];
-        __syncthreads();
-        T *V = VA, *Vn = VB;
-        for (int l = a.ls; l >= 1; l--) {
-            const LevelGeom<T> &g = a.g[l];
-            const int m1 = g.dim[1].m, m2 = g.dim[2].m;
-            const int c[3] = {g.dim[0].mc, g.dim[1].mc, g.dim[2].mc};
-            const long long n = (long long)g.dim[0].m * m1 * m2, ncl = (long long)c[0] * c[1] * c[2];
-            // 1. kept nodes, compacted
-            for (long long j = tid; j < ncl; j += blockDim.x) {
-                const int j2 = (int)(j % c[2]);
-                const long long r = j / c[2];
-                const int j1 = (int)(r % c[1]), j0 = (int)(r / c[1]);
-                const long long f = ((long long)cpos_of(g.dim[0].m, c[0], j0) * m1 + cpos_of(m1, c[1], j1)) * m2 +
-                                    cpos_of(m2, c[2], j2);
-                VK[j] = V[f];
+    T *const extra = VK + nc;                       // staged stream prefix, staged tables
+    const bool stream = MODE >= 2 && a.stream_off >= 0;
+    const T *const S = extra + (stream ? a.stream_off : 0);
+
+    // ---- staging
+    for (int i = tid; i < 3 * ls; i += nt) {
+        const int l = 1 + i / 3, k = i - (l - 1) * 3;
+        const DimTables<T> &g = a.g[l].dim[k];
+        sext[l][k] = {g.m, g.mc, a.tab_off[l][k], small_div_mul(g.m), small_div_mul(g.mc)};
+    }
+    if (tid <= ls) {
+        snprev[tid] = tid ? (int)a.g[tid].Nprev : 0;
+        if (MODE == 2) sq[tid] = q_of<T>(a.symin.sc, tid);
+    }
+    if (STG)
+        for (int task = tid >> 5; task < 18 * ls; task += nt >> 5) {
+            const int l = 1 + task / 18, r = task - (l - 1) * 18, k = r / 6, w = r - k * 6;
+            const DimTables<T> &g = a.g[l].dim[k];
+            if (!(g.m > 1)) continue;
+            const T *src = w == 0 ? g.wl : w == 1 ? g.wr : w == 2 ? g.tap : w == 3 ? g.sub : w == 4 ? g.cp : g.inv_den;
+            const int cnt = w < 2 ? g.m : w == 2 ? 5 * g.mc : g.mc;
+            T *dst = extra + a.tab_off[l][k] + (w < 2 ? w * g.m : 2 * g.m + (w == 2 ? 0 : (w + 2) * g.mc));
+            for (int i = tid & 31; i < cnt; i += 32) cp_async_elem(dst + i, src + i);
+        }
+    if (MODE <= 1) for (int i = tid; i < nl; i += nt) cp_async_elem(VA + i, a.v_in + i);
+    if (MODE == 3 && stream) for (int i = tid; i < nl; i += nt) cp_async_elem(extra + a.stream_off + i, a.coef_in + i);
+    if (MODE == 2 && stream) {
+        // symbols, then the codes of the escaped ones: every load of a batch in
+        // flight before the first use
+        T *const So = extra + a.stream_off;
+        constexpr int U = 10;
+        bool first = true;
+        for (int i0 = tid; i0 < nl || first; i0 += U * nt) {
+            unsigned sv[U];
+            long long ev[U];
+#pragma unroll
+            for (int u = 0; u < U; u++) sv[u] = i0 + u * nt < nl ? a.symin.sym[i0 + u * nt] : 1u;
+#pragma unroll
+            for (int u = 0; u < U; u++) ev[u] = sv[u] == 0u ? a.symin.esc[i0 + u * nt] : 0;
+            if (first) __syncthreads();   // the bins and the level starts
+            first = false;
+#pragma unroll
+            for (int u = 0; u < U; u++) {
+                const int i = i0 + u * nt;
+                if (i >= nl) continue;
+                int l = 0;
+                while (l < ls && i >= snprev[l + 1]) l++;
+                So[i] = sv[u] != 0u ? mul_rn((T)((int)sv[u] - (int)(a.symin.D / 2)), sq[l]) : mul_rn((T)ev[u], sq[l]);
             }
-            __syncthreads();
-            //    coefficients of the new nodes
-            const double rho = MODE == 0 ? rho64_of(a.qo.sc, l) : 0.0;
-            for (long long i = tid; i < n; i += blockDim.x) {
-                const int p2 = (int)(i % m2);
-                const long long r = i / m2;
-                const int p1 = (int)(r % m1), p0 = (int)(r / m1);
-                if (kept_pos(g.dim[0].m, p0) && kept_pos(m1, p1) && kept_pos(m2, p2)) { W[i] = (T)0; continue; }
-                const T w = sub_rn(V[i], coarse_interp<T>(g, VK, p0, p1, p2));
-                W[i] = w;
-                const long long si = stream_rank(g, p0, p1, p2);
-                if (MODE == 0) quant_emit(a.qo, nullptr, false, si, w, rho);
+        }
+    }
+    cp_async_wait_all();
+    __syncthreads();
+
+    if (MODE <= 1) {
+        T *V = VA, *Vn = VB;
+        for (int l = ls; l >= 0; l--) {
+            // quantization constants of this level, off the critical path of the phases
+            double rho = 0.0;
+            float rhi = 0.f, rlo = 0.f;
+            if (MODE == 0) { rho = rho64_of(a.qo.sc, l); rhi = a.qo.sc->rho_f[l]; rlo = a.qo.sc->rho_lo[l]; }
+            auto put = [&](long long si, T w) {
+                if (MODE == 0) quant_emit_exact(a.qo, si, w, rho, rhi, rlo);
                 else a.coef_out[si] = w;
+            };
+            if (l == 0) {
+                for (int i = tid; i < N0; i += nt) put((long long)i, V[i]);
+                break;
+            }
+            const CoarseDim<T> d[3] = {coarse_dim<T, STG>(a, sext[l][0], extra, l, 0),
+                                       coarse_dim<T, STG>(a, sext[l][1], extra, l, 1),
+                                       coarse_dim<T, STG>(a, sext[l][2], extra, l, 2)};
+            const int m0 = d[0].m, m1 = d[1].m, m2 = d[2].m, c0 = d[0].mc, c1 = d[1].mc, c2 = d[2].mc;
+            const int np = snprev[l];
+            // 1. coefficients of the new nodes
+#pragma unroll 1
+            for (int i = tid; i < c0 * c1 * c2; i += nt) {
+                const int r = small_div(i, d[2].cmul), j0 = small_div(r, d[1].cmul);
+                const int j[3] = {j0, r - j0 * c1, i - r * c2};
+                const CoarseCell<T> c = coarse_cell<T>(d, j);
+                const int base = (c.p[0] * m1 + c.p[1]) * m2 + c.p[2];
+                const int st[3] = {c.h[0] ? 2 * m1 * m2 : 0, c.h[1] ? 2 * m2 : 0, c.h[2] ? 2 : 0};
+                T x[8];
+                coarse_interp<T>(c, V + base, st, x);
+                W[base] = (T)0;
+                coarse_new_nodes<T>(c, j, m1, m2, c1, c2, [&](int q, int off, int so) {
+                    const T w = sub_rn(V[base + off], x[q]);
+                    W[base + off] = w;
+                    put((long long)np + so, w);
+                });
             }
             __syncthreads();
             // 2.-3.
-            coarse_rhs<T>(g, W, R2, R1, B);
-            coarse_solves<T>(g, c, B);
-            // 4.
-            for (long long j = tid; j < ncl; j += blockDim.x) Vn[j] = add_rn(VK[j], B[j]);
-            __syncthreads();
+            coarse_correct<T>(d, W, R2, R1, B, [&](int j, int j0, int j1, int t, T z) {
+                Vn[j] = add_rn(V[(cpos_of(m0, c0, j0) * m1 + cpos_of(m1, c1, j1)) * m2 + cpos_of(m2, c2, t)], z);
+            });
             T *t = V; V = Vn; Vn = t;
-        }
-        // level 0
-        const double rho0 = MODE == 0 ? rho64_of(a.qo.sc, 0) : 0.0;
-        for (long long i = tid; i < a.N0; i += blockDim.x) {
-            if (MODE == 0) quant_emit(a.qo, nullptr, false, i, V[i], rho0);
-            else a.coef_out[i] = V[i];
         }
     } else {
         T *V = VA, *Vn = VB;
         // the same ping-pong as compression, run backwards: level l's grid lands
-        // where compression read it (the top level in VA)
-        if ((a.ls & 1) == 1) { V = VB; Vn = VA; }
-        const T q0 = MODE == 2 ? q_of<T>(a.symin.sc, 0) : (T)0;
-        for (long long i = tid; i < a.N0; i += blockDim.x)
-            V[i] = MODE == 2 ? dequant_sym<T>(a.symin, a.symin.sym[i], i, q0) : a.coef_in[i];
-        __syncthreads();
-        for (int l = 1; l <= a.ls; l++) {
-            const LevelGeom<T> &g = a.g[l];
-            const int m1 = g.dim[1].m, m2 = g.dim[2].m;
-            const int c[3] = {g.dim[0].mc, g.dim[1].mc, g.dim[2].mc};
-            const long long n = (long long)g.dim[0].m * m1 * m2, ncl = (long long)c[0] * c[1] * c[2];
-            const T q = MODE == 2 ? q_of<T>(a.symin.sc, l) : (T)0;
-            for (long long i = tid; i < n; i += blockDim.x) {
-                const int p2 = (int)(i % m2);
-                const long long r = i / m2;
-                const int p1 = (int)(r % m1), p0 = (int)(r / m1);
-                if (kept_pos(g.dim[0].m, p0) && kept_pos(m1, p1) && kept_pos(m2, p2)) { W[i] = (T)0; continue; }
-                const long long si = stream_rank(g, p0, p1, p2);
-                W[i] = MODE == 2 ? dequant_sym<T>(a.symin, a.symin.sym[si], si, q) : a.coef_in[si];
+        // where compression read it (the top level's would be VA)
+        if ((ls & 1) == 1) { V = VB; Vn = VA; }
+        // value of stream index i of level l
+        auto value = [&](int i, int l) -> T {
+            if (stream) return S[i];
+            if (MODE == 2) return dequant_sym<T>(a.symin, a.symin.sym[i], i, sq[l]);
+            return a.coef_in[i];
+        };
+        for (int i = tid; i < N0; i += nt) V[i] = value(i, 0);
+        for (int l = 1; l <= ls; l++) {
+            const CoarseDim<T> d[3] = {coarse_dim<T, STG>(a, sext[l][0], extra, l, 0),
+                                       coarse_dim<T, STG>(a, sext[l][1], extra, l, 1),
+                                       coarse_dim<T, STG>(a, sext[l][2], extra, l, 2)};
+            const int m1 = d[1].m, m2 = d[2].m, c0 = d[0].mc, c1 = d[1].mc, c2 = d[2].mc;
+            const int np = snprev[l];
+            auto cell = [&](int i, int j[3]) {
+                const int r = small_div(i, d[2].cmul);
+                j[0] = small_div(r, d[1].cmul);
+                j[1] = r - j[0] * c1;
+                j[2] = i - r * c2;
+                return coarse_cell<T>(d, j);
+            };
+#pragma unroll 1
+            for (int i = tid; i < c0 * c1 * c2; i += nt) {
+                int j[3];
+                const CoarseCell<T> c = cell(i, j);
+                const int base = (c.p[0] * m1 + c.p[1]) * m2 + c.p[2];
+                W[base] = (T)0;
+                coarse_new_nodes<T>(c, j, m1, m2, c1, c2, [&](int, int off, int so) { W[base + off] = value(np + so, l); });
             }
             __syncthreads();
-            coarse_rhs<T>(g, W, R2, R1, B);
-            coarse_solves<T>(g, c, B);
-            for (long long j = tid; j < ncl; j += blockDim.x) VK[j] = sub_rn(V[j], B[j]);
-            __syncthreads();
-            for (long long i = tid; i < n; i += blockDim.x) {
-                const int p2 = (int)(i % m2);
-                const long long r = i / m2;
-                const int p1 = (int)(r % m1), p0 = (int)(r / m1);
-                const bool kept = kept_pos(g.dim[0].m, p0) && kept_pos(m1, p1) && kept_pos(m2, p2);
-                Vn[i] = kept ? VK[((long long)cidx_of(g.dim[0].m, c[0], p0) * c[1] + cidx_of(m1, c[1], p1)) * c[2] +
-                                  cidx_of(m2, c[2], p2)]
-                             : add_rn(W[i], coarse_interp<T>(g, VK, p0, p1, p2));
-            }
+            coarse_correct<T>(d, W, R2, R1, B, [&](int j, int, int, int, T z) { VK[j] = sub_rn(V[j], z); });
+            auto expand = [&](T *dst) {
+#pragma unroll 1
+                for (int i = tid; i < c0 * c1 * c2; i += nt) {
+                    int j[3];
+                    const CoarseCell<T> c = cell(i, j);
+                    const int base = (c.p[0] * m1 + c.p[1]) * m2 + c.p[2];
+                    const int st[3] = {c.h[0] ? c1 * c2 : 0, c.h[1] ? c2 : 0, c.h[2] ? 1 : 0};
+                    T x[8];
+                    coarse_interp<T>(c, VK + i, st, x);
+                    dst[base] = x[0];
+                    coarse_new_nodes<T>(c, j, m1, m2, c1, c2, [&](int q, int off, int) {
+                        dst[base + off] = add_rn(W[base + off], x[q]);
+                    });
+                }
+            };
+            if (l == ls) { expand(a.v_out); break; }
+            expand(Vn);
             __syncthreads();
             T *t = V; V = Vn; Vn = t;
         }
-        for (long long i = tid; i < nl; i += blockDim.x) a.v_out[i] = V[i];
     }
 }
 
 template <typename T, int MODE>
 __global__ void __launch_bounds__(kCoarseThreads, 1) coarse_kernel(CoarseArgs<T> a)
 {
-    coarse_body<T, MODE>(a);
+    if (a.staged) coarse_body<T, MODE, true>(a);
+    else coarse_body<T, MODE, false>(a);
 }
 
-// one field per block
-template <typename T, int MODE>
+// one field per block (compression)
+template <typename T>
 __global__ void __launch_bounds__(kCoarseThreads, 1) coarse_batch_kernel(const CoarseArgs<T> *jobs)
 {
-    coarse_body<T, MODE>(jobs[blockIdx.x]);
+    const CoarseArgs<T> &a = jobs[blockIdx.x];
+    if (a.staged) coarse_body<T, 0, true>(a);
+    else coarse_body<T, 0, false>(a);
 }
 
 }  // namespace
@@ -793,7 +996,7 @@ int coarse_top(const Plan *P, const LevelGeom<T> *geo)
 }
 
 template <typename T>
-CoarseArgs<T> coarse_args(const Plan *P, const LevelGeom<T> *geo, int ls, const T *v_in, T *v_out,
+CoarseArgs<T> coarse_args(int mode, const Plan *P, const LevelGeom<T> *geo, int ls, const T *v_in, T *v_out,
                           const QuantOut &qo, T *coef_out, const SymIn &symin, const T *coef_in, size_t *smem)
 {
     CoarseArgs<T> a;
@@ -802,30 +1005,46 @@ CoarseArgs<T> coarse_args(const Plan *P, const LevelGeom<T> *geo, int ls, const 
     a.ls = ls;
     a.N0 = P->N[0];
     a.v_in = v_in; a.v_out = v_out; a.qo = qo; a.coef_out = coef_out; a.symin = symin; a.coef_in = coef_in;
-    if (smem) *smem = ls >= 1 && ls <= kCoarseMaxLevels ? coarse_smem_bytes<T>(geo[ls]) : 0;
+    a.stream_off = -1;
+    size_t bytes = 0;
+    if (ls >= 1 && ls <= kCoarseMaxLevels) {
+        // the stream prefix, then the tables of every level and dimension, as far
+        // as the block's shared memory takes them (long thin grids read theirs in
+        // global memory)
+        const size_t work = coarse_smem_bytes<T>(geo[ls]);
+        const size_t room = work < kCoarseSmemMax ? (kCoarseSmemMax - work) / sizeof(T) : 0;
+        const size_t nl = (size_t)geo[ls].dim[0].m * geo[ls].dim[1].m * geo[ls].dim[2].m;
+        size_t n = 0, tab = 0;
+        for (int l = 1; l <= ls; l++)
+            for (int k = 0; k < 3; k++)
+                if (geo[l].dim[k].m > 1) tab += coarse_tab_elems(geo[l].dim[k].m, geo[l].dim[k].mc);
+        a.staged = tab <= room;
+        if (a.staged)
+            for (int l = 1; l <= ls; l++)
+                for (int k = 0; k < 3; k++) {
+                    a.tab_off[l][k] = (int)n;
+                    if (geo[l].dim[k].m > 1) n += coarse_tab_elems(geo[l].dim[k].m, geo[l].dim[k].mc);
+                }
+        if (mode >= 2 && n + nl <= room) { a.stream_off = (int)n; n += nl; }
+        bytes = work + n * sizeof(T);
+    }
+    if (smem) *smem = bytes;
     return a;
 }
 
 template <typename T>
-cudaError_t launch_coarse_batch(int mode, const CoarseArgs<T> *jobs, int n, size_t smem, cudaStream_t s)
+cudaError_t launch_coarse_batch(const CoarseArgs<T> *jobs, int n, size_t smem, cudaStream_t s)
 {
     if (n < 1) return cudaSuccess;
-    static PerDeviceOnce attr[4];
-    auto go = [&](auto kern) -> cudaError_t {
-        cudaError_t e = once_per_device(attr[mode & 3], [&] {
-            return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCoarseSmem);
-        });
-        if (e != cudaSuccess) return e;
-        kern<<<n, kCoarseThreads, smem, s>>>(jobs);
-        count_launch();
-        return cudaGetLastError();
-    };
-    switch (mode) {
-    case 0: return go(coarse_batch_kernel<T, 0>);
-    case 1: return go(coarse_batch_kernel<T, 1>);
-    case 2: return go(coarse_batch_kernel<T, 2>);
-    default: return go(coarse_batch_kernel<T, 3>);
-    }
+    static PerDeviceOnce attr;
+    cudaError_t e = once_per_device(attr, [] {
+        return cudaFuncSetAttribute(coarse_batch_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)kCoarseSmemMax);
+    });
+    if (e != cudaSuccess) return e;
+    coarse_batch_kernel<T><<<n, kCoarseThreads, smem, s>>>(jobs);
+    count_launch();
+    return cudaGetLastError();
 }
 
 template <typename T>
@@ -834,11 +1053,11 @@ cudaError_t launch_coarse(int mode, const Plan *P, const LevelGeom<T> *geo, int 
 {
     if (ls < 1 || ls > kCoarseMaxLevels) return cudaErrorInvalidValue;
     size_t sm = 0;
-    const CoarseArgs<T> a = coarse_args<T>(P, geo, ls, v_in, v_out, qo, coef_out, symin, coef_in, &sm);
+    const CoarseArgs<T> a = coarse_args<T>(mode, P, geo, ls, v_in, v_out, qo, coef_out, symin, coef_in, &sm);
     static PerDeviceOnce attr[4];
     auto go = [&](auto kern) -> cudaError_t {
         cudaError_t e = once_per_device(attr[mode], [&] {
-            return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCoarseSmem);
+            return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCoarseSmemMax);
         });
         if (e != cudaSuccess) return e;
         kern<<<1, kCoarseThreads, sm, s>>>(a);
@@ -866,9 +1085,9 @@ cudaError_t launch_coarse(int mode, const Plan *P, const LevelGeom<T> *geo, int 
     template int coarse_top<T>(const Plan *, const LevelGeom<T> *);                              \
     template cudaError_t launch_coarse<T>(int, const Plan *, const LevelGeom<T> *, int, const T *, T *, \
                                           const QuantOut &, T *, const SymIn &, const T *, cudaStream_t); \
-    template CoarseArgs<T> coarse_args<T>(const Plan *, const LevelGeom<T> *, int, const T *, T *,         \
+    template CoarseArgs<T> coarse_args<T>(int, const Plan *, const LevelGeom<T> *, int, const T *, T *,         \
                                           const QuantOut &, T *, const SymIn &, const T *, size_t *);      \
-    template cudaError_t launch_coarse_batch<T>(int, const CoarseArgs<T> *, int, size_t, cudaStream_t);
+    template cudaError_t launch_coarse_batch<T>(const CoarseArgs<T> *, int, size_t, cudaStream_t);
 INST(float)
 INST(double)
 

@@ -117,7 +117,8 @@ int norm_parts();
 // mode 0: compression (v_in -> symbols), 1: decomposition (v_in -> coef_out),
 // 2: decompression (symbols -> v_out), 3: recomposition (coef_in -> v_out).
 constexpr int kCoarseMaxLevels = 16;
-constexpr size_t kCoarseSmem = 200 * 1024;
+constexpr size_t kCoarseSmem = 200 * 1024;      // working arrays (fixes ls)
+constexpr size_t kCoarseSmemMax = 220 * 1024;   // with the staged tables and stream
 template <typename T>
 int coarse_top(const Plan *P, const LevelGeom<T> *geo);
 template <typename T>
@@ -131,18 +132,23 @@ struct CoarseArgs {
     T *coef_out;         // decomposition
     SymIn symin;         // decompression
     const T *coef_in;    // recomposition
+    // past the working arrays: element offsets of the staged tables (staged) and
+    // of the staged stream prefix (-1: read in global memory)
+    bool staged;
+    int stream_off;
+    int tab_off[kCoarseMaxLevels + 1][3];
 };
 template <typename T>
 cudaError_t launch_coarse(int mode, const Plan *P, const LevelGeom<T> *geo, int ls, const T *v_in, T *v_out,
                           const QuantOut &qo, T *coef_out, const SymIn &symin, const T *coef_in, cudaStream_t s);
 // the arguments of that launch (host), and its dynamic shared memory
 template <typename T>
-CoarseArgs<T> coarse_args(const Plan *P, const LevelGeom<T> *geo, int ls, const T *v_in, T *v_out,
+CoarseArgs<T> coarse_args(int mode, const Plan *P, const LevelGeom<T> *geo, int ls, const T *v_in, T *v_out,
                           const QuantOut &qo, T *coef_out, const SymIn &symin, const T *coef_in, size_t *smem);
-// the coarse levels of n fields in one launch (one block per field; jobs:
+// the coarse levels of n compressions in one launch (one block per field; jobs:
 // device [n]; smem: the largest of the fields' shared-memory sizes)
 template <typename T>
-cudaError_t launch_coarse_batch(int mode, const CoarseArgs<T> *jobs, int n, size_t smem, cudaStream_t s);
+cudaError_t launch_coarse_batch(const CoarseArgs<T> *jobs, int n, size_t smem, cudaStream_t s);
 
 // adjoint.cu: transposes of recomposition / decomposition over all levels.
 // ga, gb, y, R hold N_{L-1} elements; t1, t2 the partial prolongations

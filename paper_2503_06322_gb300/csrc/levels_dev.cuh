@@ -13,13 +13,17 @@ namespace {
 // whatever the data type, so that codes agree with a binary64 decision on
 // the same coefficients everywhere but at half-bin ties.  Codes whose
 // magnitude reaches 2^62 are clamped there (the escape store then flags them).
+//
+// Binary64 issue is slow on this part, so only the product, the sum and one
+// more addition use it: t >= 0, so its range is read off its high word, and
+// adding 2^52 rounded down leaves floor(t) in the low word.
 template <typename T>
 __device__ __forceinline__ long long quant_code(T x, double rho)
 {
-    const double ax = x < (T)0 ? -(double)x : (double)x;
+    const double ax = fabs((double)x);
     const double t = __dadd_rn(__dmul_rn(ax, rho), 0.5);
     long long k;
-    if (t < 1073741824.0) k = (long long)(int)floor(t);
+    if (__double2hiint(t) < 0x41D00000) k = __double2loint(__dadd_rd(t, 4503599627370496.0));   // t < 2^30
     else if (t < 4611686018427387904.0) k = (long long)floor(t);
     else k = kEscMax;
     return x < (T)0 ? -k : k;
@@ -131,6 +135,41 @@ __device__ __forceinline__ void quant_emit(const QuantOut &qo, unsigned int *hs,
     qo.sym[si] = (uint16_t)sym;
     if (smem_hist) atomicAdd(&hs[sym], 1u);
     else atomicAdd(&qo.hist[sym], 1ULL);
+}
+
+// The binary64 decision of a binary32 coefficient without binary64 arithmetic
+// almost everywhere: the double-word product of quant_small_f32 leaves
+// ax rho - n within 2^-24 of r = d + e2 (p < 2^22), so away from the decision
+// points +-1/2 by 2^-16 the code is the one that quant_code gives; closer, and
+// for codes of 2^22 and more, quant_code decides (one coefficient in 2^15).
+__device__ __noinline__ long long quant_code_call(float x, double rho) { return quant_code(x, rho); }
+__device__ __forceinline__ long long quant_exact(float x, double rho, float rho_hi, float rho_lo)
+{
+    const float ax = fabsf(x);
+    const float p = __fmul_rn(ax, rho_hi);
+    const float e2 = __fmaf_rn(ax, rho_lo, __fmaf_rn(ax, rho_hi, -p));
+    const float n = rintf(p);
+    const float r = __fadd_rn(__fsub_rn(p, n), e2);
+    if (p < kSmallQuant && fabsf(fabsf(r) - 0.5f) > 1.52587890625e-5f) {
+        const int k = __float2int_rn(n) + (r >= 0.5f ? 1 : 0) - (r < -0.5f ? 1 : 0);
+        return x < 0.0f ? -k : k;
+    }
+    return quant_code_call(x, rho);
+}
+__device__ __forceinline__ long long quant_exact(double x, double rho, float, float) { return quant_code(x, rho); }
+
+// one coefficient into the symbol stream, the global histogram and the escapes
+template <typename T>
+__device__ __forceinline__ void quant_emit_exact(const QuantOut &qo, long long si, T w, double rho, float rho_hi,
+                                                 float rho_lo)
+{
+    const long long k = quant_exact(w, rho, rho_hi, rho_lo);
+    const long long s = k + (long long)(qo.D / 2);
+    unsigned int sym = 0;
+    if (s >= 1 && s <= (long long)qo.D - 1) sym = (unsigned int)s;
+    else atomicMax(&qo.sc->esc_w, escape_store(qo, si, k));
+    qo.sym[si] = (uint16_t)sym;
+    atomicAdd(&qo.hist[sym], 1ULL);
 }
 
 template <typename T>
