@@ -243,11 +243,11 @@ enum : int { kPhLevels = 1, kPhCoarse = 2, kPhCodebook = 4, kPhEncode = 8, kPhHe
 
 // the whole compression of one field (or the selected phases of it),
 // enqueued on s without any host wait; the container size and status stay
-// in w.sc (device)
+// in w.sc (device), and in the device pair size_status where the caller gives one
 template <typename T>
 hpdr_status compress_core(hpdr_ctx *ctx, const Plan *P, const T *u, int ndim, const size_t *dims, double tol,
                           int tol_kind, int mode, unsigned D, unsigned K, uint8_t *out, size_t cap, const Ws &w,
-                          cudaStream_t s, int phases = kPhAll)
+                          cudaStream_t s, int phases = kPhAll, unsigned long long *size_status = nullptr)
 {
     const int L = P->L;
     const long long N = P->N[L];
@@ -329,7 +329,7 @@ hpdr_status compress_core(hpdr_ctx *ctx, const Plan *P, const T *u, int ndim, co
     EncodeArgs ea;
     memset(&ea, 0, sizeof(ea));
     ea.sym = w.sym; ea.N = (unsigned long long)N; ea.D = D; ea.K = K;
-    ea.len = hs.len; ea.code = hs.code;
+    ea.len = hs.len; ea.code = hs.code; ea.pack = hs.pack;
     ea.esc = w.esc;
     ea.chunk_bits = w.chunk_bits; ea.sc = w.sc;
     ea.bsum = w.bsum;
@@ -340,17 +340,14 @@ hpdr_status compress_core(hpdr_ctx *ctx, const Plan *P, const T *u, int ndim, co
         CK(launch_encode(ea, s));
     }
     if (!(phases & kPhHeader)) return HPDR_OK;
-    const HeaderArgs h = header_args<T>(P, ndim, dims, tol, tol_kind, mode, D, K, w);
-    CK(launch_header(h, hs.len, w.sc, out, s));
+    HeaderJob hj;
+    hj.h = header_args<T>(P, ndim, dims, tol, tol_kind, mode, D, K, w);
+    hj.len = hs.len;
+    hj.sc = w.sc;
+    hj.out = out;
+    hj.size_status = size_status;
+    CK(launch_header(hj, s));
     return HPDR_OK;
-}
-
-// container size and device status of one compression, for callers that
-// do not wait for it
-__global__ void size_status_kernel(const Scalars *sc, unsigned long long *dst)
-{
-    dst[0] = sc->out_bytes;
-    dst[1] = sc->status;
 }
 
 // h_size_status == null: synchronize and return the size in *out_bytes;
@@ -368,12 +365,10 @@ hpdr_status compress_t(hpdr_ctx *ctx, const Plan *P, const T *u, int ndim, const
     hpdr_status st = ensure_workspace(ctx, need);
     if (st != HPDR_OK) return st;
     carve_ws(ctx->ws.base, P, sizeof(T), D, K, true, &w);
-    st = compress_core<T>(ctx, P, u, ndim, dims, tol, tol_kind, mode, D, K, out, cap, w, s);
+    st = compress_core<T>(ctx, P, u, ndim, dims, tol, tol_kind, mode, D, K, out, cap, w, s, kPhAll,
+                          h_size_status ? d_pair : nullptr);
     if (st != HPDR_OK) return st;
     if (h_size_status) {
-        size_status_kernel<<<1, 1, 0, s>>>(w.sc, d_pair);
-        count_launch();
-        CK(cudaGetLastError());
         CK(cudaMemcpyAsync(h_size_status, d_pair, 2 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
         return HPDR_OK;
     }
@@ -459,31 +454,6 @@ hpdr_status parse_header(const uint8_t *b, size_t avail, size_t in_bytes, Hdr *h
     return HPDR_OK;
 }
 
-// the decoder-side scalars of one container, set on the device from the
-// launch parameters (no host staging buffer, so calls need not wait)
-struct ScalarInit {
-    double q[kMaxLevels + 1];
-    int L;
-    unsigned long long n_esc, total_bits;
-};
-__global__ void init_scalars_kernel(Scalars *sc, ScalarInit si)
-{
-    unsigned char *b = reinterpret_cast<unsigned char *>(sc);
-    for (unsigned i = threadIdx.x; i < sizeof(Scalars); i += blockDim.x) b[i] = 0;
-    __syncthreads();
-    for (int l = threadIdx.x; l <= si.L; l += blockDim.x) {
-        sc->q[l] = si.q[l];
-        sc->q_f[l] = __double2float_rn(si.q[l]);
-        sc->rho_d[l] = 1.0 / si.q[l];
-        sc->rho_f[l] = __double2float_rn(1.0 / si.q[l]);
-        sc->rho_lo[l] = __double2float_rn(sc->rho_d[l] - (double)sc->rho_f[l]);
-    }
-    if (threadIdx.x == 0) {
-        sc->n_esc = si.n_esc;
-        sc->total_bits = si.total_bits;
-    }
-}
-
 // status of one decompression OR-ed into an accumulated word
 __global__ void accumulate_status_kernel(const Scalars *sc, unsigned *acc)
 {
@@ -557,22 +527,21 @@ hpdr_status decompress_t(hpdr_ctx *ctx, const Plan *P, const Hdr &h, const uint8
     carve_ws(ctx->ws.base, P, sizeof(T), h.D, h.K, true, &w);
     const int L = P->L;
     Scalars *hsc = (Scalars *)ctx->host_pinned;
-    {
-        ScalarInit si;
-        memset(&si, 0, sizeof(si));
-        for (int l = 0; l <= L; l++) si.q[l] = h.q[l];
-        si.L = L;
-        si.n_esc = h.n_esc;
-        si.total_bits = h.bits;
-        init_scalars_kernel<<<1, 256, 0, s>>>(w.sc, si);
-        count_launch();
-        CK(cudaGetLastError());
-    }
     HuffScratch hs;
     huff_scratch_carve(w.huff, h.D, w.sc, &hs);
     {
+    // the decoder-side scalars come with the launch parameters (no host staging
+    // buffer, so calls need not wait)
     ProfScope ps(ctx, "d_tables", s);
-    CK(launch_decode_tables(in + h.off_len, h.s_lo, h.s_hi, h.D, hs, s));
+    TabArgs ta;
+    ta.lenb = in + h.off_len; ta.s_lo = h.s_lo; ta.s_hi = h.s_hi; ta.D = h.D;
+    ta.sc = w.sc;
+    ta.set_scalars = true;
+    for (int l = 0; l <= L; l++) ta.si.q[l] = h.q[l];
+    ta.si.L = L;
+    ta.si.n_esc = h.n_esc;
+    ta.si.total_bits = h.bits;
+    CK(launch_decode_tables(ta, hs, s));
     }
     DecodeArgs da;
     da.words = (const uint32_t *)(in + h.off_bits);
@@ -598,91 +567,6 @@ hpdr_status decompress_t(hpdr_ctx *ctx, const Plan *P, const Hdr &h, const uint8
     return HPDR_OK;
 }
 
-// ----- container header parsed on the device ---------------------------------
-// The checks of parse_header, plus agreement with the shape, type and
-// dictionary the caller expects; a failure sets DS_FORMAT, and every later
-// kernel of the decompression skips or computes on stale (in-bounds) data.
-struct HdrExpect {
-    int dtype, ndim, L;
-    unsigned long long dims[3], N;
-    unsigned D, K;
-};
-
-__device__ uint32_t crc32_dev(const uint8_t *p, int n)
-{
-    uint32_t c = 0xFFFFFFFFu;
-    for (int i = 0; i < n; i++) {
-        c ^= p[i];
-        for (int b = 0; b < 8; b++) c = (c >> 1) ^ (0xEDB88320u & (0u - (c & 1u)));
-    }
-    return c ^ 0xFFFFFFFFu;
-}
-__device__ uint32_t rd32d(const uint8_t *p) { uint32_t v = 0; for (int i = 0; i < 4; i++) v |= (uint32_t)p[i] << (8 * i); return v; }
-__device__ uint64_t rd64d(const uint8_t *p) { uint64_t v = 0; for (int i = 0; i < 8; i++) v |= (uint64_t)p[i] << (8 * i); return v; }
-__device__ unsigned long long a16d(unsigned long long x) { return (x + 15) & ~15ULL; }
-
-__global__ void hdr_parse_kernel(const uint8_t *b, unsigned long long in_bytes, HdrExpect ex, DevHdr *dh, Scalars *sc)
-{
-    unsigned char *z = reinterpret_cast<unsigned char *>(sc);
-    for (unsigned i = threadIdx.x; i < sizeof(Scalars); i += blockDim.x) z[i] = 0;
-    __shared__ int ok;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        bool g = in_bytes >= 128;
-        if (g) g = b[0] == 'H' && b[1] == 'P' && b[2] == 'D' && b[3] == 'R' && rd32d(b + 4) == 3u;
-        if (g) g = crc32_dev(b, 124) == rd32d(b + 124);
-        DevHdr h;
-        h.pad = 0;
-        if (g) {
-            g = (int)rd32d(b + 8) == ex.dtype && (int)rd32d(b + 12) == ex.ndim && (int)rd32d(b + 40) == ex.L &&
-                rd32d(b + 48) <= 1u && rd32d(b + 52) == ex.D && rd32d(b + 56) == ex.K && rd64d(b + 96) == ex.N;
-            for (int k = 0; k < 3; k++) g = g && rd64d(b + 16 + 8 * k) == ex.dims[k];
-        }
-        if (g) {
-            h.s_lo = rd32d(b + 60);
-            h.n_esc = rd64d(b + 104);
-            h.total_bits = rd64d(b + 112);
-            const uint32_t w120 = rd32d(b + 120);
-            h.s_hi = w120 & 0xFFFFu;
-            h.esc_w = (w120 >> 16) & 0xFFu;
-            g = (w120 >> 24) == 0u && h.s_hi < ex.D && h.s_lo <= h.s_hi && h.n_esc <= ex.N && h.esc_w <= 63u &&
-                ((h.n_esc > 0) == (h.esc_w > 0)) && h.total_bits >= ex.N &&
-                h.total_bits <= 63ULL * ex.N + (unsigned long long)h.esc_w * h.n_esc;
-        }
-        if (g) {
-            const unsigned long long nch = (ex.N + ex.K - 1) / ex.K;
-            h.nwords = (h.total_bits + 31) / 32;
-            h.off_len = a16d(128 + 8ULL * (ex.L + 1));
-            h.off_chunk = a16d(h.off_len + (h.s_hi - h.s_lo + 1));
-            h.off_bits = a16d(h.off_chunk + 8 * nch);
-            g = h.off_bits + 4 * h.nwords <= in_bytes;
-        }
-        if (g)
-            for (int l = 0; l <= ex.L; l++) {
-                const double q = __longlong_as_double((long long)rd64d(b + 128 + 8 * l));
-                if (!(q > 0.0) || !isfinite(q)) g = false;
-            }
-        if (g) {
-            *dh = h;
-            sc->n_esc = h.n_esc;
-            sc->total_bits = h.total_bits;
-        } else {
-            sc->status = (unsigned)DS_FORMAT;
-        }
-        ok = g ? 1 : 0;
-    }
-    __syncthreads();
-    if (!ok) return;
-    for (int l = threadIdx.x; l <= ex.L; l += blockDim.x) {
-        const double q = __longlong_as_double((long long)rd64d(b + 128 + 8 * l));
-        sc->q[l] = q;
-        sc->q_f[l] = __double2float_rn(q);
-        sc->rho_d[l] = 1.0 / q;
-        sc->rho_f[l] = __double2float_rn(1.0 / q);
-        sc->rho_lo[l] = __double2float_rn(sc->rho_d[l] - (double)sc->rho_f[l]);
-    }
-}
-
 // {status} of one call into a device word
 __global__ void status_out_kernel(const Scalars *sc, unsigned long long *dst) { dst[0] = sc->status; }
 
@@ -698,8 +582,13 @@ hpdr_status decompress_dev(hpdr_ctx *ctx, const Plan *P, int dtype, int ndim, co
     hpdr_status st = ensure_workspace(ctx, need);
     if (st != HPDR_OK) return st;
     carve_ws(ctx->ws.base, P, sizeof(T), D, K, true, &w);
-    HdrExpect ex;
-    memset(&ex, 0, sizeof(ex));
+    HuffScratch hs;
+    huff_scratch_carve(w.huff, D, w.sc, &hs);
+    TabArgs ta;
+    ta.D = D;
+    ta.sc = w.sc;
+    ta.base = in; ta.in_bytes = in_bytes; ta.dh = w.dh;
+    HdrExpect &ex = ta.ex;
     ex.dtype = dtype;
     ex.ndim = ndim;
     ex.L = P->L;
@@ -707,14 +596,9 @@ hpdr_status decompress_dev(hpdr_ctx *ctx, const Plan *P, int dtype, int ndim, co
     ex.N = (unsigned long long)P->N[P->L];
     ex.D = D;
     ex.K = K;
-    hdr_parse_kernel<<<1, 256, 0, s>>>(in, in_bytes, ex, w.dh, w.sc);
-    count_launch();
-    CK(cudaGetLastError());
-    HuffScratch hs;
-    huff_scratch_carve(w.huff, D, w.sc, &hs);
     {
     ProfScope ps(ctx, "d_tables", s);
-    CK(launch_decode_tables_dev(in, w.dh, D, hs, s));
+    CK(launch_decode_tables(ta, hs, s));
     }
     DecodeArgs da;
     da.words = nullptr; da.nwords = 0; da.chunk = nullptr; da.total_bits = 0; da.esc_w = 0;
@@ -1399,15 +1283,11 @@ hpdr_status hpdr_compress_async(hpdr_ctx *ctx, const void *d_in, hpdr_dtype dtyp
     carve_ws(ctx->ws.base, P, dtype == HPDR_F64 ? 8 : 4, D, K, true, &w);
     if (dtype == HPDR_F32)
         st = compress_core<float>(ctx, P, (const float *)d_in, ndim, dims, tol, tol_kind, mode, D, K,
-                                  (uint8_t *)d_out, out_capacity, w, s);
+                                  (uint8_t *)d_out, out_capacity, w, s, kPhAll, (unsigned long long *)d_result);
     else
         st = compress_core<double>(ctx, P, (const double *)d_in, ndim, dims, tol, tol_kind, mode, D, K,
-                                   (uint8_t *)d_out, out_capacity, w, s);
-    if (st != HPDR_OK) return st;
-    size_status_kernel<<<1, 1, 0, s>>>(w.sc, (unsigned long long *)d_result);
-    count_launch();
-    CK(cudaGetLastError());
-    return HPDR_OK;
+                                   (uint8_t *)d_out, out_capacity, w, s, kPhAll, (unsigned long long *)d_result);
+    return st;
 }
 
 hpdr_status hpdr_device_status(uint64_t code) { return map_device_status((unsigned)code); }
@@ -1506,7 +1386,7 @@ hpdr_status hpdr_huffman_encode(hpdr_ctx *ctx, const uint16_t *d_symbols, uint64
     CK(launch_codebook(hist, D, hs, s));
     EncodeArgs ea;
     memset(&ea, 0, sizeof(ea));
-    ea.sym = d_symbols; ea.N = N; ea.D = D; ea.K = K; ea.len = hs.len; ea.code = hs.code;
+    ea.sym = d_symbols; ea.N = N; ea.D = D; ea.K = K; ea.len = hs.len; ea.code = hs.code; ea.pack = hs.pack;
     ea.chunk_bits = cb; ea.sc = sc; ea.bsum = bs;
     ea.chunk_out = (unsigned long long *)d_chunk_bits;
     ea.words_out = d_words;
@@ -1585,7 +1465,7 @@ hpdr_status hpdr_lossless_compress(hpdr_ctx *ctx, const void *d_keys, uint64_t n
     CK(launch_codebook(hist, D, hs, s));
     EncodeArgs ea;
     memset(&ea, 0, sizeof(ea));
-    ea.sym = sym; ea.N = n; ea.D = D; ea.K = h.K; ea.len = hs.len; ea.code = hs.code;
+    ea.sym = sym; ea.N = n; ea.D = D; ea.K = h.K; ea.len = hs.len; ea.code = hs.code; ea.pack = hs.pack;
     ea.chunk_bits = cb; ea.sc = sc; ea.bsum = bs;
     ea.chunk_out = (unsigned long long *)(out + h.off_chunk);
     ea.words_out = (uint32_t *)(out + h.off_bits);
@@ -1651,7 +1531,9 @@ hpdr_status hpdr_lossless_decompress(hpdr_ctx *ctx, const void *d_in, size_t in_
     CK(cudaMemsetAsync(sc, 0, sizeof(Scalars), s));
     HuffScratch hs;
     huff_scratch_carve(hsb, D, sc, &hs);
-    CK(launch_decode_tables(in + kLosslessHdr, 0, D - 1, D, hs, s));
+    TabArgs ta;
+    ta.lenb = in + kLosslessHdr; ta.s_hi = D - 1; ta.D = D;
+    CK(launch_decode_tables(ta, hs, s));
     DecodeArgs da;
     da.words = (const uint32_t *)(in + h.off_bits);
     da.nwords = (h.bits + 31) / 32;
@@ -1709,7 +1591,9 @@ hpdr_status hpdr_huffman_decode(hpdr_ctx *ctx, const uint32_t *d_words, uint64_t
     CK(cudaMemsetAsync(sc, 0, sizeof(Scalars), s));
     HuffScratch hs;
     huff_scratch_carve(hb, D, sc, &hs);
-    CK(launch_decode_tables(d_lengths, 0, D - 1, D, hs, s));
+    TabArgs ta;
+    ta.lenb = d_lengths; ta.s_hi = D - 1; ta.D = D;
+    CK(launch_decode_tables(ta, hs, s));
     DecodeArgs da;
     da.words = d_words; da.nwords = (total_bits + 31) / 32;
     da.chunk = (const unsigned long long *)d_chunk_bits;

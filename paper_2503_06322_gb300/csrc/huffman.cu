@@ -126,41 +126,96 @@ __device__ unsigned count_lt(const unsigned long long *a, unsigned n, unsigned l
     return lo;
 }
 
-__device__ void length_tables(const HuffScratch &hs, unsigned *cnt)
+// canonical length tables staged in shared memory
+struct LenTabs {
+    unsigned long long first[64], lim[64];
+    unsigned start[64], count[64];
+};
+
+// Canonical tables of every code length from the per-length counts cnt[64]
+// (shared memory), by one warp; returns whether the lengths are those of a
+// prefix code (the same answer in every lane).  With
+// S_L = sum_{j <= L} cnt_j 2^(63 - j), the share of the code space that the
+// codewords of at most L bits take (2^63 is all of it):
+//   first canonical code of length L     S_{L-1} >> (63 - L)
+//   left-justified limit of length <= L  2 S_L  (all ones once the space is full)
+// The sums saturate just above 2^63, so an over-full set of lengths is seen
+// whatever its counts; a serial recurrence over the 63 lengths took 2.5 us.
+constexpr unsigned long long kFullCode = 1ULL << 63;
+__device__ __forceinline__ unsigned long long sat_add(unsigned long long a, unsigned long long b)
 {
-    // first canonical code and start index of every length
-    unsigned long long c = 0;
-    int prev = -1;
-    unsigned st = 0;
-    bool ok = true;
-    for (int L = 1; L <= kMaxCodeLen; L++) {
-        hs.start[L] = st;
-        hs.count[L] = cnt[L];
-        if (cnt[L]) {
-            if (prev >= 0) c <<= (L - prev);
-            hs.first[L] = c;
-            c += cnt[L];
-            if (c > (1ULL << L)) ok = false;   // not a prefix code
-            prev = L;
-            st += cnt[L];
-        } else {
-            hs.first[L] = 0;
+    const unsigned long long c = a + b;
+    return (a > kFullCode || b > kFullCode || c > kFullCode || c < a) ? kFullCode + 1 : c;
+}
+__device__ __forceinline__ bool length_tables(LenTabs &T, const unsigned *cnt)
+{
+    const unsigned lane = threadIdx.x & 31;
+    unsigned long long scarry = 0;
+    unsigned ncarry = 0;
+#pragma unroll
+    for (int h = 0; h < 2; h++) {
+        const unsigned L = lane + 32u * h;
+        const unsigned c = L ? cnt[L] : 0u;
+        // more codewords of L bits than the space holds: over-full
+        const unsigned long long share = (unsigned long long)c > (1ULL << L) ? kFullCode + 1
+                                                                            : (unsigned long long)c << (63 - L);
+        unsigned long long S = share;
+        unsigned n = c;
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned long long y = __shfl_up_sync(0xffffffffu, S, o);
+            const unsigned z = __shfl_up_sync(0xffffffffu, n, o);
+            if ((int)lane >= o) { S = sat_add(S, y); n += z; }
+        }
+        S = sat_add(S, scarry);
+        n += ncarry;
+        unsigned long long before = __shfl_up_sync(0xffffffffu, S, 1);
+        if (lane == 0) before = scarry;
+        T.count[L] = c;
+        T.start[L] = n - c;
+        T.first[L] = c ? before >> (63 - L) : 0ULL;
+        T.lim[L] = L == 0 ? 0ULL : S >= kFullCode ? ~0ULL : S << 1;
+        scarry = __shfl_sync(0xffffffffu, S, 31);
+        ncarry = __shfl_sync(0xffffffffu, n, 31);
+    }
+    return scarry <= kFullCode;
+}
+// the tables into the scratch that the encoder and the decoder read
+__device__ __forceinline__ void store_tables(const HuffScratch &hs, const LenTabs &T, unsigned i)
+{
+    hs.first[i] = T.first[i];
+    hs.lim[i] = T.lim[i];
+    hs.start[i] = T.start[i];
+    hs.count[i] = T.count[i];
+}
+
+// CRC-32 (reflected, polynomial 0xEDB88320, all-ones start and final xor) of
+// the first 124 bytes of a 128-byte header, by one warp: lane j < 31 holds word
+// j.  The register is linear in the message, so word j adds w_j x^(32 (31 - j))
+// mod P (the all-ones start is an xor of the first word): one product of
+// polynomials per lane and a reduction, where the bitwise or byte-table
+// recurrence over 124 bytes is serial.
+struct CrcPowers {
+    uint32_t v[32];
+    constexpr CrcPowers() : v()
+    {
+        uint32_t x = 0x80000000u;   // 1: bit 31 is the constant term
+        for (int j = 31; j >= 0; j--) {
+            v[j] = x;               // x^(32 (31 - j))
+            for (int b = 0; b < 32; b++) x = (x >> 1) ^ ((x & 1u) ? 0xEDB88320u : 0u);
         }
     }
-    hs.count[0] = 0;
-    if (!ok) atomicExch(hs.status, (unsigned)DS_FORMAT);
-    // left-justified limit of the codes of length <= L: (first_L + count_L) << (64 - L),
-    // with first_L from the canonical recurrence for every L
-    unsigned long long f = 0;
-    bool started = false;
-    for (int L = 1; L <= kMaxCodeLen; L++) {
-        if (started) f <<= 1;
-        if (cnt[L] && !started) { started = true; f = 0; }
-        const unsigned long long nxt = f + cnt[L];
-        hs.lim[L] = (nxt >= (1ULL << L)) ? ~0ULL : (nxt << (64 - L));
-        f = nxt;
+};
+__constant__ CrcPowers kCrcPowers = CrcPowers();
+__device__ __forceinline__ uint32_t crc32_warp(uint32_t word)
+{
+    const unsigned lane = threadIdx.x & 31;
+    uint32_t a = lane == 0 ? ~word : word, b = kCrcPowers.v[lane], p = 0;
+#pragma unroll
+    for (int i = 31; i >= 0; i--) {
+        p ^= (a >> i) & 1u ? b : 0u;
+        b = (b >> 1) ^ ((b & 1u) ? 0xEDB88320u : 0u);
     }
-    hs.lim[0] = 0;
+    return ~__reduce_xor_sync(0xffffffffu, lane < 31 ? p : 0u);
 }
 
 // code lengths from the frequency-sorted leaves, one block
@@ -168,6 +223,7 @@ __global__ void __launch_bounds__(1024) merge_kernel(HuffScratch hs, unsigned D)
 {
     extern __shared__ unsigned long long sm[];
     __shared__ unsigned ia, ib, nb, ka, kb, cnt[kMaxCodeLen + 2];
+    __shared__ LenTabs T;
     __shared__ int done;
     const unsigned n = *hs.nsym;
     const unsigned tid = threadIdx.x;
@@ -181,8 +237,11 @@ __global__ void __launch_bounds__(1024) merge_kernel(HuffScratch hs, unsigned D)
             hs.len[s] = 1;
             hs.keys2[0] = (1ULL << 16) | s;
             cnt[1] = 1;
-            length_tables(hs, cnt);
         }
+        __syncthreads();
+        if (tid < 32) length_tables(T, cnt);
+        __syncthreads();
+        if (tid < 64) store_tables(hs, T, tid);
         return;
     }
     const bool insm = n <= (unsigned)kSmemKeys;
@@ -275,10 +334,21 @@ __global__ void __launch_bounds__(1024) merge_kernel(HuffScratch hs, unsigned D)
         atomicAdd(&cnt[L], 1u);
     }
     __syncthreads();
-    if (tid == 0) length_tables(hs, cnt);
+    if (tid < 32 && !length_tables(T, cnt) && tid == 0) atomicExch(hs.status, (unsigned)DS_FORMAT);
+    __syncthreads();
+    if (tid < 64) store_tables(hs, T, tid);
 }
 
-// canonical codeword of every present symbol and the (length, symbol) order
+// entry of the encoder's packed codeword table: code << 6 | length for
+// codewords of at most 26 bits (0: absent symbol); kPackLong sends the symbol
+// to the full tables
+constexpr uint32_t kPackLong = 0xFFFFFFFFu;
+__device__ __forceinline__ uint32_t pack_code(unsigned long long code, unsigned L)
+{
+    return L <= 26 ? (uint32_t)((code << 6) | L) : kPackLong;
+}
+
+// canonical codeword of every present symbol
 __global__ void __launch_bounds__(256) assign_kernel(HuffScratch hs)
 {
     const unsigned n = *hs.nsym;
@@ -287,7 +357,7 @@ __global__ void __launch_bounds__(256) assign_kernel(HuffScratch hs)
         unsigned s = (unsigned)(k & 0xFFFFu), L = (unsigned)(k >> 16);
         unsigned r = hs.rank[i];
         hs.code[s] = hs.first[L] + (r - hs.start[L]);
-        hs.sorted_sym[r] = (uint16_t)s;
+        hs.pack[s] = pack_code(hs.code[s], L);
     }
 }
 
@@ -305,12 +375,6 @@ constexpr uint32_t kSubFlag = 0x20000000u;
 // decoder copy of an entry of the escape symbol 0 whose codeword and payload
 // (W bits) together fit 32 bits: L = codeword length + W
 constexpr uint32_t kEscFolded = 0x40000000u;
-
-// canonical length tables staged in shared memory
-struct LenTabs {
-    unsigned long long first[64], lim[64];
-    unsigned start[64], count[64];
-};
 
 // length of the canonical codeword at the top of the left-aligned window,
 // known to lie in [lo, hi]: the first length l in [lo, hi) whose limit lim[l]
@@ -335,194 +399,109 @@ __device__ __forceinline__ uint32_t leaf_of(const LenTabs &t, const uint16_t *so
     return idx < n ? ((uint32_t)sorted_sym[idx] | (L << 16)) : 0u;
 }
 
-// One block of 1024 threads, eight consecutive prefixes each.  The
-// second-level tables are laid out in prefix order by a block scan of their
-// sizes; prefixes past the budget keep long entries.  The sorted symbols are
-// staged in shared memory when there are at most kLutSyms of them.
-constexpr int kLutThreads = 1024;
-constexpr unsigned kLutPer = (1u << kLutBits) / kLutThreads;
-constexpr unsigned kLutSyms = 16384;
-constexpr size_t kLutSmem = (4u << kLutBits) + 2 * kLutSyms;
-__global__ void __launch_bounds__(kLutThreads, 1) lut_kernel(HuffScratch hs)
-{
-    __shared__ LenTabs T;
-    __shared__ unsigned wsum[kLutThreads / 32];
-    __shared__ unsigned total;
-    extern __shared__ __align__(16) unsigned char lsm[];
-    uint32_t *ent = reinterpret_cast<uint32_t *>(lsm);                         // [1 << kLutBits]
-    uint16_t *ssym = reinterpret_cast<uint16_t *>(ent + (1u << kLutBits));      // [kLutSyms]
-    const unsigned tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    if (tid < 64) {
-        T.first[tid] = hs.first[tid];
-        T.lim[tid] = hs.lim[tid];
-        T.start[tid] = hs.start[tid];
-        T.count[tid] = hs.count[tid];
-    }
-    const unsigned n = *hs.nsym;
-    const uint16_t *sorted = n <= kLutSyms ? ssym : hs.sorted_sym;
-    if (n <= kLutSyms)
-        for (unsigned i = tid; i < n; i += kLutThreads) ssym[i] = hs.sorted_sym[i];
-    __syncthreads();
-    const bool ok = *hs.status == 0;
-    unsigned maxL = 0;
-    for (int l = kMaxCodeLen; l >= 1; l--) if (T.count[l]) { maxL = (unsigned)l; break; }
-    const bool any = ok && maxL;
-    const unsigned t0 = tid * kLutPer;
-    constexpr unsigned long long kTail = (1ULL << (64 - kLutBits)) - 1;
-    unsigned mine = 0;
-    unsigned char sbs[kLutPer];
-#pragma unroll
-    for (unsigned j = 0; j < kLutPer; j++) {
-        const unsigned t = t0 + j;
-        uint32_t e = 0;
-        sbs[j] = 0;
-        if (any) {
-            // the codeword whose left-justified range holds t's first bit string;
-            // at most P bits long, it is a prefix of every extension of t
-            const unsigned long long w0 = (unsigned long long)t << (64 - kLutBits);
-            const unsigned lmin = code_len_in(T, w0, 1, maxL);
-            if (lmin <= (unsigned)kLutBits) {
-                e = leaf_of(T, sorted, n, w0, lmin);
-            } else {
-                const unsigned lmax = code_len_in(T, w0 | kTail, lmin, maxL);
-                e = kLongFlag | (lmin << 16) | ((lmax - lmin) << 24);
-                if (lmax <= (unsigned)(kLutBits + kSubMax)) {
-                    sbs[j] = (unsigned char)(lmax - kLutBits);
-                    mine += 1u << (lmax - kLutBits);
-                }
-            }
-        }
-        ent[t] = e;
-    }
-    // exclusive scan of the second-level sizes over the block
-    unsigned incl = mine;
-    for (int o = 1; o < 32; o <<= 1) {
-        const unsigned v = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= (unsigned)o) incl += v;
-    }
-    if (lane == 31) wsum[warp] = incl;
-    __syncthreads();
-    if (warp == 0) {
-        const unsigned v = wsum[lane];
-        unsigned x = v;
-        for (int o = 1; o < 32; o <<= 1) {
-            const unsigned y = __shfl_up_sync(0xffffffffu, x, o);
-            if (lane >= (unsigned)o) x += y;
-        }
-        wsum[lane] = x - v;
-        if (lane == 31) total = x < kSubCap ? x : kSubCap;
-    }
-    __syncthreads();
-    unsigned off = wsum[warp] + incl - mine;
-#pragma unroll
-    for (unsigned j = 0; j < kLutPer; j++) {
-        if (!sbs[j]) continue;
-        const unsigned sz = 1u << sbs[j];
-        if (off + sz <= kSubCap) ent[t0 + j] = kSubFlag | off | ((unsigned)sbs[j] << 16);
-        off += sz;
-    }
-    __syncthreads();
-    for (unsigned t = tid; t < (1u << kLutBits); t += kLutThreads) hs.lut1[t] = ent[t];
-    // second-level entries: a warp per prefix, a lane per suffix
-    for (unsigned t = warp; t < (1u << kLutBits); t += kLutThreads / 32) {
-        const uint32_t e = ent[t];
-        if ((e & (kLongFlag | kSubFlag)) != kSubFlag) continue;
-        const unsigned sb = (e >> 16) & 0xFu, base = e & 0xFFFFu;
-        const unsigned long long w0 = (unsigned long long)t << (64 - kLutBits);
-        const unsigned lo = code_len_in(T, w0, 1, maxL);
-        for (unsigned r = lane; r < (1u << sb); r += 32) {
-            const unsigned long long w = w0 | ((unsigned long long)r << (64 - kLutBits - sb));
-            hs.lut_sub[base + r] = leaf_of(T, sorted, n, w, code_len_in(T, w, lo, kLutBits + sb));
-        }
-    }
-    if (tid == 0) *hs.nsub = any ? total : 0u;
-}
-
 // Canonical codewords (Sec. IV-B): the present symbols ordered by (length,
 // symbol) get consecutive codewords within each length, so a symbol's rank is
 // start[L] plus the number of smaller symbols of its length L, and its
-// codeword first[L] plus that number.  The block (1024 threads) walks the
-// alphabet in tiles of 1024 symbols: __match_any_sync groups a warp's lanes by
-// length, wc[warp][L] holds per-warp counts that are then scanned over the
-// warps of every length on top of the running totals of the earlier tiles.
+// codeword first[L] plus that number.  A block of 1024 threads: warp w owns a
+// contiguous run of symbols, wc[w][L] counts its symbols of length L (grouped
+// by __match_any_sync, 32 at a time), a scan over the warps turns the counts
+// into offsets within each length, and a second walk over the run ranks its
+// symbols: three block barriers for the whole alphabet.
 constexpr int kWcStride = 65;     // 64 lengths, padded against bank conflicts
-__device__ void canonical_assign(const uint8_t *lens, unsigned D, const unsigned *sstart,
-                                 const unsigned long long *sfirst, unsigned *wc, unsigned *run,
-                                 unsigned long long *code, uint16_t *sorted_sym)
+__device__ __forceinline__ unsigned canonical_run(unsigned D) { return ((D + 1023) / 1024) * 32; }
+
+// wc (zeroed) <- per-warp counts, then offsets within each length; cnt[64] <-
+// counts per length.  lens must be complete; ends with a block barrier.
+__device__ __forceinline__ void canonical_counts(const uint8_t *lens, unsigned D, unsigned *wc, unsigned *cnt)
 {
     const unsigned lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    for (unsigned i = threadIdx.x; i < 64; i += blockDim.x) run[i] = 0;
-    for (unsigned t0 = 0; t0 < D; t0 += 1024) {
-        for (unsigned i = threadIdx.x; i < 32 * kWcStride; i += blockDim.x) wc[i] = 0;
-        __syncthreads();
-        const unsigned s = t0 + threadIdx.x;
+    const unsigned run = canonical_run(D), r0 = w * run;
+    for (unsigned i = 0; i < run; i += 32) {
+        const unsigned s = r0 + i + lane;
+        const unsigned L = s < D ? lens[s] : 0u;
+        const unsigned m = __match_any_sync(0xffffffffu, L);
+        if (L && (m & ((1u << lane) - 1)) == 0) wc[w * kWcStride + L] += __popc(m);
+        __syncwarp();
+    }
+    __syncthreads();
+    for (unsigned L = w; L < 64; L += 32) {
+        const unsigned x = wc[lane * kWcStride + L];
+        unsigned y = x;
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned z = __shfl_up_sync(0xffffffffu, y, o);
+            if ((int)lane >= o) y += z;
+        }
+        wc[lane * kWcStride + L] = y - x;
+        if (lane == 31) cnt[L] = y;
+    }
+    __syncthreads();
+}
+// f(s, L, k): symbol s of length L is the k-th of its length (L = 0: absent)
+template <typename F>
+__device__ __forceinline__ void canonical_ranks(const uint8_t *lens, unsigned D, unsigned *wc, F f)
+{
+    const unsigned lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const unsigned run = canonical_run(D), r0 = w * run;
+    for (unsigned i = 0; i < run; i += 32) {
+        const unsigned s = r0 + i + lane;
         const unsigned L = s < D ? lens[s] : 0u;
         const unsigned m = __match_any_sync(0xffffffffu, L);
         const unsigned below = __popc(m & ((1u << lane) - 1));
-        if (below == 0) wc[w * kWcStride + L] = __popc(m);
-        __syncthreads();
-        for (unsigned Lq = w; Lq < 64; Lq += 32) {
-            const unsigned x = wc[lane * kWcStride + Lq];
-            unsigned y = x;
-            for (int o = 1; o < 32; o <<= 1) {
-                const unsigned z = __shfl_up_sync(0xffffffffu, y, o);
-                if ((int)lane >= o) y += z;
-            }
-            const unsigned base = run[Lq];
-            __syncwarp();
-            wc[lane * kWcStride + Lq] = base + y - x;
-            if (lane == 31) run[Lq] = base + y;
-        }
-        __syncthreads();
-        if (L) {
-            const unsigned k = wc[w * kWcStride + L] + below;
-            if (code) code[s] = sfirst[L] + k;
-            sorted_sym[sstart[L] + k] = (uint16_t)s;
-        }
-        __syncthreads();
+        if (s < D) f(s, L, L ? wc[w * kWcStride + L] + below : 0u);
+        __syncwarp();
+        if (L && below == 0) wc[w * kWcStride + L] += __popc(m);
+        __syncwarp();
     }
 }
 
 // ---------------------------------------------------------------------------
 // One-block codebook for alphabets of at most kFusedMaxD symbols, everything
 // in shared memory: present symbols, their (frequency, symbol) order, the
-// two-queue code lengths in rounds (as merge_kernel), depths by pointer
-// jumping, canonical codewords.  Rounds that pick at most kWarpRound nodes,
-// the common case once the smallest weights are merged, run on warp 0 alone
-// without block barriers.
+// two-queue code lengths in rounds (as merge_kernel), depths, canonical
+// codewords.  One block, so latency bounds it: 128 -> 58 us at 8000 present
+// symbols (513^3, 1e-3), 80 -> 27 us at 129^2.  What each part does about it (the
+// cycles are those of the form it replaced, of 250 thousand at 513^3):
+//   sort      radix sort of the frequencies, eight bits a pass and only as many
+//             passes as the largest frequency has bytes; stable, so equal
+//             frequencies stay in symbol order (merge-path rounds: 125k);
+//   rounds    pair t of a round finds its two nodes by one merge-path search
+//             and sums them (a rank search and a 64-bit shared atomic per
+//             node: 75k); limits by 32-way searches; rounds of at most kWarpRound nodes run on warp 0
+//             without block barriers;
+//   depths    from the root, round by round: a node's parent is always made in
+//             a later round (pointer jumping over all nodes: 28k).
 constexpr unsigned kFusedMaxD = 8192;
 constexpr unsigned kWarpRound = 64;
+// Rounds of one build: no node of weight below 2 w survives the two rounds
+// after one whose smallest weight is w, and weights are below 2^64.
+constexpr unsigned kMaxRounds = 136;
+constexpr unsigned kDigStride = 258;   // 256 digits of 16-bit counts, padded against bank conflicts
 constexpr size_t kCodebookSmem = 16ull * kFusedMaxD            // keys + sort buffer / internal weights
-                                 + 2ull * 2 * kFusedMaxD         // parent / ancestor
-                                 + 2ull * kFusedMaxD             // depth
+                                 + 2ull * 2 * kFusedMaxD         // parents (digit counts while sorting)
+                                 + kFusedMaxD                    // depths of the internal nodes
                                  + kFusedMaxD                    // lengths by symbol
                                  + 4ull * 32 * kWcStride;        // per-warp length counts
+static_assert(32 * kDigStride * 2 <= 4 * kFusedMaxD, "digit counts fit the parents' space");
 
 // number of the first rem sorted values v(i) that are <= thr (v non-decreasing),
-// by warp ballot over the first 32 and binary search beyond
+// by one warp: 32 probes a step
 template <typename F>
 __device__ __forceinline__ unsigned warp_count_le(F v, unsigned rem, unsigned long long thr, unsigned lane)
 {
-    const bool p = lane < rem && v(lane) <= thr;
-    const unsigned c = __popc(__ballot_sync(0xffffffffu, p));
+    unsigned lo = 0, len = rem;
+    // most counts are small: the first 32 values first
+    unsigned c = __popc(__ballot_sync(0xffffffffu, lane < rem && v(lane) <= thr));
     if (c < 32 || rem <= 32) return c;
-    unsigned lo = 32, hi = rem;
-    while (lo < hi) { const unsigned m = (lo + hi) >> 1; if (v(m) <= thr) lo = m + 1; else hi = m; }
-    return lo;
-}
-
-// sorted ascending 8 keys in registers (odd-even transposition, 8 rounds)
-__device__ __forceinline__ void sort8(unsigned long long (&k)[8])
-{
-#pragma unroll
-    for (int r = 0; r < 8; r++) {
-#pragma unroll
-        for (int i = r & 1; i + 1 < 8; i += 2) {
-            const unsigned long long a = k[i], b = k[i + 1];
-            k[i] = a < b ? a : b;
-            k[i + 1] = a < b ? b : a;
-        }
+    lo = 32;
+    len = rem - 32;
+    while (len > 32) {
+        const unsigned step = (len + 31) / 32, e = (lane + 1) * step;   // probe the last value of part `lane`
+        c = __popc(__ballot_sync(0xffffffffu, e <= len && v(lo + e - 1) <= thr));
+        lo += c * step;
+        len = min(step - 1, len - c * step);                             // the part's last value is > thr, or past the end
+        if (c == 32) return lo;
     }
+    return lo + __popc(__ballot_sync(0xffffffffu, lane < len && v(lo + lane) <= thr));
 }
 
 __device__ __forceinline__ void codebook_body(const unsigned long long *hist, unsigned D, const HuffScratch &hs)
@@ -531,116 +510,177 @@ __device__ __forceinline__ void codebook_body(const unsigned long long *hist, un
     unsigned long long *key = reinterpret_cast<unsigned long long *>(csm);   // [kFusedMaxD]
     unsigned long long *aux = key + kFusedMaxD;                              // [kFusedMaxD]
     uint16_t *par = reinterpret_cast<uint16_t *>(aux + kFusedMaxD);          // [2 kFusedMaxD]
-    uint16_t *dep = par + 2 * kFusedMaxD;                                    // [kFusedMaxD] as bytes x2
-    uint8_t *lens = reinterpret_cast<uint8_t *>(dep + kFusedMaxD);           // [kFusedMaxD]
+    uint8_t *dep = reinterpret_cast<uint8_t *>(par + 2 * kFusedMaxD);        // [kFusedMaxD]
+    uint8_t *lens = dep + kFusedMaxD;                                        // [kFusedMaxD]
     unsigned *wc = reinterpret_cast<unsigned *>(lens + kFusedMaxD);          // [32 * kWcStride]
-    uint8_t *depb = reinterpret_cast<uint8_t *>(dep);                        // [2 kFusedMaxD]
-    __shared__ unsigned wcnt[32], wpre[32], cnt[64], run[64], sstart[64];
-    __shared__ unsigned long long sfirst[64];
-    __shared__ unsigned sh_n, sh_lo, sh_hi, s_ia, s_ib, s_nb, s_a, s_b;
+    __shared__ unsigned wcnt[32], wlo[32], whi[32], cnt[64], dbase[256];
+    __shared__ unsigned long long wor[32];
+    __shared__ LenTabs T;
+    __shared__ unsigned s_ia, s_ib, s_nb, s_a, s_b, s_rounds;
     __shared__ int s_done;
+    __shared__ uint16_t rstart[kMaxRounds];
     const unsigned tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     const unsigned long long INF = ~0ULL;
+    constexpr unsigned R = kFusedMaxD / 1024;   // symbols per thread
 
-    // 1. present symbols as keys (frequency << 16) | s, in symbol order
-    if (tid == 0) { sh_n = 0; sh_lo = 0xFFFFFFFFu; sh_hi = 0; }
-    for (unsigned i = tid; i < 64; i += blockDim.x) cnt[i] = 0;
-    for (unsigned i = tid; i < D; i += blockDim.x) lens[i] = 0;
-    __syncthreads();
-    for (unsigned t0 = 0; t0 < D; t0 += 1024) {
-        const unsigned s = t0 + tid;
-        const unsigned long long f = s < D ? hist[s] : 0ULL;
-        const bool p = f != 0;
-        const unsigned ball = __ballot_sync(0xffffffffu, p);
-        if (lane == 0) wcnt[w] = __popc(ball);
-        __syncthreads();
-        if (w == 0) {
-            const unsigned v = wcnt[lane];
-            unsigned x = v;
-            for (int o = 1; o < 32; o <<= 1) {
-                const unsigned y = __shfl_up_sync(0xffffffffu, x, o);
-                if ((int)lane >= o) x += y;
+    // 1. present symbols as keys (frequency << 16) | s, in symbol order: warp w
+    //    compacts its run of 32 R symbols
+    unsigned n;
+    unsigned long long orf;
+    {
+        unsigned long long f[R];
+        unsigned before[R], mycnt = 0;
+        const unsigned r0 = w * 32 * R;
+#pragma unroll
+        for (unsigned i = 0; i < R; i++) f[i] = r0 + 32 * i + lane < D ? hist[r0 + 32 * i + lane] : 0ULL;
+        for (unsigned i = tid; i < 32 * kWcStride; i += 1024) wc[i] = 0;
+        for (unsigned i = tid; i < (D + 3) / 4; i += 1024) reinterpret_cast<uint32_t *>(lens)[i] = 0;
+        unsigned lo = 0xFFFFFFFFu, hi = 0;
+        unsigned long long o = 0;
+#pragma unroll
+        for (unsigned i = 0; i < R; i++) {
+            const unsigned ball = __ballot_sync(0xffffffffu, f[i] != 0);
+            before[i] = mycnt + __popc(ball & ((1u << lane) - 1));
+            mycnt += __popc(ball);
+            if (ball) {
+                lo = min(lo, r0 + 32 * i + __ffs(ball) - 1);
+                hi = r0 + 32 * i + 31 - __clz(ball);
             }
-            wpre[lane] = x - v;
+            o |= f[i];
         }
+        const unsigned ol = __reduce_or_sync(0xffffffffu, (unsigned)o), oh = __reduce_or_sync(0xffffffffu, (unsigned)(o >> 32));
+        if (lane == 0) { wcnt[w] = mycnt; wlo[w] = lo; whi[w] = hi; wor[w] = ((unsigned long long)oh << 32) | ol; }
         __syncthreads();
-        if (p) {
-            key[sh_n + wpre[w] + __popc(ball & ((1u << lane) - 1))] = (f << 16) | s;
-            atomicMin(&sh_lo, s);
-            atomicMax(&sh_hi, s);
+        // every warp scans the warps' counts
+        const unsigned c = wcnt[lane];
+        unsigned x = c;
+        for (int d = 1; d < 32; d <<= 1) {
+            const unsigned y = __shfl_up_sync(0xffffffffu, x, d);
+            if ((int)lane >= d) x += y;
         }
-        __syncthreads();
-        if (tid == 0) sh_n += wpre[31] + wcnt[31];
-        __syncthreads();
+        const unsigned base = __shfl_sync(0xffffffffu, x - c, w);
+        n = __shfl_sync(0xffffffffu, x, 31);
+        const unsigned long long wo = wor[lane];
+        orf = ((unsigned long long)__reduce_or_sync(0xffffffffu, (unsigned)(wo >> 32)) << 32) |
+              __reduce_or_sync(0xffffffffu, (unsigned)wo);
+        if (w == 0) {
+            const unsigned l0 = __reduce_min_sync(0xffffffffu, wlo[lane]), h0 = __reduce_max_sync(0xffffffffu, whi[lane]);
+            if (lane == 0) {
+                *hs.nsym = n;
+                *hs.s_lo = n ? l0 : 0;
+                *hs.s_hi = n ? h0 : 0;
+            }
+        }
+#pragma unroll
+        for (unsigned i = 0; i < R; i++)
+            if (f[i]) key[base + before[i]] = (f[i] << 16) | (r0 + 32 * i + lane);
     }
-    const unsigned n = sh_n;
-    if (tid == 0) {
-        *hs.nsym = n;
-        *hs.s_lo = n ? sh_lo : 0;
-        *hs.s_hi = n ? sh_hi : 0;
-    }
+    __syncthreads();
     if (n == 0) {
-        for (unsigned i = tid; i < D; i += blockDim.x) hs.len[i] = 0;
+        for (unsigned i = tid; i < D; i += 1024) { hs.len[i] = 0; hs.pack[i] = 0; }
         return;
     }
 
-    // 2. sort the keys (unique) ascending: runs of 8 in registers, then
-    //    merge-path rounds in shared memory
-    unsigned P = 8;
-    while (P < n) P <<= 1;
-    unsigned rounds = 0;
-    for (unsigned r = 8; r < P; r <<= 1) rounds++;
+    // 2. radix sort by frequency: warp w ranks its contiguous run of keys
+    unsigned long long *src = key, *dst = aux;
     {
-        unsigned long long *dst = (rounds & 1) ? aux : key;
-        unsigned long long k8[8];
-        const bool act = tid * 8 < P;
-        if (act) {
+        uint16_t *dc = par;   // [32][kDigStride] digit counts of every warp
+        const unsigned per = ((n + 1023) / 1024) * 32, p0 = w * per;
+        uint16_t *mine = dc + w * kDigStride;
+        for (unsigned shift = 16; shift == 16 || (shift < 64 && (orf >> (shift - 16)) != 0); shift += 8) {
+            for (unsigned i = lane; i < kDigStride / 2; i += 32) reinterpret_cast<uint32_t *>(mine)[i] = 0;
+            __syncwarp();
+            unsigned long long k[R];
+            unsigned rk[R];
 #pragma unroll
-            for (int i = 0; i < 8; i++) k8[i] = (tid * 8 + i < n) ? key[tid * 8 + i] : INF;
-            sort8(k8);
-        }
-        __syncthreads();
-        if (act) {
+            for (unsigned i = 0; i < R; i++) {
+                const unsigned p = p0 + 32 * i + lane;
+                k[i] = 32 * i < per && p < n ? src[p] : INF;
+            }
 #pragma unroll
-            for (int i = 0; i < 8; i++) dst[tid * 8 + i] = k8[i];
-        }
-        __syncthreads();
-        unsigned long long *src = dst;
-        for (unsigned R = 8; R < P; R <<= 1) {
-            dst = (src == key) ? aux : key;
-            if (act) {
-                const unsigned o = tid * 8, pair = o / (2 * R), d = o % (2 * R);
-                const unsigned long long *A = src + pair * 2 * R, *B = A + R;
-                unsigned lo = d > R ? d - R : 0, hi = d < R ? d : R;
-                while (lo < hi) {
-                    const unsigned m = (lo + hi) >> 1;
-                    if (A[m] <= B[d - m - 1]) lo = m + 1; else hi = m;
+            for (unsigned i = 0; i < R; i++) {
+                if (32 * i >= per) break;
+                const bool in = p0 + 32 * i + lane < n;
+                const unsigned d = in ? (unsigned)(k[i] >> shift) & 0xFFu : 0x100u;
+                const unsigned m = __match_any_sync(0xffffffffu, d);
+                const unsigned below = __popc(m & ((1u << lane) - 1)), at = in ? mine[d] : 0u;
+                __syncwarp();
+                if (in && below == 0) mine[d] = (uint16_t)(at + __popc(m));
+                __syncwarp();
+                rk[i] = at + below;
+            }
+            __syncthreads();
+            // offsets of the warps within each digit, and the digits' totals
+#pragma unroll
+            for (unsigned j = 0; j < 8; j++) {
+                const unsigned d = 8 * w + j, x = dc[lane * kDigStride + d];
+                unsigned y = x;
+                for (int o = 1; o < 32; o <<= 1) {
+                    const unsigned z = __shfl_up_sync(0xffffffffu, y, o);
+                    if ((int)lane >= o) y += z;
                 }
-                unsigned i = lo, j = d - lo;
+                dc[lane * kDigStride + d] = (uint16_t)(y - x);
+                if (lane == 31) dbase[d] = y;
+            }
+            __syncthreads();
+            if (w == 0) {
+                unsigned v[8], sum = 0;
 #pragma unroll
-                for (int e = 0; e < 8; e++) {
-                    unsigned long long v;
-                    if (j >= R || (i < R && A[i] <= B[j])) { v = A[i]; i++; } else { v = B[j]; j++; }
-                    dst[o + e] = v;
+                for (int j = 0; j < 8; j++) { v[j] = sum; sum += dbase[8 * lane + j]; }
+                unsigned x = sum;
+                for (int o = 1; o < 32; o <<= 1) {
+                    const unsigned z = __shfl_up_sync(0xffffffffu, x, o);
+                    if ((int)lane >= o) x += z;
+                }
+#pragma unroll
+                for (int j = 0; j < 8; j++) dbase[8 * lane + j] = x - sum + v[j];
+            }
+            __syncthreads();
+#pragma unroll
+            for (unsigned i = 0; i < R; i++) {
+                const unsigned p = p0 + 32 * i + lane;
+                if (32 * i < per && p < n) {
+                    const unsigned d = (unsigned)(k[i] >> shift) & 0xFFu;
+                    dst[dbase[d] + mine[d] + rk[i]] = k[i];
                 }
             }
             __syncthreads();
-            src = dst;
+            unsigned long long *t = src; src = dst; dst = t;
         }
     }
-    // key[0, n) sorted; aux becomes the internal node weights
-    for (unsigned i = tid; i < n; i += blockDim.x) aux[i] = 0;
-    unsigned long long *intw = aux;
-    auto LW = [&](unsigned i) { return key[i] >> 16; };
+    const unsigned long long *leaf = src;     // [n] sorted keys
+    unsigned long long *intw = dst;           // [n - 1] weights of the internal nodes
+    auto LW = [&](unsigned i) { return leaf[i] >> 16; };
 
     // 3. two-queue merging in rounds
-    if (tid == 0) { s_ia = s_ib = s_nb = 0; s_done = 0; }
+    if (tid == 0) { s_ia = s_ib = s_nb = s_rounds = 0; s_done = 0; }
     __syncthreads();
+    // pair t of a round: the merged nodes 2t and 2t + 1 of its a leaves and b
+    // internal nodes (equal weights: the leaf first) become internal node nb + t
+    auto pair = [&](unsigned t, unsigned ia, unsigned ib, unsigned nb, unsigned a, unsigned b) {
+        const unsigned d = 2 * t;
+        unsigned lo = d > b ? d - b : 0u, hi = min(d, a);
+        while (lo < hi) {
+            const unsigned m = (lo + hi) >> 1;
+            if (LW(ia + m) <= intw[ib + d - 1 - m]) lo = m + 1; else hi = m;
+        }
+        unsigned i = lo, j = d - lo;
+        unsigned long long sum = 0;
+#pragma unroll
+        for (int e = 0; e < 2; e++) {
+            const unsigned long long x = i < a ? LW(ia + i) : INF, y = j < b ? intw[ib + j] : INF;
+            const bool l = x <= y;
+            sum += l ? x : y;
+            par[l ? ia + i : n + ib + j] = (uint16_t)(n + nb + t);
+            if (l) i++; else j++;
+        }
+        intw[nb + t] = sum;
+    };
     // s_done is read only between the barrier after warp 0 writes it and the
     // next round's barriers, so every warp leaves the loop at the same barrier
     while (n > 1) {
         if (w == 0) {
-            unsigned ia = s_ia, ib = s_ib, nb = s_nb, a = 0, b = 0;
+            unsigned ia = s_ia, ib = s_ib, nb = s_nb, rounds = s_rounds, a = 0, b = 0;
             int state = 0;
             while (true) {
                 const unsigned remA = n - ia, remB = nb - ib;
@@ -662,111 +702,71 @@ __device__ __forceinline__ void codebook_body(const unsigned long long *hist, un
                     else if (intw[ib + b - 1] >= LW(ia + a - 1)) b--;
                     else a--;
                 }
+                if (lane == 0 && rounds < kMaxRounds) rstart[rounds] = (uint16_t)nb;
+                rounds++;
                 if (a + b > kWarpRound) { state = 1; break; }
-                for (unsigned i = lane; i < a + b; i += 32) {
-                    unsigned long long wt;
-                    unsigned q, node;
-                    if (i < a) {
-                        wt = LW(ia + i);
-                        unsigned lo = 0, hi = b;     // internal weights < wt come first
-                        while (lo < hi) { const unsigned m = (lo + hi) >> 1; if (intw[ib + m] < wt) lo = m + 1; else hi = m; }
-                        q = i + lo;
-                        node = ia + i;
-                    } else {
-                        const unsigned j = i - a;
-                        wt = intw[ib + j];
-                        unsigned lo = 0, hi = a;     // leaves <= wt come first
-                        while (lo < hi) { const unsigned m = (lo + hi) >> 1; if (LW(ia + m) <= wt) lo = m + 1; else hi = m; }
-                        q = j + lo;
-                        node = n + ib + j;
-                    }
-                    const unsigned t = nb + (q >> 1);
-                    atomicAdd(&intw[t], wt);
-                    par[node] = (uint16_t)(n + t);
-                }
+                if (2 * lane < a + b) pair(lane, ia, ib, nb, a, b);
                 __syncwarp();
                 ia += a; ib += b; nb += (a + b) >> 1;
             }
             if (lane == 0) {
-                s_ia = ia; s_ib = ib; s_nb = nb; s_a = a; s_b = b;
+                s_ia = ia; s_ib = ib; s_nb = nb; s_a = a; s_b = b; s_rounds = rounds;
                 s_done = state == 2;
             }
         }
         __syncthreads();
         if (s_done) break;
-        {
-            const unsigned ia = s_ia, ib = s_ib, nb = s_nb, a = s_a, b = s_b;
-            for (unsigned i = tid; i < a + b; i += blockDim.x) {
-                unsigned long long wt;
-                unsigned q, node;
-                if (i < a) {
-                    wt = LW(ia + i);
-                    q = i + count_lt(intw + ib, b, wt);
-                    node = ia + i;
-                } else {
-                    const unsigned j = i - a;
-                    wt = intw[ib + j];
-                    unsigned lo = 0, hi = a;
-                    while (lo < hi) { const unsigned m = (lo + hi) >> 1; if (LW(ia + m) <= wt) lo = m + 1; else hi = m; }
-                    q = j + lo;
-                    node = n + ib + j;
-                }
-                const unsigned t = nb + (q >> 1);
-                atomicAdd(&intw[t], wt);
-                par[node] = (uint16_t)(n + t);
-            }
-        }
+        const unsigned ia = s_ia, ib = s_ib, nb = s_nb, a = s_a, b = s_b;
+        for (unsigned t = tid; 2 * t < a + b; t += 1024) pair(t, ia, ib, nb, a, b);
         __syncthreads();
-        if (tid == 0) { s_ia += s_a; s_ib += s_b; s_nb += (s_a + s_b) >> 1; }
+        if (tid == 0) { s_ia = ia + a; s_ib = ib + b; s_nb = nb + ((a + b) >> 1); }
         __syncthreads();
     }
 
-    // 4. depth of every node by pointer jumping (parents have larger indices)
-    const unsigned total = 2 * n - 1, root = total - 1;
-    for (unsigned i = tid; i < total; i += blockDim.x) {
-        if (i == root) par[i] = (uint16_t)root;
-        depb[i] = i == root ? 0 : 1;
-    }
-    __syncthreads();
-    for (int step = 0; step < 7; step++) {
-        uint16_t na[16];
-        uint8_t nd[16];
-#pragma unroll
-        for (int k = 0; k < 16; k++) {
-            const unsigned i = tid + 1024u * k;
-            if (i < total) {
-                const unsigned a = par[i];
-                const unsigned dd = (unsigned)depb[i] + depb[a];
-                nd[k] = (uint8_t)(dd > 255 ? 255 : dd);
-                na[k] = par[a];
+    // 4. depths of the internal nodes (the root is the last one), the rounds
+    //    from the last to the first: warp 0 alone over the small ones at the top
+    //    of the tree, then the block.  Depths saturate at 255.
+    if (n > 1) {
+        const unsigned ni = n - 1;
+        int r = (int)s_rounds - 1;
+        auto depth = [&](unsigned i) {
+            const unsigned d = i + 1 == ni ? 0u : (unsigned)dep[par[n + i] - n] + 1u;
+            dep[i] = (uint8_t)min(d, 255u);
+        };
+        unsigned end = ni;
+        for (; r >= 0 && end - rstart[r] <= kWarpRound; end = rstart[r], r--) {
+            if (w == 0) {
+                for (unsigned i = rstart[r] + lane; i < end; i += 32) depth(i);
+                __syncwarp();
             }
         }
         __syncthreads();
-#pragma unroll
-        for (int k = 0; k < 16; k++) {
-            const unsigned i = tid + 1024u * k;
-            if (i < total) { par[i] = na[k]; depb[i] = nd[k]; }
+        for (; r >= 0; end = rstart[r], r--) {
+            for (unsigned i = rstart[r] + tid; i < end; i += 1024) depth(i);
+            __syncthreads();
         }
-        __syncthreads();
     }
 
-    // 5. code lengths, per-length counts, canonical tables and codewords
-    for (unsigned i = tid; i < n; i += blockDim.x) {
-        unsigned L = n == 1 ? 1u : depb[i];
-        if (n > 1 && (par[i] != root || L > (unsigned)kMaxCodeLen || L == 0)) {
+    // 5. code lengths, canonical tables and codewords
+    for (unsigned i = tid; i < n; i += 1024) {
+        unsigned L = n == 1 ? 1u : (unsigned)dep[par[i] - n] + 1u;
+        if (L > (unsigned)kMaxCodeLen) {
             atomicExch(hs.status, (unsigned)DS_LENGTH);
             L = kMaxCodeLen;
         }
-        lens[(unsigned)(key[i] & 0xFFFFu)] = (uint8_t)L;
-        atomicAdd(&cnt[L], 1u);
+        lens[(unsigned)(leaf[i] & 0xFFFFu)] = (uint8_t)L;
     }
     __syncthreads();
-    for (unsigned i = tid; i < D; i += blockDim.x) hs.len[i] = lens[i];
-    if (tid == 0) length_tables(hs, cnt);
+    canonical_counts(lens, D, wc, cnt);
+    if (w == 0 && !length_tables(T, cnt) && lane == 0) atomicExch(hs.status, (unsigned)DS_FORMAT);
     __syncthreads();
-    if (tid < 64) { sstart[tid] = hs.start[tid]; sfirst[tid] = hs.first[tid]; }
-    __syncthreads();
-    canonical_assign(lens, D, sstart, sfirst, wc, run, hs.code, hs.sorted_sym);
+    if (tid < 64) store_tables(hs, T, tid);
+    canonical_ranks(lens, D, wc, [&](unsigned s, unsigned L, unsigned k) {
+        const unsigned long long code = L ? T.first[L] + k : 0ULL;
+        hs.len[s] = (uint8_t)L;
+        hs.code[s] = code;
+        hs.pack[s] = pack_code(code, L);
+    });
 }
 
 __global__ void __launch_bounds__(1024, 1) codebook_kernel(const unsigned long long *hist, unsigned D, HuffScratch hs)
@@ -782,47 +782,266 @@ __global__ void __launch_bounds__(1024, 1) codebook_batch_kernel(const CodebookJ
 }
 
 // Decoder tables from the code lengths of symbols s_lo..s_hi (every other
-// symbol of the alphabet absent), one block of 1024 threads: counts,
-// canonical tables, the (length, symbol) order of the symbols.
-__global__ void __launch_bounds__(1024, 1) dec_tables_kernel(const uint8_t *lenb, unsigned s_lo, unsigned s_hi,
-                                                             unsigned D, HuffScratch hs, const uint8_t *base,
-                                                             const DevHdr *dh)
+// symbol of the alphabet absent): per-length counts, canonical tables, the
+// (length, symbol) order of the symbols, the first-level table and the
+// second-level tables, laid out in prefix order by a scan of their sizes
+// (prefixes past the budget keep long entries).  With a header on the device
+// (a.dh) it is checked and parsed here first.
+//
+// Single-block latency bounds this (it was three launches of one block: 10 us
+// header, 17 us tables, 24-78 us look-up tables at 8192 symbols).  So every
+// block of a small grid does the short common part for itself, with no
+// exchange between blocks, and the blocks share only what is long: block b
+// stores its slice of the first level and its share of the second-level
+// entries, one thread per entry.  Block 0 stores everything else.
+// One launch of 17 us against 47 at 129^2 (19 against 101 at 130x67x45 and 1e-4,
+// 18 against 66 at 513^3).
+constexpr int kTabThreads = 1024;
+constexpr int kTabBlocks = 16;
+constexpr unsigned kTabPer = (1u << kLutBits) / kTabThreads;    // prefixes per thread
+constexpr unsigned kTabSyms = 16384;                            // sorted symbols staged in shared memory
+constexpr size_t kTabSmem = 4ull * 32 * kWcStride + 2ull * (4u << kLutBits) + 2ull * kTabSyms;   // + D code lengths
+
+// length of the codeword at the top of the left-aligned window: the first L in
+// [1, maxL) whose limit it stays below, else maxL
+template <int N>
+__device__ __forceinline__ void code_lens(const LenTabs &T, const unsigned long long (&win)[N], unsigned maxL,
+                                          unsigned (&L)[N])
 {
-    if (dh) {
-        // a header parsed on the device (and rejected there: nothing to build)
-        if (block_skip(hs.status)) return;
-        lenb = base + dh->off_len;
-        s_lo = dh->s_lo;
-        s_hi = dh->s_hi;
-    }
-    extern __shared__ __align__(16) unsigned char tsm[];
-    unsigned *wc = reinterpret_cast<unsigned *>(tsm);                        // [32 * kWcStride]
-    uint8_t *lens = tsm + 4 * 32 * kWcStride;                                // [D]
-    __shared__ unsigned cnt[64], run[64], sstart[64], nsum;
-    __shared__ unsigned long long sfirst[64];
+#pragma unroll
+    for (int j = 0; j < N; j++) L[j] = 1;
+#pragma unroll
+    for (unsigned s = 32; s; s >>= 1)
+#pragma unroll
+        for (int j = 0; j < N; j++)
+            if (L[j] + s <= maxL && win[j] >= T.lim[L[j] + s - 1]) L[j] += s;
+}
+
+// checks of a container header (the host's parse_header, plus agreement with
+// the shape, type and dictionary the caller expects) by one block; the same
+// answer in every thread of every block
+__device__ __forceinline__ bool parse_header_block(const uint8_t *b, unsigned long long in_bytes, const HdrExpect &ex,
+                                                   DevHdr *out)
+{
+    __shared__ uint32_t hw[32];
+    __shared__ DevHdr h;
+    __shared__ int good;
     const unsigned tid = threadIdx.x;
-    for (unsigned i = tid; i < 64; i += blockDim.x) cnt[i] = 0;
-    if (tid == 0) nsum = 0;
-    __syncthreads();
-    unsigned mine = 0;
-    for (unsigned s = tid; s < D; s += blockDim.x) {
-        unsigned L = (s >= s_lo && s <= s_hi) ? lenb[s - s_lo] : 0u;
-        if (L > (unsigned)kMaxCodeLen) { atomicExch(hs.status, (unsigned)DS_FORMAT); L = 0; }
-        lens[s] = (uint8_t)L;
-        if (L) { atomicAdd(&cnt[L], 1u); mine++; }
+    if (in_bytes < 128) return false;
+    if (tid < 32) {
+        const uint32_t w = reinterpret_cast<const uint32_t *>(b)[tid];
+        hw[tid] = w;
+        const uint32_t crc = crc32_warp(w);
+        if (tid == 31) good = crc == w;
     }
-    mine = warp_sum(mine);
-    if ((tid & 31) == 0 && mine) atomicAdd(&nsum, mine);
     __syncthreads();
+    auto w64 = [&](int at) { return (unsigned long long)hw[at / 4] | ((unsigned long long)hw[at / 4 + 1] << 32); };
     if (tid == 0) {
-        *hs.nsym = nsum;
-        if (nsum == 0) atomicExch(hs.status, (unsigned)DS_FORMAT);
-        length_tables(hs, cnt);
+        bool g = good && hw[0] == 0x52445048u && hw[1] == 3u;    // "HPDR", version 3
+        g = g && (int)hw[2] == ex.dtype && (int)hw[3] == ex.ndim && (int)hw[10] == ex.L && hw[12] <= 1u &&
+            hw[13] == ex.D && hw[14] == ex.K && w64(96) == ex.N;
+        for (int k = 0; k < 3; k++) g = g && w64(16 + 8 * k) == ex.dims[k];
+        h.pad = 0;
+        h.s_lo = hw[15];
+        h.n_esc = w64(104);
+        h.total_bits = w64(112);
+        const uint32_t w120 = hw[30];
+        h.s_hi = w120 & 0xFFFFu;
+        h.esc_w = (w120 >> 16) & 0xFFu;
+        g = g && (w120 >> 24) == 0u && h.s_hi < ex.D && h.s_lo <= h.s_hi && h.n_esc <= ex.N && h.esc_w <= 63u &&
+            ((h.n_esc > 0) == (h.esc_w > 0)) && h.total_bits >= ex.N &&
+            h.total_bits <= 63ULL * ex.N + (unsigned long long)h.esc_w * h.n_esc;
+        if (g) {
+            const unsigned long long nch = (ex.N + ex.K - 1) / ex.K;
+            h.nwords = (h.total_bits + 31) / 32;
+            h.off_len = a16(128 + 8ULL * (ex.L + 1));
+            h.off_chunk = a16(h.off_len + (h.s_hi - h.s_lo + 1));
+            h.off_bits = a16(h.off_chunk + 8 * nch);
+            g = h.off_bits + 4 * h.nwords <= in_bytes;
+        }
+        good = g;
     }
     __syncthreads();
-    if (tid < 64) { sstart[tid] = hs.start[tid]; sfirst[tid] = hs.first[tid]; }
+    bool g = good != 0;
+    if (g && (int)tid <= ex.L) {
+        const double q = reinterpret_cast<const double *>(b + 128)[tid];
+        g = q > 0.0 && isfinite(q);
+    }
+    g = __syncthreads_and(g) != 0;
+    *out = h;
+    return g;
+}
+
+__global__ void __launch_bounds__(kTabThreads, 1) dec_tables_kernel(TabArgs a, HuffScratch hs)
+{
+    extern __shared__ __align__(16) unsigned char tsm[];
+    uint32_t *ent = reinterpret_cast<uint32_t *>(tsm);                          // [1 << kLutBits] first level
+    unsigned *soff = ent + (1u << kLutBits);                                    // [1 << kLutBits] second-level offsets
+    uint16_t *ssym = reinterpret_cast<uint16_t *>(soff + (1u << kLutBits));     // [kTabSyms]
+    unsigned *wc = reinterpret_cast<unsigned *>(ssym + kTabSyms);               // [32][kWcStride]
+    uint8_t *lens = reinterpret_cast<uint8_t *>(wc + 32 * kWcStride);           // [D]
+    __shared__ LenTabs T;
+    __shared__ unsigned cnt[64], wsum[32], total_s;
+    __shared__ int okc;
+    const unsigned tid = threadIdx.x, lane = tid & 31, w = tid >> 5, D = a.D;
+    const bool lead = blockIdx.x == 0;
+    // ---- scalars and header
+    const uint8_t *lenb = a.lenb;
+    unsigned s_lo = a.s_lo, s_hi = a.s_hi;
+    if (a.dh || a.set_scalars) {
+        if (lead) {
+            unsigned char *z = reinterpret_cast<unsigned char *>(a.sc);
+            for (unsigned i = tid; i < sizeof(Scalars); i += kTabThreads) z[i] = 0;
+            __syncthreads();
+        }
+        DevHdr h;
+        bool ok = true;
+        if (a.dh) ok = parse_header_block(a.base, a.in_bytes, a.ex, &h);
+        if (!ok) {
+            if (lead && tid == 0) a.sc->status = (unsigned)DS_FORMAT;
+            return;
+        }
+        if (a.dh) { lenb = a.base + h.off_len; s_lo = h.s_lo; s_hi = h.s_hi; }
+        const int L = a.dh ? a.ex.L : a.si.L;
+        if (lead && (int)tid <= L) {
+            const double q = a.dh ? reinterpret_cast<const double *>(a.base + 128)[tid] : a.si.q[tid];
+            a.sc->q[tid] = q;
+            a.sc->q_f[tid] = __double2float_rn(q);
+            const double r = 1.0 / q;
+            a.sc->rho_d[tid] = r;
+            a.sc->rho_f[tid] = __double2float_rn(r);
+            a.sc->rho_lo[tid] = __double2float_rn(r - (double)__double2float_rn(r));
+        }
+        if (lead && tid == 0) {
+            a.sc->n_esc = a.dh ? h.n_esc : a.si.n_esc;
+            a.sc->total_bits = a.dh ? h.total_bits : a.si.total_bits;
+            if (a.dh) *a.dh = h;
+        }
+    }
+    // ---- code lengths; counts per warp and length over the warp's run of symbols
+    if (tid == 0) okc = 1;
+    for (unsigned i = tid; i < 32 * kWcStride; i += kTabThreads) wc[i] = 0;
     __syncthreads();
-    canonical_assign(lens, D, sstart, sfirst, wc, run, nullptr, hs.sorted_sym);
+    constexpr int U = 8;
+    for (unsigned s0 = tid; s0 < D; s0 += U * kTabThreads) {
+        unsigned v[U];
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            const unsigned s = s0 + u * kTabThreads;
+            v[u] = s < D && s >= s_lo && s <= s_hi ? lenb[s - s_lo] : 0u;
+        }
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            const unsigned s = s0 + u * kTabThreads;
+            if (v[u] > (unsigned)kMaxCodeLen) { okc = 0; v[u] = 0; }
+            if (s < D) lens[s] = (uint8_t)v[u];
+        }
+    }
+    __syncthreads();
+    canonical_counts(lens, D, wc, cnt);
+    if (w == 0 && !length_tables(T, cnt) && lane == 0) okc = 0;
+    __syncthreads();
+    const unsigned n = T.start[63] + T.count[63];
+    const bool ok = okc && n > 0;
+    // ---- symbols in (length, symbol) order
+    uint16_t *sorted = n <= kTabSyms ? ssym : hs.sorted_sym;
+    if (ok)
+        canonical_ranks(lens, D, wc, [&](unsigned s, unsigned L, unsigned k) {
+            if (L) sorted[T.start[L] + k] = (uint16_t)s;
+        });
+    __syncthreads();
+    if (lead) {
+        if (tid < 64) store_tables(hs, T, tid);
+        if (tid == 0) {
+            *hs.nsym = n;
+            if (!ok) atomicExch(hs.status, (unsigned)DS_FORMAT);
+        }
+        if (ok && n <= kTabSyms) for (unsigned i = tid; i < n; i += kTabThreads) hs.sorted_sym[i] = ssym[i];
+    }
+    // ---- first level: the codeword whose left-justified range holds a prefix's
+    // first bit string (at most P bits long, it is a prefix of every extension),
+    // else the range of lengths under the prefix
+    unsigned maxL = 0;
+    for (int l = kMaxCodeLen; l >= 1; l--) if (T.count[l]) { maxL = (unsigned)l; break; }
+    const unsigned t0 = tid * kTabPer;
+    constexpr unsigned long long kTail = (1ULL << (64 - kLutBits)) - 1;
+    unsigned mine = 0;
+    unsigned sbs[kTabPer];
+    {
+        unsigned long long win[kTabPer];
+        unsigned lmin[kTabPer], lmax[kTabPer];
+#pragma unroll
+        for (unsigned j = 0; j < kTabPer; j++) win[j] = (unsigned long long)(t0 + j) << (64 - kLutBits);
+        code_lens(T, win, ok ? maxL : 1u, lmin);
+#pragma unroll
+        for (unsigned j = 0; j < kTabPer; j++) win[j] |= kTail;
+        code_lens(T, win, ok ? maxL : 1u, lmax);
+#pragma unroll
+        for (unsigned j = 0; j < kTabPer; j++) {
+            uint32_t e = 0;
+            sbs[j] = 0;
+            if (ok) {
+                if (lmin[j] <= (unsigned)kLutBits) {
+                    e = leaf_of(T, sorted, n, win[j] & ~kTail, lmin[j]);
+                } else {
+                    e = kLongFlag | (lmin[j] << 16) | ((lmax[j] - lmin[j]) << 24);
+                    if (lmax[j] <= (unsigned)(kLutBits + kSubMax)) {
+                        sbs[j] = lmax[j] - kLutBits;
+                        mine += 1u << sbs[j];
+                    }
+                }
+            }
+            ent[t0 + j] = e;
+        }
+    }
+    // exclusive scan of the second-level sizes over the block
+    unsigned incl = mine;
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned v = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= (unsigned)o) incl += v;
+    }
+    if (lane == 31) wsum[w] = incl;
+    __syncthreads();
+    if (w == 0) {
+        const unsigned v = wsum[lane];
+        unsigned x = v;
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= (unsigned)o) x += y;
+        }
+        wsum[lane] = x - v;
+        if (lane == 31) total_s = x < kSubCap ? x : kSubCap;
+    }
+    __syncthreads();
+    unsigned off = wsum[w] + incl - mine;
+#pragma unroll
+    for (unsigned j = 0; j < kTabPer; j++) {
+        soff[t0 + j] = off;
+        if (!sbs[j]) continue;
+        const unsigned sz = 1u << sbs[j];
+        if (off + sz <= kSubCap) ent[t0 + j] = kSubFlag | off | (sbs[j] << 16);
+        off += sz;
+    }
+    __syncthreads();
+    // ---- this block's slice of the first level and share of the second
+    constexpr unsigned slice = (1u << kLutBits) / kTabBlocks;
+    if (tid < slice) hs.lut1[blockIdx.x * slice + tid] = ent[blockIdx.x * slice + tid];
+    for (unsigned e = blockIdx.x * kTabThreads + tid; e < total_s; e += kTabBlocks * kTabThreads) {
+        // the last prefix whose second-level table starts at or before e
+        unsigned t = 0;
+#pragma unroll
+        for (unsigned s = 1u << (kLutBits - 1); s; s >>= 1)
+            if (soff[t + s] <= e) t += s;
+        const uint32_t f = ent[t];
+        if ((f & (kLongFlag | kSubFlag)) != kSubFlag) continue;   // cut off by the budget
+        const unsigned sb = (f >> 16) & 0xFu, r = e - soff[t];
+        const unsigned long long win[1] = {((unsigned long long)t << (64 - kLutBits)) |
+                                           ((unsigned long long)r << (64 - kLutBits - sb))};
+        unsigned L[1];
+        code_lens(T, win, kLutBits + sb, L);
+        hs.lut_sub[e] = leaf_of(T, sorted, n, win[0], L[0]);
+    }
+    if (lead && tid == 0) *hs.nsub = total_s;
 }
 
 // ---------------------------------------------------------------------------
@@ -854,10 +1073,12 @@ __host__ __device__ inline unsigned enc_group(unsigned K) { return (K < 1024 && 
 // contiguous chunk range [b*cpb, (b+1)*cpb) and leaves its sum in bsum
 __global__ void __launch_bounds__(256) enc_count_kernel(EncodeArgs a)
 {
-    extern __shared__ uint8_t slen[];
+    extern __shared__ __align__(16) uint8_t slen[];
     __shared__ unsigned long long wb[8];
     if (block_skip(&a.sc->status)) return;
-    for (unsigned i = threadIdx.x; i < a.D; i += blockDim.x) slen[i] = a.len[i];
+    // the length table's space in the scratch is a multiple of 256 bytes
+    for (unsigned i = threadIdx.x; i < (a.D + 15) / 16; i += blockDim.x)
+        reinterpret_cast<uint4 *>(slen)[i] = reinterpret_cast<const uint4 *>(a.len)[i];
     __syncthreads();
     // an escape adds its payload width to its codeword
     if (a.esc && threadIdx.x == 0) slen[0] = (uint8_t)(slen[0] + a.sc->esc_w);
@@ -937,74 +1158,77 @@ __global__ void __launch_bounds__(256) enc_count_kernel(EncodeArgs a)
     }
 }
 
-// exclusive scan of the block sums (one block), container layout and capacity
-__global__ void __launch_bounds__(1024) enc_scan1_kernel(EncodeArgs a, int nb)
-{
-    __shared__ unsigned long long sb[1024];
-    if (block_skip(&a.sc->status)) return;
-    const int t = threadIdx.x;
-    sb[t] = t < nb ? a.bsum[t] : 0;
-    __syncthreads();
-    for (int o = 1; o < 1024; o <<= 1) {
-        unsigned long long x = t >= o ? sb[t - o] : 0;
-        __syncthreads();
-        sb[t] += x;
-        __syncthreads();
-    }
-    // inclusive -> exclusive
-    if (t < nb) a.bsum[t] = t ? sb[t - 1] : 0;
-    if (t == 0) {
-        const unsigned long long nch = (a.N + a.K - 1) / a.K;
-        const unsigned long long x = sb[1023];
-        if (a.container) {
-            Layout lay = container_layout(a.L, a.ncoord, a.sc->s_lo, a.sc->s_hi, nch, x);
-            if (lay.total > a.capacity) atomicExch(&a.sc->status, (unsigned)DS_CAPACITY);
-            a.sc->out_bytes = lay.total;
-        } else {
-            if ((x + 31) / 32 > a.words_cap) atomicExch(&a.sc->status, (unsigned)DS_CAPACITY);
-        }
-        a.sc->total_bits = x;
-    }
-}
-
-__device__ __forceinline__ uint32_t *enc_words(const EncodeArgs &a, unsigned long long nch)
+__device__ __forceinline__ uint32_t *enc_words(const EncodeArgs &a, unsigned long long nch, unsigned long long bits)
 {
     if (!a.container) return a.words_out;
-    Layout lay = container_layout(a.L, a.ncoord, a.sc->s_lo, a.sc->s_hi, nch, a.sc->total_bits);
+    Layout lay = container_layout(a.L, a.ncoord, a.sc->s_lo, a.sc->s_hi, nch, bits);
     return reinterpret_cast<uint32_t *>(a.container + lay.off_bits);
 }
 
-// chunk offsets within each block's range (plus the block's offset), chunk
-// table, and zeroed words where more than one writer will meet
-__global__ void __launch_bounds__(256) enc_scan2_kernel(EncodeArgs a)
+// chunk offsets and chunk table, container layout and capacity, and zeroed
+// words where more than one writer will meet.  Block b continues from the sums
+// of the blocks before it, which every block adds up for itself (a scan in a
+// launch of its own cost 5 us and a gap on every call).
+__global__ void __launch_bounds__(256) enc_scan_kernel(EncodeArgs a)
 {
-    __shared__ unsigned long long sb[256];
+    __shared__ unsigned long long spre[8], stot[8];
     if (block_skip(&a.sc->status)) return;
     const unsigned long long nch = (a.N + a.K - 1) / a.K;
     const unsigned long long cpb = (nch + gridDim.x - 1) / gridDim.x;
     const unsigned long long c0 = blockIdx.x * cpb, c1 = c0 + cpb < nch ? c0 + cpb : nch;
-    uint32_t *words = enc_words(a, nch);
-    unsigned long long *ctab = a.chunk_out;
-    if (a.container) {
-        Layout lay = container_layout(a.L, a.ncoord, a.sc->s_lo, a.sc->s_hi, nch, a.sc->total_bits);
-        ctab = reinterpret_cast<unsigned long long *>(a.container + lay.off_chunk);
+    const unsigned t = threadIdx.x, lane = t & 31, w = t >> 5;
+    unsigned long long pre = 0, total = 0;
+    for (unsigned i = t; i < gridDim.x; i += 256) {
+        const unsigned long long x = a.bsum[i];
+        total += x;
+        if (i < blockIdx.x) pre += x;
     }
-    const unsigned long long total = a.sc->total_bits;
-    unsigned long long carry = a.bsum[blockIdx.x];
-    const int t = threadIdx.x;
+    pre = warp_sum64(pre);
+    total = warp_sum64(total);
+    if (lane == 0) { spre[w] = pre; stot[w] = total; }
+    __syncthreads();
+    pre = total = 0;
+#pragma unroll
+    for (int i = 0; i < 8; i++) { pre += spre[i]; total += stot[i]; }
+    // the same decision in every block: nothing is written past the capacity
+    uint32_t *words = a.words_out;
+    unsigned long long *ctab = a.chunk_out;
+    bool fits;
+    if (a.container) {
+        const Layout lay = container_layout(a.L, a.ncoord, a.sc->s_lo, a.sc->s_hi, nch, total);
+        words = reinterpret_cast<uint32_t *>(a.container + lay.off_bits);
+        ctab = reinterpret_cast<unsigned long long *>(a.container + lay.off_chunk);
+        fits = lay.total <= a.capacity;
+        if (blockIdx.x == 0 && t == 0) a.sc->out_bytes = lay.total;
+    } else {
+        fits = (total + 31) / 32 <= a.words_cap;
+    }
+    if (blockIdx.x == 0 && t == 0) {
+        a.sc->total_bits = total;
+        a.chunk_bits[nch] = total;
+        if (!fits) atomicExch(&a.sc->status, (unsigned)DS_CAPACITY);
+    }
+    if (!fits) return;
+    unsigned long long carry = pre;
     for (unsigned long long base = c0; base < c1; base += 256) {
         const unsigned long long c = base + t;
-        unsigned long long v = c < c1 ? a.chunk_bits[c] : 0;
-        sb[t] = v;
+        const unsigned long long v = c < c1 ? a.chunk_bits[c] : 0;
+        unsigned long long x = v;
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned long long y = __shfl_up_sync(0xffffffffu, x, o);
+            if ((int)lane >= o) x += y;
+        }
         __syncthreads();
-        for (int o = 1; o < 256; o <<= 1) {
-            unsigned long long x = t >= o ? sb[t - o] : 0;
-            __syncthreads();
-            sb[t] += x;
-            __syncthreads();
+        if (lane == 31) spre[w] = x;
+        __syncthreads();
+        unsigned long long before = 0, sum = 0;
+#pragma unroll
+        for (int i = 0; i < 8; i++) {
+            if (i < (int)w) before += spre[i];
+            sum += spre[i];
         }
         if (c < c1) {
-            const unsigned long long off = carry + sb[t] - v;
+            const unsigned long long off = carry + before + x - v;
             a.chunk_bits[c] = off;
             ctab[c] = off;
             const unsigned long long cend = off + v;
@@ -1018,48 +1242,172 @@ __global__ void __launch_bounds__(256) enc_scan2_kernel(EncodeArgs a)
             if (full) {
                 if (c % r == 0) words[off >> 5] = 0u;
             } else {
-                for (unsigned long long w = off >> 5; w <= ((cend ? cend - 1 : 0) >> 5); w++) words[w] = 0u;
+                for (unsigned long long i = off >> 5; i <= ((cend ? cend - 1 : 0) >> 5); i++) words[i] = 0u;
             }
             if (c + 1 == nch && (total & 31)) words[total >> 5] = 0u;
         }
-        __syncthreads();
-        carry += sb[255];
-        __syncthreads();
+        carry += sum;
     }
-    if (blockIdx.x == 0 && t == 0) a.chunk_bits[nch] = total;
 }
 
-// one warp per group of chunks (enc_group): every lane encodes 32 (K/32 when
-// K >= 1024) consecutive symbols, assembling its bits in a 64-bit register and
-// storing whole words; the partial words at lane boundaries are merged through
-// shuffles (complete groups) or atomics (the last, partial group)
-__global__ void __launch_bounds__(256) enc_write_kernel(EncodeArgs a)
+// A complete group of 1024 symbols by one warp, 32 consecutive symbols per
+// lane; what bounds it is the issue rate and the shared-memory look-ups, so a
+// symbol is looked up once (its entry stays in a register for the emission),
+// the bits move through two 32-bit registers by funnel shifts, and finished
+// words go to shared memory, from where the group's words leave in whole
+// rows: stored by each lane as they finish, every word was a sector of its own
+// in L2.  An escape is a codeword of its total length whose payload is OR-ed in
+// from a prefetched load.  513^3: 405 -> 207 us (300x431x517 at 1e-4, where most
+// symbols are escapes: 396 -> 257 us); a 129^2 field, whose last group ran symbol
+// by symbol from global memory, 24 -> 9 us.
+constexpr unsigned kEncOutWords = 832;     // words a group may take in shared memory (26 bits per symbol)
+constexpr int kEncWarps = 8;
+// returns false (nothing done) where the group needs the general path: a
+// codeword above 26 bits, an escape above 32 bits in all, more than kEncOutWords
+// words.  PART: the stream's last group, cnt < 1024 symbols; its lanes may hold
+// few bits or none, so its words are merged in cleared shared memory.
+template <bool PART>
+__device__ __forceinline__ bool enc_fast_group(const uint32_t *spk, uint32_t *buf, const uint16_t *sym, unsigned cnt,
+                                               const long long *esc, uint32_t e0, uint32_t code0, unsigned ew,
+                                               unsigned long long start, uint32_t *words)
 {
-    extern __shared__ uint32_t esm32[];
+    const unsigned lane = threadIdx.x & 31;
+    uint32_t e[32];
+    unsigned mb = 0, worst = 0;
+    if (PART) {
+        uint16_t x[32];
+#pragma unroll
+        for (unsigned q = 0; q < 32; q++) x[q] = 32 * lane + q < cnt ? sym[32 * lane + q] : (uint16_t)0;
+#pragma unroll
+        for (unsigned q = 0; q < 32; q++) e[q] = 32 * lane + q < cnt ? spk[x[q]] : 0u;
+    } else {
+        const uint4 *v = reinterpret_cast<const uint4 *>(sym + 32 * lane);
+        uint4 x[4];
+#pragma unroll
+        for (int u = 0; u < 4; u++) x[u] = __ldcs(v + u);
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+            const uint32_t y[4] = {x[u].x, x[u].y, x[u].z, x[u].w};
+#pragma unroll
+            for (int k = 0; k < 4; k++) {
+                e[8 * u + 2 * k] = spk[y[k] & 0xFFFFu];
+                e[8 * u + 2 * k + 1] = spk[y[k] >> 16];
+            }
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < 32; q++) { mb += e[q] & 63u; worst = max(worst, e[q]); }
+    unsigned xb = mb;
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned y = __shfl_up_sync(0xffffffffu, xb, o);
+        if (lane >= (unsigned)o) xb += y;
+    }
+    const unsigned s0 = (unsigned)(start & 31), endb = s0 + __shfl_sync(0xffffffffu, xb, 31);
+    const unsigned W = (endb + 31) >> 5;
+    if (__any_sync(0xffffffffu, worst == kPackLong) || W > kEncOutWords) return false;
+    if (PART) {
+        for (unsigned i = lane; i < W; i += 32) buf[i] = 0u;
+        __syncwarp();
+    }
+    const unsigned at = s0 + xb - mb;
+    unsigned n = at & 31u;
+    uint32_t hi = 0, lo = 0;
+    uint32_t *o = buf + (at >> 5);
+    // low words of the escaped codes, eight symbols ahead of their use
+    const int *el = reinterpret_cast<const int *>(esc + 32 * lane);
+    int zn[8], zc[8];
+    auto fetch = [&](int b) {
+#pragma unroll
+        for (int q = 0; q < 8; q++) {
+            zn[q] = 0;
+            if (e[8 * b + q] == e0) zn[q] = __ldcs(el + 2 * (8 * b + q));
+        }
+    };
+    fetch(0);
+#pragma unroll
+    for (int b = 0; b < 4; b++) {
+#pragma unroll
+        for (int q = 0; q < 8; q++) zc[q] = zn[q];
+        if (b < 3) fetch(b + 1);
+#pragma unroll
+        for (int q = 0; q < 8; q++) {
+            const uint32_t f = e[8 * b + q];
+            const unsigned L = f & 63u;
+            uint32_t c = f >> 6;
+            // zigzag(k) of an escape fits its payload width (below 32 bits)
+            if (f == e0) c = (code0 << ew) | (((uint32_t)zc[q] << 1) ^ (uint32_t)(zc[q] >> 31));
+            hi = __funnelshift_lc(lo, hi, L);
+            lo = __funnelshift_lc(0u, lo, L) | c;
+            n += L;
+            if (n >= 32u) {
+                n -= 32u;
+                const uint32_t v = __funnelshift_r(lo, hi, n);
+                if (PART) atomicOr(o++, v);
+                else *o++ = v;
+            }
+        }
+    }
+    // the word a lane ends in is the next lane's first one (every lane of a
+    // complete group holds at least 32 bits); the last lane's is stored alone
+    __syncwarp();
+    if (n) {
+        const uint32_t last = lo << (32u - n);
+        if (!PART && lane == 31) *o = last;
+        else if (last) atomicOr(o, last);
+    }
+    __syncwarp();
+    uint32_t *g = words + (start >> 5);
+    for (unsigned i = lane; i < W; i += 32) {
+        const uint32_t v = buf[i];
+        // the group's first and last words are shared with its neighbours (zeroed before)
+        if ((i == 0 && s0) || (i + 1 == W && (endb & 31u))) atomicOr(g + i, v);
+        else g[i] = v;
+    }
+    __syncwarp();
+    return true;
+}
+
+__global__ void __launch_bounds__(32 * kEncWarps, 3) enc_write_kernel(EncodeArgs a)
+{
+    extern __shared__ __align__(16) uint32_t esm32[];
     if (block_skip(&a.sc->status)) return;
-    // codeword table: code << 8 | length for codewords of at most 24 bits; a
-    // length field of 0xFF sends the symbol to the global tables
+    // the packed codeword table (pack_code)
     const bool code_sm = a.D <= (unsigned)kSmemCodes;
     uint32_t *spk = esm32;
-    // per warp: the 32 symbols of every lane, 17 words per lane (conflict-free)
-    uint32_t *sw = esm32 + (code_sm ? a.D : 0) + (threadIdx.x >> 5) * (32 * 17);
+    // per warp: a group's finished words, or (general path) the 32 symbols of
+    // every lane, 17 words per lane (conflict-free)
+    const unsigned Dv = (a.D + 3) / 4;   // the table's space in the scratch is a multiple of 256 bytes
+    uint32_t *sw = esm32 + (code_sm ? 4 * Dv : 0) + (threadIdx.x >> 5) * kEncOutWords;
     const uint16_t *ss = reinterpret_cast<const uint16_t *>(sw + (threadIdx.x & 31) * 17);
-    if (code_sm)
-        for (unsigned i = threadIdx.x; i < a.D; i += blockDim.x) {
-            const unsigned L = a.len[i];
-            spk[i] = L <= 24 ? (uint32_t)((a.code[i] << 8) | L) : 0xFFu;
+    const long long *__restrict__ esc = a.esc;
+    const int ew = esc ? (int)a.sc->esc_w : 0;       // escape payload width
+    const unsigned L0 = a.len[0];
+    const uint32_t code0 = (uint32_t)a.code[0];
+    // entry of an escape: its total length, the payload comes from its code
+    const uint32_t e0 = !ew ? 0xFFFFFFFEu : L0 + ew <= 32 ? L0 + ew : kPackLong;
+    if (code_sm) {
+        const uint4 *src = reinterpret_cast<const uint4 *>(a.pack);
+        constexpr int U = 8;
+        for (unsigned i0 = threadIdx.x; i0 < Dv; i0 += U * blockDim.x) {
+            uint4 v[U];
+#pragma unroll
+            for (int u = 0; u < U; u++) v[u] = src[min(i0 + u * blockDim.x, Dv - 1)];
+#pragma unroll
+            for (int u = 0; u < U; u++)
+                if (i0 + u * blockDim.x < Dv) reinterpret_cast<uint4 *>(spk)[i0 + u * blockDim.x] = v[u];
         }
+        __syncthreads();
+        if (threadIdx.x == 0 && ew && L0) spk[0] = e0;
+    }
     __syncthreads();
     // (codeword, length) of symbol s
     auto cw_of = [&](unsigned sv, unsigned long long &cw, int &L) {
-        const uint32_t e = code_sm ? spk[sv] : 0xFFu;
-        if ((e & 0xFFu) != 0xFFu) { cw = e >> 8; L = (int)(e & 0xFFu); }
+        const uint32_t e = code_sm && !(ew && sv == 0) ? spk[sv] : kPackLong;
+        if (e != kPackLong) { cw = e >> 6; L = (int)(e & 63u); }
         else { cw = a.code[sv]; L = a.len[sv]; }
     };
     const unsigned long long nch = (a.N + a.K - 1) / a.K;
-    uint32_t *__restrict__ words = enc_words(a, nch);
-    const long long *__restrict__ esc = a.esc;
-    const int ew = esc ? (int)a.sc->esc_w : 0;       // escape payload width
+    uint32_t *__restrict__ words = enc_words(a, nch, a.sc->total_bits);
     const unsigned lane = threadIdx.x & 31;
     const unsigned r = enc_group(a.K);
     const unsigned long long G = (unsigned long long)a.K * r;   // symbols per warp group
@@ -1070,6 +1418,14 @@ __global__ void __launch_bounds__(256) enc_write_kernel(EncodeArgs a)
     for (unsigned long long c = wg; c < ngr; c += nw) {
         const unsigned long long beg = c * G;
         const unsigned long long end = beg + G < a.N ? beg + G : a.N;
+        if (code_sm && G == 1024) {
+            const unsigned long long start = a.chunk_bits[c * r];
+            const unsigned cnt = (unsigned)(end - beg);
+            const long long *ge = esc ? esc + beg : nullptr;
+            if (cnt == 1024 ? enc_fast_group<false>(spk, sw, a.sym + beg, cnt, ge, e0, code0, (unsigned)ew, start, words)
+                            : enc_fast_group<true>(spk, sw, a.sym + beg, cnt, ge, e0, code0, (unsigned)ew, start, words))
+                continue;
+        }
         unsigned long long m0 = beg + (unsigned long long)lane * spl, m1 = m0 + spl;
         if (m0 > end) m0 = end;
         if (m1 > end) m1 = end;
@@ -1091,9 +1447,10 @@ __global__ void __launch_bounds__(256) enc_write_kernel(EncodeArgs a)
             }
 #pragma unroll 4
             for (int q = 0; q < (int)spl; q++) {
-                const unsigned sv = ss[q];
-                const uint32_t e = code_sm ? spk[sv] : 0xFFu;
-                mb += ((e & 0xFFu) != 0xFFu ? (e & 0xFFu) : a.len[sv]) + (sv == 0 ? ew : 0);
+                unsigned long long cw;
+                int L;
+                cw_of(ss[q], cw, L);
+                mb += L + (ss[q] == 0 ? ew : 0);
             }
         } else {
             for (unsigned long long i = m0; i < m1; i++) {
@@ -1208,79 +1565,94 @@ __global__ void __launch_bounds__(256) enc_write_kernel(EncodeArgs a)
 }
 
 
-__device__ __forceinline__ void put32(uint8_t *p, uint32_t v) { for (int i = 0; i < 4; i++) p[i] = (uint8_t)(v >> (8 * i)); }
-__device__ __forceinline__ void put64(uint8_t *p, unsigned long long v) { for (int i = 0; i < 8; i++) p[i] = (uint8_t)(v >> (8 * i)); }
-__device__ __forceinline__ void putd(uint8_t *p, double v) { put64(p, (unsigned long long)__double_as_longlong(v)); }
-
-__device__ __forceinline__ void header_body(const HeaderArgs &h, const uint8_t *len, Scalars *sc, uint8_t *out)
+// Container header, bins, coordinates, code lengths and the zero gaps before
+// the chunk table and the bitstream.  One block: what bounds it is latency, so
+// the scalars are loaded together and put into words, one warp forms the CRC,
+// and the code lengths move a word per thread with eight words' loads in
+// flight (byte by byte, each load waiting for the store before it, they took
+// most of the 19-23 us; now 5-7 us).
+constexpr int kHeaderThreads = 512;
+__device__ __forceinline__ void header_body(const HeaderArgs &h, const uint8_t *__restrict__ len, Scalars *sc,
+                                            uint8_t *__restrict__ out)
 {
-    __shared__ uint8_t hdr[128];
-    __shared__ uint32_t crct[256];
     if (block_skip(&sc->status)) return;
+    const unsigned tid = threadIdx.x, nt = blockDim.x;
+    const unsigned s_lo = sc->s_lo, s_hi = sc->s_hi;
+    const unsigned long long bits = sc->total_bits;
     const unsigned long long nch = (h.N + h.K - 1) / h.K;
-    Layout lay = container_layout(h.L, h.ncoord, sc->s_lo, sc->s_hi, nch, sc->total_bits);
-    const unsigned long long n_esc = h.hist ? h.hist[0] : 0ULL;
-    // CRC-32 (reflected, polynomial 0xEDB88320) by a byte table, one entry per thread
-    for (int i = threadIdx.x; i < 256; i += blockDim.x) {
-        uint32_t c = (uint32_t)i;
-        for (int b = 0; b < 8; b++) c = (c >> 1) ^ (0xEDB88320u & (0u - (c & 1u)));
-        crct[i] = c;
+    const Layout lay = container_layout(h.L, h.ncoord, s_lo, s_hi, nch, bits);
+    if (tid < 32) {
+        __shared__ uint32_t hw[32];
+        if (tid == 0) {
+            const unsigned long long n_esc = h.hist ? h.hist[0] : 0ULL;
+            const unsigned esc_w = sc->esc_w;
+            const double tau = sc->tau_abs, mx = sc->maxabs, rms = sqrt(sc->sumsq / (double)h.N);
+            auto w64 = [&](int at, unsigned long long v) { hw[at / 4] = (uint32_t)v; hw[at / 4 + 1] = (uint32_t)(v >> 32); };
+            auto wd = [&](int at, double v) { w64(at, (unsigned long long)__double_as_longlong(v)); };
+            hw[0] = 0x52445048u;   // "HPDR"
+            hw[1] = 3;
+            hw[2] = (uint32_t)h.dtype;
+            hw[3] = (uint32_t)h.ndim;
+            for (int k = 0; k < 3; k++) w64(16 + 8 * k, h.dims[k]);
+            hw[10] = (uint32_t)h.L;
+            hw[11] = (uint32_t)h.mode;
+            hw[12] = (uint32_t)h.tol_kind | (h.ncoord ? 0x100u : 0u);
+            hw[13] = h.D;
+            hw[14] = h.K;
+            hw[15] = s_lo;
+            wd(64, h.tol);
+            wd(72, tau);
+            wd(80, mx);
+            wd(88, rms);
+            w64(96, h.N);
+            w64(104, n_esc);
+            w64(112, bits);
+            hw[30] = s_hi | ((n_esc ? esc_w : 0u) << 16);
+            hw[31] = 0;
+            sc->n_esc = n_esc;
+        }
+        __syncwarp();
+        const uint32_t w = hw[tid], crc = crc32_warp(w);
+        reinterpret_cast<uint32_t *>(out)[tid] = tid == 31 ? crc : w;
     }
-    for (int i = threadIdx.x; i < 128; i += blockDim.x) hdr[i] = 0;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        hdr[0] = 'H'; hdr[1] = 'P'; hdr[2] = 'D'; hdr[3] = 'R';
-        put32(hdr + 4, 3);
-        put32(hdr + 8, (uint32_t)h.dtype);
-        put32(hdr + 12, (uint32_t)h.ndim);
-        for (int k = 0; k < 3; k++) put64(hdr + 16 + 8 * k, h.dims[k]);
-        put32(hdr + 40, (uint32_t)h.L);
-        put32(hdr + 44, (uint32_t)h.mode);
-        put32(hdr + 48, (uint32_t)h.tol_kind | (h.ncoord ? 0x100u : 0u));
-        put32(hdr + 52, h.D);
-        put32(hdr + 56, h.K);
-        put32(hdr + 60, sc->s_lo);
-        putd(hdr + 64, h.tol);
-        putd(hdr + 72, sc->tau_abs);
-        putd(hdr + 80, sc->maxabs);
-        putd(hdr + 88, sqrt(sc->sumsq / (double)h.N));
-        put64(hdr + 96, h.N);
-        put64(hdr + 104, n_esc);
-        sc->n_esc = n_esc;
-        put64(hdr + 112, sc->total_bits);
-        put32(hdr + 120, sc->s_hi | ((n_esc ? sc->esc_w : 0u) << 16));
-        uint32_t c = 0xFFFFFFFFu;
-        for (int i = 0; i < 124; i++) c = crct[(c ^ hdr[i]) & 0xFFu] ^ (c >> 8);
-        put32(hdr + 124, c ^ 0xFFFFFFFFu);
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < 128; i += blockDim.x) out[i] = hdr[i];
     const unsigned long long qend = 128 + 8ULL * (h.L + 1);
-    for (int l = threadIdx.x; l <= h.L; l += blockDim.x) putd(out + 128 + 8 * l, sc->q[l]);
-    for (unsigned long long i = threadIdx.x; i < h.ncoord; i += blockDim.x) putd(out + qend + 8 * i, h.coords[i]);
-    for (unsigned long long i = qend + 8 * h.ncoord + threadIdx.x; i < lay.off_len; i += blockDim.x) out[i] = 0;
-    const unsigned nlen = sc->s_hi - sc->s_lo + 1;
-    for (unsigned i = threadIdx.x; i < nlen; i += blockDim.x) out[lay.off_len + i] = len[sc->s_lo + i];
-    for (unsigned long long i = lay.off_len + nlen + threadIdx.x; i < lay.off_chunk; i += blockDim.x) out[i] = 0;
-    for (unsigned long long i = lay.off_chunk + 8 * nch + threadIdx.x; i < lay.off_bits; i += blockDim.x) out[i] = 0;
-}
-
-__global__ void __launch_bounds__(256)
-header_kernel(HeaderArgs h, const uint8_t *len, Scalars *sc, uint8_t *out)
-{
-    header_body(h, len, sc, out);
+    for (int l = tid; l <= h.L; l += nt) reinterpret_cast<double *>(out + 128)[l] = sc->q[l];
+    for (unsigned long long i = tid; i < h.ncoord; i += nt) reinterpret_cast<double *>(out + qend)[i] = h.coords[i];
+    for (unsigned long long i = qend + 8 * h.ncoord + tid; i < lay.off_len; i += nt) out[i] = 0;
+    const unsigned nlen = s_hi - s_lo + 1, nw = nlen / 4;
+    const uint8_t *lsrc = len + s_lo;
+    uint32_t *lw = reinterpret_cast<uint32_t *>(out + lay.off_len);
+    constexpr int U = 4;
+    for (unsigned i0 = tid; i0 < nw; i0 += U * nt) {
+        uint32_t v[U];
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            const unsigned i = min(i0 + u * nt, nw - 1);
+            v[u] = (uint32_t)lsrc[4 * i] | ((uint32_t)lsrc[4 * i + 1] << 8) | ((uint32_t)lsrc[4 * i + 2] << 16) |
+                   ((uint32_t)lsrc[4 * i + 3] << 24);
+        }
+#pragma unroll
+        for (int u = 0; u < U; u++) if (i0 + u * nt < nw) lw[i0 + u * nt] = v[u];
+    }
+    for (unsigned i = 4 * nw + tid; i < nlen; i += nt) out[lay.off_len + i] = lsrc[i];
+    for (unsigned long long i = lay.off_len + nlen + tid; i < lay.off_chunk; i += nt) out[i] = 0;
+    for (unsigned long long i = lay.off_chunk + 8 * nch + tid; i < lay.off_bits; i += nt) out[i] = 0;
 }
 
 // one container header per block, then the field's {bytes, status} pair
-__global__ void __launch_bounds__(256) header_batch_kernel(const HeaderJob *jobs)
+__device__ __forceinline__ void header_job(const HeaderJob &j)
 {
-    const HeaderJob &j = jobs[blockIdx.x];
     header_body(j.h, j.len, j.sc, j.out);
     __syncthreads();
     if (threadIdx.x == 0 && j.size_status) {
         j.size_status[0] = j.sc->out_bytes;
         j.size_status[1] = j.sc->status;
     }
+}
+__global__ void __launch_bounds__(kHeaderThreads) header_kernel(HeaderJob j) { header_job(j); }
+__global__ void __launch_bounds__(kHeaderThreads) header_batch_kernel(const HeaderJob *jobs)
+{
+    header_job(jobs[blockIdx.x]);
 }
 
 // ---------------------------------------------------------------------------
@@ -1640,15 +2012,13 @@ cudaError_t set_attrs_now()
                                  (int)kCodebookSmem);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(dec_tables_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 4 * 32 * kWcStride + 65536);
+                                 (int)kTabSmem + 65536);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(enc_write_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(enc_count_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 65536);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(decode_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDecSmem);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(lut_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLutSmem);
     return e;
 }
 cudaError_t set_attrs() { return once_per_device(g_attr_done, set_attrs_now); }
@@ -1666,7 +2036,7 @@ size_t huff_scratch_bytes(unsigned int D)
     add(4); add(8 * 64); add(4 * 64); add(4 * 64);     // nsym, first, count, start
     add(d); add(8 * d); add(2 * d); add(4u << kLutBits);
     add(8 * 64);
-    add(4 * kSubCap); add(4);
+    add(4 * kSubCap); add(4); add(4 * d);
     return b;
 }
 
@@ -1695,6 +2065,7 @@ void huff_scratch_carve(void *base, unsigned int D, Scalars *sc, HuffScratch *hs
     hs->lim = (unsigned long long *)take(8 * 64);
     hs->lut_sub = (uint32_t *)take(4 * kSubCap);
     hs->nsub = (unsigned *)take(4);
+    hs->pack = (uint32_t *)take(4 * d);
     hs->status = &sc->status;
     hs->s_lo = &sc->s_lo;
     hs->s_hi = &sc->s_hi;
@@ -1719,25 +2090,12 @@ cudaError_t launch_codebook(const unsigned long long *hist, unsigned int D, cons
     return cudaGetLastError();
 }
 
-cudaError_t launch_decode_tables(const uint8_t *lenb, unsigned int s_lo, unsigned int s_hi, unsigned int D,
-                                 const HuffScratch &hs, cudaStream_t s)
+cudaError_t launch_decode_tables(const TabArgs &a, const HuffScratch &hs, cudaStream_t s)
 {
     cudaError_t e = set_attrs();
     if (e != cudaSuccess) return e;
-    dec_tables_kernel<<<1, 1024, 4 * 32 * kWcStride + D, s>>>(lenb, s_lo, s_hi, D, hs, nullptr, nullptr);
-    lut_kernel<<<1, kLutThreads, kLutSmem, s>>>(hs);
-    count_launch(2);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_decode_tables_dev(const uint8_t *base, const DevHdr *dh, unsigned int D, const HuffScratch &hs,
-                                     cudaStream_t s)
-{
-    cudaError_t e = set_attrs();
-    if (e != cudaSuccess) return e;
-    dec_tables_kernel<<<1, 1024, 4 * 32 * kWcStride + D, s>>>(nullptr, 0u, 0u, D, hs, base, dh);
-    lut_kernel<<<1, kLutThreads, kLutSmem, s>>>(hs);
-    count_launch(2);
+    dec_tables_kernel<<<kTabBlocks, kTabThreads, kTabSmem + a.D, s>>>(a, hs);
+    count_launch();
     return cudaGetLastError();
 }
 
@@ -1745,28 +2103,30 @@ cudaError_t launch_encode(const EncodeArgs &a, cudaStream_t s)
 {
     cudaError_t e = set_attrs();
     if (e != cudaSuccess) return e;
-    enc_count_kernel<<<kEncBlocks, 256, a.D, s>>>(a);
-    enc_scan1_kernel<<<1, 1024, 0, s>>>(a, kEncBlocks);
-    enc_scan2_kernel<<<kEncBlocks, 256, 0, s>>>(a);
+    // eight warps a block, a group each: no more blocks than the stream has groups
+    const unsigned long long groups = ((a.N + a.K - 1) / a.K + enc_group(a.K) - 1) / enc_group(a.K);
+    const unsigned nb = (unsigned)std::min<unsigned long long>(kEncBlocks, (groups + 7) / 8);
+    enc_count_kernel<<<nb, 256, (a.D + 15) / 16 * 16, s>>>(a);
+    enc_scan_kernel<<<nb, 256, 0, s>>>(a);
     const bool code_sm = a.D <= (unsigned)kSmemCodes;
-    const size_t sm = (code_sm ? 4 * (size_t)a.D : 0) + 8 * 32 * 17 * 4;
+    const size_t sm = ((code_sm ? (size_t)(a.D + 3) / 4 * 4 : 0) + kEncWarps * kEncOutWords) * 4;
     int per_sm = 0, nsm = 0, dev = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, enc_write_kernel, 256, sm) != cudaSuccess ||
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, enc_write_kernel, 32 * kEncWarps, sm) != cudaSuccess ||
         cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
         cudaGetLastError();
         per_sm = 3;
         nsm = 152;
     }
-    enc_write_kernel<<<(unsigned)(nsm * std::max(1, per_sm)), 256, sm, s>>>(a);
-    count_launch(4);
+    const unsigned long long full = (unsigned long long)nsm * std::max(1, per_sm);
+    enc_write_kernel<<<(unsigned)std::min(full, (groups + kEncWarps - 1) / kEncWarps), 32 * kEncWarps, sm, s>>>(a);
+    count_launch(3);
     return cudaGetLastError();
 }
 
-cudaError_t launch_header(const HeaderArgs &h, const uint8_t *len, Scalars *sc, uint8_t *container,
-                          cudaStream_t s)
+cudaError_t launch_header(const HeaderJob &j, cudaStream_t s)
 {
-    header_kernel<<<1, 256, 0, s>>>(h, len, sc, container);
+    header_kernel<<<1, kHeaderThreads, 0, s>>>(j);
     count_launch();
     return cudaGetLastError();
 }
@@ -1786,7 +2146,7 @@ cudaError_t launch_codebook_batch(const CodebookJob *jobs, int n, cudaStream_t s
 cudaError_t launch_header_batch(const HeaderJob *jobs, int n, cudaStream_t s)
 {
     if (n < 1) return cudaSuccess;
-    header_batch_kernel<<<n, 256, 0, s>>>(jobs);
+    header_batch_kernel<<<n, kHeaderThreads, 0, s>>>(jobs);
     count_launch();
     return cudaGetLastError();
 }

@@ -38,6 +38,7 @@ struct HuffScratch {
     unsigned int *start;          // [64]
     uint8_t *len;                 // [D]
     unsigned long long *code;     // [D]
+    uint32_t *pack;               // [D] encoder: codeword << 8 | length, short codewords (pack_code)
     uint16_t *sorted_sym;         // [D]
     uint32_t *lut1;               // [1 << kLutBits] first-level decoder table of every 13-bit prefix
     uint32_t *lut_sub;            // [kSubCap] second-level entries of longer codewords
@@ -60,13 +61,37 @@ void huff_scratch_carve(void *base, unsigned int D, Scalars *sc, HuffScratch *hs
 // Codebook from a histogram hist[D] (two-queue lengths, canonical codes).
 cudaError_t launch_codebook(const unsigned long long *hist, unsigned int D, const HuffScratch &hs,
                             cudaStream_t s);
-// Canonical tables + LUT from the code lengths lenb[0 .. s_hi - s_lo] of the
-// symbols s_lo..s_hi (device bytes; every other symbol absent), decoder side.
-cudaError_t launch_decode_tables(const uint8_t *lenb, unsigned int s_lo, unsigned int s_hi, unsigned int D,
-                                 const HuffScratch &hs, cudaStream_t s);
-// the same with the length table located through a device-parsed header
-cudaError_t launch_decode_tables_dev(const uint8_t *base, const DevHdr *dh, unsigned int D, const HuffScratch &hs,
-                                     cudaStream_t s);
+// What the caller of a device-parsed header expects of it.
+struct HdrExpect {
+    int dtype, ndim, L;
+    unsigned long long dims[3], N;
+    unsigned D, K;
+};
+// The decoder-side scalars of one container whose header the host has parsed.
+struct ScalarInit {
+    double q[kMaxLevels + 1];
+    int L;
+    unsigned long long n_esc, total_bits;
+};
+// Canonical tables and look-up tables from the code lengths of the symbols
+// s_lo..s_hi (device bytes; every other symbol absent), decoder side.
+struct TabArgs {
+    const uint8_t *lenb = nullptr;    // lengths of s_lo..s_hi (dh null)
+    unsigned s_lo = 0, s_hi = 0, D = 0;
+    Scalars *sc = nullptr;
+    // set_scalars: *sc is cleared and takes si
+    bool set_scalars = false;
+    ScalarInit si;
+    // dh non-null: the header of the container at base (in_bytes) is checked
+    // against ex and parsed into *dh, *sc cleared and set from it; a bad header
+    // leaves DS_FORMAT there, and every later kernel of the decompression skips or
+    // computes on stale (in-bounds) data
+    const uint8_t *base = nullptr;
+    unsigned long long in_bytes = 0;
+    DevHdr *dh = nullptr;
+    HdrExpect ex;
+};
+cudaError_t launch_decode_tables(const TabArgs &a, const HuffScratch &hs, cudaStream_t s);
 
 // Encoder.  Layout of the destination: chunk table at chunk_out, bitstream at
 // words (both device pointers, possibly inside a container whose offsets are
@@ -78,6 +103,7 @@ struct EncodeArgs {
     unsigned int D, K;
     const uint8_t *len;
     const unsigned long long *code;
+    const uint32_t *pack;
     const long long *esc;             // null: plain symbols; else symbol 0 is the quantizer's
                                       // escape and esc[i] its code k (payload after the codeword,
                                       // in sc->esc_w bits)
@@ -105,11 +131,6 @@ struct HeaderArgs {
     const double *coords;             // node coordinates (device), ncoord values, or null
     unsigned long long ncoord;
 };
-cudaError_t launch_header(const HeaderArgs &h, const uint8_t *len, Scalars *sc, uint8_t *container,
-                          cudaStream_t s);
-
-// Batched forms for many fields at once (one block per field, the same
-// device code as the single-field launches, so the same bytes).
 struct CodebookJob {
     const unsigned long long *hist;
     unsigned int D;
@@ -122,6 +143,10 @@ struct HeaderJob {
     uint8_t *out;
     unsigned long long *size_status;   // [2]: container bytes and device status (may be null)
 };
+cudaError_t launch_header(const HeaderJob &j, cudaStream_t s);
+
+// Batched forms for many fields at once (one block per field, the same
+// device code as the single-field launches, so the same bytes).
 // whether launch_codebook builds an alphabet of D symbols in one block
 // (launch_codebook_batch takes only such alphabets)
 bool codebook_fused(unsigned int D);
