@@ -84,7 +84,7 @@ long long total_of(int ndim, const size_t *dims)
     return n;
 }
 
-// workspace of one field: scalars, partials, hist, level buffers, symbols,
+// workspace of one field: scalars, hist, partials, level buffers, symbols,
 // escaped codes, chunk tables, Huffman scratch
 struct Ws {
     Scalars *sc;
@@ -106,8 +106,8 @@ size_t carve_ws(void *base, const Plan *P, size_t esz, unsigned D, unsigned K, b
     long long Nl1 = P->L >= 1 ? P->N[P->L - 1] : 1;
     unsigned long long nch = (N + K - 1) / K;
     w->sc = c.take<Scalars>(1);
-    w->partials = c.take<double>(2 * norm_parts());
     w->hist = c.take<unsigned long long>(D);
+    w->partials = c.take<double>(2 * norm_parts());
     w->va = c.take<char>(Nl1 * esz);
     w->vb = c.take<char>(Nl1 * esz);
     w->b = c.take<char>(Nl1 * esz);
@@ -199,7 +199,7 @@ void l2s_weights(const Plan *P, L2sArgs &a)
     }
 }
 
-// runs after bins_kernel (which set the norm, tau and the status of the
+// runs after the norm pass (which set the norm, tau and the status of the
 // bound) and replaces its bins; a rejected bound or a zero field keeps them
 __global__ void bins_l2s_kernel(L2sArgs a, Scalars *sc)
 {
@@ -261,12 +261,8 @@ hpdr_status compress_core(hpdr_ctx *ctx, const Plan *P, const T *u, int ndim, co
     HuffScratch hs;
     huff_scratch_carve(w.huff, D, w.sc, &hs);
     if (phases & kPhLevels) {
-    CK(cudaMemsetAsync(w.sc, 0, sizeof(Scalars), s));
-    CK(cudaMemsetAsync(w.hist, 0, sizeof(unsigned long long) * D, s));
-    {
-    ProfScope ps(ctx, "norm", s);
-    CK(launch_norm<T>(u, N, w.partials, norm_parts(), s));
-    }
+    // the scalars and the histogram are neighbours in the workspace
+    CK(cudaMemsetAsync(w.sc, 0, (size_t)((char *)(w.hist + D) - (char *)w.sc), s));
     BinArgs ba;
     memset(&ba, 0, sizeof(ba));
     ba.L = L;
@@ -276,7 +272,10 @@ hpdr_status compress_core(hpdr_ctx *ctx, const Plan *P, const T *u, int ndim, co
     ba.mode = mode == 2 ? 1 : mode;   // both L2 modes take the RMS norm
     ba.eps = sizeof(T) == 4 ? ldexp(1.0, -24) : ldexp(1.0, -53);
     ba.N = N;
-    CK(launch_bins(ba, w.partials, norm_parts(), w.sc, s));
+    {
+    ProfScope ps(ctx, "norm", s);
+    CK(launch_norm<T>(u, N, w.partials, ba, w.sc, s));
+    }
     if (mode == 2) {
         L2sArgs la;
         memset(&la, 0, sizeof(la));

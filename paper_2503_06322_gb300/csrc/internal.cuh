@@ -78,8 +78,7 @@ struct Scalars {
     unsigned int status;          // 0 ok, else an hpdr_status magnitude
     unsigned int esc_w;           // escape payload width: largest bit length of zigzag(k)
     unsigned int s_lo, s_hi;
-    unsigned int maxbits_f32;     // max|u| as float bits (atomicMax)
-    unsigned long long maxbits_f64;
+    unsigned int blocks_done;     // norm pass: blocks that have stored their partials
 };
 
 // escaped codes must satisfy |k| < 2^62 (payload of at most 63 bits)

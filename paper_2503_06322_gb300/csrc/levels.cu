@@ -258,18 +258,95 @@ __global__ void level0_in_kernel(const T *coef_in, SymIn symin, long long N0, T 
 }
 
 // --------------------------------------------------------------------------
-// max|u| and sum u^2: fixed grid, fixed per-thread order -> deterministic.
+// max|u| and sum u^2, then the level bins by the last block to finish: fixed
+// grid, fixed per-thread order and a fixed tree over the blocks' partials ->
+// deterministic.  Binary64 issue is slow on this part (about two lanes per
+// cycle and SM), so a magnitude is compared as an integer (the order of
+// non-negative values, with every NaN above infinity) and binary64 fields
+// spend one binary64 instruction a value, the multiply-add of the sum, where
+// they spent four (500 x 500 x 100: 300 -> NORM64 us).
 
-template <typename T>
-__device__ __forceinline__ void nan_max(T &m, T x)
+template <typename T> struct BitsOf;
+template <> struct BitsOf<float> { using type = unsigned; };
+template <> struct BitsOf<double> { using type = unsigned long long; };
+__device__ __forceinline__ unsigned abs_bits(float x) { return __float_as_uint(x) & 0x7FFFFFFFu; }
+__device__ __forceinline__ unsigned long long abs_bits(double x)
 {
-    if (x > m || x != x) m = (m != m) ? m : x;
+    return (unsigned long long)__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFull;
+}
+__device__ __forceinline__ double abs_value(unsigned b) { return (double)__uint_as_float(b); }
+__device__ __forceinline__ double abs_value(unsigned long long b) { return __longlong_as_double((long long)b); }
+
+// the bins from the partials, by one block of 256 threads
+__device__ __forceinline__ void bins_body(const BinArgs &ba, const volatile double *partials, int nparts, Scalars *sc)
+{
+    __shared__ unsigned long long smx[256];
+    __shared__ double sss[256];
+    // five loads in flight, then the sums in the order of the partials
+    unsigned long long mx = 0;
+    double ss = 0.0;
+    constexpr int U = 5;
+    for (int i0 = threadIdx.x; i0 < nparts; i0 += U * 256) {
+        double m[U], v[U];
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            const int i = i0 + 256 * u;
+            m[u] = i < nparts ? partials[2 * i] : 0.0;
+            v[u] = i < nparts ? partials[2 * i + 1] : 0.0;
+        }
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            mx = max(mx, abs_bits(m[u]));
+            ss += v[u];
+        }
+    }
+    smx[threadIdx.x] = mx;
+    sss[threadIdx.x] = ss;
+    __syncthreads();
+    for (int s = 128; s > 0; s >>= 1) {
+        if ((int)threadIdx.x < s) {
+            smx[threadIdx.x] = max(smx[threadIdx.x], smx[threadIdx.x + s]);
+            sss[threadIdx.x] += sss[threadIdx.x + s];
+        }
+        __syncthreads();
+    }
+    const double mxv = abs_value(smx[0]);
+    ss = sss[0];
+    if (threadIdx.x == 0) {
+        sc->maxabs = mxv;
+        sc->sumsq = ss;
+    }
+    const int L = ba.L;
+    bool ok = mxv <= DBL_MAX;
+    double nrm = ba.mode == 0 ? mxv : sqrt(__ddiv_rn(ss, (double)ba.N));
+    double tau = ba.tol_kind == 1 ? __dmul_rn(ba.tol, nrm) : ba.tol;
+    if (threadIdx.x == 0) sc->tau_abs = tau;
+    double tp = 0.0;
+    if (ok && mxv > 0.0) {
+        tp = __dsub_rn(tau, __dmul_rn(__dmul_rn(__dmul_rn(32.0, (double)(L + 1)), ba.eps), mxv));
+        if (!(tp > 0.0)) ok = false;
+    }
+    // one level per thread (two FP64 divisions each)
+    for (int l = threadIdx.x; l <= L; l += blockDim.x) {
+        double q;
+        if (!ok || mxv == 0.0) q = 1.0;
+        else if (l == 0) q = __ddiv_rn(__dmul_rn(2.0, tp), (double)(L + 1));
+        else q = __ddiv_rn(__dmul_rn(2.0, tp), __dmul_rn((double)(L + 1), __dadd_rn(1.0, ba.c[l])));
+        sc->q[l] = q;
+        double r = __ddiv_rn(1.0, q);
+        sc->rho_d[l] = r;
+        sc->rho_f[l] = __double2float_rn(r);
+        sc->rho_lo[l] = __double2float_rn(__dsub_rn(r, (double)sc->rho_f[l]));
+        sc->q_f[l] = __double2float_rn(q);
+    }
+    if (!ok && threadIdx.x == 0) atomicExch(&sc->status, (unsigned int)DS_ARG);
 }
 
 template <typename T>
-__global__ void __launch_bounds__(256) norm_kernel(const T *__restrict__ u, long long N, double *partials)
+__global__ void __launch_bounds__(256) norm_kernel(const T *__restrict__ u, long long N, double *partials, BinArgs ba,
+                                                   Scalars *sc)
 {
-    T mx = (T)0;
+    typename BitsOf<T>::type mx = 0;
     T ssT = (T)0;   // per-thread partial sum in T (binary64 arithmetic is slow on this part)
     double ss = 0.0;
     const long long tid = blockIdx.x * (long long)blockDim.x + threadIdx.x;
@@ -285,89 +362,40 @@ __global__ void __launch_bounds__(256) norm_kernel(const T *__restrict__ u, long
             const T *e = reinterpret_cast<const T *>(&x);
 #pragma unroll
             for (int k = 0; k < V; k++) {
-                T ax = e[k] < (T)0 ? -e[k] : e[k];
-                nan_max(mx, ax);
+                mx = max(mx, abs_bits(e[k]));
                 ssT = fma_rn(e[k], e[k], ssT);
             }
         }
     }
     for (long long i = nv * V + tid; i < N; i += nth) {
         T x = u[i];
-        T ax = x < (T)0 ? -x : x;
-        nan_max(mx, ax);
+        mx = max(mx, abs_bits(x));
         ssT = fma_rn(x, x, ssT);
     }
     ss = (double)ssT;
     for (int o = 16; o > 0; o >>= 1) {
-        T om = __shfl_down_sync(0xffffffffu, mx, o);
-        double os = __shfl_down_sync(0xffffffffu, ss, o);
-        nan_max(mx, om);
-        ss += os;
+        mx = max(mx, __shfl_down_sync(0xffffffffu, mx, o));
+        ss += __shfl_down_sync(0xffffffffu, ss, o);
     }
-    __shared__ T smx[8];
+    __shared__ typename BitsOf<T>::type smx[8];
     __shared__ double sss[8];
+    __shared__ bool last;
     int w = threadIdx.x >> 5;
     if ((threadIdx.x & 31) == 0) { smx[w] = mx; sss[w] = ss; }
     __syncthreads();
     if (threadIdx.x == 0) {
-        T m = smx[0];
+        typename BitsOf<T>::type m = smx[0];
         double s = sss[0];
-        for (int i = 1; i < (int)(blockDim.x >> 5); i++) { nan_max(m, smx[i]); s += sss[i]; }
-        partials[2 * blockIdx.x] = (double)m;
+        for (int i = 1; i < (int)(blockDim.x >> 5); i++) { m = max(m, smx[i]); s += sss[i]; }
+        partials[2 * blockIdx.x] = abs_value(m);
         partials[2 * blockIdx.x + 1] = s;
+        __threadfence();
+        last = atomicAdd(&sc->blocks_done, 1u) + 1 == gridDim.x;
     }
-}
-
-__global__ void bins_kernel(BinArgs ba, const double *partials, int nparts, Scalars *sc)
-{
-    __shared__ double smx[256], sss[256];
-    double mx = 0.0, ss = 0.0;
-    for (int i = threadIdx.x; i < nparts; i += blockDim.x) {
-        double m = partials[2 * i];
-        if (m > mx || m != m) mx = (mx != mx) ? mx : m;
-        ss += partials[2 * i + 1];
-    }
-    smx[threadIdx.x] = mx;
-    sss[threadIdx.x] = ss;
     __syncthreads();
-    for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-        if ((int)threadIdx.x < s) {
-            double m = smx[threadIdx.x + s];
-            if (m > smx[threadIdx.x] || m != m) smx[threadIdx.x] = (smx[threadIdx.x] != smx[threadIdx.x]) ? smx[threadIdx.x] : m;
-            sss[threadIdx.x] += sss[threadIdx.x + s];
-        }
-        __syncthreads();
-    }
-    mx = smx[0];
-    ss = sss[0];
-    if (threadIdx.x == 0) {
-        sc->maxabs = mx;
-        sc->sumsq = ss;
-    }
-    const int L = ba.L;
-    bool ok = mx <= DBL_MAX;
-    double nrm = ba.mode == 0 ? mx : sqrt(__ddiv_rn(ss, (double)ba.N));
-    double tau = ba.tol_kind == 1 ? __dmul_rn(ba.tol, nrm) : ba.tol;
-    if (threadIdx.x == 0) sc->tau_abs = tau;
-    double tp = 0.0;
-    if (ok && mx > 0.0) {
-        tp = __dsub_rn(tau, __dmul_rn(__dmul_rn(__dmul_rn(32.0, (double)(L + 1)), ba.eps), mx));
-        if (!(tp > 0.0)) ok = false;
-    }
-    // one level per thread (two FP64 divisions each)
-    for (int l = threadIdx.x; l <= L; l += blockDim.x) {
-        double q;
-        if (!ok || mx == 0.0) q = 1.0;
-        else if (l == 0) q = __ddiv_rn(__dmul_rn(2.0, tp), (double)(L + 1));
-        else q = __ddiv_rn(__dmul_rn(2.0, tp), __dmul_rn((double)(L + 1), __dadd_rn(1.0, ba.c[l])));
-        sc->q[l] = q;
-        double r = __ddiv_rn(1.0, q);
-        sc->rho_d[l] = r;
-        sc->rho_f[l] = __double2float_rn(r);
-        sc->rho_lo[l] = __double2float_rn(__dsub_rn(r, (double)sc->rho_f[l]));
-        sc->q_f[l] = __double2float_rn(q);
-    }
-    if (!ok && threadIdx.x == 0) atomicExch(&sc->status, (unsigned int)DS_ARG);
+    if (!last) return;
+    __threadfence();
+    bins_body(ba, partials, (int)gridDim.x, sc);
 }
 
 // --------------------------------------------------------------------------
@@ -961,21 +989,17 @@ cudaError_t launch_level0_in(WSrc src, const T *coef_in, const SymIn &symin, lon
 }
 
 template <typename T>
-cudaError_t launch_norm(const T *u, long long N, double *partials, int nparts, cudaStream_t s)
+cudaError_t launch_norm(const T *u, long long N, double *partials, const BinArgs &ba, Scalars *sc, cudaStream_t s)
 {
-    norm_kernel<T><<<nparts, 256, 0, s>>>(u, N, partials);
+    // a block per 256 16-byte vectors, at most norm_parts() of them: with fewer
+    // vectors than the full grid has threads the smaller grid gives every value
+    // the same thread, and the blocks left out would add zeros
+    const long long need = (N * (long long)sizeof(T) / 16 + 255) / 256 + 1;
+    const int blocks = (((uintptr_t)u) & 15) == 0 && need < kNormBlocks ? (int)need : kNormBlocks;
+    norm_kernel<T><<<blocks, 256, 0, s>>>(u, N, partials, ba, sc);
     count_launch();
     return cudaGetLastError();
 }
-
-cudaError_t launch_bins(const BinArgs &ba, const double *partials, int nparts, Scalars *sc,
-                        cudaStream_t s)
-{
-    bins_kernel<<<1, 256, 0, s>>>(ba, partials, nparts, sc);
-    count_launch();
-    return cudaGetLastError();
-}
-
 
 template <typename T>
 size_t coarse_smem_bytes(const LevelGeom<T> &g)
@@ -1081,7 +1105,7 @@ cudaError_t launch_coarse(int mode, const Plan *P, const LevelGeom<T> *geo, int 
                                           cudaStream_t);                                         \
     template cudaError_t launch_level0_in<T>(WSrc, const T *, const SymIn &, long long, T *,      \
                                              cudaStream_t);                                      \
-    template cudaError_t launch_norm<T>(const T *, long long, double *, int, cudaStream_t);      \
+    template cudaError_t launch_norm<T>(const T *, long long, double *, const BinArgs &, Scalars *, cudaStream_t); \
     template int coarse_top<T>(const Plan *, const LevelGeom<T> *);                              \
     template cudaError_t launch_coarse<T>(int, const Plan *, const LevelGeom<T> *, int, const T *, T *, \
                                           const QuantOut &, T *, const SymIn &, const T *, cudaStream_t); \

@@ -91,9 +91,8 @@ template <typename T>
 cudaError_t launch_level0_in(WSrc src, const T *coef_in, const SymIn &symin, long long N0, T *v0,
                              cudaStream_t s);
 
-// max|u| and sum u^2 (deterministic), then bins (one thread block).
-template <typename T>
-cudaError_t launch_norm(const T *u, long long N, double *partials, int nparts, cudaStream_t s);
+// max|u| and sum u^2 (deterministic), then the bins, in one launch; sc must be
+// zero before (its blocks_done counts the blocks), partials holds 2 norm_parts().
 struct BinArgs {
     int L;
     double c[kMaxLevels + 1];
@@ -102,8 +101,8 @@ struct BinArgs {
     double eps;
     long long N;
 };
-cudaError_t launch_bins(const BinArgs &ba, const double *partials, int nparts, Scalars *sc,
-                        cudaStream_t s);
+template <typename T>
+cudaError_t launch_norm(const T *u, long long N, double *partials, const BinArgs &ba, Scalars *sc, cudaStream_t s);
 
 // Transposes: dense level-l array from a coarse array through (x)_k M_l P
 template <typename T>
