@@ -50,11 +50,15 @@ solve_strided_kernel(T *b, int n, long long stride, long long nlines, const T *_
 // One thread per line, 32 adjacent lines per warp (every step one coalesced
 // row), the line swept in place in global memory: the loads of the next sixteen
 // steps are in flight while the current sixteen are computed; the Thomas
-// factors sit in shared memory.
+// factors sit in shared memory.  Blocks of two warps: the sweeps are bound by
+// the recurrence, in binary64 by the FP64 pipe of the SMs that hold a line, so
+// lines have to spread over all SMs (256 threads before: 65 -> 56 us for the
+// finest level of 500x500x100 in binary64).
 constexpr int kSolvePre = 16;
+constexpr int kSolveThreads = 64;
 
 template <typename T>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(kSolveThreads)
 solve_stream_kernel(T *b, int n, long long st, long long ostride, long long ninner, long long nlines,
                     const T *__restrict__ sub, const T *__restrict__ cp, const T *__restrict__ inv_den)
 {
@@ -136,106 +140,165 @@ __device__ __forceinline__ void cp_async_wait_all()
     asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
 }
 
-// 32 lines per CTA, staged in shared memory as [n][32]: line i's element t at
-// base + t*st + i (the 32 lines are contiguous), so every load and store of a
-// step t is one coalesced 128-byte row; one warp then runs the 32 sweeps.
-template <typename T>
-__global__ void __launch_bounds__(128)
-solve_tile_kernel(T *b, int n, long long st, long long ostride, int ninner,
-                  const T *__restrict__ sub, const T *__restrict__ cp, const T *__restrict__ inv_den)
+// U steps of a Thomas sweep from step t0 on, every load issued before the
+// recurrence (in a plain loop each load waits for the store before it): forward
+// y_t = (p_t - sub_t y) inv_t in place, backward x_t = p_t - cp_t x down from t0
+// with fin(t, x) taking the solution.  One warp's chain is bound by its issue
+// rate, so the steps carry no bound checks.
+template <int U, typename T>
+__device__ __forceinline__ T sweep_fwd(T *p, int st, const T *sub, const T *inv, int t0, T y)
 {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    T *S = reinterpret_cast<T *>(smem_raw);
-    T *csub = S + n * 32, *ccp = csub + n, *cinv = ccp + n;   // Thomas factors, staged
-    for (int t = threadIdx.x; t < n; t += blockDim.x) { csub[t] = sub[t]; ccp[t] = cp[t]; cinv[t] = inv_den[t]; }
-    const int nblk = (ninner + 31) >> 5;
-    const long long o = blockIdx.x / nblk;
-    const int jb = (int)(blockIdx.x - o * nblk);
-    const int nl = min(32, ninner - jb * 32);
-    T *base = b + o * ostride + (long long)jb * 32;
-    for (int idx = threadIdx.x; idx < n * 32; idx += blockDim.x) {
-        const int t = idx >> 5, i = idx & 31;
-        if (i < nl) cp_async_elem(&S[idx], base + (long long)t * st + i);
-    }
-    cp_async_wait_all();
-    __syncthreads();
-    if ((int)threadIdx.x < nl) {
-        T *p = S + threadIdx.x;
-        T y = (T)0;
-        for (int t = 0; t < n; t++) { y = mul_rn(fma_rn(-csub[t], y, p[t * 32]), cinv[t]); p[t * 32] = y; }
-        T x = (T)0;
-        for (int t = n - 1; t >= 0; t--) { x = fma_rn(-ccp[t], x, p[t * 32]); p[t * 32] = x; }
-    }
-    __syncthreads();
-    for (int idx = threadIdx.x; idx < n * 32; idx += blockDim.x) {
-        const int t = idx >> 5, i = idx & 31;
-        if (i < nl) base[(long long)t * st + i] = S[idx];
-    }
+    T v[U], f[U], g[U];
+#pragma unroll
+    for (int u = 0; u < U; u++) { v[u] = p[(t0 + u) * st]; f[u] = sub[t0 + u]; g[u] = inv[t0 + u]; }
+#pragma unroll
+    for (int u = 0; u < U; u++) { y = mul_rn(fma_rn(-f[u], y, v[u]), g[u]); p[(t0 + u) * st] = y; }
+    return y;
+}
+template <int U, typename T, typename Fin>
+__device__ __forceinline__ T sweep_bwd(const T *p, int st, const T *cp, int t0, T x, Fin fin)
+{
+    T v[U], f[U];
+#pragma unroll
+    for (int u = 0; u < U; u++) { v[u] = p[(t0 - u) * st]; f[u] = cp[t0 - u]; }
+#pragma unroll
+    for (int u = 0; u < U; u++) { x = fma_rn(-f[u], x, v[u]); v[u] = x; }
+    fin(t0, v);
+    return x;
+}
+// both sweeps of a line of n nodes; fin(t, x): x[u] is the solution at t - u
+template <typename T, typename Fin>
+__device__ __forceinline__ void sweep_line(T *p, int st, int n, const T *sub, const T *cp, const T *inv, Fin fin)
+{
+    constexpr int U = sizeof(T) == 4 ? 8 : 4;
+    T y = (T)0;
+    int t = 0;
+    for (; t + U <= n; t += U) y = sweep_fwd<U>(p, st, sub, inv, t, y);
+    if (U > 4 && t + 4 <= n) { y = sweep_fwd<4>(p, st, sub, inv, t, y); t += 4; }
+    for (; t < n; t++) y = sweep_fwd<1>(p, st, sub, inv, t, y);
+    T x = (T)0;
+    t = n - 1;
+    for (; t + 1 >= U; t -= U) x = sweep_bwd<U>(p, st, cp, t, x, [&](int q, const T(&v)[U]) { fin(q, v); });
+    if (U > 4 && t + 1 >= 4) { x = sweep_bwd<4>(p, st, cp, t, x, [&](int q, const T(&v)[4]) { fin(q, v); }); t -= 4; }
+    for (; t >= 0; t--) x = sweep_bwd<1>(p, st, cp, t, x, [&](int q, const T(&v)[1]) { fin(q, v); });
 }
 
+// a contiguous run of cnt elements between global and shared memory in 16-byte
+// pieces, single elements at its ends; dst and src agree modulo 16 bytes
+__device__ __forceinline__ void cp_async16(void *dst_smem, const void *src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst_smem)), "l"(src) : "memory");
+}
 template <typename T>
-__global__ void __launch_bounds__(256)
-solve_contig_kernel(T *b, int n, long long nlines, int rows, int pitch, const T *__restrict__ sub,
-                    const T *__restrict__ cp, const T *__restrict__ inv_den, T *vc, int sign)
+__device__ __forceinline__ int run_head(const T *g, int cnt)
+{
+    const int h = (int)((16 - ((uintptr_t)g & 15)) & 15) / (int)sizeof(T);
+    return h < cnt ? h : cnt;
+}
+template <typename T>
+__device__ __forceinline__ void run_load(T *dst, const T *src, int cnt)
+{
+    constexpr int V = 16 / sizeof(T);
+    const int h = run_head(src, cnt), nv = (cnt - h) / V;
+    for (int i = threadIdx.x; i < nv; i += blockDim.x) cp_async16(dst + h + i * V, src + h + i * V);
+    if ((int)threadIdx.x < h) cp_async_elem(dst + threadIdx.x, src + threadIdx.x);
+    for (int i = h + nv * V + threadIdx.x; i < cnt; i += blockDim.x) cp_async_elem(dst + i, src + i);
+}
+template <typename T>
+__device__ __forceinline__ void run_store(T *dst, const T *src, int cnt)
+{
+    constexpr int V = 16 / sizeof(T);
+    const int h = run_head(dst, cnt), nv = (cnt - h) / V;
+#pragma unroll 4
+    for (int i = threadIdx.x; i < nv; i += blockDim.x)
+        *reinterpret_cast<uint4 *>(dst + h + i * V) = *reinterpret_cast<const uint4 *>(src + h + i * V);
+    if ((int)threadIdx.x < h) dst[threadIdx.x] = src[threadIdx.x];
+    for (int i = h + nv * V + threadIdx.x; i < cnt; i += blockDim.x) dst[i] = src[i];
+}
+
+// Contiguous lines: a tile of up to 32 lines, one lane of a warp each, with the
+// tile of v_c that takes the result beside it.  A tile is one contiguous run of
+// memory, so both tiles arrive by 16-byte asynchronous copies in flight together
+// and leave by 16-byte stores: element-wise copies and a read-modify-write of v_c
+// after the sweeps kept the kernel at 2.4 TB/s.  Lines of 257: 84 -> 60 us at
+// 513^3 (204 MB), lines of 129: 19 -> 10 us.
+// The lines keep the pitch n they have in memory, so the lanes of a warp meet in
+// gcd(n, 32) words of a bank: where n is a multiple of kContigLag, lane i runs i
+// steps behind, which makes the stride between lanes odd (not below that: the
+// lag adds 31 steps with bound checks, and 2- and 4-fold conflicts cost less).
+constexpr int kContigRows = 32;
+constexpr int kContigLag = 8;
+constexpr int kContigThreads = 128;
+constexpr size_t kContigMaxKb = 220;
+template <typename T>
+__global__ void __launch_bounds__(kContigThreads)
+solve_contig_kernel(T *b, int n, long long nlines, int rows, const T *__restrict__ sub, const T *__restrict__ cp,
+                    const T *__restrict__ inv_den, T *vc, int sign)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    T *S = reinterpret_cast<T *>(smem_raw);
-    T *csub = S + (size_t)rows * pitch, *ccp = csub + n, *cinv = ccp + n;
-    for (int t = threadIdx.x; t < n; t += blockDim.x) { csub[t] = sub[t]; ccp[t] = cp[t]; cinv[t] = inv_den[t]; }
-    const long long row0 = blockIdx.x * (long long)rows;
-    const int nr = (int)min((long long)rows, nlines - row0);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
-    // one warp per row: coalesced, no per-element division
-    for (int r = warp; r < nr; r += nwarp) {
-        const T *srow = b + (row0 + r) * n;
-        T *drow = S + r * pitch;
-        for (int t = lane; t < n; t += 32) cp_async_elem(&drow[t], srow + t);
+    constexpr int V = 16 / sizeof(T);
+    T *csub = reinterpret_cast<T *>(smem_raw), *ccp = csub + n, *cinv = ccp + n;
+    T *tile = csub + (3 * n + V - 1) / V * V;
+    const long long row0 = blockIdx.x * (long long)rows, first = row0 * n;
+    const int nr = (int)min((long long)rows, nlines - row0), cnt = nr * n;
+    T *B = tile + ((uintptr_t)(b + first) & 15) / sizeof(T);
+    run_load(B, b + first, cnt);
+    T *X = B;
+    if (sign != 0) {
+        X = tile + (rows * n + 2 * V - 1) / V * V + ((uintptr_t)(vc + first) & 15) / sizeof(T);
+        run_load(X, vc + first, cnt);
     }
+    for (int t = threadIdx.x; t < n; t += blockDim.x) { csub[t] = sub[t]; ccp[t] = cp[t]; cinv[t] = inv_den[t]; }
     cp_async_wait_all();
     __syncthreads();
     if ((int)threadIdx.x < nr) {
-        T *p = S + threadIdx.x * pitch;
-        T y = (T)0;
-#pragma unroll 8
-        for (int t = 0; t < n; t++) { y = mul_rn(fma_rn(-csub[t], y, p[t]), cinv[t]); p[t] = y; }
-        T x = (T)0;
-#pragma unroll 8
-        for (int t = n - 1; t >= 0; t--) { x = fma_rn(-ccp[t], x, p[t]); p[t] = x; }
-    }
-    __syncthreads();
-    if (sign == 0) {
-        for (int r = warp; r < nr; r += nwarp) {
-            const T *srow = S + r * pitch;
-            const long long g0 = (row0 + r) * n;
-            for (int t = lane; t < n; t += 32) b[g0 + t] = srow[t];
-        }
-        return;
-    }
-    // the read-modify-write of vc: a warp's elements j (row warp + nwarp (j / nk),
-    // column lane + 32 (j mod nk)) in batches of U, every load of a batch
-    // issued before its stores, so U loads per lane are in flight
-    const int nk = (n + 31) / 32;
-    const int rows_w = nr > warp ? (nr - warp + nwarp - 1) / nwarp : 0;
-    const int nj = rows_w * nk;
-    constexpr int U = sizeof(T) == 4 ? 12 : 8;
-    for (int j0 = 0; j0 < nj; j0 += U) {
-        T old[U];
+        T *p = B + threadIdx.x * n, *xo = X + threadIdx.x * n;
+        if (n % kContigLag) {
+            sweep_line<T>(p, 1, n, csub, ccp, cinv, [&](int t, const auto &v) {
+                constexpr int U = sizeof(v) / sizeof(T);
+                T old[U];
+                if (sign != 0) {
 #pragma unroll
-        for (int u = 0; u < U; u++) {
-            const int j = j0 + u, q = j / nk, t = lane + 32 * (j - q * nk);
-            old[u] = (j < nj && t < n) ? vc[(row0 + warp + (long long)q * nwarp) * n + t] : (T)0;
-        }
+                    for (int u = 0; u < U; u++) old[u] = xo[t - u];
+                }
 #pragma unroll
-        for (int u = 0; u < U; u++) {
-            const int j = j0 + u, q = j / nk, t = lane + 32 * (j - q * nk);
-            if (j < nj && t < n) {
-                const int r = warp + q * nwarp;
-                const T z = S[r * pitch + t];
-                const long long g = (row0 + r) * n + t;
-                vc[g] = sign > 0 ? add_rn(old[u], z) : sub_rn(old[u], z);
+                for (int u = 0; u < U; u++)
+                    xo[t - u] = sign == 0 ? v[u] : sign > 0 ? add_rn(old[u], v[u]) : sub_rn(old[u], v[u]);
+            });
+        } else {
+            const int lag = (int)threadIdx.x;
+            constexpr int U = 8;
+            T y = (T)0;
+            for (int k0 = -lag; k0 < n; k0 += U) {
+                T v[U], f[U], g[U];
+#pragma unroll
+                for (int u = 0; u < U; u++) {
+                    const int t = min(max(k0 + u, 0), n - 1);
+                    v[u] = p[t]; f[u] = csub[t]; g[u] = cinv[t];
+                }
+#pragma unroll
+                for (int u = 0; u < U; u++)
+                    if (k0 + u >= 0 && k0 + u < n) { y = mul_rn(fma_rn(-f[u], y, v[u]), g[u]); p[k0 + u] = y; }
+            }
+            T x = (T)0;
+            for (int k0 = n - 1 + lag; k0 >= 0; k0 -= U) {
+                T v[U], f[U], old[U];
+#pragma unroll
+                for (int u = 0; u < U; u++) {
+                    const int t = min(max(k0 - u, 0), n - 1);
+                    v[u] = p[t]; f[u] = ccp[t]; old[u] = xo[t];
+                }
+#pragma unroll
+                for (int u = 0; u < U; u++)
+                    if (k0 - u >= 0 && k0 - u < n) {
+                        x = fma_rn(-f[u], x, v[u]);
+                        xo[k0 - u] = sign == 0 ? x : sign > 0 ? add_rn(old[u], x) : sub_rn(old[u], x);
+                    }
             }
         }
     }
+    __syncthreads();
+    run_store(sign == 0 ? b + first : vc + first, X, cnt);
 }
 
 // --------------------------------------------------------------------------
@@ -589,46 +652,13 @@ __device__ __forceinline__ void coarse_restrict(const CoarseDim<T> &d, int n0, i
     __syncthreads();
 }
 
-// Thomas sweeps of one line p[0], p[st], ...; fin(t, x) takes the solution
-template <typename T, typename Fin>
-__device__ __forceinline__ void coarse_line(const CoarseDim<T> &d, T *p, int st, Fin fin)
-{
-    constexpr int U = sizeof(T) == 4 ? 8 : 4;
-    const int n = d.mc;
-    const T *sub = d.sub, *inv = d.inv, *cp = d.cp;
-    T y = (T)0;
-#pragma unroll 1
-    for (int t0 = 0; t0 < n; t0 += U) {
-        T v[U], f[U], g[U];
-#pragma unroll
-        for (int u = 0; u < U; u++) {
-            const int t = min(t0 + u, n - 1);
-            v[u] = p[t * st]; f[u] = sub[t]; g[u] = inv[t];
-        }
-#pragma unroll
-        for (int u = 0; u < U; u++)
-            if (t0 + u < n) { y = mul_rn(fma_rn(-f[u], y, v[u]), g[u]); p[(t0 + u) * st] = y; }
-    }
-    T x = (T)0;
-#pragma unroll 1
-    for (int t0 = n - 1; t0 >= 0; t0 -= U) {
-        T v[U], f[U];
-#pragma unroll
-        for (int u = 0; u < U; u++) {
-            const int t = max(t0 - u, 0);
-            v[u] = p[t * st]; f[u] = cp[t];
-        }
-#pragma unroll
-        for (int u = 0; u < U; u++)
-            if (t0 - u >= 0) { x = fma_rn(-f[u], x, v[u]); fin(t0 - u, x); }
-    }
-}
-
 // b = (x)_k P^T M_l W, then z = (x)_k M_{l-1}^{-1} b in place (R2, R1, B
-// scratch); fin(j, j0, j1, t, z) takes z at the coarse node (j0, j1, t) of flat
-// index j (the dimension-2 sweep always runs: a field's last dimension is active)
-template <typename T, typename Fin>
-__device__ __forceinline__ void coarse_correct(const CoarseDim<T> *d, const T *W, T *R2, T *R1, T *B, Fin fin)
+// scratch).  out[j] = sign z + base at the coarse node (j0, j1, t) of flat index
+// j, with base read at base0(j0, j1) + at(t) (the dimension-2 sweep always runs:
+// a field's last dimension is active)
+template <typename T, bool SUB, typename Base, typename At>
+__device__ __forceinline__ void coarse_correct(const CoarseDim<T> *d, const T *W, T *R2, T *R1, T *B, T *out, Base base0,
+                                               At at)
 {
     const int c0 = d[0].mc, c1 = d[1].mc, c2 = d[2].mc, m0 = d[0].m, m1 = d[1].m;
     // an inactive dimension (one node) keeps its values: no pass
@@ -640,7 +670,10 @@ __device__ __forceinline__ void coarse_correct(const CoarseDim<T> *d, const T *W
         const int pl = c1 * c2;
         for (int i = threadIdx.x; i < pl; i += blockDim.x) {
             T *p = rhs + i;
-            coarse_line<T>(d[0], p, pl, [&](int t, T x) { p[t * pl] = x; });
+            sweep_line<T>(p, pl, c0, d[0].sub, d[0].cp, d[0].inv, [&](int t, const auto &v) {
+#pragma unroll
+                for (int u = 0; u < (int)(sizeof(v) / sizeof(T)); u++) p[(t - u) * pl] = v[u];
+            });
         }
         __syncthreads();
     }
@@ -648,13 +681,25 @@ __device__ __forceinline__ void coarse_correct(const CoarseDim<T> *d, const T *W
         for (int i = threadIdx.x; i < c0 * c2; i += blockDim.x) {
             const int j0 = small_div(i, d[2].cmul);
             T *p = rhs + j0 * c1 * c2 + (i - j0 * c2);
-            coarse_line<T>(d[1], p, c2, [&](int t, T x) { p[t * c2] = x; });
+            sweep_line<T>(p, c2, c1, d[1].sub, d[1].cp, d[1].inv, [&](int t, const auto &v) {
+#pragma unroll
+                for (int u = 0; u < (int)(sizeof(v) / sizeof(T)); u++) p[(t - u) * c2] = v[u];
+            });
         }
         __syncthreads();
     }
     for (int i = threadIdx.x; i < c0 * c1; i += blockDim.x) {
         const int j0 = small_div(i, d[1].cmul), j1 = i - j0 * c1;
-        coarse_line<T>(d[2], rhs + i * c2, 1, [&](int t, T x) { fin(i * c2 + t, j0, j1, t, x); });
+        const T *src = base0(j0, j1);
+        T *dst = out + i * c2;
+        sweep_line<T>(rhs + i * c2, 1, c2, d[2].sub, d[2].cp, d[2].inv, [&](int t, const auto &v) {
+            constexpr int U = sizeof(v) / sizeof(T);
+            T old[U];
+#pragma unroll
+            for (int u = 0; u < U; u++) old[u] = src[at(t - u)];
+#pragma unroll
+            for (int u = 0; u < U; u++) dst[t - u] = SUB ? sub_rn(old[u], v[u]) : add_rn(old[u], v[u]);
+        });
     }
     __syncthreads();
 }
@@ -772,9 +817,10 @@ __device__ __forceinline__ void coarse_body(const CoarseArgs<T> &a)
             }
             __syncthreads();
             // 2.-3.
-            coarse_correct<T>(d, W, R2, R1, B, [&](int j, int j0, int j1, int t, T z) {
-                Vn[j] = add_rn(V[(cpos_of(m0, c0, j0) * m1 + cpos_of(m1, c1, j1)) * m2 + cpos_of(m2, c2, t)], z);
-            });
+            coarse_correct<T, false>(
+                d, W, R2, R1, B, Vn,
+                [&](int j0, int j1) { return V + (cpos_of(m0, c0, j0) * m1 + cpos_of(m1, c1, j1)) * m2; },
+                [&](int t) { return cpos_of(m2, c2, t); });
             T *t = V; V = Vn; Vn = t;
         }
     } else {
@@ -811,7 +857,8 @@ __device__ __forceinline__ void coarse_body(const CoarseArgs<T> &a)
                 coarse_new_nodes<T>(c, j, m1, m2, c1, c2, [&](int, int off, int so) { W[base + off] = value(np + so, l); });
             }
             __syncthreads();
-            coarse_correct<T>(d, W, R2, R1, B, [&](int j, int, int, int, T z) { VK[j] = sub_rn(V[j], z); });
+            coarse_correct<T, true>(
+                d, W, R2, R1, B, VK, [&](int j0, int j1) { return V + (j0 * c1 + j1) * c2; }, [&](int t) { return t; });
             auto expand = [&](T *dst) {
 #pragma unroll 1
                 for (int i = tid; i < c0 * c1 * c2; i += nt) {
@@ -885,8 +932,6 @@ cudaError_t launch_restrict(WSrc src, Sink sink, const RestrictArgs<T> &a, cudaS
     return launch_restrict_planes<T>(src, a, s);
 }
 
-constexpr bool kSolveStream = true;   // strided dimensions: streaming sweeps
-
 template <typename T>
 cudaError_t launch_solves(const LevelGeom<T> &g, T *b, T *vc, int sign, cudaStream_t s)
 {
@@ -899,29 +944,15 @@ cudaError_t launch_solves(const LevelGeom<T> &g, T *b, T *vc, int sign, cudaStre
         int sg = (k == last) ? sign : 0;
         // the streaming sweep keeps the three factor tables in shared memory
         // (at most the default 48 KB); longer lines take the strided kernel
-        if (k < 2 && sg == 0 && kSolveStream && 3 * (size_t)d.mc * sizeof(T) <= 48 * 1024) {
+        if (k < 2 && sg == 0 && 3 * (size_t)d.mc * sizeof(T) <= 48 * 1024) {
             // dim 0: lines (j1, j2), step c1*c2; dim 1: lines (j0, j2), step c2
             const long long st = (k == 0) ? c1 * c2 : c2;
             const long long outer = (k == 0) ? c1 : c0;
             const long long ostride = (k == 0) ? c2 : c1 * c2;
             const long long nlines = outer * c2;
-            solve_stream_kernel<T><<<(unsigned)((nlines + 255) / 256), 256, 3 * (size_t)d.mc * sizeof(T), s>>>(
+            solve_stream_kernel<T><<<(unsigned)((nlines + kSolveThreads - 1) / kSolveThreads), kSolveThreads,
+                                     3 * (size_t)d.mc * sizeof(T), s>>>(
                 b, d.mc, st, ostride, c2, nlines, d.sub, d.cp, d.inv_den);
-        } else if (k < 2 && sg == 0 && (size_t)d.mc * 35 * sizeof(T) <= 160 * 1024) {
-            // dim 0: lines (j1, j2), step c1*c2; dim 1: lines (j0, j2), step c2
-            const long long st = (k == 0) ? c1 * c2 : c2;
-            const long long outer = (k == 0) ? c1 : c0;
-            const long long ostride = (k == 0) ? c2 : c1 * c2;
-            const int ninner = (int)c2;
-            static PerDeviceOnce attr;
-            cudaError_t ea = once_per_device(attr, [] {
-                return cudaFuncSetAttribute(solve_tile_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                            164 * 1024);
-            });
-            if (ea != cudaSuccess) return ea;
-            const long long grid = outer * ((ninner + 31) / 32);
-            solve_tile_kernel<T><<<(unsigned)grid, 128, (size_t)d.mc * 35 * sizeof(T), s>>>(
-                b, d.mc, st, ostride, ninner, d.sub, d.cp, d.inv_den);
         } else if (k < 2) {
             long long stride = (k == 0) ? c1 * c2 : c2;
             long long nlines = (k == 0) ? c1 * c2 : c0 * c2;
@@ -931,12 +962,12 @@ cudaError_t launch_solves(const LevelGeom<T> &g, T *b, T *vc, int sign, cudaStre
         } else {
             int n = d.mc;
             long long nlines = c0 * c1;
-            int pitch = n | 1;
-            size_t rowbytes = (size_t)pitch * sizeof(T);
-            // the row tile and the three factor tables share the 100 KB limit
-            const size_t tab = 3 * (size_t)n * sizeof(T);
-            const size_t budget = std::min<size_t>(90 * 1024, tab < 100 * 1024 ? 100 * 1024 - tab : 0);
-            int rows = (int)std::min<size_t>(64, budget / rowbytes);
+            // one tile of lines (two with v_c) and the three factor tables in 100 KB,
+            // two or three CTAs per SM; long lines take the SM's shared memory
+            const size_t line = (size_t)n * sizeof(T) * (sg ? 2 : 1), fixed = 3 * (size_t)n * sizeof(T) + 96;
+            const auto lines_in = [&](size_t kb) { return kb * 1024 > fixed ? (kb * 1024 - fixed) / line : 0; };
+            size_t rows = std::min<size_t>(kContigRows, lines_in(100));
+            if (rows < 8) rows = std::min<size_t>(8, lines_in(kContigMaxKb));
             if (rows < 1) {
                 solve_strided_kernel<T><<<(unsigned)((nlines + 255) / 256), 256, 0, s>>>(
                     b, n, 1, nlines, d.sub, d.cp, d.inv_den, vc, sg);
@@ -944,12 +975,11 @@ cudaError_t launch_solves(const LevelGeom<T> &g, T *b, T *vc, int sign, cudaStre
                 static PerDeviceOnce attr;
                 cudaError_t ea = once_per_device(attr, [] {
                     return cudaFuncSetAttribute(solve_contig_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                100 * 1024);
+                                                (int)(kContigMaxKb * 1024));
                 });
                 if (ea != cudaSuccess) return ea;
-                solve_contig_kernel<T><<<(unsigned)((nlines + rows - 1) / rows), 256,
-                                         rows * rowbytes + 3 * (size_t)n * sizeof(T), s>>>(
-                    b, n, nlines, rows, pitch, d.sub, d.cp, d.inv_den, vc, sg);
+                solve_contig_kernel<T><<<(unsigned)((nlines + rows - 1) / rows), kContigThreads, fixed + rows * line, s>>>(
+                    b, n, nlines, (int)rows, d.sub, d.cp, d.inv_den, vc, sg);
             }
         }
         count_launch();
