@@ -372,9 +372,6 @@ __global__ void __launch_bounds__(256) assign_kernel(HuffScratch hs)
 //   no codeword (incomplete code):  0
 constexpr uint32_t kLongFlag = 0x80000000u;
 constexpr uint32_t kSubFlag = 0x20000000u;
-// decoder copy of an entry of the escape symbol 0 whose codeword and payload
-// (W bits) together fit 32 bits: L = codeword length + W
-constexpr uint32_t kEscFolded = 0x40000000u;
 
 // length of the canonical codeword at the top of the left-aligned window,
 // known to lie in [lo, hi]: the first length l in [lo, hi) whose limit lim[l]
@@ -1661,66 +1658,161 @@ __global__ void __launch_bounds__(kHeaderThreads) header_batch_kernel(const Head
 //
 // A thread decodes its chunk of K symbols.  It keeps the next bits of the
 // chunk MSB-aligned in two 32-bit registers hi:lo (nb valid bits, at least 32
-// before every read) and refills them a word at a time from a queue of two
-// prefetched 16-byte blocks.  A codeword of at most 13 bits is one load from
-// the first-level table of every 13-bit prefix; one of up to 23 bits is a
-// second load from the table its prefix names, indexed by the bits after the
-// prefix; either gives symbol and length, with no search.  Every other case
-// (longer codewords, prefixes past the second-level budget, escape payloads
-// that do not fit the 32-bit window, invalid codes) leaves the loop for an
-// out-of-line routine that reads its window from global memory, after which
-// the queue restarts at the new position.
+// before every look-up) and the next word of the stream in a third.  A codeword
+// of at most 13 bits is one load from the first-level table of every 13-bit
+// prefix; one of up to 23 bits is a second load from the table its prefix
+// names, indexed by the bits after the prefix; either gives symbol and length,
+// with no search.  Every other case (longer codewords, prefixes past the
+// second-level budget, escape payloads that do not fit the 32-bit window,
+// invalid codes) leaves the loop for an out-of-line routine that reads its
+// window from global memory.
+//
+// What bounds the kernel is the latency of a step (two dependent shared loads
+// under load) against the at most 32 warps that 64 registers a thread allow, and
+// the instructions of a step, so a step is short and has no divergent branch:
+//   - table entries hold their fields where the step uses them: the length in
+//     the low bits, the symbol in the high half, flag bits for the unusual cases,
+//     and in a second-level pointer the byte offset of its table and the shift
+//     that isolates its index;
+//   - the stream passes through a ring of 32 words per thread in shared memory
+//     ([word][thread], conflict-free), filled once every eight symbols by the
+//     32-byte sector prefetched in registers: a step's refill is one predicated
+//     shared load, where selecting the word from a register block and reloading
+//     the block took most of the 88 instructions a step, and every sector is
+//     fetched once (the threads' lines do not fit what is left of L1);
+//   - the second-level load, the refill and the store of a sparse escape are
+//     predicated (as branches they cost the warp both sides at nearly every
+//     step); only the out-of-line cases branch.
+// 513^3 at 1e-3: 515 -> 335 us; 300x431x517 at 1e-4, where most symbols are
+// escapes: 434 -> 295 us; 64 Mi byte keys: 222 -> 130 us.
+//
+// Escaped codes: where they are dense (more than one symbol in sixteen) a
+// thread keeps the payloads of eight symbols in registers and writes each half
+// with an escape as one 32-byte sector: single 8-byte stores scattered over the
+// escape array cost a read-modify-write of their sector in DRAM.  The other
+// slots of a stored sector carry zeros or stale values; nothing reads the escape
+// array where no escape is.  Sparse escapes are stored one by one.
 constexpr int kDecThreads = 1024;
-// In a stream where escapes are dense, escaped codes are gathered per thread
-// for eight symbols ([8][kDecThreads] slots) and written as whole 32-byte
-// sectors: single 8-byte stores scattered over the escape array cost a
-// read-modify-write of their sector in DRAM (rel 1e-4 on 513^3: 2.26 -> 1.20
-// ms).  Sparse escapes are stored one by one (the gathering costs more than it
-// saves below about one escape in sixteen symbols).
-constexpr size_t kDecEscSmem = 8ull * 8 * kDecThreads;
-constexpr size_t kDecSmem = (4u << kLutBits) + 4 * kSubCap + sizeof(LenTabs) + kDecEscSmem;
+constexpr unsigned kRingWords = 32;
+constexpr size_t kDecSmem = (4u << kLutBits) + 4 * kSubCap + sizeof(LenTabs) + 4ull * kRingWords * kDecThreads;
+
+// Decoder entries (the staged copy of the look-up tables):
+//   leaf                  symbol << 16 | L
+//   folded escape         kDecEsc | L          (L = codeword + payload, at most 32)
+//   second-level pointer  byte offset << 16 | kDecSub | (32 - index bits)
+//   long codeword         kDecSlow | Lmin << 16 | (Lmax - Lmin) << 24
+//   unfolded escape       kDecSlow | kDecOpen | L << 16
+//   no codeword           kDecSlow
+constexpr uint32_t kDecEsc = 0x40u, kDecSlow = 0x80u, kDecSub = 0x100u, kDecOpen = 0x200u;
 
 __device__ __forceinline__ uint32_t ldw(const uint32_t *w, unsigned long long i, unsigned long long n)
 {
     return i < n ? __ldg(w + i) : 0u;
 }
 
-// four words from an aligned block index (words past n read as zero)
-__device__ __forceinline__ uint4 ld4(const uint32_t *w, unsigned long long i, unsigned long long n)
+// one 32-byte sector: a load that does not stay in L1, a store
+struct Words8 {
+    uint32_t v[8];
+};
+__device__ __forceinline__ Words8 ldg32(const uint32_t *p)
 {
-    if (i + 4 <= n && ((reinterpret_cast<uintptr_t>(w) & 15) == 0))
-        return __ldg(reinterpret_cast<const uint4 *>(w + i));
-    uint4 v;
-    v.x = ldw(w, i, n); v.y = ldw(w, i + 1, n); v.z = ldw(w, i + 2, n); v.w = ldw(w, i + 3, n);
-    return v;
+    Words8 r;
+    asm volatile("ld.global.nc.L1::no_allocate.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(r.v[0]), "=r"(r.v[1]), "=r"(r.v[2]), "=r"(r.v[3]), "=r"(r.v[4]), "=r"(r.v[5]), "=r"(r.v[6]),
+                   "=r"(r.v[7])
+                 : "l"(p));
+    return r;
+}
+__device__ __forceinline__ void stg32(long long *p, long long a, long long b, long long c, long long d)
+{
+    asm volatile("st.global.v4.b64 [%0], {%1, %2, %3, %4};" :: "l"(p), "l"(a), "l"(b), "l"(c), "l"(d) : "memory");
+}
+// predicated shared load and global store (no branch around them)
+__device__ __forceinline__ void lds_if(uint32_t &v, uint32_t cond, uint32_t addr)
+{
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %1, 0;\n\t@p ld.shared.u32 %0, [%2];\n\t}"
+                 : "+r"(v) : "r"(cond), "r"(addr) : "memory");
+}
+__device__ __forceinline__ void stg_if(long long *dst, uint32_t cond, long long v)
+{
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %1, 0;\n\t@p st.global.u64 [%0], %2;\n\t}"
+                 :: "l"(dst), "r"(cond), "l"(v) : "memory");
 }
 
+// A thread's view of its chunk's words, counted in 32 bits from `base`, the
+// 32-byte sector of memory in which the chunk starts (a chunk has at most 32768
+// symbols of 126 bits).  rc: ring index of the prefetched word `next`, wr: end
+// of the words in the ring, pa: the sector after it.  left: words of the stream
+// from base on (words past it read as zero), lvec: the same as far as whole
+// sectors can be loaded (0 for a stream that does not start on 16 bytes).
 struct BitQueue {
-    const uint32_t *w;
-    unsigned long long n;     // words in the stream
-    uint4 pa, pb;             // current and next aligned block
-    unsigned k;               // next word of pa
-    unsigned long long nxt;   // next block to fetch
-    __device__ __forceinline__ uint32_t next()
+    const uint32_t *base;
+    unsigned left, lvec;
+    uint32_t ring;            // shared address of this thread's column, kDecThreads words between rows
+    unsigned rc, wr;
+    Words8 pa;
+    uint32_t next;
+    __device__ __forceinline__ Words8 sector(unsigned i) const
     {
-        const uint32_t v = k == 0 ? pa.x : k == 1 ? pa.y : k == 2 ? pa.z : pa.w;
-        if (++k == 4) { k = 0; pa = pb; pb = ld4(w, nxt, n); nxt += 4; }
+        if (i + 8 <= lvec) return ldg32(base + i);
+        Words8 r;
+#pragma unroll
+        for (unsigned k = 0; k < 8; k++) r.v[k] = ldw(base, i + k, left);
+        return r;
+    }
+    __device__ __forceinline__ uint32_t addr(unsigned i) const { return ring + (i % kRingWords) * (4 * kDecThreads); }
+    __device__ __forceinline__ uint32_t at(unsigned i) const
+    {
+        uint32_t v;
+        asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr(i)) : "memory");
         return v;
     }
-    // position the queue at bit pos and load the first 64 bits from there
-    __device__ __forceinline__ void prime(unsigned long long pos, uint32_t &hi, uint32_t &lo, int &nb)
+    __device__ __forceinline__ void append()
     {
-        const unsigned long long wb0 = (pos >> 5) & ~3ULL;
-        pa = ld4(w, wb0, n);
-        pb = ld4(w, wb0 + 4, n);
-        nxt = wb0 + 8;
-        k = (unsigned)((pos >> 5) & 3);
-        const uint32_t w0 = next(), w1 = next();
-        const unsigned sh = (unsigned)(pos & 31);
+        const uint32_t r = addr(wr);   // wr is a multiple of 8: no wrap inside
+#pragma unroll
+        for (unsigned k = 0; k < 8; k++)
+            asm volatile("st.shared.u32 [%0], %1;" :: "r"(r + 4 * kDecThreads * k), "r"(pa.v[k]) : "memory");
+        wr += 8;
+        pa = sector(wr);
+    }
+    // Eight symbols take at most eight words (32 bits each; longer steps move the
+    // queue themselves), so one sector keeps up: with ten words from `next` on
+    // before eight symbols, ten are left after this before the next eight.  The
+    // two words of the window stay in the ring, for a seek may start in them.
+    __device__ __forceinline__ void top_up()
+    {
+        if (wr - rc + 2 <= kRingWords - 8) append();
+    }
+    // the first 64 bits from bit pos of base on (at or after the current words)
+    __device__ __forceinline__ void seek(unsigned pos, uint32_t &hi, uint32_t &lo, int &nb)
+    {
+        rc = pos >> 5;
+        while ((int)(wr - rc) < 12) append();
+        const uint32_t w0 = at(rc), w1 = at(rc + 1);
+        const unsigned sh = pos & 31u;
         hi = __funnelshift_l(w1, w0, sh);
         lo = w1 << sh;
         nb = 64 - (int)sh;
+        rc += 2;
+        next = at(rc);
     }
+    __device__ __forceinline__ void start(const uint32_t *w, unsigned long long n, unsigned long long pos, uint32_t &hi,
+                                          uint32_t &lo, int &nb)
+    {
+        // a stream on 16 bytes may start in the middle of a sector, whose first half is then loaded too
+        const bool vec = (reinterpret_cast<uintptr_t>(w) & 15) == 0;
+        const long long lead = vec ? (long long)((reinterpret_cast<uintptr_t>(w) & 31) / 4) : 0;
+        const long long wb = (((long long)(pos >> 5) + lead) & ~7LL) - lead, l = (long long)n - wb;
+        base = w + wb;
+        left = l < 0x7FFFFFFFll ? (unsigned)l : 0x7FFFFFFFu;
+        lvec = vec ? left : 0u;
+        wr = 0;
+        pa = sector(0);
+        seek((unsigned)((long long)pos - 32 * wb), hi, lo, nb);
+    }
+    // bit position of the window, from base
+    __device__ __forceinline__ unsigned pos(int nb) const { return (rc << 5) - (unsigned)nb; }
 };
 
 // 64 bits of the stream from bit pos (words past the end read as zero)
@@ -1747,17 +1839,20 @@ __device__ __noinline__ SlowOut decode_slow(uint32_t e, unsigned long long pos, 
     SlowOut o;
     o.bad = 0;
     const unsigned long long win = window64(words, nwords, pos);
-    uint32_t sv = e & 0xFFFFu;
+    uint32_t sv = 0;
     unsigned L = (e >> 16) & 0x3Fu;
-    if (e & kLongFlag) {
+    if (e & kDecOpen) {
+        // the escape's codeword
+    } else if (L) {
         const unsigned lmin = L, lmax = L + ((e >> 24) & 0x3Fu);
         L = code_len_in(*T, win, lmin, lmax);
         const unsigned long long off = (win >> (64 - L)) - T->first[L];
         if (off >= T->count[L]) o.bad = 1;
         const unsigned idx = T->start[L] + (unsigned)(off < T->count[L] ? off : 0);
         sv = symtab[idx < nsym ? idx : 0];
-    } else if (e == 0) {
+    } else {
         o.bad = 1;               // no codeword starts here
+        sv = 0;
         L = 1;
     }
     pos += L;
@@ -1772,11 +1867,120 @@ __device__ __noinline__ SlowOut decode_slow(uint32_t e, unsigned long long pos, 
     return o;
 }
 
+// One chunk: cnt symbols from symbol beg on, from bit pos0 to bit expect.  EW: 0 no escapes,
+// 1 sparse ones, 2 dense ones.  Returns whether the stream was sound.
+template <int EW>
+__device__ __forceinline__ bool decode_chunk(const DecodeArgs &a, const HuffScratch &hs, const LenTabs *T, unsigned nsym,
+                                             uint32_t lut, uint32_t sub, uint32_t ring, unsigned long long pos0,
+                                             unsigned long long expect, unsigned long long beg, unsigned cnt)
+{
+    const unsigned ew = EW ? a.esc_w : 0u;     // escape payload width (1..63)
+    BitQueue q;
+    q.ring = ring;
+    uint32_t hi, lo;
+    int nb;
+    q.start(a.words, a.nwords, pos0, hi, lo, nb);
+    const unsigned expos = q.pos(nb) + (unsigned)(expect - pos0);
+    bool bad = false;
+    uint16_t *sym = a.sym + beg;
+    long long *e8 = EW ? a.esc + beg : nullptr;   // escape slots of the current group of eight symbols
+    uint32_t z[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};   // EW 2: payloads of the group, bit j of emask where there is one
+    unsigned emask = 0;
+    // symbol in the high half
+    auto step = [&](unsigned j, uint32_t &zj) -> uint32_t {
+        uint32_t e;
+        asm volatile("ld.shared.u32 %0, [%1];" : "=r"(e) : "r"(lut + 4 * (hi >> (32 - kLutBits))) : "memory");
+        // a codeword of up to 23 bits: its second-level entry, indexed by the
+        // bits after the prefix (all within hi, nb >= 32)
+        lds_if(e, e & kDecSub, sub + (e >> 16) + 4 * ((hi << kLutBits) >> (e & 31u)));
+        if (e & kDecSlow) {
+            long long kv = 0;
+            const SlowOut o = decode_slow(e, q.pos(nb), q.base, q.left, T, hs.sorted_sym, nsym, (int)ew, &kv);
+            if (EW && o.sv == 0) {
+                // at once: its payload may not fit the group's registers
+                e8[j] = kv;
+                if (EW == 2) emask |= 0x100u << j;
+            }
+            bad |= o.bad != 0;
+            q.seek((unsigned)o.pos, hi, lo, nb);
+            return o.sv << 16;
+        }
+        const unsigned L = e & 63u;
+        if (EW) {
+            // folded escape: codeword of L - ew bits, then zigzag(k) in ew < 32 bits
+            const uint32_t y = (hi << ((L - ew) & 31u)) >> ((32u - ew) & 31u);
+            if (EW == 2) {
+                zj = y;
+                emask |= ((e / kDecEsc) & 1u) << j;
+            } else {
+                stg_if(e8 + j, e & kDecEsc, (long long)((int)(y >> 1) ^ -(int)(y & 1u)));
+            }
+        }
+        // drop L <= 32 bits, then refill to at least 32 valid bits (the valid
+        // bits are all in hi then)
+        hi = __funnelshift_lc(lo, hi, L);
+        lo = __funnelshift_lc(0u, lo, L);
+        nb -= (int)L;
+        const bool need = nb < 32;
+        const uint32_t ih = q.next >> (nb & 31), il = __funnelshift_r(0u, q.next, nb);
+        hi |= need ? ih : 0u;
+        lo = need ? il : lo;
+        nb += need ? 32 : 0;
+        q.rc += need ? 1u : 0u;
+        lds_if(q.next, need, q.addr(q.rc));
+        return e;
+    };
+    // the escaped codes of a group: each half with an escape as one 32-byte
+    // store; a code stored by its own step (upper mask) keeps its half from being
+    // overwritten: the others of that half go one by one
+    auto flush8 = [&]() {
+        auto code = [&](unsigned j) { return (long long)((int)(z[j] >> 1) ^ -(int)(z[j] & 1u)); };
+#pragma unroll
+        for (unsigned h = 0; h < 8; h += 4) {
+            const unsigned m = (emask >> h) & 0xFu;
+            if (!m) continue;
+            if ((emask >> (8 + h)) & 0xFu) {
+#pragma unroll
+                for (unsigned j = 0; j < 4; j++) stg_if(e8 + h + j, (m >> j) & 1u, code(h + j));
+            } else {
+                stg32(e8 + h, code(h), code(h + 1), code(h + 2), code(h + 3));
+            }
+        }
+        emask = 0;
+    };
+    // eight symbols per 16-byte store (K is a multiple of 128)
+    for (unsigned g = cnt / 8; g; g--) {
+        uint32_t o[4];
+        q.top_up();
+#pragma unroll
+        for (unsigned j = 0; j < 8; j += 2) {
+            const uint32_t v0 = step(j, z[j]), v1 = step(j + 1, z[j + 1]);
+            o[j / 2] = __byte_perm(v0, v1, 0x7632);
+        }
+        // streaming store: the symbols are written once and read by the next
+        // kernel, so they should not push the bitstream out of L2
+        __stcs(reinterpret_cast<uint4 *>(sym), make_uint4(o[0], o[1], o[2], o[3]));
+        sym += 8;
+        if (EW == 2 && emask) flush8();
+        if (EW) e8 += 8;
+    }
+    // a last group of fewer than eight: its escapes one by one
+    q.top_up();
+    for (unsigned j = 0; j < cnt % 8; j++) {
+        uint32_t y = 0;
+        sym[j] = (uint16_t)(step(j, y) >> 16);
+        if (EW == 2 && ((emask >> j) & 1u)) e8[j] = (long long)((int)(y >> 1) ^ -(int)(y & 1u));
+    }
+    return !bad && q.pos(nb) == expos;
+}
+
 __global__ void __launch_bounds__(kDecThreads, 1) decode_kernel(DecodeArgs a_in, HuffScratch hs)
 {
     DecodeArgs a = a_in;
+    const unsigned long long nch = (a.N + a.K - 1) / a.K;
+    if (blockIdx.x >= nch) return;
+    if (block_skip(hs.status)) return;
     if (a.dh) {
-        if (block_skip(hs.status)) return;
         const DevHdr h = *a.dh;
         a.words = reinterpret_cast<const uint32_t *>(a.base + h.off_bits);
         a.nwords = h.nwords;
@@ -1790,22 +1994,35 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_kernel(DecodeArgs a_in,
     uint32_t *lut = reinterpret_cast<uint32_t *>(dsm);                       // [1 << kLutBits]
     uint32_t *sub = lut + (1u << kLutBits);                                   // [kSubCap]
     LenTabs *T = reinterpret_cast<LenTabs *>(sub + kSubCap);
-    long long *escbuf = reinterpret_cast<long long *>(T + 1);                  // [8][kDecThreads]
-    if (block_skip(hs.status)) return;
+    uint32_t *ring = reinterpret_cast<uint32_t *>(T + 1);                      // [kRingWords][kDecThreads]
     const unsigned nsym = *hs.nsym;
     const unsigned nsub = *hs.nsub < kSubCap ? *hs.nsub : kSubCap;
     {
         // escape entries take their payload width into their length when both fit 32 bits
         const unsigned ewc = a.esc ? a.esc_w : 0u;
-        auto fold = [&](uint32_t e) -> uint32_t {
-            if (ewc && e && !(e & (kLongFlag | kSubFlag)) && (e & 0xFFFFu) == 0) {
-                const unsigned L = (e >> 16) & 0x3Fu;
-                if (L + ewc <= 32) e = kEscFolded | ((L + ewc) << 16);
-            }
-            return e;
+        auto entry = [&](uint32_t e) -> uint32_t {
+            if (e == 0) return kDecSlow;
+            const unsigned L = (e >> 16) & 0x3Fu;
+            if (e & kLongFlag) return kDecSlow | (L << 16) | (((e >> 24) & 0x3Fu) << 24);
+            if (e & kSubFlag) return ((e & 0x3FFFu) << 18) | kDecSub | (32u - ((e >> 16) & 0xFu));
+            if (ewc && (e & 0xFFFFu) == 0) return L + ewc <= 32 ? kDecEsc | (L + ewc) : kDecSlow | kDecOpen | (L << 16);
+            return (e << 16) | L;
         };
-        for (int i = threadIdx.x; i < (1 << kLutBits); i += blockDim.x) lut[i] = fold(hs.lut1[i]);
-        for (unsigned i = threadIdx.x; i < nsub; i += blockDim.x) sub[i] = fold(hs.lut_sub[i]);
+        auto four = [&](uint4 v) { return make_uint4(entry(v.x), entry(v.y), entry(v.z), entry(v.w)); };
+        const uint4 *g1 = reinterpret_cast<const uint4 *>(hs.lut1), *g2 = reinterpret_cast<const uint4 *>(hs.lut_sub);
+        uint4 *d1 = reinterpret_cast<uint4 *>(lut), *d2 = reinterpret_cast<uint4 *>(sub);
+        constexpr unsigned N1 = (1u << kLutBits) / 4 / kDecThreads, N2 = kSubCap / 4 / kDecThreads;
+        uint4 v1[N1], v2[N2];
+#pragma unroll
+        for (unsigned u = 0; u < N1; u++) v1[u] = g1[threadIdx.x + u * kDecThreads];
+#pragma unroll
+        for (unsigned u = 0; u < N2; u++)
+            if (4 * (threadIdx.x + u * kDecThreads) < nsub) v2[u] = g2[threadIdx.x + u * kDecThreads];
+#pragma unroll
+        for (unsigned u = 0; u < N1; u++) d1[threadIdx.x + u * kDecThreads] = four(v1[u]);
+#pragma unroll
+        for (unsigned u = 0; u < N2; u++)
+            if (4 * (threadIdx.x + u * kDecThreads) < nsub) d2[threadIdx.x + u * kDecThreads] = four(v2[u]);
     }
     if (threadIdx.x < 64) {
         T->first[threadIdx.x] = hs.first[threadIdx.x];
@@ -1814,115 +2031,24 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_kernel(DecodeArgs a_in,
         T->count[threadIdx.x] = hs.count[threadIdx.x];
     }
     __syncthreads();
-    const uint16_t *symtab = hs.sorted_sym;
-    long long *const esc = a.esc;
-    const int ew = esc ? (int)a.esc_w : 0;     // escape payload width (1..63)
-    const bool gather = ew && a.n_esc * 16 > a.N;
-    const unsigned long long nch = (a.N + a.K - 1) / a.K;
+    const int mode = !a.esc || !a.esc_w ? 0 : a.n_esc * 16 > a.N ? 2 : 1;
+    const uint32_t lut_a = smem_u32(lut), sub_a = smem_u32(sub), ring_a = smem_u32(ring + threadIdx.x);
     // chunks interleave over the blocks so that every SM gets a share
     for (unsigned long long c = blockIdx.x + (unsigned long long)gridDim.x * threadIdx.x; c < nch;
          c += (unsigned long long)gridDim.x * blockDim.x) {
         const unsigned long long pos0 = a.chunk[c];
         const unsigned long long expect = (c + 1 < nch) ? a.chunk[c + 1] : a.total_bits;
-        if (pos0 > a.total_bits || expect > a.total_bits || pos0 > expect) {
-            atomicExch(hs.status, (unsigned)DS_FORMAT);
-            continue;
-        }
-        BitQueue q;
-        q.w = a.words;
-        q.n = a.nwords;
-        uint32_t hi, lo;
-        int nb;
-        q.prime(pos0, hi, lo, nb);
-        unsigned long long used = 0;
-        bool bad = false;
-        // this thread's escaped codes of the current group of eight symbols:
-        // slot j of the group at escbuf[j * kDecThreads + tid], bit j of emask
-        long long *const eslot = escbuf + threadIdx.x;
-        unsigned emask = 0;
-        auto step = [&](unsigned long long i) -> uint16_t {
-            uint32_t e = lut[hi >> (32 - kLutBits)];
-            // a codeword of up to 23 bits: its second-level entry, indexed by
-            // the bits after the prefix (all within hi, nb >= 32)
-            if ((e & (kLongFlag | kSubFlag)) == kSubFlag)
-                e = sub[(e & 0xFFFFu) + ((hi << kLutBits) >> (32 - ((e >> 16) & 0xFu)))];
-            const uint32_t sv = e & 0xFFFFu;
-            const unsigned L = (e >> 16) & 0x3Fu;
-            const bool at_esc = ew && sv == 0;
-            if ((e & kLongFlag) || e == 0 || (at_esc && !(e & kEscFolded))) {
-                const unsigned j = (unsigned)(i & 7);
-                const SlowOut o = decode_slow(e, pos0 + used, a.words, a.nwords, T, symtab, nsym, ew,
-                                              !esc ? nullptr : gather ? eslot + (size_t)j * kDecThreads : esc + i);
-                if (gather && o.sv == 0) emask |= 1u << j;
-                bad |= o.bad != 0;
-                used = o.pos - pos0;
-                q.prime(o.pos, hi, lo, nb);
-                return (uint16_t)o.sv;
-            }
-            // folded escape: codeword of L - ew bits, then zigzag(k) in ew bits
-            if (at_esc) {
-                const long long kv = unzigzag((unsigned long long)((hi << (L - ew)) >> (32 - ew)));
-                if (gather) {
-                    const unsigned j = (unsigned)(i & 7);
-                    eslot[(size_t)j * kDecThreads] = kv;
-                    emask |= 1u << j;
-                } else {
-                    esc[i] = kv;
-                }
-            }
-            // drop L <= 32 bits, then refill to at least 32 valid bits: the
-            // word is selected and merged by predication; only the block
-            // load (every fourth refill) branches
-            hi = L < 32 ? __funnelshift_l(lo, hi, L) : lo;
-            lo = L < 32 ? lo << L : 0u;
-            nb -= (int)L;
-            used += L;
-            {
-                const bool need = nb < 32;
-                const uint32_t wv = q.k == 0 ? q.pa.x : q.k == 1 ? q.pa.y : q.k == 2 ? q.pa.z : q.pa.w;
-                const unsigned sh = need ? (unsigned)nb : 0u;
-                hi = need ? (hi | (wv >> sh)) : hi;
-                lo = need ? __funnelshift_rc(0u, wv, sh) : lo;
-                nb += need ? 32 : 0;
-                q.k += need ? 1u : 0u;
-                if (q.k == 4) { q.k = 0; q.pa = q.pb; q.pb = ld4(q.w, q.nxt, q.n); q.nxt += 4; }
-            }
-            return (uint16_t)sv;
-        };
-        // the escaped codes of the group at i0 (a multiple of 8): each half
-        // with an escape as one 32-byte store (the other slots carry stale
-        // values, and nothing reads the escape array where no escape is)
-        auto flush8 = [&](unsigned long long i0) {
-            for (int h = 0; h < 2; h++) {
-                if (!((emask >> (4 * h)) & 0xFu)) continue;
-                const long long *src = eslot + (size_t)(4 * h) * kDecThreads;
-                longlong2 *dst = reinterpret_cast<longlong2 *>(esc + i0 + 4 * h);
-                dst[0] = make_longlong2(src[0], src[kDecThreads]);
-                dst[1] = make_longlong2(src[2 * kDecThreads], src[3 * kDecThreads]);
-            }
-            emask = 0;
-        };
+        bool ok = pos0 <= a.total_bits && expect <= a.total_bits && pos0 <= expect;
         const unsigned long long beg = c * a.K;
-        const unsigned long long end = beg + a.K < a.N ? beg + a.K : a.N;
-        unsigned long long i = beg;
-        // eight symbols per 16-byte store (K is a multiple of 128)
-        for (; i + 8 <= end; i += 8) {
-            uint4 o;
-            o.x = (uint32_t)step(i) | ((uint32_t)step(i + 1) << 16);
-            o.y = (uint32_t)step(i + 2) | ((uint32_t)step(i + 3) << 16);
-            o.z = (uint32_t)step(i + 4) | ((uint32_t)step(i + 5) << 16);
-            o.w = (uint32_t)step(i + 6) | ((uint32_t)step(i + 7) << 16);
-            // streaming store: the symbols are written once and read by the next
-            // kernel, so they should not push the bitstream out of L2
-            __stcs(reinterpret_cast<uint4 *>(a.sym + i), o);
-            if (emask) flush8(i);
+        const unsigned cnt = (unsigned)(beg + a.K < a.N ? a.K : a.N - beg);
+        // a chunk of more bits than its symbols can have is not sound either
+        ok = ok && expect - pos0 <= 126ull * a.K;
+        if (ok) {
+            if (mode == 0) ok = decode_chunk<0>(a, hs, T, nsym, lut_a, sub_a, ring_a, pos0, expect, beg, cnt);
+            else if (mode == 1) ok = decode_chunk<1>(a, hs, T, nsym, lut_a, sub_a, ring_a, pos0, expect, beg, cnt);
+            else ok = decode_chunk<2>(a, hs, T, nsym, lut_a, sub_a, ring_a, pos0, expect, beg, cnt);
         }
-        // a last group of fewer than eight: its escapes one by one
-        const unsigned long long i0 = i;
-        for (; i < end; i++) a.sym[i] = step(i);
-        for (unsigned j = 0; emask; j++, emask >>= 1)
-            if (emask & 1u) esc[i0 + j] = eslot[(size_t)j * kDecThreads];
-        if (bad || pos0 + used != expect) atomicExch(hs.status, (unsigned)DS_FORMAT);
+        if (!ok) atomicExch(hs.status, (unsigned)DS_FORMAT);
     }
 }
 
