@@ -1049,8 +1049,6 @@ void lossless_layout(LosslessHdr *h)
     h->off_bits = a16(h->off_chunk + 8 * h->nch);
     h->total = h->off_bits + 4 * ((h->bits + 31) / 32);
 }
-void wr32(uint8_t *p, uint32_t v) { for (int i = 0; i < 4; i++) p[i] = (uint8_t)(v >> (8 * i)); }
-void wr64(uint8_t *p, uint64_t v) { for (int i = 0; i < 8; i++) p[i] = (uint8_t)(v >> (8 * i)); }
 uint32_t rd32l(const uint8_t *p) { uint32_t v = 0; for (int i = 0; i < 4; i++) v |= (uint32_t)p[i] << (8 * i); return v; }
 uint64_t rd64l(const uint8_t *p) { uint64_t v = 0; for (int i = 0; i < 8; i++) v |= (uint64_t)p[i] << (8 * i); return v; }
 
@@ -1435,68 +1433,58 @@ hpdr_status hpdr_lossless_compress(hpdr_ctx *ctx, const void *d_keys, uint64_t n
     DevGuard g(ctx->device);
     cudaStream_t s = (cudaStream_t)stream;
     const unsigned D = h.D;
+    // byte keys are counted and encoded where they are; a pointer that does not
+    // start on 16 bytes has them widened in the workspace first
+    const bool bytes = key_bytes == 1 && ((uintptr_t)d_keys & 15) == 0, widen = key_bytes == 1 && !bytes;
     Carver c(nullptr);
-    c.take<Scalars>(1); c.take<unsigned long long>(D); c.take<unsigned long long>(h.nch + 2);
-    c.take<unsigned long long>(1024); c.take<char>(huff_scratch_bytes(D));
-    if (key_bytes == 1) c.take<uint16_t>(n + 8);
+    const auto carve = [&](Carver &w, Scalars *&sc, unsigned long long *&hist, unsigned long long *&cb,
+                           unsigned long long *&bs, void *&hb, uint16_t *&wide) {
+        sc = w.take<Scalars>(1);
+        hist = w.take<unsigned long long>(D);
+        cb = w.take<unsigned long long>(h.nch + 2);
+        bs = w.take<unsigned long long>(1024);
+        hb = w.take<char>(huff_scratch_bytes(D));
+        wide = widen ? w.take<uint16_t>(n + 8) : nullptr;
+    };
+    Scalars *sc;
+    unsigned long long *hist, *cb, *bs;
+    void *hb;
+    uint16_t *wide;
+    carve(c, sc, hist, cb, bs, hb, wide);
     hpdr_status st = ensure_workspace(ctx, c.used + 256);
     if (st != HPDR_OK) return st;
     Carver w(ctx->ws.base);
-    Scalars *sc = w.take<Scalars>(1);
-    unsigned long long *hist = w.take<unsigned long long>(D);
-    unsigned long long *cb = w.take<unsigned long long>(h.nch + 2);
-    unsigned long long *bs = w.take<unsigned long long>(1024);
-    void *hb = w.take<char>(huff_scratch_bytes(D));
-    const uint16_t *sym = (const uint16_t *)d_keys;
-    if (key_bytes == 1) {
-        uint16_t *wide = w.take<uint16_t>(n + 8);
+    carve(w, sc, hist, cb, bs, hb, wide);
+    if (widen) {
         widen_keys_kernel<<<152 * 8, 256, 0, s>>>((const uint8_t *)d_keys, n, wide);
         count_launch();
         CK(cudaGetLastError());
-        sym = wide;
     }
     uint8_t *out = (uint8_t *)d_out;
-    CK(cudaMemsetAsync(sc, 0, sizeof(Scalars), s));
-    CK(cudaMemsetAsync(hist, 0, 8ULL * D, s));
-    CK(launch_histogram(sym, n, D, hist, &sc->status, s));
+    // the scalars and the histogram are neighbours in the workspace
+    CK(cudaMemsetAsync(sc, 0, (size_t)((char *)(hist + D) - (char *)sc), s));
+    if (bytes) CK(launch_histogram_bytes((const uint8_t *)d_keys, n, hist, s));
+    else CK(launch_histogram(widen ? wide : (const uint16_t *)d_keys, n, D, hist, &sc->status, s));
     HuffScratch hs;
     huff_scratch_carve(hb, D, sc, &hs);
     CK(launch_codebook(hist, D, hs, s));
     EncodeArgs ea;
     memset(&ea, 0, sizeof(ea));
-    ea.sym = sym; ea.N = n; ea.D = D; ea.K = h.K; ea.len = hs.len; ea.code = hs.code; ea.pack = hs.pack;
+    ea.sym = widen ? wide : d_keys; ea.bytes = bytes;
+    ea.N = n; ea.D = D; ea.K = h.K; ea.len = hs.len; ea.code = hs.code; ea.pack = hs.pack;
     ea.chunk_bits = cb; ea.sc = sc; ea.bsum = bs;
     ea.chunk_out = (unsigned long long *)(out + h.off_chunk);
     ea.words_out = (uint32_t *)(out + h.off_bits);
     ea.words_cap = (out_capacity - h.off_bits) / 4;
     CK(launch_encode(ea, s));
-    CK(cudaMemcpyAsync(out + kLosslessHdr, hs.len, D, cudaMemcpyDeviceToDevice, s));
+    LosslessHeader lh = {h.key_bytes, h.D, h.K, h.n, h.nch, h.off_chunk, h.off_bits};
+    CK(launch_lossless_header(lh, hs.len, sc, out, s));
     Scalars *hsc = (Scalars *)ctx->host_pinned;
     CK(cudaMemcpyAsync(hsc, sc, sizeof(Scalars), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
     if (hsc->status) return map_device_status(hsc->status);
     h.bits = hsc->total_bits;
     lossless_layout(&h);
-    if (h.total > out_capacity) return HPDR_ERR_CAPACITY;
-    uint8_t *hdr = (uint8_t *)ctx->host_pinned + 48 * 1024;
-    memset(hdr, 0, kLosslessHdr);
-    memcpy(hdr, "HPDL", 4);
-    wr32(hdr + 4, 1);
-    wr32(hdr + 8, h.key_bytes);
-    wr32(hdr + 12, h.D);
-    wr32(hdr + 16, h.K);
-    wr64(hdr + 24, h.n);
-    wr64(hdr + 32, h.bits);
-    wr64(hdr + 40, h.off_chunk);
-    wr64(hdr + 48, h.off_bits);
-    wr32(hdr + 60, crc32_host(hdr, 60));
-    CK(cudaMemcpyAsync(out, hdr, kLosslessHdr, cudaMemcpyHostToDevice, s));
-    // the gaps before the chunk table and the bitstream are zero
-    if (h.off_chunk > kLosslessHdr + D)
-        CK(cudaMemsetAsync(out + kLosslessHdr + D, 0, h.off_chunk - kLosslessHdr - D, s));
-    if (h.off_bits > h.off_chunk + 8 * h.nch)
-        CK(cudaMemsetAsync(out + h.off_chunk + 8 * h.nch, 0, h.off_bits - h.off_chunk - 8 * h.nch, s));
-    CK(cudaStreamSynchronize(s));
     *out_bytes = (size_t)h.total;
     return HPDR_OK;
 }
@@ -1518,14 +1506,17 @@ hpdr_status hpdr_lossless_decompress(hpdr_ctx *ctx, const void *d_in, size_t in_
     if (h.key_bytes == 2 && ((uintptr_t)d_keys & 15)) return HPDR_ERR_ARG;
     const unsigned D = h.D;
     Carver c(nullptr);
+    // bytes are decoded in place; a pointer that does not start on 8 bytes takes
+    // them from 16-bit symbols in the workspace
+    const bool bytes = h.key_bytes == 1 && ((uintptr_t)d_keys & 7) == 0, narrow = h.key_bytes == 1 && !bytes;
     c.take<Scalars>(1); c.take<char>(huff_scratch_bytes(D));
-    if (h.key_bytes == 1) c.take<uint16_t>(h.n + 8);
+    if (narrow) c.take<uint16_t>(h.n + 8);
     st = ensure_workspace(ctx, c.used + 256);
     if (st != HPDR_OK) return st;
     Carver w(ctx->ws.base);
     Scalars *sc = w.take<Scalars>(1);
     void *hsb = w.take<char>(huff_scratch_bytes(D));
-    uint16_t *sym = h.key_bytes == 1 ? w.take<uint16_t>(h.n + 8) : (uint16_t *)d_keys;
+    uint16_t *wide = narrow ? w.take<uint16_t>(h.n + 8) : nullptr;
     const uint8_t *in = (const uint8_t *)d_in;
     CK(cudaMemsetAsync(sc, 0, sizeof(Scalars), s));
     HuffScratch hs;
@@ -1537,10 +1528,10 @@ hpdr_status hpdr_lossless_decompress(hpdr_ctx *ctx, const void *d_in, size_t in_
     da.words = (const uint32_t *)(in + h.off_bits);
     da.nwords = (h.bits + 31) / 32;
     da.chunk = (const unsigned long long *)(in + h.off_chunk);
-    da.N = h.n; da.K = h.K; da.sym = sym; da.total_bits = h.bits; da.esc = nullptr; da.esc_w = 0;
+    da.N = h.n; da.K = h.K; da.sym = narrow ? wide : d_keys; da.bytes = bytes; da.total_bits = h.bits; da.esc = nullptr; da.esc_w = 0;
     CK(launch_decode(da, hs, s));
-    if (h.key_bytes == 1) {
-        narrow_keys_kernel<<<152 * 8, 256, 0, s>>>(sym, h.n, (uint8_t *)d_keys);
+    if (narrow) {
+        narrow_keys_kernel<<<152 * 8, 256, 0, s>>>(wide, h.n, (uint8_t *)d_keys);
         count_launch();
         CK(cudaGetLastError());
     }

@@ -98,7 +98,8 @@ cudaError_t launch_decode_tables(const TabArgs &a, const HuffScratch &hs, cudaSt
 // only known on the device: then pass the base and the Scalars-derived
 // offsets through ContainerLayout).
 struct EncodeArgs {
-    const uint16_t *sym;
+    const void *sym;                  // uint16 symbols, or bytes (bytes != 0; alphabets of 256), 16-byte aligned
+    int bytes;
     unsigned long long N;
     unsigned int D, K;
     const uint8_t *len;
@@ -159,7 +160,8 @@ struct DecodeArgs {
     const unsigned long long *chunk;  // chunk table (device)
     unsigned long long N, total_bits;
     unsigned int K;
-    uint16_t *sym;
+    void *sym;                        // uint16 symbols (16-byte aligned), or bytes (bytes != 0; 8-byte aligned)
+    int bytes = 0;
     long long *esc;                   // null: plain symbols; else receives k of every escape
     unsigned int esc_w;               // payload width of the escapes
     unsigned long long n_esc = 0;     // escapes in the stream (selects the escape stores)
@@ -169,6 +171,15 @@ struct DecodeArgs {
     const DevHdr *dh = nullptr;
 };
 cudaError_t launch_decode(const DecodeArgs &a, const HuffScratch &hs, cudaStream_t s);
+// histogram of n bytes (16-byte aligned), added to hist[256]
+cudaError_t launch_histogram_bytes(const uint8_t *in, unsigned long long n, unsigned long long *hist, cudaStream_t s);
+// the lossless container's header, code lengths and gaps (the bits come from sc)
+struct LosslessHeader {
+    unsigned key_bytes, D, K;
+    unsigned long long n, nch, off_chunk, off_bits;
+};
+cudaError_t launch_lossless_header(const LosslessHeader &h, const uint8_t *len, const Scalars *sc, uint8_t *out,
+                                   cudaStream_t s);
 cudaError_t launch_histogram(const uint16_t *sym, unsigned long long N, unsigned D,
                              unsigned long long *hist, unsigned *status, cudaStream_t s);
 

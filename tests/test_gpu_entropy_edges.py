@@ -45,3 +45,31 @@ def test_codebooks(oracle, present, top):
     assert np.array_equal(words.cpu().numpy().view(np.uint32), words_ref)
     dec = H.hpdr_huffman_decode(words, bits, chunk, sym.size, ln, D=D, K=K)
     assert np.array_equal(dec.cpu().numpy().view(np.uint16), sym)
+
+
+@pytest.mark.parametrize("n", [1, 7, 16, 33, 1023, 1024, 1025, 4099, 200003])
+@pytest.mark.parametrize("shift", [0, 1, 8])
+def test_byte_keys_in_place(oracle, n, shift):
+    """Byte keys counted, encoded and decoded as bytes, or through 16-bit
+    symbols where the pointer does not allow it (shift bytes into a buffer)."""
+    from paper_2503_06322_gb300 import hpdr as H
+    x = np.clip(np.round(np.random.default_rng(n).laplace(128, 6.0, size=n)), 0, 255).astype(np.uint8)
+    store = torch.zeros(n + 16, dtype=torch.uint8, device="cuda")
+    keys = store[shift:shift + n]
+    keys.copy_(torch.from_numpy(x))
+    out = torch.zeros(H.lossless_bound(n, 1, 128), dtype=torch.uint8, device="cuda")
+    buf = H.hpdr_lossless_compress(keys, K=128, out=out)
+    b = buf.cpu().numpy()
+    ln = oracle.code_lengths(oracle.histogram(x.astype(np.uint16), 256))
+    words, chunk, bits = oracle.encode(x.astype(np.uint16), ln, K=128)
+    off_chunk, off_bits = (int(v) for v in b[40:56].view(np.uint64))
+    assert b[:4].tobytes() == b"HPDL" and int(b[60:64].view(np.uint32)[0]) == oracle.crc32(b[:60].tobytes())
+    assert np.array_equal(b[64:320], ln) and int(b[32:40].view(np.uint64)[0]) == bits
+    assert np.array_equal(b[off_chunk:off_chunk + 8 * chunk.size].view(np.uint64), chunk)
+    assert not b[320:off_chunk].any() and not b[off_chunk + 8 * chunk.size:off_bits].any()
+    assert np.array_equal(b[off_bits:].view(np.uint32), words)
+    back = torch.full((n + 16,), 7, dtype=torch.uint8, device="cuda")
+    H.hpdr_lossless_decompress(buf, out=back[shift:shift + n])
+    got = back.cpu().numpy()
+    assert np.array_equal(got[shift:shift + n], x)
+    assert (got[:shift] == 7).all() and (got[shift + n:] == 7).all()
