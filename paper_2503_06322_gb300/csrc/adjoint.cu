@@ -10,92 +10,132 @@
 //     h = g_{c_l} + E_new^T ((x)M_l P) (x)M_{l-1}^{-1} g_{v_{l-1}},
 //     g_{v_l} = E_new h + E_kept (g_{v_{l-1}} - P^T E_new h).
 // P^T is the restriction kernel with the interpolation taps, M_{l-1}^{-1} the
-// Thomas solves, and (x)M_l P is applied one dimension at a time below.
+// Thomas solves, and (x)M_l P runs in one pass over the fine grid below.
 #include <cstring>
 #include "internal.cuh"
 #include "levels.cuh"
+#include "levels_dev.cuh"
 
 namespace hpdr {
 namespace {
 
-enum { MP_PLAIN = 0, MP_RT_FINAL = 1, MP_DT_FINAL = 2 };
+enum { MP_RT_FINAL = 1, MP_DT_FINAL = 2 };
 
-// out (dims s0 x s1 x s2) = (M_l P) along dim k of in (dim k of size mc_k).
-// Final modes (k = 0, output on the level-l grid):
-//   MP_RT_FINAL: stream[rank(p)] = gsrc[p] - value   at the new nodes
-//   MP_DT_FINAL: out[p] = coef[rank(p)] + value       at the new nodes
-// One warp per output row (i0, i1), lanes along i2: the row's dimension-0
-// and dimension-1 indices, the taps of a dimension-0 or -1 pass and, in the
-// final modes, whether the row holds only new nodes and where its new nodes
-// start in the stream are computed once per row; every load and store is
-// coalesced along i2 (the kept rows of a kept plane write every other stream
-// slot: only odd i2 are new there).
+// y_f = (x)_k M_l P_k y on the level-l grid, only at its new nodes:
+//   MP_RT_FINAL: stream[rank(p)] = gsrc[p] - y_f(p)
+//   MP_DT_FINAL: out[p] = coef[rank(p)] + y_f(p)
+// One pass over the fine grid is all it needs from memory (a pass per dimension,
+// through two partial grids, moved 2.6 times the bytes and took 173 us for the
+// finest level of 257^3, this 78).  A warp owns coarse row j1 of a tile,
+// lane l coarse column j2, and the CTA marches along the coarse planes of its
+// segment; for each plane a lane forms the dimension-2, then the dimension-1
+// products at its 2 x 2 fine nodes (rows Ra, Ra + 1, columns Ca, Ca + 1) from the
+// four rows and four columns of y around it (cached loads, coalesced per row)
+// and keeps the last three planes' for the dimension-0 products.  Every value
+// sums its taps in a fixed order, so nothing depends on the tiling.
 constexpr int kMpWarps = 8;
 template <typename T, int MODE>
 __global__ void __launch_bounds__(32 * kMpWarps)
-mass_prolong_kernel(const T *__restrict__ in, T *__restrict__ out, long long s0, long long s1, long long s2, int k,
-                    int mck, const T *__restrict__ etap, const int *__restrict__ efirst, LevelGeom<T> g,
-                    const T *__restrict__ gsrc, T *__restrict__ stream, const T *__restrict__ coef)
+prolong_kernel(LevelGeom<T> g, const T *__restrict__ y, const T *__restrict__ gsrc, T *__restrict__ stream,
+               const T *__restrict__ coef, T *__restrict__ out, int seg_len)
 {
-    const long long rows = s0 * s1;
-    const long long in1 = (k == 1) ? mck : s1, in2 = (k == 2) ? mck : s2;
-    const int lane = threadIdx.x & 31;
-    for (long long row = blockIdx.x * (long long)kMpWarps + (threadIdx.x >> 5); row < rows;
-         row += (long long)gridDim.x * kMpWarps) {
-        const long long i0 = row / s1, i1 = row - i0 * s1;
-        // dimension-0 or -1 pass: the row's taps
-        int rj0 = 0;
-        T rt[3] = {(T)0, (T)0, (T)0};
-        if (k != 2) {
-            const long long pr = (k == 0) ? i0 : i1;
-            rj0 = efirst[pr];
+    const DimTables<T> &d0 = g.dim[0], &d1 = g.dim[1], &d2 = g.dim[2];
+    const int m0 = d0.m, m1 = d1.m, m2 = d2.m, mc0 = d0.mc, mc1 = d1.mc, mc2 = d2.mc;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int j2 = blockIdx.x * 32 + lane, j1 = blockIdx.y * kMpWarps + warp;
+    const int J0a = blockIdx.z * seg_len, J0b = min(J0a + seg_len, mc0);
+    if (J0a >= J0b || j1 >= mc1 || j2 >= mc2) return;
+    const int Ca = cpos_of(m2, mc2, j2), Ra = cpos_of(m1, mc1, j1);
+    const bool hb = Ca + 1 < m2 && !kept_pos(m2, Ca + 1), hr = Ra + 1 < m1 && !kept_pos(m1, Ra + 1);
+    // taps of the two fine columns and rows; the second ones start at the same
+    // coarse index or one later
+    T e2[2][3], e1[2][3];
+    const int c2 = d2.efirst[Ca], c1 = d1.efirst[Ra];
+    const bool s2 = hb && d2.efirst[Ca + 1] != c2, s1 = hr && d1.efirst[Ra + 1] != c1;
 #pragma unroll
-            for (int i = 0; i < 3; i++) rt[i] = etap[pr * 3 + i];
-        }
-        bool rownew = true;
-        long long sbase = 0;
-        if (MODE != MP_PLAIN) {
-            const int p0 = (int)i0, p1 = (int)i1;
-            const bool k0 = kept_pos(g.dim[0].m, p0), k1 = kept_pos(g.dim[1].m, p1);
-            rownew = !k0 || !k1;
-            long long cr = (long long)kept_before(p0) * g.dim[1].mc * g.dim[2].mc;
-            if (k0) cr += (long long)kept_before(p1) * g.dim[2].mc;
-            sbase = g.Nprev + row * s2 - cr;
-        }
-        // four columns per lane in flight (the buffers do not alias)
-#pragma unroll 4
-        for (long long i2 = lane; i2 < s2; i2 += 32) {
-            const long long idx = row * s2 + i2;
-            int j0;
-            T tp[3];
-            if (k == 2) {
-                j0 = efirst[i2];
+    for (int i = 0; i < 3; i++) {
+        e2[0][i] = d2.etap[Ca * 3 + i];
+        e2[1][i] = hb ? d2.etap[(Ca + 1) * 3 + i] : (T)0;
+        e1[0][i] = d1.etap[Ra * 3 + i];
+        e1[1][i] = hr ? d1.etap[(Ra + 1) * 3 + i] : (T)0;
+    }
+    const int nc2 = mc2 - c2, nc1 = mc1 - c1;   // columns and rows from the first on
+    const long long cplane = (long long)mc1 * mc2;
+    struct D4 { T v[2][2]; };
+    // dimension-2 and -1 products of coarse plane j at the lane's nodes
+    auto plane = [&](int j) -> D4 {
+        const T *p = y + j * cplane + (long long)c1 * mc2 + c2;
+        T r2[4][2];   // rows c1.., the two columns
 #pragma unroll
-                for (int i = 0; i < 3; i++) tp[i] = etap[i2 * 3 + i];
-            } else {
-                j0 = rj0;
+        for (int r = 0; r < 4; r++) {
+            T x[4];
 #pragma unroll
-                for (int i = 0; i < 3; i++) tp[i] = rt[i];
-            }
-            T v = (T)0;
+            for (int c = 0; c < 4; c++) x[c] = r < nc1 && c < nc2 ? p[r * mc2 + c] : (T)0;
+            T a = (T)0, b = (T)0;
 #pragma unroll
             for (int i = 0; i < 3; i++) {
-                const int j = j0 + i;
-                if (j < mck) {
-                    const long long a0 = (k == 0) ? j : i0, a1 = (k == 1) ? j : i1, a2 = (k == 2) ? j : i2;
-                    v = fma_rn(tp[i], in[(a0 * in1 + a1) * in2 + a2], v);
-                }
+                if (i < nc2) a = fma_rn(e2[0][i], x[i], a);
+                if (i + (s2 ? 1 : 0) < nc2) b = fma_rn(e2[1][i], s2 ? x[i + 1] : x[i], b);
             }
-            if (MODE == MP_PLAIN) {
-                out[idx] = v;
-            } else {
-                const int p2 = (int)i2;
-                if (!rownew && kept_pos(g.dim[2].m, p2)) continue;
-                const long long si = sbase + i2 - (rownew ? 0 : kept_before(p2));
-                if (MODE == MP_RT_FINAL) stream[si] = sub_rn(gsrc[idx], v);
-                else out[idx] = add_rn(coef[si], v);
+            r2[r][0] = a;
+            r2[r][1] = b;
+        }
+        D4 d;
+#pragma unroll
+        for (int c = 0; c < 2; c++) {
+            T a = (T)0, b = (T)0;
+#pragma unroll
+            for (int i = 0; i < 3; i++) {
+                if (i < nc1) a = fma_rn(e1[0][i], r2[i][c], a);
+                if (i + (s1 ? 1 : 0) < nc1) b = fma_rn(e1[1][i], s1 ? r2[i + 1][c] : r2[i][c], b);
+            }
+            d.v[0][c] = a;
+            d.v[1][c] = b;
+        }
+        return d;
+    };
+    // fine plane P from the products A, B, C of coarse planes j - 1, j, j + 1: its
+    // three taps start at plane j - 1, or one later (the start of the grid, a new
+    // plane) or earlier (its end), where the tap that falls outside is zero
+    D4 A, B, C;
+    auto emit = [&](int P, int j) {
+        const bool k0 = kept_pos(m0, P);
+        const int o = d0.efirst[P] - (j - 1);
+        const T *e = d0.etap + P * 3;
+        const T tA = o == 0 ? e[0] : o < 0 ? e[1] : (T)0, tB = o == 0 ? e[1] : o < 0 ? e[2] : e[0];
+        const T tC = o == 0 ? e[2] : o < 0 ? (T)0 : e[1];
+        const bool useA = j > 0 && o <= 0, useC = j + 1 < mc0 && o >= 0;
+        const long long cr = (long long)kept_before(P) * cplane;
+#pragma unroll
+        for (int r = 0; r < 2; r++) {
+            if (r && !hr) continue;
+            const int R = Ra + r;
+            const bool rownew = !k0 || r;
+            const long long row = ((long long)P * m1 + R) * m2;
+            const long long sb = g.Nprev + row - cr - (k0 ? (long long)kept_before(R) * mc2 : 0LL);
+#pragma unroll
+            for (int c = 0; c < 2; c++) {
+                if ((c && !hb) || (!rownew && !c)) continue;
+                T v = (T)0;
+                if (useA) v = fma_rn(tA, A.v[r][c], v);
+                v = fma_rn(tB, B.v[r][c], v);
+                if (useC) v = fma_rn(tC, C.v[r][c], v);
+                const long long si = sb + (rownew ? Ca + c : (Ca >> 1));
+                if (MODE == MP_RT_FINAL) stream[si] = sub_rn(gsrc[row + Ca + c], v);
+                else out[row + Ca + c] = add_rn(coef[si], v);
             }
         }
+    };
+    A = plane(J0a > 0 ? J0a - 1 : 0);
+    B = J0a > 0 ? plane(J0a) : A;
+    for (int j = J0a; j < J0b; j++) {
+        if (j + 1 < mc0) C = plane(j + 1);
+        const int P = cpos_of(m0, mc0, j);
+        emit(P, j);
+        // the new plane between j and j + 1
+        if (P + 1 < m0 && !kept_pos(m0, P + 1)) emit(P + 1, j);
+        A = B;
+        B = C;
     }
 }
 
@@ -133,27 +173,17 @@ __global__ void copy_kernel(T *dst, const T *src, long long n)
 }
 
 unsigned grid_for(long long n) { return (unsigned)std::min<long long>((n + 255) / 256, 152LL * 16); }
-// rows of kMpWarps warps per block, capped at 16 blocks per SM
-unsigned grid_rows(long long rows) { return (unsigned)std::min<long long>((rows + kMpWarps - 1) / kMpWarps, 152LL * 16); }
 
-// y_f = (x)_k M_l P_k y, the last dimension-0 pass in a final mode
 template <typename T, int MODE>
-cudaError_t mass_prolong_all(const LevelGeom<T> &g, const T *y, T *t1, T *t2, T *out, const T *gsrc,
-                             T *stream, const T *coef, cudaStream_t s)
+cudaError_t launch_prolong(const LevelGeom<T> &g, const T *y, T *out, const T *gsrc, T *stream, const T *coef,
+                           cudaStream_t s)
 {
-    const long long m0 = g.dim[0].m, m1 = g.dim[1].m, m2 = g.dim[2].m;
-    const long long c0 = g.dim[0].mc, c1 = g.dim[1].mc;
-    // dim 2: c0 x c1 x c2 -> c0 x c1 x m2
-    constexpr int B = 32 * kMpWarps;
-    mass_prolong_kernel<T, MP_PLAIN><<<grid_rows(c0 * c1), B, 0, s>>>(y, t1, c0, c1, m2, 2, g.dim[2].mc, g.dim[2].etap,
-                                                                     g.dim[2].efirst, g, nullptr, nullptr, nullptr);
-    // dim 1: -> c0 x m1 x m2
-    mass_prolong_kernel<T, MP_PLAIN><<<grid_rows(c0 * m1), B, 0, s>>>(t1, t2, c0, m1, m2, 1, g.dim[1].mc, g.dim[1].etap,
-                                                                     g.dim[1].efirst, g, nullptr, nullptr, nullptr);
-    // dim 0: -> m0 x m1 x m2, final
-    mass_prolong_kernel<T, MODE><<<grid_rows(m0 * m1), B, 0, s>>>(t2, out, m0, m1, m2, 0, g.dim[0].mc, g.dim[0].etap,
-                                                                 g.dim[0].efirst, g, gsrc, stream, coef);
-    count_launch(3);
+    const int mc0 = g.dim[0].mc, mc1 = g.dim[1].mc, mc2 = g.dim[2].mc;
+    const int gx = (mc2 + 31) / 32, gy = (mc1 + kMpWarps - 1) / kMpWarps;
+    const int seg = choose_segment(mc0, (long long)gx * gy, resident_ctas(prolong_kernel<T, MODE>, 32 * kMpWarps, 0));
+    prolong_kernel<T, MODE><<<dim3(gx, gy, (mc0 + seg - 1) / seg), 32 * kMpWarps, 0, s>>>(g, y, gsrc, stream, coef, out,
+                                                                                       seg);
+    count_launch();
     return cudaGetLastError();
 }
 
@@ -161,7 +191,7 @@ cudaError_t mass_prolong_all(const LevelGeom<T> &g, const T *y, T *t1, T *t2, T 
 
 template <typename T>
 cudaError_t recompose_adjoint_run(const Plan &P, const LevelGeom<T> *geo, const T *gu, T *gcoef, T *ga, T *gb,
-                                  T *y, T *t1, T *t2, unsigned *status, cudaStream_t s)
+                                  T *y, unsigned *status, cudaStream_t s)
 {
     const int L = P.L;
     const T *gl = gu;
@@ -178,12 +208,9 @@ cudaError_t recompose_adjoint_run(const Plan &P, const LevelGeom<T> *geo, const 
         a.status = status;
         cudaError_t e = launch_restrict<T>(WSrc::DENSE, Sink::NONE, a, s);
         if (e != cudaSuccess) return e;
-        const long long nc = P.N[l - 1];
-        copy_kernel<T><<<grid_for(nc), 256, 0, s>>>(y, gc, nc);
-        count_launch();
-        e = launch_solves<T>(g, y, nullptr, 0, s);
+        e = launch_solves<T>(g, y, nullptr, 0, s, gc);
         if (e != cudaSuccess) return e;
-        e = mass_prolong_all<T, MP_RT_FINAL>(g, y, t1, t2, nullptr, gl, gcoef, nullptr, s);
+        e = launch_prolong<T, MP_RT_FINAL>(g, y, nullptr, gl, gcoef, nullptr, s);
         if (e != cudaSuccess) return e;
         gl = gc;
     }
@@ -194,7 +221,7 @@ cudaError_t recompose_adjoint_run(const Plan &P, const LevelGeom<T> *geo, const 
 
 template <typename T>
 cudaError_t decompose_adjoint_run(const Plan &P, const LevelGeom<T> *geo, const T *gcoef, T *gu, T *ga, T *gb,
-                                  T *y, T *t1, T *t2, T *R, unsigned *status, cudaStream_t s)
+                                  T *y, T *R, unsigned *status, cudaStream_t s)
 {
     const int L = P.L;
     T *gv = (L == 0) ? gu : ((L % 2 == 1) ? ga : gb);
@@ -204,12 +231,10 @@ cudaError_t decompose_adjoint_run(const Plan &P, const LevelGeom<T> *geo, const 
         const LevelGeom<T> &g = geo[l];
         T *G = (l == L) ? gu : (((L - l) % 2 == 1) ? ga : gb);
         const long long nc = P.N[l - 1];
-        copy_kernel<T><<<grid_for(nc), 256, 0, s>>>(y, gv, nc);
-        count_launch();
-        cudaError_t e = launch_solves<T>(g, y, nullptr, 0, s);
+        cudaError_t e = launch_solves<T>(g, y, nullptr, 0, s, gv);
         if (e != cudaSuccess) return e;
         // new nodes: G = h = g_c + ((x)M_l P) y
-        e = mass_prolong_all<T, MP_DT_FINAL>(g, y, t1, t2, G, nullptr, nullptr, gcoef, s);
+        e = launch_prolong<T, MP_DT_FINAL>(g, y, G, nullptr, nullptr, gcoef, s);
         if (e != cudaSuccess) return e;
         // kept nodes: G = gv - P^T E_new h
         RestrictArgs<T> a;
@@ -229,17 +254,12 @@ cudaError_t decompose_adjoint_run(const Plan &P, const LevelGeom<T> *geo, const 
     return cudaGetLastError();
 }
 
-template cudaError_t recompose_adjoint_run<float>(const Plan &, const LevelGeom<float> *, const float *, float *,
-                                                  float *, float *, float *, float *, float *, unsigned *,
-                                                  cudaStream_t);
-template cudaError_t recompose_adjoint_run<double>(const Plan &, const LevelGeom<double> *, const double *,
-                                                   double *, double *, double *, double *, double *, double *,
-                                                   unsigned *, cudaStream_t);
-template cudaError_t decompose_adjoint_run<float>(const Plan &, const LevelGeom<float> *, const float *, float *,
-                                                  float *, float *, float *, float *, float *, float *,
-                                                  unsigned *, cudaStream_t);
-template cudaError_t decompose_adjoint_run<double>(const Plan &, const LevelGeom<double> *, const double *,
-                                                   double *, double *, double *, double *, double *, double *,
-                                                   double *, unsigned *, cudaStream_t);
+#define INST(T)                                                                                                    \
+    template cudaError_t recompose_adjoint_run<T>(const Plan &, const LevelGeom<T> *, const T *, T *, T *, T *, T *, \
+                                                  unsigned *, cudaStream_t);                                       \
+    template cudaError_t decompose_adjoint_run<T>(const Plan &, const LevelGeom<T> *, const T *, T *, T *, T *, T *, \
+                                                  T *, unsigned *, cudaStream_t);
+INST(float)
+INST(double)
 
 }  // namespace hpdr

@@ -736,30 +736,22 @@ template <typename T>
 hpdr_status adjoint_t(hpdr_ctx *ctx, const Plan *P, const T *in, T *out, bool recompose, cudaStream_t s)
 {
     const int L = P->L;
-    size_t n1 = L >= 1 ? (size_t)P->N[L - 1] : 1, t1n = 1, t2n = 1;
-    for (int l = 1; l <= L; l++) {
-        const size_t c0 = P->m[0][l - 1], c1 = P->m[1][l - 1], m1 = P->m[1][l], m2 = P->m[2][l];
-        t1n = std::max(t1n, c0 * c1 * m2);
-        t2n = std::max(t2n, c0 * m1 * m2);
-    }
+    const size_t n1 = L >= 1 ? (size_t)P->N[L - 1] : 1;
     Carver c(nullptr);
     c.take<Scalars>(1);
     for (int i = 0; i < 4; i++) c.take<T>(n1);
-    c.take<T>(t1n);
-    c.take<T>(t2n);
     hpdr_status st = ensure_workspace(ctx, c.used + 256);
     if (st != HPDR_OK) return st;
     Carver w(ctx->ws.base);
     Scalars *sc = w.take<Scalars>(1);
     T *ga = w.take<T>(n1), *gb = w.take<T>(n1), *y = w.take<T>(n1), *R = w.take<T>(n1);
-    T *t1 = w.take<T>(t1n), *t2 = w.take<T>(t2n);
     CK(cudaMemsetAsync(sc, 0, sizeof(Scalars), s));
     if (recompose) {
         ProfScope ps(ctx, "adj_recompose", s);
-        CK(recompose_adjoint_run<T>(*P, geos<T>(P), in, out, ga, gb, y, t1, t2, &sc->status, s));
+        CK(recompose_adjoint_run<T>(*P, geos<T>(P), in, out, ga, gb, y, &sc->status, s));
     } else {
         ProfScope ps(ctx, "adj_decompose", s);
-        CK(decompose_adjoint_run<T>(*P, geos<T>(P), in, out, ga, gb, y, t1, t2, R, &sc->status, s));
+        CK(decompose_adjoint_run<T>(*P, geos<T>(P), in, out, ga, gb, y, R, &sc->status, s));
     }
     return HPDR_OK;
 }

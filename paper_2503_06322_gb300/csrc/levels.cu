@@ -23,17 +23,18 @@ constexpr int kNormBlocks = 152 * 8;
 
 template <typename T>
 __global__ void __launch_bounds__(256)
-solve_strided_kernel(T *b, int n, long long stride, long long nlines, const T *__restrict__ sub,
+solve_strided_kernel(T *b, const T *src, int n, long long stride, long long nlines, const T *__restrict__ sub,
                      const T *__restrict__ cp, const T *__restrict__ inv_den, T *vc, int sign)
 {
     long long line = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (line >= nlines) return;
     long long o = line / stride, i = line - o * stride;
     T *p = b + o * (long long)n * stride + i;
+    const T *f = src + o * (long long)n * stride + i;   // the right-hand side: b, or an array that is kept
     T y = (T)0;
 #pragma unroll 4
     for (int t = 0; t < n; t++) {
-        y = mul_rn(fma_rn(-sub[t], y, p[(long long)t * stride]), inv_den[t]);
+        y = mul_rn(fma_rn(-sub[t], y, f[(long long)t * stride]), inv_den[t]);
         p[(long long)t * stride] = y;
     }
     T x = (T)0;
@@ -59,7 +60,7 @@ constexpr int kSolveThreads = 64;
 
 template <typename T>
 __global__ void __launch_bounds__(kSolveThreads)
-solve_stream_kernel(T *b, int n, long long st, long long ostride, long long ninner, long long nlines,
+solve_stream_kernel(T *b, const T *src, int n, long long st, long long ostride, long long ninner, long long nlines,
                     const T *__restrict__ sub, const T *__restrict__ cp, const T *__restrict__ inv_den)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -73,6 +74,7 @@ solve_stream_kernel(T *b, int n, long long st, long long ostride, long long ninn
     else if (nlines <= 0xFFFFFFFFll) { o = (unsigned)line / (unsigned)ninner; i = line - o * ninner; }
     else { o = line / ninner; i = line - o * ninner; }     // 64-bit division only for huge grids
     T *p = b + o * ostride + i;
+    const T *f = src + o * ostride + i;   // the right-hand side: b, or an array that is kept
     constexpr int P = kSolvePre;
     const int nfull = n / P;   // blocks of P steps
     // forward sweep: y_t = (d_t - sub_t y_{t-1}) / den_t
@@ -80,13 +82,13 @@ solve_stream_kernel(T *b, int n, long long st, long long ostride, long long ninn
     T cur[P], nxt[P];
     if (nfull > 0) {
 #pragma unroll
-        for (int u = 0; u < P; u++) cur[u] = p[(long long)u * st];
+        for (int u = 0; u < P; u++) cur[u] = f[(long long)u * st];
     }
     for (int k = 0; k < nfull; k++) {
         const int t0 = k * P;
         if (k + 1 < nfull) {
 #pragma unroll
-            for (int u = 0; u < P; u++) nxt[u] = p[(long long)(t0 + P + u) * st];
+            for (int u = 0; u < P; u++) nxt[u] = f[(long long)(t0 + P + u) * st];
         }
 #pragma unroll
         for (int u = 0; u < P; u++) {
@@ -97,7 +99,7 @@ solve_stream_kernel(T *b, int n, long long st, long long ostride, long long ninn
         for (int u = 0; u < P; u++) cur[u] = nxt[u];
     }
     for (int t = nfull * P; t < n; t++) {
-        y = mul_rn(fma_rn(-csub[t], y, p[(long long)t * st]), cinv[t]);
+        y = mul_rn(fma_rn(-csub[t], y, f[(long long)t * st]), cinv[t]);
         p[(long long)t * st] = y;
     }
     // backward sweep: x_t = y_t - cp_t x_{t+1}, from the end
@@ -232,7 +234,7 @@ constexpr int kContigThreads = 128;
 constexpr size_t kContigMaxKb = 220;
 template <typename T>
 __global__ void __launch_bounds__(kContigThreads)
-solve_contig_kernel(T *b, int n, long long nlines, int rows, const T *__restrict__ sub, const T *__restrict__ cp,
+solve_contig_kernel(T *b, const T *src, int n, long long nlines, int rows, const T *__restrict__ sub, const T *__restrict__ cp,
                     const T *__restrict__ inv_den, T *vc, int sign)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -241,8 +243,10 @@ solve_contig_kernel(T *b, int n, long long nlines, int rows, const T *__restrict
     T *tile = csub + (3 * n + V - 1) / V * V;
     const long long row0 = blockIdx.x * (long long)rows, first = row0 * n;
     const int nr = (int)min((long long)rows, nlines - row0), cnt = nr * n;
-    T *B = tile + ((uintptr_t)(b + first) & 15) / sizeof(T);
-    run_load(B, b + first, cnt);
+    // the right-hand side (b, or an array that is kept) and where it sits modulo
+    // 16 bytes; without v_c the solution takes its place, so b has to agree
+    T *B = tile + ((uintptr_t)(src + first) & 15) / sizeof(T);
+    run_load(B, src + first, cnt);
     T *X = B;
     if (sign != 0) {
         X = tile + (rows * n + 2 * V - 1) / V * V + ((uintptr_t)(vc + first) & 15) / sizeof(T);
@@ -933,8 +937,9 @@ cudaError_t launch_restrict(WSrc src, Sink sink, const RestrictArgs<T> &a, cudaS
 }
 
 template <typename T>
-cudaError_t launch_solves(const LevelGeom<T> &g, T *b, T *vc, int sign, cudaStream_t s)
+cudaError_t launch_solves(const LevelGeom<T> &g, T *b, T *vc, int sign, cudaStream_t s, const T *src)
 {
+    if (!src) src = b;   // the first solve reads src, the others b
     const long long c0 = g.dim[0].mc, c1 = g.dim[1].mc, c2 = g.dim[2].mc;
     int last = -1;
     for (int k = 0; k < 3; k++) if (g.dim[k].mc > 1 && g.dim[k].m > 1) last = k;
@@ -952,13 +957,13 @@ cudaError_t launch_solves(const LevelGeom<T> &g, T *b, T *vc, int sign, cudaStre
             const long long nlines = outer * c2;
             solve_stream_kernel<T><<<(unsigned)((nlines + kSolveThreads - 1) / kSolveThreads), kSolveThreads,
                                      3 * (size_t)d.mc * sizeof(T), s>>>(
-                b, d.mc, st, ostride, c2, nlines, d.sub, d.cp, d.inv_den);
+                b, src, d.mc, st, ostride, c2, nlines, d.sub, d.cp, d.inv_den);
         } else if (k < 2) {
             long long stride = (k == 0) ? c1 * c2 : c2;
             long long nlines = (k == 0) ? c1 * c2 : c0 * c2;
             int n = d.mc;
             solve_strided_kernel<T><<<(unsigned)((nlines + 255) / 256), 256, 0, s>>>(
-                b, n, stride, nlines, d.sub, d.cp, d.inv_den, vc, sg);
+                b, src, n, stride, nlines, d.sub, d.cp, d.inv_den, vc, sg);
         } else {
             int n = d.mc;
             long long nlines = c0 * c1;
@@ -970,7 +975,7 @@ cudaError_t launch_solves(const LevelGeom<T> &g, T *b, T *vc, int sign, cudaStre
             if (rows < 8) rows = std::min<size_t>(8, lines_in(kContigMaxKb));
             if (rows < 1) {
                 solve_strided_kernel<T><<<(unsigned)((nlines + 255) / 256), 256, 0, s>>>(
-                    b, n, 1, nlines, d.sub, d.cp, d.inv_den, vc, sg);
+                    b, src, n, 1, nlines, d.sub, d.cp, d.inv_den, vc, sg);
             } else {
                 static PerDeviceOnce attr;
                 cudaError_t ea = once_per_device(attr, [] {
@@ -979,9 +984,10 @@ cudaError_t launch_solves(const LevelGeom<T> &g, T *b, T *vc, int sign, cudaStre
                 });
                 if (ea != cudaSuccess) return ea;
                 solve_contig_kernel<T><<<(unsigned)((nlines + rows - 1) / rows), kContigThreads, fixed + rows * line, s>>>(
-                    b, n, nlines, (int)rows, d.sub, d.cp, d.inv_den, vc, sg);
+                    b, src, n, nlines, (int)rows, d.sub, d.cp, d.inv_den, vc, sg);
             }
         }
+        src = b;
         count_launch();
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
@@ -1128,7 +1134,7 @@ cudaError_t launch_coarse(int mode, const Plan *P, const LevelGeom<T> *geo, int 
 
 #define INST(T)                                                                                   \
     template cudaError_t launch_restrict<T>(WSrc, Sink, const RestrictArgs<T> &, cudaStream_t);  \
-    template cudaError_t launch_solves<T>(const LevelGeom<T> &, T *, T *, int, cudaStream_t);    \
+    template cudaError_t launch_solves<T>(const LevelGeom<T> &, T *, T *, int, cudaStream_t, const T *); \
     template cudaError_t launch_expand<T>(WSrc, const LevelGeom<T> &, const T *, const T *,       \
                                           const SymIn &, T *, cudaStream_t);                     \
     template cudaError_t launch_level0<T>(Sink, const T *, long long, T *, const QuantOut &,      \

@@ -72,9 +72,10 @@ extern int g_wait_limit;
 
 // Solve (x)_k M_{l-1} along every active dimension of the coarse array b, in
 // place; the last solve optionally adds (sign=+1) or subtracts (sign=-1) the
-// result into vc instead of storing it into b.
+// result into vc instead of storing it into b.  src non-null: the right-hand
+// side is read there and left as it is (b need not be set).
 template <typename T>
-cudaError_t launch_solves(const LevelGeom<T> &g, T *b, T *vc, int sign, cudaStream_t s);
+cudaError_t launch_solves(const LevelGeom<T> &g, T *b, T *vc, int sign, cudaStream_t s, const T *src = nullptr);
 
 // Recomposition of level l: out (level-l grid) = kept nodes from vc (level
 // l-1 grid), new nodes = coefficient + interpolant of vc.
@@ -103,11 +104,6 @@ struct BinArgs {
 };
 template <typename T>
 cudaError_t launch_norm(const T *u, long long N, double *partials, const BinArgs &ba, Scalars *sc, cudaStream_t s);
-
-// Transposes: dense level-l array from a coarse array through (x)_k M_l P
-template <typename T>
-cudaError_t launch_mass_prolong(const LevelGeom<T> &g, const T *yc, T *yf, T *tmp,
-                                cudaStream_t s);
 
 int norm_parts();
 
@@ -150,13 +146,12 @@ template <typename T>
 cudaError_t launch_coarse_batch(const CoarseArgs<T> *jobs, int n, size_t smem, cudaStream_t s);
 
 // adjoint.cu: transposes of recomposition / decomposition over all levels.
-// ga, gb, y, R hold N_{L-1} elements; t1, t2 the partial prolongations
-// (max over levels of c0*c1*m2 and c0*m1*m2 elements).
+// ga, gb, y, R hold N_{L-1} elements.
 template <typename T>
 cudaError_t recompose_adjoint_run(const Plan &P, const LevelGeom<T> *geo, const T *gu, T *gcoef, T *ga, T *gb,
-                                  T *y, T *t1, T *t2, unsigned *status, cudaStream_t s);
+                                  T *y, unsigned *status, cudaStream_t s);
 template <typename T>
 cudaError_t decompose_adjoint_run(const Plan &P, const LevelGeom<T> *geo, const T *gcoef, T *gu, T *ga, T *gb,
-                                  T *y, T *t1, T *t2, T *R, unsigned *status, cudaStream_t s);
+                                  T *y, T *R, unsigned *status, cudaStream_t s);
 
 }  // namespace hpdr
