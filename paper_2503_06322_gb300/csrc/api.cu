@@ -97,6 +97,7 @@ struct Ws {
     unsigned long long *bsum;
     void *huff;
     DevHdr *dh;   // a container header parsed on the device
+    double *deq;  // binary64 fields: symbol values per level (null for binary32 and large alphabets)
 };
 
 size_t carve_ws(void *base, const Plan *P, size_t esz, unsigned D, unsigned K, bool need_sym, Ws *w)
@@ -117,6 +118,7 @@ size_t carve_ws(void *base, const Plan *P, size_t esz, unsigned D, unsigned K, b
     w->bsum = c.take<unsigned long long>(1024);
     w->huff = c.take<char>(huff_scratch_bytes(D));
     w->dh = c.take<DevHdr>(1);
+    w->deq = esz == 8 && need_sym && D <= kDeqMaxD ? c.take<double>((size_t)(P->L + 1) * D) : nullptr;
     return c.used + 256;
 }
 
@@ -472,6 +474,7 @@ hpdr_status decompress_levels(hpdr_ctx *ctx, const Plan *P, unsigned D, unsigned
     SymIn si;
     si.sym = w.sym; si.D = D; si.sc = w.sc; si.esc = w.esc;
     si.status = &w.sc->status;
+    si.deq = w.deq;
     // level buffers: v_{l-1} in X, v_l written to Y (or to out at l = L)
     T *bufs[2] = {(T *)w.va, (T *)w.vb};
     const LevelGeom<T> *geo = &geom<T>(P, 0);
@@ -536,6 +539,7 @@ hpdr_status decompress_t(hpdr_ctx *ctx, const Plan *P, const Hdr &h, const uint8
     ta.lenb = in + h.off_len; ta.s_lo = h.s_lo; ta.s_hi = h.s_hi; ta.D = h.D;
     ta.sc = w.sc;
     ta.set_scalars = true;
+    ta.deq = w.deq;
     for (int l = 0; l <= L; l++) ta.si.q[l] = h.q[l];
     ta.si.L = L;
     ta.si.n_esc = h.n_esc;
@@ -587,6 +591,7 @@ hpdr_status decompress_dev(hpdr_ctx *ctx, const Plan *P, int dtype, int ndim, co
     ta.D = D;
     ta.sc = w.sc;
     ta.base = in; ta.in_bytes = in_bytes; ta.dh = w.dh;
+    ta.deq = w.deq;
     HdrExpect &ex = ta.ex;
     ex.dtype = dtype;
     ex.ndim = ndim;

@@ -534,6 +534,12 @@ decomp_kernel(RestrictArgs<T> a, int seg_len)
             const T mai = i <= 4 ? wr.ma[i <= 4 ? i : 0] : (T)0;
             if (mai != (T)0 || mbi != (T)0) mrows |= 1u << i;
         }
+        // Away from a short last interval the mass rows have taps at the kept
+        // nodes of the window only (offsets -2, 0 and 2): a fused multiply-add
+        // with a zero tap changes no bit, and binary64, bound by the FP64 pipe,
+        // skips it (in binary32 the test costs what the products do).
+        const bool even2 = sizeof(T) == 8 && __all_sync(0xffffffffu, lc.m2t[1] == (T)0 && lc.m2t[3] == (T)0);
+        const bool even1 = sizeof(T) == 8 && wr.ma[1] == (T)0 && wr.ma[3] == (T)0 && wr.mb[1] == (T)0 && wr.mb[3] == (T)0;
         T acc[2][3];
 #pragma unroll
         for (int u = 0; u < 2; u++) acc[u][0] = acc[u][1] = acc[u][2] = (T)0;
@@ -554,16 +560,18 @@ decomp_kernel(RestrictArgs<T> a, int seg_len)
                     sm[i] = (T)0;
                     if ((mrows >> i) & 1u) {
                         const T *ad = rowaddr(slot, p0, i);
-                        T m = (T)0;
-#pragma unroll
-                        for (int o = 0; o < 5; o++) m = fma_rn(lc.m2t[o], ad[o], m);
-                        sm[i] = m;
+                        T m = fma_rn(lc.m2t[0], ad[0], (T)0);
+                        if (!even2) m = fma_rn(lc.m2t[1], ad[1], m);
+                        m = fma_rn(lc.m2t[2], ad[2], m);
+                        if (!even2) m = fma_rn(lc.m2t[3], ad[3], m);
+                        sm[i] = fma_rn(lc.m2t[4], ad[4], m);
                     }
                 }
                 T ca_ = (T)0, cb_ = (T)0;
                 const bool two = wr.offb == 2;
 #pragma unroll
                 for (int o = 0; o < 5; o++) {
+                    if ((o & 1) && even1) continue;
                     ca_ = fma_rn(wr.ma[o], sm[o], ca_);
                     cb_ = fma_rn(wr.mb[o], two ? sm[o + 2] : sm[o + 1], cb_);
                 }
@@ -1047,6 +1055,17 @@ expand_kernel(LevelGeom<T> g, const T *__restrict__ vc, const T *__restrict__ co
     const int j2 = blockIdx.x * 32 + lane, j1 = blockIdx.y * XW + warp;
     const int J0a = blockIdx.z * seg_len, J0b = min(J0a + seg_len, mc0);
     if (J0a >= J0b || blockIdx.y * XW >= mc1) return;
+    extern __shared__ __align__(16) unsigned char xsm[];
+    // binary64 symbols: the level's values, behind the escape slots
+    const double *deq = nullptr;
+    if (SRC == (int)WSrc::SYMBOLS && deq_bytes<T>(symin)) {
+        double *d = reinterpret_cast<double *>(xsm + (size_t)2 * XTHREADS * 7 * sizeof(long long));
+        deq_stage(d, symin, g.level);
+        cp_async_commit();
+        cp_async_wait0();
+        __syncthreads();
+        deq = d;
+    }
     const bool rowv = j1 < mc1;                // warp-uniform
     const bool colv = rowv && j2 < mc2;
     const int jc2 = min(j2, mc2 - 1), jr1 = min(j1, mc1 - 1);
@@ -1120,7 +1139,6 @@ expand_kernel(LevelGeom<T> g, const T *__restrict__ vc, const T *__restrict__ co
     // Escaped codes (symbol 0) travel into shared slots by asynchronous
     // copies, one plane ahead of their use; with a register destination a
     // warp would wait on every node at which any lane escapes.
-    extern __shared__ __align__(16) unsigned char xsm[];
     long long *eslot = reinterpret_cast<long long *>(xsm) + threadIdx.x * 7;   // [2][XTHREADS][7]
     bool pend = false;   // escapes of the current plane in flight
     auto issue_esc = [&](const Raw &r, int b) -> bool {
@@ -1148,7 +1166,7 @@ expand_kernel(LevelGeom<T> g, const T *__restrict__ vc, const T *__restrict__ co
         if constexpr (SRC == (int)WSrc::STREAM) {
             return wv;
         } else {
-            return wv != 0u ? mul_rn((T)((int)wv - halfD), q) : mul_rn((T)eslot[(size_t)b * XTHREADS * 7 + j], q);
+            return wv != 0u ? dequant_code<T>(deq, wv, halfD, q) : mul_rn((T)eslot[(size_t)b * XTHREADS * 7 + j], q);
         }
     };
     auto step = [&](int j0, Raw &cur, const Raw &nxt, int b) {
@@ -1286,7 +1304,14 @@ cudaError_t launch_expand_planes(WSrc src, const LevelGeom<T> &g, const T *vc, c
     const int mc0 = g.dim[0].mc, mc1 = g.dim[1].mc, mc2 = g.dim[2].mc;
     const int gx = (mc2 + 31) / 32, gy = (mc1 + XW - 1) / XW;
     const bool stream = src == WSrc::STREAM;
-    const size_t sm = stream ? 0 : (size_t)2 * XTHREADS * 7 * sizeof(long long);   // escape slots
+    // escape slots, symbol values
+    const size_t sm = stream ? 0 : (size_t)2 * XTHREADS * 7 * sizeof(long long) + deq_bytes<T>(symin);
+    static PerDeviceOnce attr;
+    cudaError_t e = once_per_device(attr, [] {
+        return cudaFuncSetAttribute(expand_kernel<T, (int)WSrc::SYMBOLS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    100 * 1024);
+    });
+    if (e != cudaSuccess) return e;
     const int per_sm = stream ? resident_ctas(expand_kernel<T, (int)WSrc::STREAM>, XTHREADS, 0)
                               : resident_ctas(expand_kernel<T, (int)WSrc::SYMBOLS>, XTHREADS, sm);
     const int seg = choose_segment(mc0, (long long)gx * gy, per_sm);

@@ -916,6 +916,12 @@ __global__ void __launch_bounds__(kTabThreads, 1) dec_tables_kernel(TabArgs a, H
             a.sc->total_bits = a.dh ? h.total_bits : a.si.total_bits;
             if (a.dh) *a.dh = h;
         }
+        if (a.deq)
+            for (unsigned i = blockIdx.x * kTabThreads + tid; i < (unsigned)(L + 1) * D; i += kTabBlocks * kTabThreads) {
+                const unsigned l = i / D;
+                const double q = a.dh ? reinterpret_cast<const double *>(a.base + 128)[l] : a.si.q[l];
+                a.deq[i] = __dmul_rn((double)((int)(i - l * D) - (int)(D / 2)), q);
+            }
     }
     // ---- code lengths; counts per warp and length over the warp's run of symbols
     if (tid == 0) okc = 1;

@@ -90,6 +90,8 @@ struct TabArgs {
     unsigned long long in_bytes = 0;
     DevHdr *dh = nullptr;
     HdrExpect ex;
+    // non-null: [L + 1][D], the binary64 value (s - D/2) q_l of every symbol on every level
+    double *deq = nullptr;
 };
 cudaError_t launch_decode_tables(const TabArgs &a, const HuffScratch &hs, cudaStream_t s);
 

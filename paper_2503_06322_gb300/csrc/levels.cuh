@@ -28,7 +28,11 @@ struct SymIn {
     const Scalars *sc;               // q per level
     const long long *esc;            // [N] code k at every escaped stream position
     unsigned int *status;
+    const double *deq;               // binary64: value of every symbol on every level, [L + 1][D], or null
 };
+// The expansion of binary64 fields dequantizes symbols through a table per
+// level for alphabets whose table leaves two blocks an SM
+constexpr unsigned kDeqMaxD = 8192;
 
 template <typename T>
 struct RestrictArgs {
@@ -144,7 +148,6 @@ CoarseArgs<T> coarse_args(int mode, const Plan *P, const LevelGeom<T> *geo, int 
 // device [n]; smem: the largest of the fields' shared-memory sizes)
 template <typename T>
 cudaError_t launch_coarse_batch(const CoarseArgs<T> *jobs, int n, size_t smem, cudaStream_t s);
-
 // adjoint.cu: transposes of recomposition / decomposition over all levels.
 // ga, gb, y, R hold N_{L-1} elements.
 template <typename T>

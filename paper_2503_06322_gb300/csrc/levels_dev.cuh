@@ -14,18 +14,28 @@ namespace {
 // the same coefficients everywhere but at half-bin ties.  Codes whose
 // magnitude reaches 2^62 are clamped there (the escape store then flags them).
 //
-// Binary64 issue is slow on this part, so only the product, the sum and one
-// more addition use it: t >= 0, so its range is read off its high word, and
-// adding 2^52 rounded down leaves floor(t) in the low word.
+// Binary64 issue is slow on this part, so only the product and one addition use
+// it below 2^30: adding 2^51 + 1/2 rounded down leaves floor(2 (p + 1/2)) in the
+// low word (its last place is worth 1/2).  That is the floor of the exact
+// p + 1/2; the rounded sum of the definition reaches the next integer only from
+// p = n + 1/2 - ulp(p), whose low 20 bits are all ones (p < 2^30): such p, and
+// larger ones, take the definition as it stands.
+__device__ __noinline__ long long quant_code_slow(double p)
+{
+    const double t = __dadd_rn(p, 0.5);
+    if (t < 1073741824.0) return (long long)(int)floor(t);
+    if (t < 4611686018427387904.0) return (long long)floor(t);
+    return kEscMax;
+}
 template <typename T>
 __device__ __forceinline__ long long quant_code(T x, double rho)
 {
-    const double ax = fabs((double)x);
-    const double t = __dadd_rn(__dmul_rn(ax, rho), 0.5);
+    const double p = __dmul_rn(fabs((double)x), rho);
     long long k;
-    if (__double2hiint(t) < 0x41D00000) k = __double2loint(__dadd_rd(t, 4503599627370496.0));   // t < 2^30
-    else if (t < 4611686018427387904.0) k = (long long)floor(t);
-    else k = kEscMax;
+    if (__double2hiint(p) < 0x41D00000 && (__double2loint(p) & 0xFFFFF) != 0xFFFFF)
+        k = (unsigned)__double2loint(__dadd_rd(p, 2251799813685248.5)) >> 1;
+    else
+        k = quant_code_slow(p);
     return x < (T)0 ? -k : k;
 }
 
@@ -177,6 +187,33 @@ __device__ __forceinline__ T dequant_sym(const SymIn &si_, unsigned s, long long
 {
     if (s != 0) return mul_rn((T)((int)s - (int)(si_.D / 2)), q);
     return mul_rn((T)si_.esc[idx], q);
+}
+
+// Binary64 issue is slow on this part: the conversion and the product of a
+// symbol were a third of the binary64 instructions of the expansion of a level.
+// It takes the value from a table instead, 64 KB per level, which its blocks
+// copy into shared memory (bytes: size of it, 0 without): 419 -> 328 us for the
+// finest level of 500x500x100.  The restriction stays with the product (the
+// table made it 778 -> 814 us: it waits for shared memory more than for the pipe).
+template <typename T>
+__host__ __device__ inline size_t deq_bytes(const SymIn &si)
+{
+    return sizeof(T) == 8 && si.deq ? sizeof(double) * si.D : 0;
+}
+// starts the copy of a level's table (all threads; cp.async, committed by the caller)
+__device__ __forceinline__ void deq_stage(double *dst, const SymIn &si, int level)
+{
+    const double *src = si.deq + (size_t)level * si.D;
+    for (unsigned i = 2 * threadIdx.x; i < si.D; i += 2 * blockDim.x)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst + i)), "l"(src + i) : "memory");
+}
+// value of symbol s != 0; after a rejected header the symbols are another
+// stream's, and any of them has to stay inside the table
+template <typename T>
+__device__ __forceinline__ T dequant_code(const double *deq, unsigned s, int halfD, T q)
+{
+    if (sizeof(T) == 8 && deq) return (T)deq[min(s, 2u * (unsigned)halfD - 1u)];
+    return mul_rn((T)((int)s - halfD), q);
 }
 
 template <typename T>
