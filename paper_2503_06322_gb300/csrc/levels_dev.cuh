@@ -128,6 +128,33 @@ __device__ __noinline__ unsigned escape_f32(const QuantOut &qo, long long si, fl
     return escape_store(qo, si, k);
 }
 
+// The fast half of that decision: y = x rho_hi + 3 2^22 rounded to nearest holds
+// the integer n nearest to x rho_hi in its low bits, and r = x rho - n (two fused
+// multiply-adds, exact to 2^-24) tells whether n is the code: |r| safely below
+// 1/2 leaves one integer within 1/2 of x rho.  Everything else -- a half-bin
+// point nearby, a product near 2^22 and beyond, a NaN -- answers false.
+__device__ __forceinline__ bool quant_near_f32(float x, float rho_hi, float rho_lo, int &n)
+{
+    const float magic = 12582912.0f;
+    const float y = __fmaf_rn(x, rho_hi, magic);
+    const float nf = __fsub_rn(y, magic);
+    const float r = __fmaf_rn(x, rho_lo, __fmaf_rn(x, rho_hi, -nf));
+    n = __float_as_int(y) - 0x4B400000;
+    return fabsf(r) < 0.49998f && fabsf(nf) < 4194000.0f;
+}
+// The other half, out of line: the symbol in the low half (0: an escape, stored
+// at its stream position), the payload's bit length in the high half.
+__device__ __noinline__ unsigned quant_far_f32(const QuantOut &qo, long long si, float w, float rho_hi, float rho_lo,
+                                               double rho)
+{
+    const int halfD = (int)(qo.D / 2);
+    const float ax = fabsf(w);
+    int ki = halfD;   // a code of 2^22 or more: an escape
+    if (__fmul_rn(ax, rho_hi) < kSmallQuant) ki = quant_small_f32(ax, rho_hi, rho_lo);
+    if (ki < halfD) return (unsigned)(halfD + (w < 0.0f ? -ki : ki));
+    return escape_f32(qo, si, w, rho_hi, rho_lo, rho) << 16;
+}
+
 // quantize one coefficient into the symbol stream (+ block histogram / escapes)
 template <typename T>
 __device__ __forceinline__ void quant_emit(const QuantOut &qo, unsigned int *hs, bool smem_hist,
