@@ -195,7 +195,8 @@ cudaError_t recompose_adjoint_run(const Plan &P, const LevelGeom<T> *geo, const 
 {
     const int L = P.L;
     const T *gl = gu;
-    for (int l = L; l >= 1; l--) {
+    const int ls = coarse_adjoint_top<T>(P, geo);
+    for (int l = L; l > ls; l--) {
         const LevelGeom<T> &g = geo[l];
         T *gc = ((L - l) % 2 == 0) ? ga : gb;   // g_{l-1} = P^T g_l
         RestrictArgs<T> a;
@@ -214,6 +215,7 @@ cudaError_t recompose_adjoint_run(const Plan &P, const LevelGeom<T> *geo, const 
         if (e != cudaSuccess) return e;
         gl = gc;
     }
+    if (ls >= 1) return launch_coarse_adjoint<T>(P, geo, ls, gl, gcoef, s);
     copy_kernel<T><<<grid_for(P.N[0]), 256, 0, s>>>(gcoef, gl, P.N[0]);
     count_launch();
     return cudaGetLastError();

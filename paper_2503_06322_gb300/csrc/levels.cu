@@ -902,6 +902,174 @@ __global__ void __launch_bounds__(kCoarseThreads, 1) coarse_batch_kernel(const C
     else coarse_body<T, 0, false>(a);
 }
 
+// The coarse levels of the adjoint of recomposition in one CTA, like
+// coarse_kernel: for l = ls..1, from the level-l gradient g_l,
+//   g_{l-1} = P^T g_l,   y = (x)_k M_{l-1}^{-1} g_{l-1},
+//   g_{c_l} = g_l - (x)_k M_l P_k y at the new nodes,
+// and g_{c_0} = g_0.  Latency-bound: five launches a level took 100 us with their
+// gaps on grids this small (257^3, levels 4..1), one CTA takes 18 us.  The sums
+// run in the order of the launches it replaces.  Tables per dimension: ptap[5 mc],
+// sub[mc], cp[mc], inv[mc], etap[3 m], efirst[m].
+__host__ __device__ inline int adjoint_tab_elems(int m, int mc) { return 4 * m + 8 * mc; }
+template <typename T>
+struct AdjointSizes {
+    long long nl, nc, ra, rb, tab;   // level grid, coarse grid, the two scratch arrays, tables of levels 1..l
+};
+template <typename T>
+__host__ __device__ inline AdjointSizes<T> adjoint_sizes(const LevelGeom<T> *g, int ls)
+{
+    AdjointSizes<T> z;
+    long long r2, r1;
+    coarse_sizes<T>(g[ls], z.nl, z.nc, r2, r1);
+    const long long t2 = (long long)g[ls].dim[0].mc * g[ls].dim[1].m * g[ls].dim[2].m;
+    const long long t1 = (long long)g[ls].dim[0].mc * g[ls].dim[1].mc * g[ls].dim[2].m;
+    z.ra = r2 > t2 ? r2 : t2;
+    z.rb = r1 > t1 ? r1 : t1;
+    z.tab = 0;
+    for (int l = 1; l <= ls; l++)
+        for (int k = 0; k < 3; k++) z.tab += adjoint_tab_elems(g[l].dim[k].m, g[l].dim[k].mc);
+    return z;
+}
+
+// out = (M_l P) in along dimension k; out has extents n0 x n1 x n2 (extent k =
+// m), in the same with extent k = mc; fin(idx, v) takes the products
+template <typename T, int k, typename Fin>
+__device__ __forceinline__ void coarse_prolong(const T *etap, const int *efirst, int mc, int n0, int n1, int n2,
+                                               unsigned mul2, unsigned mul1, const T *in, Fin fin)
+{
+    const int i1 = k == 1 ? mc : n1, i2 = k == 2 ? mc : n2;
+    const int is = k == 0 ? i1 * i2 : k == 1 ? i2 : 1;
+    for (int idx = threadIdx.x; idx < n0 * n1 * n2; idx += blockDim.x) {
+        const int r = small_div(idx, mul2), p2 = idx - r * n2, p0 = small_div(r, mul1), p1 = r - p0 * n1;
+        const int p = k == 0 ? p0 : k == 1 ? p1 : p2;
+        const int f = efirst[p];
+        const T *x = in + ((k == 0 ? f : p0) * i1 + (k == 1 ? f : p1)) * i2 + (k == 2 ? f : p2);
+        T v = (T)0;
+#pragma unroll
+        for (int i = 0; i < 3; i++)
+            if (f + i < mc) v = fma_rn(etap[p * 3 + i], x[i * is], v);
+        fin(idx, p0, p1, p2, v);
+    }
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kCoarseThreads, 1) coarse_adjoint_kernel(AdjointArgs<T> a)
+{
+    extern __shared__ __align__(16) unsigned char coarse_smem[];
+    __shared__ CoarseExt sext[kCoarseMaxLevels + 1][3];
+    const int ls = a.ls, tid = threadIdx.x, nt = blockDim.x;
+    const AdjointSizes<T> z = adjoint_sizes<T>(a.g, ls);
+    const int nl = (int)z.nl, nc = (int)z.nc;
+    T *VA = reinterpret_cast<T *>(coarse_smem);   // [nl] the level's gradient, by turns
+    T *VB = VA + nl;                                // [nc]
+    T *Y = VB + nc;                                 // [nc]
+    T *RA = Y + nc;                                 // [ra]
+    T *RB = RA + z.ra;                              // [rb]
+    T *tab = RB + z.rb;
+    // extents and offsets of every dimension (thread 0: a few dozen), then the tables
+    if (tid == 0) {
+        int off = 0;
+        for (int l = 1; l <= ls; l++)
+            for (int k = 0; k < 3; k++) {
+                const int m = a.g[l].dim[k].m, mc = a.g[l].dim[k].mc;
+                sext[l][k] = {m, mc, off, small_div_mul(m), small_div_mul(mc)};
+                off += adjoint_tab_elems(m, mc);
+            }
+    }
+    for (int i = tid; i < nl; i += nt) cp_async_elem(VA + i, a.g_in + i);
+    __syncthreads();
+    for (int task = tid >> 5; task < 18 * ls; task += nt >> 5) {
+        const int l = 1 + task / 18, r = task - (l - 1) * 18, k = r / 6, w = r - k * 6;
+        const DimTables<T> &g = a.g[l].dim[k];
+        const CoarseExt &e = sext[l][k];
+        T *t = tab + e.off;
+        if (w == 5) {
+            int *d = reinterpret_cast<int *>(t + 8 * e.mc + 3 * e.m);
+            for (int i = tid & 31; i < e.m; i += 32) d[i] = g.efirst[i];
+            continue;
+        }
+        const T *src = w == 0 ? g.ptap : w == 1 ? g.sub : w == 2 ? g.cp : w == 3 ? g.inv_den : g.etap;
+        const int cnt = w == 0 ? 5 * e.mc : w < 4 ? e.mc : 3 * e.m;
+        T *dst = t + (w == 0 ? 0 : w < 4 ? (4 + w) * e.mc : 8 * e.mc);
+        for (int i = tid & 31; i < cnt; i += 32) cp_async_elem(dst + i, src + i);
+    }
+    cp_async_wait_all();
+    __syncthreads();
+    T *G = VA, *GC = VB;
+    for (int l = ls; l >= 1; l--) {
+        CoarseDim<T> d[3];
+        const T *etap[3];
+        const int *efirst[3];
+#pragma unroll
+        for (int k = 0; k < 3; k++) {
+            const CoarseExt &e = sext[l][k];
+            const T *t = tab + e.off;
+            d[k].m = e.m; d[k].mc = e.mc; d[k].mmul = e.mmul; d[k].cmul = e.cmul;
+            d[k].wl = d[k].wr = nullptr;
+            d[k].tap = t; d[k].sub = t + 5 * e.mc; d[k].cp = t + 6 * e.mc; d[k].inv = t + 7 * e.mc;
+            etap[k] = t + 8 * e.mc;
+            efirst[k] = reinterpret_cast<const int *>(t + 8 * e.mc + 3 * e.m);
+        }
+        const int m0 = d[0].m, m1 = d[1].m, m2 = d[2].m, c0 = d[0].mc, c1 = d[1].mc, c2 = d[2].mc;
+        // g_{l-1} = P^T g_l
+        coarse_restrict<T, 2>(d[2], m0, m1, m2, d[2].cmul, d[1].mmul, G, RA);
+        coarse_restrict<T, 1>(d[1], m0, m1, c2, d[2].cmul, d[1].cmul, RA, RB);
+        coarse_restrict<T, 0>(d[0], m0, c1, c2, d[2].cmul, d[1].cmul, RB, GC);
+        // y
+        for (int i = tid; i < c0 * c1 * c2; i += nt) Y[i] = GC[i];
+        __syncthreads();
+        if (m0 > 1) {
+            const int pl = c1 * c2;
+            for (int i = tid; i < pl; i += nt) {
+                T *p = Y + i;
+                sweep_line<T>(p, pl, c0, d[0].sub, d[0].cp, d[0].inv, [&](int t, const auto &v) {
+#pragma unroll
+                    for (int u = 0; u < (int)(sizeof(v) / sizeof(T)); u++) p[(t - u) * pl] = v[u];
+                });
+            }
+            __syncthreads();
+        }
+        if (m1 > 1) {
+            for (int i = tid; i < c0 * c2; i += nt) {
+                const int j0 = small_div(i, d[2].cmul);
+                T *p = Y + j0 * c1 * c2 + (i - j0 * c2);
+                sweep_line<T>(p, c2, c1, d[1].sub, d[1].cp, d[1].inv, [&](int t, const auto &v) {
+#pragma unroll
+                    for (int u = 0; u < (int)(sizeof(v) / sizeof(T)); u++) p[(t - u) * c2] = v[u];
+                });
+            }
+            __syncthreads();
+        }
+        for (int i = tid; i < c0 * c1; i += nt) {
+            T *p = Y + i * c2;
+            sweep_line<T>(p, 1, c2, d[2].sub, d[2].cp, d[2].inv, [&](int t, const auto &v) {
+#pragma unroll
+                for (int u = 0; u < (int)(sizeof(v) / sizeof(T)); u++) p[t - u] = v[u];
+            });
+        }
+        __syncthreads();
+        // the prolonged correction, taken from g_l at the new nodes
+        coarse_prolong<T, 2>(etap[2], efirst[2], c2, c0, c1, m2, d[2].mmul, d[1].cmul, Y,
+                             [&](int i, int, int, int, T v) { RB[i] = v; });
+        __syncthreads();
+        coarse_prolong<T, 1>(etap[1], efirst[1], c1, c0, m1, m2, d[2].mmul, d[1].mmul, RB,
+                             [&](int i, int, int, int, T v) { RA[i] = v; });
+        __syncthreads();
+        const long long np = a.g[l].Nprev;
+        coarse_prolong<T, 0>(etap[0], efirst[0], c0, m0, m1, m2, d[2].mmul, d[1].mmul, RA,
+                             [&](int i, int p0, int p1, int p2, T v) {
+                                 const bool k0 = kept_pos(m0, p0), k1 = kept_pos(m1, p1);
+                                 if (k0 && k1 && kept_pos(m2, p2)) return;
+                                 int cr = kept_before(p0) * c1 * c2;
+                                 if (k0) cr += kept_before(p1) * c2 + (k1 ? kept_before(p2) : 0);
+                                 a.coef_out[np + i - cr] = sub_rn(G[i], v);
+                             });
+        __syncthreads();
+        T *t = G; G = GC; GC = t;
+    }
+    for (int i = tid; i < (int)a.N0; i += nt) a.coef_out[i] = G[i];
+}
+
 }  // namespace
 
 int norm_parts() { return kNormBlocks; }
@@ -1132,6 +1300,43 @@ cudaError_t launch_coarse(int mode, const Plan *P, const LevelGeom<T> *geo, int 
     }
 }
 
+template <typename T>
+int coarse_adjoint_top(const Plan &P, const LevelGeom<T> *geo)
+{
+    int ls = 0;
+    for (int l = 1; l <= P.L && l <= kCoarseMaxLevels; l++) {
+        const AdjointSizes<T> z = adjoint_sizes<T>(geo, l);
+        // small_div takes indices below 2^16
+        if (z.nl >= 65536 || (size_t)(z.nl + 2 * z.nc + z.ra + z.rb + z.tab) * sizeof(T) > kCoarseSmemMax) break;
+        ls = l;
+    }
+    return ls;
+}
+
+template <typename T>
+cudaError_t launch_coarse_adjoint(const Plan &P, const LevelGeom<T> *geo, int ls, const T *g_in, T *coef_out,
+                                  cudaStream_t s)
+{
+    if (ls < 1 || ls > kCoarseMaxLevels) return cudaErrorInvalidValue;
+    AdjointArgs<T> a;
+    memset(&a, 0, sizeof(a));
+    for (int l = 1; l <= ls; l++) a.g[l] = geo[l];
+    a.ls = ls;
+    a.N0 = P.N[0];
+    a.g_in = g_in;
+    a.coef_out = coef_out;
+    const AdjointSizes<T> z = adjoint_sizes<T>(geo, ls);
+    static PerDeviceOnce attr;
+    cudaError_t e = once_per_device(attr, [] {
+        return cudaFuncSetAttribute(coarse_adjoint_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)kCoarseSmemMax);
+    });
+    if (e != cudaSuccess) return e;
+    coarse_adjoint_kernel<T><<<1, kCoarseThreads, (size_t)(z.nl + 2 * z.nc + z.ra + z.rb + z.tab) * sizeof(T), s>>>(a);
+    count_launch();
+    return cudaGetLastError();
+}
+
 #define INST(T)                                                                                   \
     template cudaError_t launch_restrict<T>(WSrc, Sink, const RestrictArgs<T> &, cudaStream_t);  \
     template cudaError_t launch_solves<T>(const LevelGeom<T> &, T *, T *, int, cudaStream_t, const T *); \
@@ -1147,6 +1352,8 @@ cudaError_t launch_coarse(int mode, const Plan *P, const LevelGeom<T> *geo, int 
                                           const QuantOut &, T *, const SymIn &, const T *, cudaStream_t); \
     template CoarseArgs<T> coarse_args<T>(int, const Plan *, const LevelGeom<T> *, int, const T *, T *,         \
                                           const QuantOut &, T *, const SymIn &, const T *, size_t *);      \
+    template int coarse_adjoint_top<T>(const Plan &, const LevelGeom<T> *);                      \
+    template cudaError_t launch_coarse_adjoint<T>(const Plan &, const LevelGeom<T> *, int, const T *, T *, cudaStream_t); \
     template cudaError_t launch_coarse_batch<T>(const CoarseArgs<T> *, int, size_t, cudaStream_t);
 INST(float)
 INST(double)

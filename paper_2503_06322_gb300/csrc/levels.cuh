@@ -148,6 +148,24 @@ CoarseArgs<T> coarse_args(int mode, const Plan *P, const LevelGeom<T> *geo, int 
 // device [n]; smem: the largest of the fields' shared-memory sizes)
 template <typename T>
 cudaError_t launch_coarse_batch(const CoarseArgs<T> *jobs, int n, size_t smem, cudaStream_t s);
+
+// The coarse levels ls..1 and 0 of the adjoint of recomposition in one CTA: g_in
+// is the gradient on the level-ls grid, coef_out the coefficient gradient's
+// stream.  ls = coarse_adjoint_top(), the largest level that fits (0: none).
+template <typename T>
+struct AdjointArgs {
+    LevelGeom<T> g[kCoarseMaxLevels + 1];
+    int ls;
+    long long N0;
+    const T *g_in;
+    T *coef_out;
+};
+template <typename T>
+int coarse_adjoint_top(const Plan &P, const LevelGeom<T> *geo);
+template <typename T>
+cudaError_t launch_coarse_adjoint(const Plan &P, const LevelGeom<T> *geo, int ls, const T *g_in, T *coef_out,
+                                  cudaStream_t s);
+
 // adjoint.cu: transposes of recomposition / decomposition over all levels.
 // ga, gb, y, R hold N_{L-1} elements.
 template <typename T>
