@@ -41,7 +41,7 @@ prolong_kernel(LevelGeom<T> g, const T *__restrict__ y, const T *__restrict__ gs
 {
     const DimTables<T> &d0 = g.dim[0], &d1 = g.dim[1], &d2 = g.dim[2];
     const int m0 = d0.m, m1 = d1.m, m2 = d2.m, mc0 = d0.mc, mc1 = d1.mc, mc2 = d2.mc;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31, warp = warp_index();
     const int j2 = blockIdx.x * 32 + lane, j1 = blockIdx.y * kMpWarps + warp;
     const int J0a = blockIdx.z * seg_len, J0b = min(J0a + seg_len, mc0);
     if (J0a >= J0b || j1 >= mc1 || j2 >= mc2) return;

@@ -341,7 +341,7 @@ decomp_kernel(RestrictArgs<T> a, int seg_len)
     PlaneInfo<T> *pinfo = reinterpret_cast<PlaneInfo<T> *>(smem_raw + S::off_info);
     unsigned int *hs = reinterpret_cast<unsigned int *>(smem_raw + S::off_hist);
     const unsigned char *stage_p = smem_raw + S::off_stage;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tid = threadIdx.x, lane = tid & 31, warp = warp_index();
     const int hhalf = QUANT ? min((int)a.qo.D / 2, kHistWin) : 0;
     const int hlo = (int)(a.qo.D / 2) - hhalf, hn = 2 * hhalf;
     const int nact = (tg.n1 + 1) >> 1;   // consumer warps with at least one coarse row
@@ -787,7 +787,7 @@ rsym_kernel(RestrictArgs<T> a, int seg_len)
     PlaneInfo<T> *pinfo = reinterpret_cast<PlaneInfo<T> *>(smem_raw + S::off_info);
     T *W0 = reinterpret_cast<T *>(smem_raw + S::off_w);
     SymRow *rowinfo = reinterpret_cast<SymRow *>(smem_raw + S::off_rows);
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tid = threadIdx.x, lane = tid & 31, warp = warp_index();
     const int limit = a.wait_limit;
     const SymIn &si_ = a.symin;
 
@@ -1061,7 +1061,7 @@ expand_kernel(LevelGeom<T> g, const T *__restrict__ vc, const T *__restrict__ co
 {
     const int m0 = g.dim[0].m, m1 = g.dim[1].m, m2 = g.dim[2].m;
     const int mc0 = g.dim[0].mc, mc1 = g.dim[1].mc, mc2 = g.dim[2].mc;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31, warp = warp_index();
     const int j2 = blockIdx.x * 32 + lane, j1 = blockIdx.y * XW + warp;
     const int J0a = blockIdx.z * seg_len, J0b = min(J0a + seg_len, mc0);
     if (J0a >= J0b || blockIdx.y * XW >= mc1) return;
@@ -1090,55 +1090,63 @@ expand_kernel(LevelGeom<T> g, const T *__restrict__ vc, const T *__restrict__ co
     // coarse column offsets of this lane and of the next column (lane 31 loads its own)
     const int c0 = jc2, c1 = min(jc2 + 1, mc2 - 1);
     const int r0 = jr1, r1 = min(jr1 + 1, mc1 - 1);
-    // stream offsets inside a fine plane of the rows Ra (kept) and Ra + 1
-    const int nro0 = Ra * m2, nro1 = (Ra + 1) * m2;
-    const int kro0 = Ra * m2 - kept_before(Ra) * mc2, kro1 = (Ra + 1) * m2 - kept_before(Ra + 1) * mc2;
+    // offsets of the lane's nodes inside a fine plane, dense (new planes of the
+    // stream, the output; rows Ra and Ra + 1) and in a kept plane of the stream;
+    // inside a coarse plane
+    const unsigned ox0 = (unsigned)(Ra * m2 + Ca), ox1 = ox0 + (unsigned)m2;
+    const unsigned ok0 = (unsigned)(Ra * m2 - kept_before(Ra) * mc2 + (Ca >> 1));
+    const unsigned ok1 = (unsigned)((Ra + 1) * m2 - kept_before(Ra + 1) * mc2 + Ca);
+    const unsigned ov0 = (unsigned)(r0 * mc2 + c0), ov1 = (unsigned)(r1 * mc2 + c0);
+    const unsigned dv = (unsigned)(c1 - c0);
     // the raw inputs of one coarse plane j0: its coarse values and the
     // coefficient words of the new fine plane before it (x) and of its kept
-    // fine plane (k); loaded one plane ahead of their use
+    // fine plane (k); loaded one plane ahead of their use.  Plane offsets depend
+    // on j0 alone and are added to the base pointers once per warp, and words
+    // that do not exist hold no escape, so one minimum finds a plane's escapes
+    // (513^3 binary32, finest level: 328 -> 270 us, bound by issue and latency).
     using W = typename std::conditional<SRC == (int)WSrc::SYMBOLS, unsigned, T>::type;
+    using E = typename std::conditional<SRC == (int)WSrc::SYMBOLS, uint16_t, T>::type;
+    const E *const src = SRC == (int)WSrc::SYMBOLS ? reinterpret_cast<const E *>(symin.sym)
+                                                   : reinterpret_cast<const E *>(coef_in);
     struct Raw {
         T a00, a10, a01, a11;
         W x00, x01, x10, x11, k01, k10, k11;
-        long long pbx, pbk;
     };
     const int jend = min(J0b, mc0 - 1);     // the new plane after the segment's last kept plane needs J(J0b)
-    auto word = [&](long long si) -> W {
-        if constexpr (SRC == (int)WSrc::STREAM) return coef_in[si];
-        else return symin.sym[si];
+    // the new fine plane before coarse plane j0, if there is one and it belongs to this segment
+    auto new_plane = [&](int j0) -> int {
+        if (j0 <= J0a) return -1;
+        const int Pn = cpos_of(m0, mc0, j0 - 1) + 1;
+        return Pn < cpos_of(m0, mc0, j0) ? Pn : -1;
     };
     auto load = [&](int j0) -> Raw {
         Raw r;
         const T *pl = vc + (long long)j0 * cplane;
-        r.a00 = pl[(long long)r0 * mc2 + c0];
-        r.a10 = pl[(long long)r1 * mc2 + c0];
+        const T *p0 = pl + ov0, *p1 = pl + ov1;
+        r.a00 = p0[0];
+        r.a10 = p1[0];
         r.a01 = r.a11 = (T)0;
-        if (lane == 31) { r.a01 = pl[(long long)r0 * mc2 + c1]; r.a11 = pl[(long long)r1 * mc2 + c1]; }
-        const W z = (W)0;
+        if (lane == 31) { r.a01 = p0[dv]; r.a11 = p1[dv]; }
+        const W z = (W)1;    // words that do not exist: any symbol but the escape
         r.x00 = r.x01 = r.x10 = r.x11 = r.k01 = r.k10 = r.k11 = z;
-        r.pbx = 0;    // no new plane before j0 (a new plane never starts the stream)
-        r.pbk = -1;   // no kept plane of j0 in this segment
-        const int P0 = cpos_of(m0, mc0, j0);
-        if (j0 > J0a && colv) {
-            const int Pn = cpos_of(m0, mc0, j0 - 1) + 1;
-            if (Pn < P0) {
-                const long long pb = plane_base_of(g, Pn);
-                r.pbx = pb;
-                r.x00 = word(pb + nro0 + Ca);
-                if (hb) r.x01 = word(pb + nro0 + Ca + 1);
-                if (hr) {
-                    r.x10 = word(pb + nro1 + Ca);
-                    if (hb) r.x11 = word(pb + nro1 + Ca + 1);
-                }
+        const int Pn = new_plane(j0);
+        if (Pn >= 0 && colv) {
+            const E *pp = src + plane_base_of(g, Pn);
+            const E *px = pp + ox0, *py = pp + ox1;
+            r.x00 = px[0];
+            if (hb) r.x01 = px[1];
+            if (hr) {
+                r.x10 = py[0];
+                if (hb) r.x11 = py[1];
             }
         }
         if (j0 < J0b && colv) {
-            const long long pb = plane_base_of(g, P0);
-            r.pbk = pb;
-            if (hb) r.k01 = word(pb + kro0 + (Ca >> 1));
+            const E *pp = src + plane_base_of(g, cpos_of(m0, mc0, j0));
+            const E *py = pp + ok1;
+            if (hb) r.k01 = pp[ok0];
             if (hr) {
-                r.k10 = word(pb + kro1 + Ca);
-                if (hb) r.k11 = word(pb + kro1 + Ca + 1);
+                r.k10 = py[0];
+                if (hb) r.k11 = py[1];
             }
         }
         return r;
@@ -1151,21 +1159,23 @@ expand_kernel(LevelGeom<T> g, const T *__restrict__ vc, const T *__restrict__ co
     // warp would wait on every node at which any lane escapes.
     long long *eslot = reinterpret_cast<long long *>(xsm) + threadIdx.x * 7;   // [2][XTHREADS][7]
     bool pend = false;   // escapes of the current plane in flight
-    auto issue_esc = [&](const Raw &r, int b) -> bool {
+    auto issue_esc = [&](const Raw &r, int j0, int b) -> bool {
         if constexpr (SRC == (int)WSrc::SYMBOLS) {
-            const bool any = (r.x00 == 0u && colv && r.pbx) || (r.x01 == 0u && hb && r.pbx) ||
-                             (r.x10 == 0u && hr && r.pbx) || (r.x11 == 0u && hr && hb && r.pbx) ||
-                             (r.k01 == 0u && hb && r.pbk >= 0) || (r.k10 == 0u && hr && r.pbk >= 0) ||
-                             (r.k11 == 0u && hr && hb && r.pbk >= 0);
-            if (!__any_sync(0xffffffffu, any)) return false;
+            const unsigned m = min(min(min(r.x00, r.x01), min(r.x10, r.x11)), min(min(r.k01, r.k10), r.k11));
+            if (!__any_sync(0xffffffffu, m == 0u)) return false;
             long long *e = eslot + (size_t)b * XTHREADS * 7;
-            if (r.x00 == 0u && colv && r.pbx) cp_async8(e + 0, symin.esc + r.pbx + nro0 + Ca);
-            if (r.x01 == 0u && hb && r.pbx) cp_async8(e + 1, symin.esc + r.pbx + nro0 + Ca + 1);
-            if (r.x10 == 0u && hr && r.pbx) cp_async8(e + 2, symin.esc + r.pbx + nro1 + Ca);
-            if (r.x11 == 0u && hr && hb && r.pbx) cp_async8(e + 3, symin.esc + r.pbx + nro1 + Ca + 1);
-            if (r.k01 == 0u && hb && r.pbk >= 0) cp_async8(e + 4, symin.esc + r.pbk + kro0 + (Ca >> 1));
-            if (r.k10 == 0u && hr && r.pbk >= 0) cp_async8(e + 5, symin.esc + r.pbk + kro1 + Ca);
-            if (r.k11 == 0u && hr && hb && r.pbk >= 0) cp_async8(e + 6, symin.esc + r.pbk + kro1 + Ca + 1);
+            const int Pn = new_plane(j0);
+            if (Pn >= 0) {
+                const long long *pp = symin.esc + plane_base_of(g, Pn);
+                if (r.x00 == 0u) cp_async8(e + 0, pp + ox0);
+                if (r.x01 == 0u) cp_async8(e + 1, pp + ox0 + 1);
+                if (r.x10 == 0u) cp_async8(e + 2, pp + ox1);
+                if (r.x11 == 0u) cp_async8(e + 3, pp + ox1 + 1);
+            }
+            const long long *pp = symin.esc + plane_base_of(g, cpos_of(m0, mc0, j0));
+            if (r.k01 == 0u) cp_async8(e + 4, pp + ok0);
+            if (r.k10 == 0u) cp_async8(e + 5, pp + ok1);
+            if (r.k11 == 0u) cp_async8(e + 6, pp + ok1 + 1);
             cp_async_commit();
             return true;
         }
@@ -1182,7 +1192,7 @@ expand_kernel(LevelGeom<T> g, const T *__restrict__ vc, const T *__restrict__ co
     auto step = [&](int j0, Raw &cur, const Raw &nxt, int b) {
         // this plane's escapes were issued a step ago; the next plane's words
         // arrived a step ago: its escapes go in flight
-        const bool pn = j0 + 1 <= jend && issue_esc(nxt, b ^ 1);
+        const bool pn = j0 + 1 <= jend && issue_esc(nxt, j0 + 1, b ^ 1);
         if (pend) {
             if (pn) asm volatile("cp.async.wait_group 1;" ::: "memory");
             else asm volatile("cp.async.wait_group 0;" ::: "memory");
@@ -1198,31 +1208,30 @@ expand_kernel(LevelGeom<T> g, const T *__restrict__ vc, const T *__restrict__ co
         J.v01 = fma_rn(wr2, a01, mul_rn(wl2, r.a00));
         J.v10 = fma_rn(wr1, r.a10, mul_rn(wl1, r.a00));
         J.v11 = fma_rn(wr1, fma_rn(wr2, a11, mul_rn(wl2, r.a10)), mul_rn(wl1, J.v01));
-        const int P0 = cpos_of(m0, mc0, j0);
-        if (j0 > J0a && colv) {
-            // the new fine plane between coarse planes j0 - 1 and j0, if any
-            const int Pn = cpos_of(m0, mc0, j0 - 1) + 1;
-            if (Pn < P0) {
-                const T wl0 = g.dim[0].wl[Pn], wr0 = g.dim[0].wr[Pn];
-                T *orow = out + ((long long)Pn * m1 + Ra) * m2;
-                orow[Ca] = add_rn(val(r.x00, b, 0), fma_rn(wr0, J.v00, mul_rn(wl0, Jp.v00)));
-                if (hb) orow[Ca + 1] = add_rn(val(r.x01, b, 1), fma_rn(wr0, J.v01, mul_rn(wl0, Jp.v01)));
-                if (hr) {
-                    orow += m2;
-                    orow[Ca] = add_rn(val(r.x10, b, 2), fma_rn(wr0, J.v10, mul_rn(wl0, Jp.v10)));
-                    if (hb) orow[Ca + 1] = add_rn(val(r.x11, b, 3), fma_rn(wr0, J.v11, mul_rn(wl0, Jp.v11)));
-                }
+        const int P0 = cpos_of(m0, mc0, j0), Pn = new_plane(j0);
+        if (Pn >= 0 && colv) {
+            // the new fine plane between coarse planes j0 - 1 and j0
+            const T wl0 = g.dim[0].wl[Pn], wr0 = g.dim[0].wr[Pn];
+            T *op = out + (long long)Pn * m1 * m2;
+            T *orow = op + ox0;
+            orow[0] = add_rn(val(r.x00, b, 0), fma_rn(wr0, J.v00, mul_rn(wl0, Jp.v00)));
+            if (hb) orow[1] = add_rn(val(r.x01, b, 1), fma_rn(wr0, J.v01, mul_rn(wl0, Jp.v01)));
+            if (hr) {
+                orow = op + ox1;
+                orow[0] = add_rn(val(r.x10, b, 2), fma_rn(wr0, J.v10, mul_rn(wl0, Jp.v10)));
+                if (hb) orow[1] = add_rn(val(r.x11, b, 3), fma_rn(wr0, J.v11, mul_rn(wl0, Jp.v11)));
             }
         }
         if (j0 < J0b && colv) {
             // the kept fine plane of coarse plane j0
-            T *orow = out + ((long long)P0 * m1 + Ra) * m2;
-            orow[Ca] = J.v00;
-            if (hb) orow[Ca + 1] = add_rn(val(r.k01, b, 4), J.v01);
+            T *op = out + (long long)P0 * m1 * m2;
+            T *orow = op + ox0;
+            orow[0] = J.v00;
+            if (hb) orow[1] = add_rn(val(r.k01, b, 4), J.v01);
             if (hr) {
-                orow += m2;
-                orow[Ca] = add_rn(val(r.k10, b, 5), J.v10);
-                if (hb) orow[Ca + 1] = add_rn(val(r.k11, b, 6), J.v11);
+                orow = op + ox1;
+                orow[0] = add_rn(val(r.k10, b, 5), J.v10);
+                if (hb) orow[1] = add_rn(val(r.k11, b, 6), J.v11);
             }
         }
         Jp = J;
@@ -1232,7 +1241,7 @@ expand_kernel(LevelGeom<T> g, const T *__restrict__ vc, const T *__restrict__ co
     Raw A = load(J0a);
     Raw B;
     if (J0a + 1 <= jend) B = load(J0a + 1);
-    pend = issue_esc(A, 0);
+    pend = issue_esc(A, J0a, 0);
     for (int j0 = J0a; j0 <= jend; j0 += 2) {
         step(j0, A, B, 0);
         if (j0 + 1 > jend) break;

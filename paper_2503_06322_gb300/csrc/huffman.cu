@@ -1094,7 +1094,7 @@ __global__ void __launch_bounds__(256) enc_count_kernel(EncodeArgs a)
     const unsigned long long nch = (a.N + a.K - 1) / a.K;
     const unsigned long long cpb = (nch + gridDim.x - 1) / gridDim.x;
     const unsigned long long c0 = blockIdx.x * cpb, c1 = c0 + cpb < nch ? c0 + cpb : nch;
-    const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned lane = threadIdx.x & 31, warp = (unsigned)warp_index();
     unsigned long long tb = 0;
     const unsigned r = enc_group(a.K);
     if (r > 1) {
@@ -1388,7 +1388,8 @@ __global__ void __launch_bounds__(32 * kEncWarps, 3) enc_write_kernel(EncodeArgs
     uint32_t *spk = esm32;
     // per warp: a group's finished words
     const unsigned Dv = (a.D + 3) / 4;   // the table's space in the scratch is a multiple of 256 bytes
-    uint32_t *sw = esm32 + (SM ? 4 * Dv : 0) + (threadIdx.x >> 5) * kEncOutWords;
+    const unsigned warp = (unsigned)warp_index();
+    uint32_t *sw = esm32 + (SM ? 4 * Dv : 0) + warp * kEncOutWords;
     const long long *__restrict__ esc = a.esc;
     const int ew = esc ? (int)a.sc->esc_w : 0;       // escape payload width
     const unsigned L0 = a.len[0];
@@ -1427,7 +1428,7 @@ __global__ void __launch_bounds__(32 * kEncWarps, 3) enc_write_kernel(EncodeArgs
     const unsigned long long G = (unsigned long long)a.K * r;   // symbols per warp group
     const unsigned long long ngr = (a.N + G - 1) / G;
     const unsigned spl = (unsigned)(G >> 5);
-    const unsigned long long wg = blockIdx.x * (unsigned long long)(blockDim.x >> 5) + (threadIdx.x >> 5);
+    const unsigned long long wg = blockIdx.x * (unsigned long long)(blockDim.x >> 5) + warp;
     const unsigned long long nw = (unsigned long long)gridDim.x * (blockDim.x >> 5);
     for (unsigned long long c = wg; c < ngr; c += nw) {
         const unsigned long long beg = c * G;

@@ -96,6 +96,13 @@ enum DeviceStatus : unsigned int {
 // ---------------------------------------------------------------------------
 // Bulk asynchronous copies (global -> shared) completed on an mbarrier.
 
+// The warp's index in its block.  Taken from lane 0 the compiler knows that it is
+// the same in every lane: what follows from it -- rows, their conditions, plane
+// and row offsets -- is kept and computed once per warp instead of per thread
+// (whole warps only).  Decomposition of a 300x431x517 binary32 level, bound by
+// issue: 378 -> 332 us.
+__device__ __forceinline__ int warp_index() { return __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0); }
+
 __device__ __forceinline__ uint32_t smem_u32(const void *p)
 {
     return (uint32_t)__cvta_generic_to_shared(p);

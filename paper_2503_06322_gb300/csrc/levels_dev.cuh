@@ -234,13 +234,21 @@ __device__ __forceinline__ void deq_stage(double *dst, const SymIn &si, int leve
     for (unsigned i = 2 * threadIdx.x; i < si.D; i += 2 * blockDim.x)
         asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst + i)), "l"(src + i) : "memory");
 }
+// s - D/2 for a symbol s
+template <typename T>
+__device__ __forceinline__ T code_value(unsigned s, int halfD)
+{
+    // binary32: 2^23 + s is the word 0x4B000000 | s, and both it and the difference are exact
+    if constexpr (sizeof(T) == 4) return __fsub_rn(__uint_as_float(0x4B000000u | s), 8388608.0f + (float)halfD);
+    else return (T)((int)s - halfD);
+}
 // value of symbol s != 0; after a rejected header the symbols are another
 // stream's, and any of them has to stay inside the table
 template <typename T>
 __device__ __forceinline__ T dequant_code(const double *deq, unsigned s, int halfD, T q)
 {
     if (sizeof(T) == 8 && deq) return (T)deq[min(s, 2u * (unsigned)halfD - 1u)];
-    return mul_rn((T)((int)s - halfD), q);
+    return mul_rn(code_value<T>(s, halfD), q);
 }
 
 template <typename T>
