@@ -19,8 +19,12 @@
 // nodes plus a two-node halo) into a ring of shared-memory stages, one bulk
 // asynchronous copy per row, completed on a "full" mbarrier per stage; seven
 // consumer warps compute and hand each stage back on an "empty" mbarrier.
-// Two CTAs of eight warps per SM leave each SM sub-partition four warps, so
-// a thread may hold 128 registers.
+// decomp_kernel: two CTAs of eight warps per SM leave each SM sub-partition four
+// warps, so a thread may hold 128 registers (three CTAs of 80 spill: 513^3
+// compression 1534 -> 1658 us).  rsym_kernel meets a barrier every plane and waits
+// for shared memory, so binary32 runs four CTAs of 64 registers, with two tiles,
+// one escape tile and two or three stages each (two CTAs: 513^3 decompression
+// 1713 us, three 1583, four 1536).
 // Every wait is bounded; a wait that runs out sets DS_TIMEOUT, the consumers
 // leave their plane loop and the producer waits (with a long bound of its
 // own) for every copy still in flight before the CTA exits.
@@ -64,7 +68,7 @@ template <typename E> __host__ __device__ constexpr int stage_pitch();
 template <typename E> __host__ __device__ constexpr int guard_bytes() { return 3 * stage_pitch<E>(); }
 
 template <typename T> __host__ __device__ constexpr int decomp_stages() { return sizeof(T) == 4 ? 6 : 3; }
-template <typename T> __host__ __device__ constexpr int rsym_stages() { return 6; }
+template <typename T> __host__ __device__ constexpr int rsym_stages(bool sym) { return sizeof(T) == 8 ? 4 : sym ? 2 : 3; }
 // bytes per staged row: the region plus the 16-byte alignment of its copy
 template <typename E> __host__ __device__ constexpr int stage_pitch() { return ((DR2 * (int)sizeof(E) + 32) + 15) & ~15; }
 
@@ -709,27 +713,29 @@ decomp_kernel(RestrictArgs<T> a, int seg_len)
 // is kept in dim 1 holds only its odd positions); the consumers expand the
 // region together into one of the shared tiles W, meet at one named barrier
 // per plane (which also carries their vote on a wait that ran out), hand the
-// stage back, and restrict W as decomp_kernel restricts v.
+// stage back, and restrict W as decomp_kernel restricts v.  Two tiles are enough:
+// tile k & 1 is filled again only after the barrier that follows its restriction;
+// one escape tile is, since a thread waits for its own copies before that barrier.
 
 template <typename T, int SRC>
 struct RsymSmem {
     // staged element: symbols (SYMBOLS) or values (STREAM, DENSE)
     using E = typename std::conditional<SRC == (int)WSrc::SYMBOLS, uint16_t, T>::type;
     static constexpr bool ESC = SRC == (int)WSrc::SYMBOLS;
-    static constexpr int NST = rsym_stages<T>();
+    static constexpr int NST = rsym_stages<T>(SRC == (int)WSrc::SYMBOLS);
     static constexpr int PB = stage_pitch<E>();
     static constexpr size_t stage_bytes = (size_t)DR1 * PB;
     static constexpr int WROWS = DR1 + 6;     // zero rows around the region: two before, up to four after
     static constexpr size_t wtile_bytes = (size_t)WROWS * kWPitch * sizeof(T);
     static constexpr size_t off_w = 0;
-    static constexpr size_t off_stage = off_w + 3 * wtile_bytes;   // three dequantized tiles
+    static constexpr size_t off_stage = off_w + 2 * wtile_bytes;   // two dequantized tiles
     static constexpr size_t off_full = off_stage + NST * stage_bytes;
     static constexpr size_t off_empty = off_full + NST * 8;
     static constexpr size_t off_info = off_empty + NST * 8;
     static constexpr size_t off_rows = (off_info + NST * sizeof(PlaneInfo<T>) + 15) & ~size_t(15);
     static constexpr int EPITCH = DR2;           // escaped codes of a plane: [DR1][DR2] int64
     static constexpr size_t off_esc = off_rows + (size_t)NST * DR1 * 16;
-    static constexpr size_t bytes = off_esc + (ESC ? 2 * (size_t)DR1 * EPITCH * 8 : 0);
+    static constexpr size_t bytes = off_esc + (ESC ? (size_t)DR1 * EPITCH * 8 : 0);
 };
 
 // an asynchronous 8-byte global -> shared copy (its own completion group per thread)
@@ -766,7 +772,7 @@ __device__ __forceinline__ bool named_sync_or(int id, int nthreads, bool pred)
 }
 
 template <typename T, int SRC>
-__global__ void __launch_bounds__(DTHREADS, 2)
+__global__ void __launch_bounds__(DTHREADS, sizeof(T) == 4 ? 4 : 2)
 rsym_kernel(RestrictArgs<T> a, int seg_len)
 {
     using S = RsymSmem<T, SRC>;
@@ -885,7 +891,7 @@ rsym_kernel(RestrictArgs<T> a, int seg_len)
     bool failed = false;
     const int nplanes = tg.hi0 - tg.lo0 + 1;
     const int nq = (tg.r2n + 3) >> 2;
-    auto tile = [&](int kk) -> T * { return W0 + (size_t)(kk % 3) * (S::wtile_bytes / sizeof(T)) + 2 * kWPitch + 4; };
+    auto tile = [&](int kk) -> T * { return W0 + (size_t)(kk & 1) * (S::wtile_bytes / sizeof(T)) + 2 * kWPitch + 4; };
     // The dequantized tile of plane kk is filled one iteration before its
     // restriction: the values of its symbols now; its escaped codes travel
     // from global memory into a shared escape tile by asynchronous copies and
@@ -902,7 +908,7 @@ rsym_kernel(RestrictArgs<T> a, int seg_len)
         const int sl = kk % NST;
         const unsigned char *st = smem_raw + S::off_stage + sl * S::stage_bytes;
         const SymRow *ri = rowinfo + sl * DR1;
-        long long *et = esc_tile0 + (size_t)(kk & 1) * DR1 * S::EPITCH;
+        long long *et = esc_tile0;
         unsigned escm = 0;
 #pragma unroll
         for (int it = 0; it < kDqItems; it++) {
@@ -948,7 +954,7 @@ rsym_kernel(RestrictArgs<T> a, int seg_len)
     // the escaped codes of plane kk (this thread's, copied one iteration ago) into its tile
     auto patch = [&](int kk, T *Wt, unsigned escm) {
         if (!SYM || !escm) return;
-        const long long *et = esc_tile0 + (size_t)(kk & 1) * DR1 * S::EPITCH;
+        const long long *et = esc_tile0;
 #pragma unroll
         for (int it = 0; it < kDqItems; it++) {
             const int u = tid + it * DCW * 32;
