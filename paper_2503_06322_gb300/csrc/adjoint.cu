@@ -36,14 +36,15 @@ enum { MP_RT_FINAL = 1, MP_DT_FINAL = 2 };
 constexpr int kMpWarps = 8;
 template <typename T, int MODE>
 __global__ void __launch_bounds__(32 * kMpWarps)
-prolong_kernel(LevelGeom<T> g, const T *__restrict__ y, const T *__restrict__ gsrc, T *__restrict__ stream,
-               const T *__restrict__ coef, T *__restrict__ out, int seg_len)
+prolong_kernel(LevelGeom<T> g, const T *y, const T *gsrc, T *__restrict__ stream, const T *coef, T *__restrict__ out,
+               int seg_len)
 {
     const DimTables<T> &d0 = g.dim[0], &d1 = g.dim[1], &d2 = g.dim[2];
     const int m0 = d0.m, m1 = d1.m, m2 = d2.m, mc0 = d0.mc, mc1 = d1.mc, mc2 = d2.mc;
     const int lane = threadIdx.x & 31, warp = warp_index();
     const int j2 = blockIdx.x * 32 + lane, j1 = blockIdx.y * kMpWarps + warp;
     const int J0a = blockIdx.z * seg_len, J0b = min(J0a + seg_len, mc0);
+    next_begin();
     if (J0a >= J0b || j1 >= mc1 || j2 >= mc2) return;
     const int Ca = cpos_of(m2, mc2, j2), Ra = cpos_of(m1, mc1, j1);
     const bool hb = Ca + 1 < m2 && !kept_pos(m2, Ca + 1), hr = Ra + 1 < m1 && !kept_pos(m1, Ra + 1);
@@ -143,6 +144,7 @@ prolong_kernel(LevelGeom<T> g, const T *__restrict__ y, const T *__restrict__ gs
 template <typename T>
 __global__ void set_kept_kernel(T *G, const T *gv, const T *R, LevelGeom<T> g)
 {
+    next_begin();
     const long long c1 = g.dim[1].mc, c2 = g.dim[2].mc;
     const long long n = (long long)g.dim[0].mc * c1 * c2;
     for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < n; q += (long long)gridDim.x * blockDim.x) {
@@ -168,6 +170,7 @@ __global__ void set_kept_kernel(T *G, const T *gv, const T *R, LevelGeom<T> g)
 template <typename T>
 __global__ void copy_kernel(T *dst, const T *src, long long n)
 {
+    next_begin();
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
         dst[i] = src[i];
 }
@@ -181,10 +184,9 @@ cudaError_t launch_prolong(const LevelGeom<T> &g, const T *y, T *out, const T *g
     const int mc0 = g.dim[0].mc, mc1 = g.dim[1].mc, mc2 = g.dim[2].mc;
     const int gx = (mc2 + 31) / 32, gy = (mc1 + kMpWarps - 1) / kMpWarps;
     const int seg = choose_segment(mc0, (long long)gx * gy, resident_ctas(prolong_kernel<T, MODE>, 32 * kMpWarps, 0));
-    prolong_kernel<T, MODE><<<dim3(gx, gy, (mc0 + seg - 1) / seg), 32 * kMpWarps, 0, s>>>(g, y, gsrc, stream, coef, out,
-                                                                                       seg);
     count_launch();
-    return cudaGetLastError();
+    return launch_next(prolong_kernel<T, MODE>, dim3(gx, gy, (mc0 + seg - 1) / seg), 32 * kMpWarps, 0, s, g, y, gsrc, stream,
+                       coef, out, seg);
 }
 
 }  // namespace
@@ -216,9 +218,8 @@ cudaError_t recompose_adjoint_run(const Plan &P, const LevelGeom<T> *geo, const 
         gl = gc;
     }
     if (ls >= 1) return launch_coarse_adjoint<T>(P, geo, ls, gl, gcoef, s);
-    copy_kernel<T><<<grid_for(P.N[0]), 256, 0, s>>>(gcoef, gl, P.N[0]);
     count_launch();
-    return cudaGetLastError();
+    return launch_next(copy_kernel<T>, grid_for(P.N[0]), 256, 0, s, gcoef, gl, P.N[0]);
 }
 
 template <typename T>
@@ -227,13 +228,14 @@ cudaError_t decompose_adjoint_run(const Plan &P, const LevelGeom<T> *geo, const 
 {
     const int L = P.L;
     T *gv = (L == 0) ? gu : ((L % 2 == 1) ? ga : gb);
-    copy_kernel<T><<<grid_for(P.N[0]), 256, 0, s>>>(gv, gcoef, P.N[0]);
     count_launch();
+    cudaError_t e = launch_next(copy_kernel<T>, grid_for(P.N[0]), 256, 0, s, gv, gcoef, P.N[0]);
+    if (e != cudaSuccess) return e;
     for (int l = 1; l <= L; l++) {
         const LevelGeom<T> &g = geo[l];
         T *G = (l == L) ? gu : (((L - l) % 2 == 1) ? ga : gb);
         const long long nc = P.N[l - 1];
-        cudaError_t e = launch_solves<T>(g, y, nullptr, 0, s, gv);
+        e = launch_solves<T>(g, y, nullptr, 0, s, gv);
         if (e != cudaSuccess) return e;
         // new nodes: G = h = g_c + ((x)M_l P) y
         e = launch_prolong<T, MP_DT_FINAL>(g, y, G, nullptr, nullptr, gcoef, s);
@@ -249,8 +251,9 @@ cudaError_t decompose_adjoint_run(const Plan &P, const LevelGeom<T> *geo, const 
         a.status = status;
         e = launch_restrict<T>(WSrc::DENSE, Sink::NONE, a, s);
         if (e != cudaSuccess) return e;
-        set_kept_kernel<T><<<grid_for(nc), 256, 0, s>>>(G, gv, R, g);
         count_launch();
+        e = launch_next(set_kept_kernel<T>, grid_for(nc), 256, 0, s, G, gv, R, g);
+        if (e != cudaSuccess) return e;
         gv = G;
     }
     return cudaGetLastError();

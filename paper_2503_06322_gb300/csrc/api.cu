@@ -205,6 +205,7 @@ void l2s_weights(const Plan *P, L2sArgs &a)
 // bound) and replaces its bins; a rejected bound or a zero field keeps them
 __global__ void bins_l2s_kernel(L2sArgs a, Scalars *sc)
 {
+    next_begin();
     if (sc->status) return;
     const double mx = sc->maxabs;
     if (!(mx > 0.0)) return;
@@ -283,9 +284,8 @@ hpdr_status compress_core(hpdr_ctx *ctx, const Plan *P, const T *u, int ndim, co
         memset(&la, 0, sizeof(la));
         l2s_weights(P, la);
         la.eps = ba.eps;
-        bins_l2s_kernel<<<1, 32, 0, s>>>(la, w.sc);
         count_launch();
-        CK(cudaGetLastError());
+        CK(launch_next(bins_l2s_kernel, 1, 32, 0, s, la, w.sc));
     }
 
     const T *v = u;
@@ -458,6 +458,7 @@ hpdr_status parse_header(const uint8_t *b, size_t avail, size_t in_bytes, Hdr *h
 // status of one decompression OR-ed into an accumulated word
 __global__ void accumulate_status_kernel(const Scalars *sc, unsigned *acc)
 {
+    next_begin();
     if (sc->status) atomicOr(acc, sc->status);
 }
 
@@ -559,9 +560,8 @@ hpdr_status decompress_t(hpdr_ctx *ctx, const Plan *P, const Hdr &h, const uint8
     st = decompress_levels<T>(ctx, P, h.D, h.N, w, out, s);
     if (st != HPDR_OK) return st;
     if (err_acc) {
-        accumulate_status_kernel<<<1, 1, 0, s>>>(w.sc, err_acc);
         count_launch();
-        CK(cudaGetLastError());
+        CK(launch_next(accumulate_status_kernel, 1, 1, 0, s, w.sc, err_acc));
         return HPDR_OK;
     }
     CK(cudaMemcpyAsync(hsc, w.sc, sizeof(Scalars), cudaMemcpyDeviceToHost, s));
@@ -571,7 +571,11 @@ hpdr_status decompress_t(hpdr_ctx *ctx, const Plan *P, const Hdr &h, const uint8
 }
 
 // {status} of one call into a device word
-__global__ void status_out_kernel(const Scalars *sc, unsigned long long *dst) { dst[0] = sc->status; }
+__global__ void status_out_kernel(const Scalars *sc, unsigned long long *dst)
+{
+    next_begin();
+    dst[0] = sc->status;
+}
 
 // decompression whose header is read on the device: no host wait
 template <typename T>
@@ -614,9 +618,8 @@ hpdr_status decompress_dev(hpdr_ctx *ctx, const Plan *P, int dtype, int ndim, co
     }
     st = decompress_levels<T>(ctx, P, D, ex.N, w, out, s);
     if (st != HPDR_OK) return st;
-    status_out_kernel<<<1, 1, 0, s>>>(w.sc, d_result);
     count_launch();
-    CK(cudaGetLastError());
+    CK(launch_next(status_out_kernel, 1, 1, 0, s, w.sc, d_result));
     return HPDR_OK;
 }
 

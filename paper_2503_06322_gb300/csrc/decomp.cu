@@ -337,7 +337,7 @@ decomp_kernel(RestrictArgs<T> a, int seg_len)
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const LevelGeom<T> &g = a.g;
     const TileGeom tg = tile_geom(g, seg_len);
-    if (tg.J0a >= tg.J0b) return;
+    if (tg.J0a >= tg.J0b) { next_begin(); return; }
     const int m0 = g.dim[0].m, m1 = g.dim[1].m, m2 = g.dim[2].m;
     const int mc0 = g.dim[0].mc, mc1 = g.dim[1].mc, mc2 = g.dim[2].mc;
     unsigned long long *full = reinterpret_cast<unsigned long long *>(smem_raw + S::off_full);
@@ -368,6 +368,7 @@ decomp_kernel(RestrictArgs<T> a, int seg_len)
             mbar_fence_init();
         }
     }
+    next_begin();
     __syncthreads();
 
     if (warp == DCW) {
@@ -785,7 +786,7 @@ rsym_kernel(RestrictArgs<T> a, int seg_len)
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const LevelGeom<T> &g = a.g;
     const TileGeom tg = tile_geom(g, seg_len);
-    if (tg.J0a >= tg.J0b) return;
+    if (tg.J0a >= tg.J0b) { next_begin(); return; }
     const int m0 = g.dim[0].m, m1 = g.dim[1].m, m2 = g.dim[2].m;
     const int mc1 = g.dim[1].mc, mc2 = g.dim[2].mc;
     unsigned long long *full = reinterpret_cast<unsigned long long *>(smem_raw + S::off_full);
@@ -810,6 +811,7 @@ rsym_kernel(RestrictArgs<T> a, int seg_len)
             mbar_fence_init();
         }
     }
+    next_begin();
     __syncthreads();
 
     if (warp == DCW) {
@@ -1062,7 +1064,7 @@ constexpr int XTHREADS = XW * 32;
 
 template <typename T, int SRC>
 __global__ void __launch_bounds__(XTHREADS)
-expand_kernel(LevelGeom<T> g, const T *__restrict__ vc, const T *__restrict__ coef_in, SymIn symin,
+expand_kernel(LevelGeom<T> g, const T *vc, const T *coef_in, SymIn symin,
               T *__restrict__ out, int seg_len)
 {
     const int m0 = g.dim[0].m, m1 = g.dim[1].m, m2 = g.dim[2].m;
@@ -1070,6 +1072,7 @@ expand_kernel(LevelGeom<T> g, const T *__restrict__ vc, const T *__restrict__ co
     const int lane = threadIdx.x & 31, warp = warp_index();
     const int j2 = blockIdx.x * 32 + lane, j1 = blockIdx.y * XW + warp;
     const int J0a = blockIdx.z * seg_len, J0b = min(J0a + seg_len, mc0);
+    next_begin();
     if (J0a >= J0b || blockIdx.y * XW >= mc1) return;
     extern __shared__ __align__(16) unsigned char xsm[];
     // binary64 symbols: the level's values, behind the escape slots
@@ -1278,9 +1281,8 @@ cudaError_t launch_decomp(Sink sink, const RestrictArgs<T> &a0, cudaStream_t s)
         if (e != cudaSuccess) return e;
         const int seg = choose_segment(mc0, (long long)gx * gy, resident_ctas(kern, DTHREADS, sm));
         const int gz = (mc0 + seg - 1) / seg;
-        kern<<<dim3(gx, gy, gz), DTHREADS, sm, s>>>(a, seg);
         count_launch();
-        return cudaGetLastError();
+        return launch_next(kern, dim3(gx, gy, gz), DTHREADS, sm, s, a, seg);
     };
     if (sink == Sink::QUANT) return go(decomp_kernel<T, (int)Sink::QUANT>, attr_quant);
     return go(decomp_kernel<T, (int)Sink::STREAM>, attr_stream);
@@ -1310,9 +1312,8 @@ cudaError_t launch_restrict_planes(WSrc src, const RestrictArgs<T> &a0, cudaStre
         if (e != cudaSuccess) return e;
         const int seg = choose_segment(mc0, (long long)gx * gy, resident_ctas(kern, DTHREADS, sm));
         const int gz = (mc0 + seg - 1) / seg;
-        kern<<<dim3(gx, gy, gz), DTHREADS, sm, s>>>(a, seg);
         count_launch();
-        return cudaGetLastError();
+        return launch_next(kern, dim3(gx, gy, gz), DTHREADS, sm, s, a, seg);
     };
     static PerDeviceOnce attr_sym, attr_stream, attr_dense;
     if (src == WSrc::STREAM)
@@ -1341,12 +1342,9 @@ cudaError_t launch_expand_planes(WSrc src, const LevelGeom<T> &g, const T *vc, c
                               : resident_ctas(expand_kernel<T, (int)WSrc::SYMBOLS>, XTHREADS, sm);
     const int seg = choose_segment(mc0, (long long)gx * gy, per_sm);
     const int gz = (mc0 + seg - 1) / seg;
-    if (stream)
-        expand_kernel<T, (int)WSrc::STREAM><<<dim3(gx, gy, gz), XTHREADS, 0, s>>>(g, vc, coef_in, symin, out, seg);
-    else
-        expand_kernel<T, (int)WSrc::SYMBOLS><<<dim3(gx, gy, gz), XTHREADS, sm, s>>>(g, vc, coef_in, symin, out, seg);
     count_launch();
-    return cudaGetLastError();
+    return launch_next(stream ? expand_kernel<T, (int)WSrc::STREAM> : expand_kernel<T, (int)WSrc::SYMBOLS>,
+                       dim3(gx, gy, gz), XTHREADS, sm, s, g, vc, coef_in, symin, out, seg);
 }
 
 template cudaError_t launch_decomp<float>(Sink, const RestrictArgs<float> &, cudaStream_t);

@@ -770,6 +770,7 @@ __device__ __forceinline__ void codebook_body(const unsigned long long *hist, un
 
 __global__ void __launch_bounds__(1024, 1) codebook_kernel(const unsigned long long *hist, unsigned D, HuffScratch hs)
 {
+    next_begin();
     codebook_body(hist, D, hs);
 }
 
@@ -884,6 +885,7 @@ __global__ void __launch_bounds__(kTabThreads, 1) dec_tables_kernel(TabArgs a, H
     __shared__ int okc;
     const unsigned tid = threadIdx.x, lane = tid & 31, w = tid >> 5, D = a.D;
     const bool lead = blockIdx.x == 0;
+    next_begin();
     // ---- scalars and header
     const uint8_t *lenb = a.lenb;
     unsigned s_lo = a.s_lo, s_hi = a.s_hi;
@@ -1083,6 +1085,7 @@ __global__ void __launch_bounds__(256) enc_count_kernel(EncodeArgs a)
     const S *__restrict__ sym = reinterpret_cast<const S *>(a.sym);
     extern __shared__ __align__(16) uint8_t slen[];
     __shared__ unsigned long long wb[8];
+    next_begin();
     if (block_skip(&a.sc->status)) return;
     // the length table's space in the scratch is a multiple of 256 bytes
     for (unsigned i = threadIdx.x; i < (a.D + 15) / 16; i += blockDim.x)
@@ -1180,6 +1183,7 @@ __device__ __forceinline__ uint32_t *enc_words(const EncodeArgs &a, unsigned lon
 __global__ void __launch_bounds__(256) enc_scan_kernel(EncodeArgs a)
 {
     __shared__ unsigned long long spre[8], stot[8];
+    next_begin();
     if (block_skip(&a.sc->status)) return;
     const unsigned long long nch = (a.N + a.K - 1) / a.K;
     const unsigned long long cpb = (nch + gridDim.x - 1) / gridDim.x;
@@ -1383,6 +1387,7 @@ template <typename S, bool SM>
 __global__ void __launch_bounds__(32 * kEncWarps, 3) enc_write_kernel(EncodeArgs a)
 {
     extern __shared__ __align__(16) uint32_t esm32[];
+    next_begin();
     if (block_skip(&a.sc->status)) return;
     const S *__restrict__ sym = reinterpret_cast<const S *>(a.sym);
     uint32_t *spk = esm32;
@@ -1636,7 +1641,11 @@ __device__ __forceinline__ void header_job(const HeaderJob &j)
         j.size_status[1] = j.sc->status;
     }
 }
-__global__ void __launch_bounds__(kHeaderThreads) header_kernel(HeaderJob j) { header_job(j); }
+__global__ void __launch_bounds__(kHeaderThreads) header_kernel(HeaderJob j)
+{
+    next_begin();
+    header_job(j);
+}
 __global__ void __launch_bounds__(kHeaderThreads) header_batch_kernel(const HeaderJob *jobs)
 {
     header_job(jobs[blockIdx.x]);
@@ -1972,6 +1981,7 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_kernel(DecodeArgs a_in,
 {
     DecodeArgs a = a_in;
     const unsigned long long nch = (a.N + a.K - 1) / a.K;
+    next_begin();
     if (blockIdx.x >= nch) return;
     if (block_skip(hs.status)) return;
     if (a.dh) {
@@ -2262,9 +2272,8 @@ cudaError_t launch_codebook(const unsigned long long *hist, unsigned int D, cons
     cudaError_t e = set_attrs();
     if (e != cudaSuccess) return e;
     if (D <= kFusedMaxD) {
-        codebook_kernel<<<1, 1024, kCodebookSmem, s>>>(hist, D, hs);
         count_launch();
-        return cudaGetLastError();
+        return launch_next(codebook_kernel, 1, 1024, kCodebookSmem, s, hist, D, hs);
     }
     compact_kernel<<<1, 1024, 0, s>>>(hist, nullptr, D, hs.keys, hs.nsym, hs.s_lo, hs.s_hi);
     rank_kernel<<<kRankBlocks, 256, kSmemKeys * 8, s>>>(hs.keys, hs.nsym, hs.sorted, nullptr);
@@ -2279,9 +2288,8 @@ cudaError_t launch_decode_tables(const TabArgs &a, const HuffScratch &hs, cudaSt
 {
     cudaError_t e = set_attrs();
     if (e != cudaSuccess) return e;
-    dec_tables_kernel<<<kTabBlocks, kTabThreads, kTabSmem + a.D, s>>>(a, hs);
     count_launch();
-    return cudaGetLastError();
+    return launch_next(dec_tables_kernel, kTabBlocks, kTabThreads, kTabSmem + a.D, s, a, hs);
 }
 
 cudaError_t launch_encode(const EncodeArgs &a, cudaStream_t s)
@@ -2293,30 +2301,27 @@ cudaError_t launch_encode(const EncodeArgs &a, cudaStream_t s)
     const unsigned nb = (unsigned)std::min<unsigned long long>(kEncBlocks, (groups + 7) / 8);
     const bool code_sm = a.D <= (unsigned)kSmemCodes;
     const size_t smc = (a.D + 15) / 16 * 16, smw = ((code_sm ? (size_t)(a.D + 3) / 4 * 4 : 0) + kEncWarps * kEncOutWords) * 4;
-    if (a.bytes) enc_count_kernel<uint8_t><<<nb, 256, smc, s>>>(a);
-    else enc_count_kernel<uint16_t><<<nb, 256, smc, s>>>(a);
-    enc_scan_kernel<<<nb, 256, 0, s>>>(a);
-    const auto write = [&](auto kern) {
+    e = launch_next(a.bytes ? enc_count_kernel<uint8_t> : enc_count_kernel<uint16_t>, nb, 256, smc, s, a);
+    if (e == cudaSuccess) e = launch_next(enc_scan_kernel, nb, 256, 0, s, a);
+    if (e != cudaSuccess) return e;
+    const auto write = [&](auto kern) -> cudaError_t {
         int per_sm = 0;
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * kEncWarps, smw) != cudaSuccess) {
             cudaGetLastError();
             per_sm = 3;
         }
         const unsigned long long full = (unsigned long long)sm_count() * std::max(1, per_sm);
-        kern<<<(unsigned)std::min(full, (groups + kEncWarps - 1) / kEncWarps), 32 * kEncWarps, smw, s>>>(a);
+        return launch_next(kern, (unsigned)std::min(full, (groups + kEncWarps - 1) / kEncWarps), 32 * kEncWarps, smw, s, a);
     };
-    if (a.bytes) write(enc_write_kernel<uint8_t, true>);
-    else if (code_sm) write(enc_write_kernel<uint16_t, true>);
-    else write(enc_write_kernel<uint16_t, false>);
     count_launch(3);
-    return cudaGetLastError();
+    if (a.bytes) return write(enc_write_kernel<uint8_t, true>);
+    return code_sm ? write(enc_write_kernel<uint16_t, true>) : write(enc_write_kernel<uint16_t, false>);
 }
 
 cudaError_t launch_header(const HeaderJob &j, cudaStream_t s)
 {
-    header_kernel<<<1, kHeaderThreads, 0, s>>>(j);
     count_launch();
-    return cudaGetLastError();
+    return launch_next(header_kernel, 1, kHeaderThreads, 0, s, j);
 }
 
 bool codebook_fused(unsigned int D) { return D <= kFusedMaxD; }
@@ -2388,10 +2393,8 @@ cudaError_t launch_decode(const DecodeArgs &a, const HuffScratch &hs, cudaStream
 {
     cudaError_t e = set_attrs();
     if (e != cudaSuccess) return e;
-    if (a.bytes) decode_kernel<uint8_t><<<sm_count(), kDecThreads, kDecSmem, s>>>(a, hs);
-    else decode_kernel<uint16_t><<<sm_count(), kDecThreads, kDecSmem, s>>>(a, hs);
     count_launch();
-    return cudaGetLastError();
+    return launch_next(a.bytes ? decode_kernel<uint8_t> : decode_kernel<uint16_t>, sm_count(), kDecThreads, kDecSmem, s, a, hs);
 }
 
 }  // namespace hpdr

@@ -166,6 +166,50 @@ __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t by
 constexpr int kWaitPolls = 1 << 20;
 
 // ---------------------------------------------------------------------------
+// A call is a chain of up to fifty launches, many of them a few microseconds
+// long, so the gap between one kernel's end and the next one's start counts.
+// The chain's kernels are launched as programmatic dependents (launch_next): the
+// next kernel's blocks start as the last blocks of this one leave, and wait in
+// next_begin(), the first thing a kernel does before it touches memory that an
+// earlier one writes.  The wait ends when the kernel before has completed with
+// its writes visible, and that kernel waited for its own predecessor, so the order
+// of the chain is that of a plain stream.  No kernel triggers the next one
+// earlier: blocks that become resident beside a kernel with few free registers
+// crowd on the SMs it leaves empty (round trips of 500x500x100 binary64: 3758 ->
+// 3840 us with a trigger at the start, 3782 -> 3651 without one; of 130x67x45
+// 363 -> 296, training steps at 257^3 778 -> 676).  What the kernel before writes
+// is not read through pointers that promise it to be constant (__restrict__ on a
+// const pointer), whose loads may be moved up.
+__device__ __forceinline__ void next_begin()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+// A stream that is being captured takes a plain launch (its graph orders the
+// kernels by full dependencies).
+template <typename... P, typename... A>
+cudaError_t launch_next(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A &&...args)
+{
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) {
+        cudaGetLastError();   // the launch itself decides whether it is allowed
+        cap = cudaStreamCaptureStatusActive;
+    }
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t c = {};
+    c.gridDim = grid;
+    c.blockDim = block;
+    c.dynamicSmemBytes = smem;
+    c.stream = s;
+    c.attrs = &at;
+    c.numAttrs = cap == cudaStreamCaptureStatusNone ? 1 : 0;
+    cudaError_t e = cudaLaunchKernelEx(&c, kern, static_cast<P>(args)...);
+    if (e != cudaSuccess) cudaGetLastError();
+    return e;
+}
+
+// ---------------------------------------------------------------------------
 // Plans: hierarchy + device tables for one (shape, dtype).
 
 struct Plan {

@@ -26,6 +26,7 @@ __global__ void __launch_bounds__(256)
 solve_strided_kernel(T *b, const T *src, int n, long long stride, long long nlines, const T *__restrict__ sub,
                      const T *__restrict__ cp, const T *__restrict__ inv_den, T *vc, int sign)
 {
+    next_begin();
     long long line = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (line >= nlines) return;
     long long o = line / stride, i = line - o * stride;
@@ -65,7 +66,9 @@ solve_stream_kernel(T *b, const T *src, int n, long long st, long long ostride, 
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     T *csub = reinterpret_cast<T *>(smem_raw), *ccp = csub + n, *cinv = ccp + n;
+    // the plan's tables do not change: staged before the wait
     for (int t = threadIdx.x; t < n; t += blockDim.x) { csub[t] = sub[t]; ccp[t] = cp[t]; cinv[t] = inv_den[t]; }
+    next_begin();
     __syncthreads();
     const long long line = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (line >= nlines) return;
@@ -243,6 +246,8 @@ solve_contig_kernel(T *b, const T *src, int n, long long nlines, int rows, const
     T *tile = csub + (3 * n + V - 1) / V * V;
     const long long row0 = blockIdx.x * (long long)rows, first = row0 * n;
     const int nr = (int)min((long long)rows, nlines - row0), cnt = nr * n;
+    for (int t = threadIdx.x; t < n; t += blockDim.x) { csub[t] = sub[t]; ccp[t] = cp[t]; cinv[t] = inv_den[t]; }
+    next_begin();
     // the right-hand side (b, or an array that is kept) and where it sits modulo
     // 16 bytes; without v_c the solution takes its place, so b has to agree
     T *B = tile + ((uintptr_t)(src + first) & 15) / sizeof(T);
@@ -252,7 +257,6 @@ solve_contig_kernel(T *b, const T *src, int n, long long nlines, int rows, const
         X = tile + (rows * n + 2 * V - 1) / V * V + ((uintptr_t)(vc + first) & 15) / sizeof(T);
         run_load(X, vc + first, cnt);
     }
-    for (int t = threadIdx.x; t < n; t += blockDim.x) { csub[t] = sub[t]; ccp[t] = cp[t]; cinv[t] = inv_den[t]; }
     cp_async_wait_all();
     __syncthreads();
     if ((int)threadIdx.x < nr) {
@@ -309,6 +313,7 @@ solve_contig_kernel(T *b, const T *src, int n, long long nlines, int rows, const
 template <typename T, int SINK>
 __global__ void level0_kernel(const T *v0, long long N0, T *coef_out, QuantOut qo)
 {
+    next_begin();
     long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (i >= N0) return;
     T x = v0[i];
@@ -319,6 +324,7 @@ __global__ void level0_kernel(const T *v0, long long N0, T *coef_out, QuantOut q
 template <typename T, int SRC>
 __global__ void level0_in_kernel(const T *coef_in, SymIn symin, long long N0, T *v0)
 {
+    next_begin();
     long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (i >= N0) return;
     v0[i] = (SRC == (int)WSrc::STREAM) ? coef_in[i] : dequant<T>(symin, i, 0);
@@ -410,9 +416,10 @@ __device__ __forceinline__ void bins_body(const BinArgs &ba, const volatile doub
 }
 
 template <typename T>
-__global__ void __launch_bounds__(256) norm_kernel(const T *__restrict__ u, long long N, double *partials, BinArgs ba,
+__global__ void __launch_bounds__(256) norm_kernel(const T *u, long long N, double *partials, BinArgs ba,
                                                    Scalars *sc)
 {
+    next_begin();
     typename BitsOf<T>::type mx = 0;
     T ssT = (T)0;   // per-thread partial sum in T (binary64 arithmetic is slow on this part)
     double ss = 0.0;
@@ -889,6 +896,7 @@ __device__ __forceinline__ void coarse_body(const CoarseArgs<T> &a)
 template <typename T, int MODE>
 __global__ void __launch_bounds__(kCoarseThreads, 1) coarse_kernel(CoarseArgs<T> a)
 {
+    next_begin();
     if (a.staged) coarse_body<T, MODE, true>(a);
     else coarse_body<T, MODE, false>(a);
 }
@@ -966,6 +974,7 @@ __global__ void __launch_bounds__(kCoarseThreads, 1) coarse_adjoint_kernel(Adjoi
     T *RA = Y + nc;                                 // [ra]
     T *RB = RA + z.ra;                              // [rb]
     T *tab = RB + z.rb;
+    next_begin();
     // extents and offsets of every dimension (thread 0: a few dozen), then the tables
     if (tid == 0) {
         int off = 0;
@@ -1115,6 +1124,7 @@ cudaError_t launch_solves(const LevelGeom<T> &g, T *b, T *vc, int sign, cudaStre
         const DimTables<T> &d = g.dim[k];
         if (!(d.m > 1)) continue;
         int sg = (k == last) ? sign : 0;
+        cudaError_t e;
         // the streaming sweep keeps the three factor tables in shared memory
         // (at most the default 48 KB); longer lines take the strided kernel
         if (k < 2 && sg == 0 && 3 * (size_t)d.mc * sizeof(T) <= 48 * 1024) {
@@ -1123,15 +1133,14 @@ cudaError_t launch_solves(const LevelGeom<T> &g, T *b, T *vc, int sign, cudaStre
             const long long outer = (k == 0) ? c1 : c0;
             const long long ostride = (k == 0) ? c2 : c1 * c2;
             const long long nlines = outer * c2;
-            solve_stream_kernel<T><<<(unsigned)((nlines + kSolveThreads - 1) / kSolveThreads), kSolveThreads,
-                                     3 * (size_t)d.mc * sizeof(T), s>>>(
-                b, src, d.mc, st, ostride, c2, nlines, d.sub, d.cp, d.inv_den);
+            e = launch_next(solve_stream_kernel<T>, (unsigned)((nlines + kSolveThreads - 1) / kSolveThreads), kSolveThreads,
+                            3 * (size_t)d.mc * sizeof(T), s, b, src, d.mc, st, ostride, c2, nlines, d.sub, d.cp, d.inv_den);
         } else if (k < 2) {
             long long stride = (k == 0) ? c1 * c2 : c2;
             long long nlines = (k == 0) ? c1 * c2 : c0 * c2;
             int n = d.mc;
-            solve_strided_kernel<T><<<(unsigned)((nlines + 255) / 256), 256, 0, s>>>(
-                b, src, n, stride, nlines, d.sub, d.cp, d.inv_den, vc, sg);
+            e = launch_next(solve_strided_kernel<T>, (unsigned)((nlines + 255) / 256), 256, 0, s, b, src, n, stride, nlines,
+                            d.sub, d.cp, d.inv_den, vc, sg);
         } else {
             int n = d.mc;
             long long nlines = c0 * c1;
@@ -1142,8 +1151,8 @@ cudaError_t launch_solves(const LevelGeom<T> &g, T *b, T *vc, int sign, cudaStre
             size_t rows = std::min<size_t>(kContigRows, lines_in(100));
             if (rows < 8) rows = std::min<size_t>(8, lines_in(kContigMaxKb));
             if (rows < 1) {
-                solve_strided_kernel<T><<<(unsigned)((nlines + 255) / 256), 256, 0, s>>>(
-                    b, src, n, 1, nlines, d.sub, d.cp, d.inv_den, vc, sg);
+                e = launch_next(solve_strided_kernel<T>, (unsigned)((nlines + 255) / 256), 256, 0, s, b, src, n, 1, nlines,
+                                d.sub, d.cp, d.inv_den, vc, sg);
             } else {
                 static PerDeviceOnce attr;
                 cudaError_t ea = once_per_device(attr, [] {
@@ -1151,13 +1160,12 @@ cudaError_t launch_solves(const LevelGeom<T> &g, T *b, T *vc, int sign, cudaStre
                                                 (int)(kContigMaxKb * 1024));
                 });
                 if (ea != cudaSuccess) return ea;
-                solve_contig_kernel<T><<<(unsigned)((nlines + rows - 1) / rows), kContigThreads, fixed + rows * line, s>>>(
-                    b, src, n, nlines, (int)rows, d.sub, d.cp, d.inv_den, vc, sg);
+                e = launch_next(solve_contig_kernel<T>, (unsigned)((nlines + rows - 1) / rows), kContigThreads,
+                                fixed + rows * line, s, b, src, n, nlines, (int)rows, d.sub, d.cp, d.inv_den, vc, sg);
             }
         }
         src = b;
         count_launch();
-        cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
@@ -1175,10 +1183,9 @@ cudaError_t launch_level0(Sink sink, const T *v0, long long N0, T *coef_out, con
                           cudaStream_t s)
 {
     unsigned blocks = (unsigned)((N0 + 255) / 256);
-    if (sink == Sink::STREAM) level0_kernel<T, 1><<<blocks, 256, 0, s>>>(v0, N0, coef_out, qo);
-    else level0_kernel<T, 2><<<blocks, 256, 0, s>>>(v0, N0, coef_out, qo);
     count_launch();
-    return cudaGetLastError();
+    return launch_next(sink == Sink::STREAM ? level0_kernel<T, 1> : level0_kernel<T, 2>, blocks, 256, 0, s, v0, N0, coef_out,
+                       qo);
 }
 
 template <typename T>
@@ -1186,10 +1193,9 @@ cudaError_t launch_level0_in(WSrc src, const T *coef_in, const SymIn &symin, lon
                              cudaStream_t s)
 {
     unsigned blocks = (unsigned)((N0 + 255) / 256);
-    if (src == WSrc::STREAM) level0_in_kernel<T, 1><<<blocks, 256, 0, s>>>(coef_in, symin, N0, v0);
-    else level0_in_kernel<T, 2><<<blocks, 256, 0, s>>>(coef_in, symin, N0, v0);
     count_launch();
-    return cudaGetLastError();
+    return launch_next(src == WSrc::STREAM ? level0_in_kernel<T, 1> : level0_in_kernel<T, 2>, blocks, 256, 0, s, coef_in, symin,
+                       N0, v0);
 }
 
 template <typename T>
@@ -1200,9 +1206,8 @@ cudaError_t launch_norm(const T *u, long long N, double *partials, const BinArgs
     // the same thread, and the blocks left out would add zeros
     const long long need = (N * (long long)sizeof(T) / 16 + 255) / 256 + 1;
     const int blocks = (((uintptr_t)u) & 15) == 0 && need < kNormBlocks ? (int)need : kNormBlocks;
-    norm_kernel<T><<<blocks, 256, 0, s>>>(u, N, partials, ba, sc);
     count_launch();
-    return cudaGetLastError();
+    return launch_next(norm_kernel<T>, blocks, 256, 0, s, u, N, partials, ba, sc);
 }
 
 template <typename T>
@@ -1288,9 +1293,8 @@ cudaError_t launch_coarse(int mode, const Plan *P, const LevelGeom<T> *geo, int 
             return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCoarseSmemMax);
         });
         if (e != cudaSuccess) return e;
-        kern<<<1, kCoarseThreads, sm, s>>>(a);
         count_launch();
-        return cudaGetLastError();
+        return launch_next(kern, 1, kCoarseThreads, sm, s, a);
     };
     switch (mode) {
     case 0: return go(coarse_kernel<T, 0>);
@@ -1332,9 +1336,9 @@ cudaError_t launch_coarse_adjoint(const Plan &P, const LevelGeom<T> *geo, int ls
                                     (int)kCoarseSmemMax);
     });
     if (e != cudaSuccess) return e;
-    coarse_adjoint_kernel<T><<<1, kCoarseThreads, (size_t)(z.nl + 2 * z.nc + z.ra + z.rb + z.tab) * sizeof(T), s>>>(a);
     count_launch();
-    return cudaGetLastError();
+    return launch_next(coarse_adjoint_kernel<T>, 1, kCoarseThreads,
+                       (size_t)(z.nl + 2 * z.nc + z.ra + z.rb + z.tab) * sizeof(T), s, a);
 }
 
 #define INST(T)                                                                                   \
