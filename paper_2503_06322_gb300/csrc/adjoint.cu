@@ -26,7 +26,8 @@ enum { MP_RT_FINAL = 1, MP_DT_FINAL = 2 };
 //   MP_DT_FINAL: out[p] = coef[rank(p)] + y_f(p)
 // One pass over the fine grid is all it needs from memory (a pass per dimension,
 // through two partial grids, moved 2.6 times the bytes and took 173 us for the
-// finest level of 257^3, this 78).  A warp owns coarse row j1 of a tile,
+// finest level of 257^3; this takes 62, bound by instruction issue: 78 with 64-bit offsets
+// and the window's edges tested at every node).  A warp owns coarse row j1 of a tile,
 // lane l coarse column j2, and the CTA marches along the coarse planes of its
 // segment; for each plane a lane forms the dimension-2, then the dimension-1
 // products at its 2 x 2 fine nodes (rows Ra, Ra + 1, columns Ca, Ca + 1) from the
@@ -45,8 +46,10 @@ prolong_kernel(LevelGeom<T> g, const T *y, const T *gsrc, T *__restrict__ stream
     const int j2 = blockIdx.x * 32 + lane, j1 = blockIdx.y * kMpWarps + warp;
     const int J0a = blockIdx.z * seg_len, J0b = min(J0a + seg_len, mc0);
     next_begin();
-    if (J0a >= J0b || j1 >= mc1 || j2 >= mc2) return;
-    const int Ca = cpos_of(m2, mc2, j2), Ra = cpos_of(m1, mc1, j1);
+    if (J0a >= J0b || j1 >= mc1) return;
+    const bool live = j2 < mc2;
+    const int jc = live ? j2 : mc2 - 1;
+    const int Ca = cpos_of(m2, mc2, jc), Ra = cpos_of(m1, mc1, j1);
     const bool hb = Ca + 1 < m2 && !kept_pos(m2, Ca + 1), hr = Ra + 1 < m1 && !kept_pos(m1, Ra + 1);
     // taps of the two fine columns and rows; the second ones start at the same
     // coarse index or one later
@@ -61,12 +64,37 @@ prolong_kernel(LevelGeom<T> g, const T *y, const T *gsrc, T *__restrict__ stream
         e1[1][i] = hr ? d1.etap[(Ra + 1) * 3 + i] : (T)0;
     }
     const int nc2 = mc2 - c2, nc1 = mc1 - c1;   // columns and rows from the first on
+    // away from the grid's edges the window is whole and the second taps start one later
+    const bool inner = __all_sync(0xffffffffu, s2 && s1 && nc2 >= 4 && nc1 >= 4);
+    if (!live) return;
     const long long cplane = (long long)mc1 * mc2;
+    // offsets inside a coarse plane, a fine plane, and a kept plane of the stream
+    const unsigned oy = (unsigned)(c1 * mc2 + c2);
+    const unsigned ox0 = (unsigned)(Ra * m2 + Ca), ox1 = ox0 + (unsigned)m2;
+    const unsigned ok0 = (unsigned)(Ra * m2 - kept_before(Ra) * mc2 + (Ca >> 1));
+    const unsigned ok1 = (unsigned)((Ra + 1) * m2 - kept_before(Ra + 1) * mc2 + Ca);
     struct D4 { T v[2][2]; };
     // dimension-2 and -1 products of coarse plane j at the lane's nodes
     auto plane = [&](int j) -> D4 {
-        const T *p = y + j * cplane + (long long)c1 * mc2 + c2;
+        const T *p = y + j * cplane;
         T r2[4][2];   // rows c1.., the two columns
+        D4 d;
+        if (inner) {
+#pragma unroll
+            for (int r = 0; r < 4; r++) {
+                const T *q = p + (oy + (unsigned)(r * mc2));
+                const T x0 = q[0], x1 = q[1], x2 = q[2], x3 = q[3];
+                r2[r][0] = fma_rn(e2[0][2], x2, fma_rn(e2[0][1], x1, fma_rn(e2[0][0], x0, (T)0)));
+                r2[r][1] = fma_rn(e2[1][2], x3, fma_rn(e2[1][1], x2, fma_rn(e2[1][0], x1, (T)0)));
+            }
+#pragma unroll
+            for (int c = 0; c < 2; c++) {
+                d.v[0][c] = fma_rn(e1[0][2], r2[2][c], fma_rn(e1[0][1], r2[1][c], fma_rn(e1[0][0], r2[0][c], (T)0)));
+                d.v[1][c] = fma_rn(e1[1][2], r2[3][c], fma_rn(e1[1][1], r2[2][c], fma_rn(e1[1][0], r2[1][c], (T)0)));
+            }
+            return d;
+        }
+        p += oy;
 #pragma unroll
         for (int r = 0; r < 4; r++) {
             T x[4];
@@ -81,7 +109,6 @@ prolong_kernel(LevelGeom<T> g, const T *y, const T *gsrc, T *__restrict__ stream
             r2[r][0] = a;
             r2[r][1] = b;
         }
-        D4 d;
 #pragma unroll
         for (int c = 0; c < 2; c++) {
             T a = (T)0, b = (T)0;
@@ -106,14 +133,14 @@ prolong_kernel(LevelGeom<T> g, const T *y, const T *gsrc, T *__restrict__ stream
         const T tA = o == 0 ? e[0] : o < 0 ? e[1] : (T)0, tB = o == 0 ? e[1] : o < 0 ? e[2] : e[0];
         const T tC = o == 0 ? e[2] : o < 0 ? (T)0 : e[1];
         const bool useA = j > 0 && o <= 0, useC = j + 1 < mc0 && o >= 0;
-        const long long cr = (long long)kept_before(P) * cplane;
+        const long long fp = (long long)P * m1 * m2, sp = plane_base_of(g, P);
 #pragma unroll
         for (int r = 0; r < 2; r++) {
             if (r && !hr) continue;
-            const int R = Ra + r;
             const bool rownew = !k0 || r;
-            const long long row = ((long long)P * m1 + R) * m2;
-            const long long sb = g.Nprev + row - cr - (k0 ? (long long)kept_before(R) * mc2 : 0LL);
+            const unsigned f = r ? ox1 : ox0, k = k0 ? (r ? ok1 : ok0) : f;   // of column Ca, or the row's first new one
+            const T *gp = MODE == MP_RT_FINAL ? gsrc + fp + f : coef + sp + k;
+            T *op = MODE == MP_RT_FINAL ? stream + sp + k : out + fp + f;
 #pragma unroll
             for (int c = 0; c < 2; c++) {
                 if ((c && !hb) || (!rownew && !c)) continue;
@@ -121,9 +148,9 @@ prolong_kernel(LevelGeom<T> g, const T *y, const T *gsrc, T *__restrict__ stream
                 if (useA) v = fma_rn(tA, A.v[r][c], v);
                 v = fma_rn(tB, B.v[r][c], v);
                 if (useC) v = fma_rn(tC, C.v[r][c], v);
-                const long long si = sb + (rownew ? Ca + c : (Ca >> 1));
-                if (MODE == MP_RT_FINAL) stream[si] = sub_rn(gsrc[row + Ca + c], v);
-                else out[row + Ca + c] = add_rn(coef[si], v);
+                const int ks = rownew ? c : 0;   // the stream's step to column Ca + c
+                if (MODE == MP_RT_FINAL) op[ks] = sub_rn(gp[c], v);
+                else op[c] = add_rn(gp[ks], v);
             }
         }
     };
