@@ -14,14 +14,15 @@
 //                  new nodes, through P^T M_l or P^T (the adjoints).
 //
 // Both are warp-specialised plane pipelines.  A CTA owns a tile of 14 x 32
-// coarse nodes in dims (1, 2) and a segment of coarse planes of dim 0.  One
+// (decomp_kernel in binary32: 18 x 32) coarse nodes in dims (1, 2) and a segment of coarse planes of dim 0.  One
 // producer warp streams the fine planes of the tile's region (the owned
 // nodes plus a two-node halo) into a ring of shared-memory stages, one bulk
 // asynchronous copy per row, completed on a "full" mbarrier per stage; seven
-// consumer warps compute and hand each stage back on an "empty" mbarrier.
-// decomp_kernel: two CTAs of eight warps per SM leave each SM sub-partition four
-// warps, so a thread may hold 128 registers (three CTAs of 80 spill: 513^3
-// compression 1534 -> 1658 us).  rsym_kernel meets a barrier every plane and waits
+// (or nine) consumer warps compute and hand each stage back on an "empty" mbarrier.
+// decomp_kernel in binary32: two CTAs of ten warps per SM, 96 registers a thread
+// (eight warps of 121 registers: 513^3 compression 1469 us, nine 1482, ten 1408;
+// three CTAs of eight at 80 spill, 1534 -> 1658); in binary64 one of eight, bound
+// by the FP64 pipe.  rsym_kernel meets a barrier every plane and waits
 // for shared memory, so binary32 runs four CTAs of 64 registers, with two tiles,
 // one escape tile and two or three stages each (two CTAs: 513^3 decompression
 // 1713 us, three 1583, four 1536).
@@ -60,6 +61,8 @@ constexpr int DCW = 7;                     // consumer warps, two coarse rows ea
 constexpr int DT1 = 2 * DCW, DT2 = 32;     // coarse tile, dims 1 and 2
 constexpr int DTHREADS = (DCW + 1) * 32;   // plus one producer warp
 constexpr int DR1 = 2 * DT1 + 4;           // largest region: fine rows
+// decomp_kernel's consumer warps: nine in binary32
+template <typename T> __host__ __device__ constexpr int decomp_warps() { return sizeof(T) == 4 ? 9 : 7; }
 constexpr int DR2 = 2 * DT2 + 4;           //                 fine columns
 constexpr int kHistWin = 4096;             // shared histogram: D/2 +- kHistWin and the escape symbol
 // zero rows before the first stage and after the last: the window rows of a
@@ -130,17 +133,17 @@ struct TileGeom {
 };
 
 template <typename T>
-__device__ __forceinline__ TileGeom tile_geom(const LevelGeom<T> &g, int seg_len)
+__device__ __forceinline__ TileGeom tile_geom(const LevelGeom<T> &g, int seg_len, int dt1 = DT1)
 {
     TileGeom t;
     const int m0 = g.dim[0].m, m1 = g.dim[1].m, m2 = g.dim[2].m;
     const int mc0 = g.dim[0].mc, mc1 = g.dim[1].mc, mc2 = g.dim[2].mc;
     t.J2 = blockIdx.x * DT2;
-    t.J1 = blockIdx.y * DT1;
+    t.J1 = blockIdx.y * dt1;
     t.J0a = blockIdx.z * seg_len;
     t.J0b = min(t.J0a + seg_len, mc0);
     t.n2 = min(DT2, mc2 - t.J2);
-    t.n1 = min(DT1, mc1 - t.J1);
+    t.n1 = min(dt1, mc1 - t.J1);
     t.lo2 = max(0, cpos_of(m2, mc2, t.J2) - 2) & ~1;
     t.hi2 = min(m2 - 1, cpos_of(m2, mc2, t.J2 + t.n2 - 1) + 2);
     t.lo1 = max(0, cpos_of(m1, mc1, t.J1) - 2) & ~1;
@@ -316,9 +319,10 @@ __device__ __forceinline__ void restrict_plane(const WarpRows<T> &w, const T t2[
 
 template <typename T>
 struct DecompSmem {
+    static constexpr int W = decomp_warps<T>(), ROWS = 4 * W + 4;   // consumer warps, largest region's fine rows
     static constexpr int NST = decomp_stages<T>();
     static constexpr int PB = stage_pitch<T>();
-    static constexpr size_t stage_bytes = (size_t)DR1 * PB;
+    static constexpr size_t stage_bytes = (size_t)ROWS * PB;
     static constexpr size_t off_stage = guard_bytes<T>();
     static constexpr size_t off_full = off_stage + NST * stage_bytes + guard_bytes<T>();
     static constexpr size_t off_empty = off_full + NST * 8;
@@ -328,7 +332,7 @@ struct DecompSmem {
 };
 
 template <typename T, int SINK>
-__global__ void __launch_bounds__(DTHREADS, sizeof(T) == 4 ? 2 : 1)
+__global__ void __launch_bounds__((decomp_warps<T>() + 1) * 32, sizeof(T) == 4 ? 2 : 1)
 decomp_kernel(RestrictArgs<T> a, int seg_len)
 {
     using S = DecompSmem<T>;
@@ -336,7 +340,7 @@ decomp_kernel(RestrictArgs<T> a, int seg_len)
     constexpr bool QUANT = SINK == (int)Sink::QUANT;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const LevelGeom<T> &g = a.g;
-    const TileGeom tg = tile_geom(g, seg_len);
+    const TileGeom tg = tile_geom(g, seg_len, 2 * S::W);
     if (tg.J0a >= tg.J0b) { next_begin(); return; }
     const int m0 = g.dim[0].m, m1 = g.dim[1].m, m2 = g.dim[2].m;
     const int mc0 = g.dim[0].mc, mc1 = g.dim[1].mc, mc2 = g.dim[2].mc;
@@ -356,9 +360,9 @@ decomp_kernel(RestrictArgs<T> a, int seg_len)
     {
         uint4 *z = reinterpret_cast<uint4 *>(smem_raw);
         const int n16 = (int)(S::off_full / 16);
-        for (int i = tid; i < n16; i += DTHREADS) z[i] = make_uint4(0u, 0u, 0u, 0u);
+        for (int i = tid; i < n16; i += ((S::W + 1) * 32)) z[i] = make_uint4(0u, 0u, 0u, 0u);
         if (QUANT)
-            for (int i = tid; i <= hn; i += DTHREADS) hs[i] = 0u;
+            for (int i = tid; i <= hn; i += ((S::W + 1) * 32)) hs[i] = 0u;
         fence_proxy_async();
         if (tid == 0) {
             for (int i = 0; i < NST; i++) {
@@ -371,7 +375,7 @@ decomp_kernel(RestrictArgs<T> a, int seg_len)
     next_begin();
     __syncthreads();
 
-    if (warp == DCW) {
+    if (warp == S::W) {
         // ---------------- producer ----------------
         // the dim-0 taps of the next plane are loaded while this plane's
         // copies are issued, so their latency overlaps the ring's wait
@@ -695,8 +699,8 @@ decomp_kernel(RestrictArgs<T> a, int seg_len)
             if (ew) atomicMax(&a.qo.sc->esc_w, ew);
             if (nesc) atomicAdd(&hs[hn], nesc);
         }
-        named_sync(1, DCW * 32);
-        for (int i = tid; i < hn; i += DCW * 32)
+        named_sync(1, S::W * 32);
+        for (int i = tid; i < hn; i += S::W * 32)
             if (hs[i]) atomicAdd(&a.qo.hist[hlo + i], (unsigned long long)hs[i]);
         if (tid == 0 && hs[hn]) atomicAdd(&a.qo.hist[0], (unsigned long long)hs[hn]);
     }
@@ -1269,7 +1273,8 @@ cudaError_t launch_decomp(Sink sink, const RestrictArgs<T> &a0, cudaStream_t s)
     RestrictArgs<T> a = a0;
     a.wait_limit = g_wait_limit;
     const int mc0 = a.g.dim[0].mc, mc1 = a.g.dim[1].mc, mc2 = a.g.dim[2].mc;
-    const int gx = (mc2 + DT2 - 1) / DT2, gy = (mc1 + DT1 - 1) / DT1;
+    constexpr int rows = 2 * decomp_warps<T>(), threads = (decomp_warps<T>() + 1) * 32;
+    const int gx = (mc2 + DT2 - 1) / DT2, gy = (mc1 + rows - 1) / rows;
     const int hn = sink == Sink::QUANT ? 2 * (int)std::min<unsigned>(a.qo.D / 2, kHistWin) : 0;
     const size_t sm = DecompSmem<T>::bytes(hn);
     // one set-up flag per kernel (both instantiations share a function type)
@@ -1279,10 +1284,10 @@ cudaError_t launch_decomp(Sink sink, const RestrictArgs<T> &a0, cudaStream_t s)
             return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
         });
         if (e != cudaSuccess) return e;
-        const int seg = choose_segment(mc0, (long long)gx * gy, resident_ctas(kern, DTHREADS, sm));
+        const int seg = choose_segment(mc0, (long long)gx * gy, resident_ctas(kern, threads, sm));
         const int gz = (mc0 + seg - 1) / seg;
         count_launch();
-        return launch_next(kern, dim3(gx, gy, gz), DTHREADS, sm, s, a, seg);
+        return launch_next(kern, dim3(gx, gy, gz), threads, sm, s, a, seg);
     };
     if (sink == Sink::QUANT) return go(decomp_kernel<T, (int)Sink::QUANT>, attr_quant);
     return go(decomp_kernel<T, (int)Sink::STREAM>, attr_stream);
