@@ -886,6 +886,7 @@ rsym_kernel(RestrictArgs<T> a, int seg_len)
     LaneCols<T> lc;
     lane_cols(g, tg, lane, false, lc, ptap);
     const T q = SYM ? q_of<T>(si_.sc, g.level) : (T)0;
+    const int halfD = SYM ? (int)(si_.D / 2) : 0;
     const bool new_only = a.dense_new_only != 0;
     const int lanecol = lc.ca - 2;
     const long long cstride = (long long)mc1 * mc2;
@@ -936,7 +937,7 @@ rsym_kernel(RestrictArgs<T> a, int seg_len)
                     if constexpr (SYM) {
                         const unsigned sv = sr[sx];
                         if (sv != 0u) {
-                            wv[e] = mul_rn((T)((int)sv - (int)(si_.D / 2)), q);
+                            wv[e] = mul_rn(code_value<T>(sv, halfD), q);
                         } else {
                             cp_async8(et + i1 * S::EPITCH + i2, si_.esc + r.rb + (r.rownew ? p2 : (p2 - 1) >> 1));
                             escm |= 1u << (4 * it + e);

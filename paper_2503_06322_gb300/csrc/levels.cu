@@ -343,9 +343,12 @@ template <typename T> struct BitsOf;
 template <> struct BitsOf<float> { using type = unsigned; };
 template <> struct BitsOf<double> { using type = unsigned long long; };
 __device__ __forceinline__ unsigned abs_bits(float x) { return __float_as_uint(x) & 0x7FFFFFFFu; }
+// (by halves: masking the whole word is recognised as an absolute value and sent
+// through the FP64 pipe, which is what bounds the norm of a binary64 field: 25
+// million values 108 -> 61 us)
 __device__ __forceinline__ unsigned long long abs_bits(double x)
 {
-    return (unsigned long long)__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFull;
+    return (unsigned long long)((unsigned)__double2hiint(x) & 0x7FFFFFFFu) << 32 | (unsigned)__double2loint(x);
 }
 __device__ __forceinline__ double abs_value(unsigned b) { return (double)__uint_as_float(b); }
 __device__ __forceinline__ double abs_value(unsigned long long b) { return __longlong_as_double((long long)b); }
@@ -782,7 +785,7 @@ __device__ __forceinline__ void coarse_body(const CoarseArgs<T> &a)
                 if (i >= nl) continue;
                 int l = 0;
                 while (l < ls && i >= snprev[l + 1]) l++;
-                So[i] = sv[u] != 0u ? mul_rn((T)((int)sv[u] - (int)(a.symin.D / 2)), sq[l]) : mul_rn((T)ev[u], sq[l]);
+                So[i] = sv[u] != 0u ? mul_rn(code_value<T>(sv[u], (int)(a.symin.D / 2)), sq[l]) : mul_rn((T)ev[u], sq[l]);
             }
         }
     }

@@ -216,12 +216,11 @@ __device__ __forceinline__ T dequant_sym(const SymIn &si_, unsigned s, long long
     return mul_rn((T)si_.esc[idx], q);
 }
 
-// Binary64 issue is slow on this part: the conversion and the product of a
-// symbol were a third of the binary64 instructions of the expansion of a level.
-// It takes the value from a table instead, 64 KB per level, which its blocks
-// copy into shared memory (bytes: size of it, 0 without): 419 -> 328 us for the
-// finest level of 500x500x100.  The restriction stays with the product (the
-// table made it 778 -> 814 us: it waits for shared memory more than for the pipe).
+// Binary64 issue is slow on this part, so the expansion takes the value of a
+// symbol from a table, 64 KB per level, which its blocks copy into shared memory
+// (bytes: size of it, 0 without): finest level of 500x500x100 229 us, round trip
+// 3386 -> 3337 us against the product at every node.  The restriction stays with
+// the product: it waits for shared memory more than for the pipe.
 template <typename T>
 __host__ __device__ inline size_t deq_bytes(const SymIn &si)
 {
@@ -238,9 +237,17 @@ __device__ __forceinline__ void deq_stage(double *dst, const SymIn &si, int leve
 template <typename T>
 __device__ __forceinline__ T code_value(unsigned s, int halfD)
 {
-    // binary32: 2^23 + s is the word 0x4B000000 | s, and both it and the difference are exact
-    if constexpr (sizeof(T) == 4) return __fsub_rn(__uint_as_float(0x4B000000u | s), 8388608.0f + (float)halfD);
-    else return (T)((int)s - halfD);
+    if constexpr (sizeof(T) == 4) {
+        // 2^23 + s is the word 0x4B000000 | s, and both it and the difference are exact
+        return __fsub_rn(__uint_as_float(0x4B000000u | s), 8388608.0f + (float)halfD);
+    } else {
+        // a conversion to binary64 takes the FP64 pipe more than the product does;
+        // binary32 holds the code exactly, and its bits widen in integers
+        // (500x500x100 round trip, with the norm's halves: 3590 -> 3315 us)
+        const unsigned f = __float_as_uint((float)((int)s - halfD));
+        const unsigned hi = (f & 0x80000000u) | (((f & 0x7FFFFFFFu) >> 3) + 0x38000000u);
+        return __hiloint2double(f ? (int)hi : 0, (int)(f << 29));
+    }
 }
 // value of symbol s != 0; after a rejected header the symbols are another
 // stream's, and any of them has to stay inside the table
