@@ -71,7 +71,10 @@ template <typename E> __host__ __device__ constexpr int stage_pitch();
 template <typename E> __host__ __device__ constexpr int guard_bytes() { return 3 * stage_pitch<E>(); }
 
 template <typename T> __host__ __device__ constexpr int decomp_stages() { return sizeof(T) == 4 ? 6 : 3; }
-template <typename T> __host__ __device__ constexpr int rsym_stages(bool sym) { return sizeof(T) == 8 ? 4 : sym ? 2 : 3; }
+template <typename T> __host__ __device__ constexpr int rsym_stages(bool sym)
+{
+    return sizeof(T) == 8 ? (sym ? 4 : 2) : sym ? 2 : 3;
+}
 // bytes per staged row: the region plus the 16-byte alignment of its copy
 template <typename E> __host__ __device__ constexpr int stage_pitch() { return ((DR2 * (int)sizeof(E) + 32) + 15) & ~15; }
 
@@ -733,7 +736,11 @@ struct RsymSmem {
     static constexpr int WROWS = DR1 + 6;     // zero rows around the region: two before, up to four after
     static constexpr size_t wtile_bytes = (size_t)WROWS * kWPitch * sizeof(T);
     static constexpr size_t off_w = 0;
-    static constexpr size_t off_stage = off_w + 2 * wtile_bytes;   // two dequantized tiles
+    static constexpr size_t off_sums = off_w + 2 * wtile_bytes;   // two dequantized tiles
+    // binary64: the dim-2 sums of the tiles' rows, two planes
+    static constexpr bool SHARE = sizeof(T) == 8;
+    static constexpr size_t sums_bytes = SHARE ? (size_t)WROWS * 32 * sizeof(T) : 0;
+    static constexpr size_t off_stage = off_sums + 2 * sums_bytes;
     static constexpr size_t off_full = off_stage + NST * stage_bytes;
     static constexpr size_t off_empty = off_full + NST * 8;
     static constexpr size_t off_info = off_empty + NST * 8;
@@ -979,9 +986,61 @@ rsym_kernel(RestrictArgs<T> a, int seg_len)
         t.tr[0] = pi.tr[0]; t.tr[1] = pi.tr[1]; t.tr[2] = pi.tr[2];
         return t;
     };
+    // Binary64 waits for the FP64 pipe, and the rows that two warps read would be
+    // summed along dim 2 twice: the warps share out the rows of a plane, and take
+    // the dim-1 products of its sums after the barrier, one iteration later
+    // (round trip of 500x500x100: 3303 -> 3180 us).
+    T *const sums0 = reinterpret_cast<T *>(smem_raw + S::off_sums) + 2 * 32 + lane;
+    const auto sums = [&](int kk) -> T * { return sums0 + (size_t)(kk & 1) * (S::sums_bytes / sizeof(T)); };
+    const auto sum_rows = [&](int kk) {
+        const T *w = tile(kk) + lanecol;
+        T *d = sums(kk);
+#pragma unroll
+        for (int it = 0; it < (DR1 + DCW - 1) / DCW; it++) {
+            const int r = warp + it * DCW;
+            if (r < tg.r1n) {
+                T acc = (T)0;
+#pragma unroll
+                for (int o = 0; o < 5; o++) acc = fma_rn(lc.t2[o], w[r * kWPitch + o], acc);
+                d[r * 32] = acc;
+            }
+        }
+    };
+    const auto accumulate = [&](const Taps &t, T ra, T rb) {
+        while (jb < t.jlo && jb < tg.J0b) {
+            if (lc.colv) {
+                a.b[(long long)jb * cstride + out_a] = acc[0][0];
+                if (wr.vb) a.b[(long long)jb * cstride + out_b] = acc[1][0];
+            }
+#pragma unroll
+            for (int u = 0; u < 2; u++) { acc[u][0] = acc[u][1]; acc[u][1] = acc[u][2]; acc[u][2] = (T)0; }
+            jb++;
+        }
+#pragma unroll
+        for (int i = 0; i < 3; i++) {
+            acc[0][i] = fma_rn(t.tr[i], ra, acc[0][i]);
+            acc[1][i] = fma_rn(t.tr[i], rb, acc[1][i]);
+        }
+    };
+    // the dim-1 products of plane kk's sums
+    const auto restrict_sums = [&](int kk, const Taps &t) {
+        const T *w = sums(kk) + wr.rl0 * 32;
+        T s[7];
+#pragma unroll
+        for (int i = 0; i < 7; i++) s[i] = w[i * 32];
+        T ra = (T)0, rb = (T)0;
+        const bool two = wr.offb == 2;
+#pragma unroll
+        for (int o = 0; o < 5; o++) {
+            ra = fma_rn(wr.t1a[o], s[o], ra);
+            rb = fma_rn(wr.t1b[o], two ? s[o + 2] : s[o + 1], rb);
+        }
+        accumulate(t, ra, rb);
+    };
     unsigned ec = 0;
-    Taps tc;
+    Taps tc, tp;
     tc.jlo = 0; tc.tr[0] = tc.tr[1] = tc.tr[2] = (T)0;
+    tp = tc;
     {
         const bool ok = warp_wait(&full[0], 0u, limit);
         if (ok) {
@@ -1008,24 +1067,14 @@ rsym_kernel(RestrictArgs<T> a, int seg_len)
             ok = warp_wait(&full[(k + 1) % NST], (uint32_t)(((k + 1) / NST) & 1), limit);
             if (ok) { tn = taps_of(k + 1); en = fill(k + 1, tile(k + 1)); }
         }
-        if (wr.va) {
+        if constexpr (S::SHARE) {
+            sum_rows(k);
+            if (k > 0 && wr.va) restrict_sums(k - 1, tp);
+        } else if (wr.va) {
             T ra, rb;
             restrict_plane<T>(wr, lc.t2, [&](int i) -> const T * { return W + (wr.rl0 + i) * kWPitch + lanecol; },
                               ra, rb);
-            while (jb < tc.jlo && jb < tg.J0b) {
-                if (lc.colv) {
-                    a.b[(long long)jb * cstride + out_a] = acc[0][0];
-                    if (wr.vb) a.b[(long long)jb * cstride + out_b] = acc[1][0];
-                }
-#pragma unroll
-                for (int u = 0; u < 2; u++) { acc[u][0] = acc[u][1]; acc[u][1] = acc[u][2]; acc[u][2] = (T)0; }
-                jb++;
-            }
-#pragma unroll
-            for (int i = 0; i < 3; i++) {
-                acc[0][i] = fma_rn(tc.tr[i], ra, acc[0][i]);
-                acc[1][i] = fma_rn(tc.tr[i], rb, acc[1][i]);
-            }
+            accumulate(tc, ra, rb);
         }
         if (k + 1 < nplanes) {
             // the next plane's escaped codes (copied during the restriction) into its tile
@@ -1035,11 +1084,16 @@ rsym_kernel(RestrictArgs<T> a, int seg_len)
             if (named_sync_or(1, DCW * 32, !ok)) { failed = true; break; }
             if (tid == 0) mbar_arrive(&empty[(k + 1) % NST]);
         }
+        tp = tc;
         tc = tn;
     }
     if (failed) {
         if (tid == 0) atomicExch(a.status, (unsigned)DS_TIMEOUT);
         return;
+    }
+    if constexpr (S::SHARE) {
+        named_sync(1, DCW * 32);
+        if (wr.va) restrict_sums(nplanes - 1, tp);
     }
     if (wr.va && lc.colv) {
         while (jb < tg.J0b) {
