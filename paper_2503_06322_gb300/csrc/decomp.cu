@@ -38,7 +38,7 @@
 // identity P^T M_l P = M_{l-1} of nested P1 spaces,
 //     b = P^T M_l (v - P v_c) = ((x)_k P^T M_l) v - ((x)_k M_{l-1}) v_c,
 // so it restricts the staged values of v directly and no warp needs another
-// warp's coefficients: the consumers run without block barriers.  The
+// warp's coefficients: in binary32 the consumers run without block barriers.  The
 // coefficients of the lane's own 2 x 2 nodes per owned row pair take the
 // multilinear interpolant of the kept planes around them; the interpolant
 // J = I_1 I_2 v of a kept plane is formed once, while that plane is staged,
@@ -121,6 +121,19 @@ __device__ __forceinline__ bool warp_wait(unsigned long long *bar, uint32_t pari
 __device__ __forceinline__ void named_sync(int id, int nthreads)
 {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
+}
+__device__ __forceinline__ bool named_sync_or(int id, int nthreads, bool pred)
+{
+    uint32_t r;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.u32 p, %1, 0;\n\t"
+        "bar.red.or.pred q, %2, %3, p;\n\t"
+        "selp.u32 %0, 1, 0, q;\n\t}"
+        : "=r"(r)
+        : "r"((uint32_t)pred), "r"(id), "r"(nthreads)
+        : "memory");
+    return r != 0;
 }
 __device__ __forceinline__ void fence_proxy_async()
 {
@@ -327,12 +340,57 @@ struct DecompSmem {
     static constexpr int PB = stage_pitch<T>();
     static constexpr size_t stage_bytes = (size_t)ROWS * PB;
     static constexpr size_t off_stage = guard_bytes<T>();
-    static constexpr size_t off_full = off_stage + NST * stage_bytes + guard_bytes<T>();
+    // binary64: the dim-2 restriction and mass sums of the region's rows, two planes
+    static constexpr bool SHARE = sizeof(T) == 8;
+    static constexpr size_t sums_bytes = SHARE ? (size_t)(ROWS + 6) * 32 * sizeof(T) : 0;
+    static constexpr size_t off_sums = off_stage + NST * stage_bytes + guard_bytes<T>();
+    static constexpr size_t off_full = off_sums + 4 * sums_bytes;
     static constexpr size_t off_empty = off_full + NST * 8;
     static constexpr size_t off_info = off_empty + NST * 8;
     static constexpr size_t off_hist = (off_info + NST * sizeof(PlaneInfo<T>) + 15) & ~size_t(15);
     static size_t bytes(int hn) { return off_hist + (size_t)(hn + 1) * 4; }
 };
+
+// Binary64 waits for the FP64 pipe, and most of the rows that a warp reads belong
+// to the windows of two warps: the active warps share out the dim-2 sums of a
+// plane's rows (restriction, then mass on kept rows of kept planes), one plane
+// ahead, and meet once a plane (round trip of 500x500x100: 3198 -> 3116 us; nine
+// consumer warps 3165).
+// plane_sums: row 0 of plane kk's restriction sums.
+template <typename T>
+__device__ __forceinline__ T *plane_sums(unsigned char *smem, int kk)
+{
+    using S = DecompSmem<T>;
+    return reinterpret_cast<T *>(smem + S::off_sums + (kk & 1) * 2 * S::sums_bytes) + 2 * 32;
+}
+template <typename T>
+__device__ __forceinline__ void sum_rows(const LevelGeom<T> &g, const TileGeom &tg, const LaneCols<T> &lc, bool even2,
+                                         int warp, int nact, unsigned char *smem, uint32_t bel, int kk, int slot, int p)
+{
+    using S = DecompSmem<T>;
+    constexpr uint32_t VM = 16 / sizeof(T) - 1;
+    const int m1 = g.dim[1].m, m2 = g.dim[2].m, lane = threadIdx.x & 31;
+    T *const d = plane_sums<T>(smem, kk) + lane, *const dm = d + S::sums_bytes / sizeof(T);
+    const bool kp = kept_pos(g.dim[0].m, p);
+    uint32_t t = bel + (uint32_t)p * ((uint32_t)m1 * (uint32_t)m2) + (uint32_t)(tg.lo1 + warp) * (uint32_t)m2;
+    const unsigned char *st = smem + S::off_stage + slot * S::stage_bytes;
+    for (int r = warp; r < tg.r1n; r += nact, t += (uint32_t)(nact * m2)) {
+        const T *w = reinterpret_cast<const T *>(st + r * S::PB) + (int)(t & VM) + (lc.ca - 2);
+        T v[5], x = (T)0;
+#pragma unroll
+        for (int o = 0; o < 5; o++) v[o] = w[o];
+#pragma unroll
+        for (int o = 0; o < 5; o++) x = fma_rn(lc.t2[o], v[o], x);
+        d[r * 32] = x;
+        if (kp && kept_pos(m1, tg.lo1 + r)) {
+            T m = fma_rn(lc.m2t[0], v[0], (T)0);
+            if (!even2) m = fma_rn(lc.m2t[1], v[1], m);
+            m = fma_rn(lc.m2t[2], v[2], m);
+            if (!even2) m = fma_rn(lc.m2t[3], v[3], m);
+            dm[r * 32] = fma_rn(lc.m2t[4], v[4], m);
+        }
+    }
+}
 
 template <typename T, int SINK>
 __global__ void __launch_bounds__((decomp_warps<T>() + 1) * 32, sizeof(T) == 4 ? 2 : 1)
@@ -564,19 +622,49 @@ decomp_kernel(RestrictArgs<T> a, int seg_len)
         int jb = tg.J0a;
         bool ok = true;
         int k = 0, slot = 0;
-        for (int p0 = tg.lo0; p0 <= tg.hi0; p0++, k++, slot = (slot + 1 == NST) ? 0 : slot + 1) {
-            if (!warp_wait(&full[slot], (uint32_t)((k / NST) & 1), limit)) { ok = false; break; }
+        if constexpr (S::SHARE) {
+            ok = warp_wait(&full[0], 0u, limit);
+            if (ok) sum_rows<T>(g, tg, lc, even2, warp, nact, smem_raw, bel, 0, 0, tg.lo0);
+            ok = !named_sync_or(2, nact * 32, !ok);
+        }
+        for (int p0 = tg.lo0; (!S::SHARE || ok) && p0 <= tg.hi0; p0++, k++, slot = (slot + 1 == NST) ? 0 : slot + 1) {
+            bool next_ok = true;
+            if constexpr (S::SHARE) {
+                if (p0 < tg.hi0) {
+                    const int ns = (slot + 1 == NST) ? 0 : slot + 1;
+                    next_ok = warp_wait(&full[ns], (uint32_t)(((k + 1) / NST) & 1), limit);
+                    if (next_ok) sum_rows<T>(g, tg, lc, even2, warp, nact, smem_raw, bel, k + 1, ns, p0 + 1);
+                }
+            } else {
+                if (!warp_wait(&full[slot], (uint32_t)((k / NST) & 1), limit)) { ok = false; break; }
+            }
             const PlaneInfo<T> pi = pinfo[slot];
             const bool k0 = kept_pos(m0, p0);
             // ---- restriction of v, and of v_c through the coarse mass matrix
             T ra, rb;
-            restrict_plane<T>(wr, lc.t2, [&](int i) { return rowaddr(slot, p0, i); }, ra, rb);
+            if constexpr (S::SHARE) {
+                const T *const sr = plane_sums<T>(smem_raw, k) + wr.rl0 * 32 + lane;   // the sums of local row 0
+                T s7[7];
+#pragma unroll
+                for (int i = 0; i < 7; i++) s7[i] = sr[i * 32];
+                ra = rb = (T)0;
+                const bool two = wr.offb == 2;
+#pragma unroll
+                for (int o = 0; o < 5; o++) {
+                    ra = fma_rn(wr.t1a[o], s7[o], ra);
+                    rb = fma_rn(wr.t1b[o], two ? s7[o + 2] : s7[o + 1], rb);
+                }
+            } else {
+                restrict_plane<T>(wr, lc.t2, [&](int i) { return rowaddr(slot, p0, i); }, ra, rb);
+            }
             if (k0) {
                 T sm[7];
 #pragma unroll
                 for (int i = 0; i < 7; i++) {
                     sm[i] = (T)0;
-                    if ((mrows >> i) & 1u) {
+                    if constexpr (S::SHARE) {
+                        if ((mrows >> i) & 1u) sm[i] = plane_sums<T>(smem_raw, k)[S::sums_bytes / sizeof(T) + (wr.rl0 + i) * 32 + lane];
+                    } else if ((mrows >> i) & 1u) {
                         const T *ad = rowaddr(slot, p0, i);
                         T m = fma_rn(lc.m2t[0], ad[0], (T)0);
                         if (!even2) m = fma_rn(lc.m2t[1], ad[1], m);
@@ -654,7 +742,8 @@ decomp_kernel(RestrictArgs<T> a, int seg_len)
                 } else {
                     // a new plane: the kept plane after it is staged in the next slot
                     const int nslot = (slot + 1 == NST) ? 0 : slot + 1;
-                    if (!warp_wait(&full[nslot], (uint32_t)(((k + 1) / NST) & 1), limit)) { ok = false; break; }
+                    if constexpr (!S::SHARE)
+                        if (!warp_wait(&full[nslot], (uint32_t)(((k + 1) / NST) & 1), limit)) { ok = false; break; }
                     const Interp<T> Jn = form_J(nslot, p0 + 1);
                     const T *a2 = rowaddr(slot, p0, 2) + 2;
                     const T *a3 = rowaddr(slot, p0, 3) + 2;
@@ -682,6 +771,8 @@ decomp_kernel(RestrictArgs<T> a, int seg_len)
                 }
             }
             __syncwarp();
+            if constexpr (S::SHARE)
+                if (p0 < tg.hi0 && named_sync_or(2, nact * 32, !next_ok)) { ok = false; break; }
             if (lane == 0) mbar_arrive(&empty[slot]);
         }
         if (ok && lc.colv) {
@@ -768,20 +859,6 @@ struct SymRow {
     int off;
     short rownew, allnew;
 };
-
-__device__ __forceinline__ bool named_sync_or(int id, int nthreads, bool pred)
-{
-    uint32_t r;
-    asm volatile(
-        "{\n\t.reg .pred p, q;\n\t"
-        "setp.ne.u32 p, %1, 0;\n\t"
-        "bar.red.or.pred q, %2, %3, p;\n\t"
-        "selp.u32 %0, 1, 0, q;\n\t}"
-        : "=r"(r)
-        : "r"((uint32_t)pred), "r"(id), "r"(nthreads)
-        : "memory");
-    return r != 0;
-}
 
 template <typename T, int SRC>
 __global__ void __launch_bounds__(DTHREADS, sizeof(T) == 4 ? 4 : 2)
