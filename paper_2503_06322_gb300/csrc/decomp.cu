@@ -1084,8 +1084,9 @@ rsym_kernel(RestrictArgs<T> a, int seg_len)
             const int i1 = u / NQ, i2b = (u - i1 * NQ) * 4;
 #pragma unroll
             for (int e = 0; e < 4; e++)
-                if ((escm >> (4 * it + e)) & 1u)
-                    Wt[i1 * kWPitch + i2b + e] = mul_rn((T)et[i1 * S::EPITCH + i2b + e], q);
+                if ((escm >> (4 * it + e)) & 1u)   // binary32: few enough here for the 64-bit conversion
+                    Wt[i1 * kWPitch + i2b + e] = mul_rn(sizeof(T) == 8 ? escape_value<T>(et[i1 * S::EPITCH + i2b + e])
+                                               : (T)et[i1 * S::EPITCH + i2b + e], q);
         }
     };
     auto taps_of = [&](int kk) -> Taps {
@@ -1364,7 +1365,7 @@ expand_kernel(LevelGeom<T> g, const T *vc, const T *coef_in, SymIn symin,
         if constexpr (SRC == (int)WSrc::STREAM) {
             return wv;
         } else {
-            return wv != 0u ? dequant_code<T>(deq, wv, halfD, q) : mul_rn((T)eslot[(size_t)b * XTHREADS * 7 + j], q);
+            return wv != 0u ? dequant_code<T>(deq, wv, halfD, q) : mul_rn(escape_value<T>(eslot[(size_t)b * XTHREADS * 7 + j]), q);
         }
     };
     auto step = [&](int j0, Raw &cur, const Raw &nxt, int b) {

@@ -785,7 +785,7 @@ __device__ __forceinline__ void coarse_body(const CoarseArgs<T> &a)
                 if (i >= nl) continue;
                 int l = 0;
                 while (l < ls && i >= snprev[l + 1]) l++;
-                So[i] = sv[u] != 0u ? mul_rn(code_value<T>(sv[u], (int)(a.symin.D / 2)), sq[l]) : mul_rn((T)ev[u], sq[l]);
+                So[i] = sv[u] != 0u ? mul_rn(code_value<T>(sv[u], (int)(a.symin.D / 2)), sq[l]) : mul_rn(escape_value<T>(ev[u]), sq[l]);
             }
         }
     }

@@ -233,6 +233,31 @@ __device__ __forceinline__ void deq_stage(double *dst, const SymIn &si, int leve
     for (unsigned i = 2 * threadIdx.x; i < si.D; i += 2 * blockDim.x)
         asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst + i)), "l"(src + i) : "memory");
 }
+// The value of an escaped code k, (T)k.  Converting 64-bit integers (and anything
+// to binary64) takes the FP64 pipe, and where it is one side of a selection it is
+// done for every symbol; so codes convert through 32 bits -- exactly for binary64
+// below 2^24, its bits widened in integers -- and the rest out of line (the
+// expansion kept the FP64 pipe 79% busy in binary32: decompression of 513^3 1448 ->
+// 1402 us, round trip of 500x500x100 binary64 3154 -> 2943).
+__device__ __forceinline__ double widen_bits(float x)   // x: an integer
+{
+    const unsigned f = __float_as_uint(x);
+    const unsigned hi = (f & 0x80000000u) | (((f & 0x7FFFFFFFu) >> 3) + 0x38000000u);
+    return __hiloint2double(f ? (int)hi : 0, (int)(f << 29));
+}
+template <typename T>
+__device__ __noinline__ T escape_value_wide(long long k) { return (T)k; }
+template <typename T>
+__device__ __forceinline__ T escape_value(long long k)
+{
+    const int lo = (int)k;
+    if constexpr (sizeof(T) == 4) {
+        if (lo == k) return (T)lo;
+    } else {
+        if (lo == k && abs(lo) < (1 << 24)) return widen_bits((float)lo);
+    }
+    return escape_value_wide<T>(k);
+}
 // s - D/2 for a symbol s
 template <typename T>
 __device__ __forceinline__ T code_value(unsigned s, int halfD)
@@ -244,9 +269,7 @@ __device__ __forceinline__ T code_value(unsigned s, int halfD)
         // a conversion to binary64 takes the FP64 pipe more than the product does;
         // binary32 holds the code exactly, and its bits widen in integers
         // (500x500x100 round trip, with the norm's halves: 3590 -> 3315 us)
-        const unsigned f = __float_as_uint((float)((int)s - halfD));
-        const unsigned hi = (f & 0x80000000u) | (((f & 0x7FFFFFFFu) >> 3) + 0x38000000u);
-        return __hiloint2double(f ? (int)hi : 0, (int)(f << 29));
+        return widen_bits((float)((int)s - halfD));
     }
 }
 // value of symbol s != 0; after a rejected header the symbols are another
