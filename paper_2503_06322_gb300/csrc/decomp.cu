@@ -1282,7 +1282,8 @@ expand_kernel(LevelGeom<T> g, const T *vc, const T *coef_in, SymIn symin,
     // fine plane (k); loaded one plane ahead of their use.  Plane offsets depend
     // on j0 alone and are added to the base pointers once per warp, and words
     // that do not exist hold no escape, so one minimum finds a plane's escapes
-    // (513^3 binary32, finest level: 328 -> 270 us, bound by issue and latency).
+    // (513^3 binary32, finest level: 328 -> 270 us, bound by issue and latency; 222
+    // with escapes converted through 32 bits).
     using W = typename std::conditional<SRC == (int)WSrc::SYMBOLS, unsigned, T>::type;
     using E = typename std::conditional<SRC == (int)WSrc::SYMBOLS, uint16_t, T>::type;
     const E *const src = SRC == (int)WSrc::SYMBOLS ? reinterpret_cast<const E *>(symin.sym)

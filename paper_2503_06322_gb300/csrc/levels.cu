@@ -477,7 +477,7 @@ __global__ void __launch_bounds__(256) norm_kernel(const T *u, long long N, doub
 
 // --------------------------------------------------------------------------
 // The coarse levels in one CTA.  Every level l <= ls (the largest level whose
-// working arrays fit in shared memory) and level 0 run in a single 1024-thread
+// working arrays fit in shared memory) and level 0 run in a single 512-thread
 // block out of shared memory, instead of four or five launches per level.  A
 // level of compression (Alg. 1) here:
 //   1. w = v - P v_c on the new nodes (0 on kept ones; v_c are the kept nodes

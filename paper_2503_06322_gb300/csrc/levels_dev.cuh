@@ -218,8 +218,8 @@ __device__ __forceinline__ T dequant_sym(const SymIn &si_, unsigned s, long long
 
 // Binary64 issue is slow on this part, so the expansion takes the value of a
 // symbol from a table, 64 KB per level, which its blocks copy into shared memory
-// (bytes: size of it, 0 without): finest level of 500x500x100 229 us, round trip
-// 3386 -> 3337 us against the product at every node.  The restriction stays with
+// (bytes: size of it, 0 without): round trip of 500x500x100 3386 -> 3337 us against
+// the product at every node.  The restriction stays with
 // the product: it waits for shared memory more than for the pipe.
 template <typename T>
 __host__ __device__ inline size_t deq_bytes(const SymIn &si)
