@@ -544,6 +544,7 @@ hpdr_status decompress_t(hpdr_ctx *ctx, const Plan *P, const Hdr &h, const uint8
     for (int l = 0; l <= L; l++) ta.si.q[l] = h.q[l];
     ta.si.L = L;
     ta.si.n_esc = h.n_esc;
+    ta.si.esc_w = h.esc_w;
     ta.si.total_bits = h.bits;
     CK(launch_decode_tables(ta, hs, s));
     }

@@ -1001,6 +1001,7 @@ rsym_kernel(RestrictArgs<T> a, int seg_len)
     lane_cols(g, tg, lane, false, lc, ptap);
     const T q = SYM ? q_of<T>(si_.sc, g.level) : (T)0;
     const int halfD = SYM ? (int)(si_.D / 2) : 0;
+    const bool narrow = SYM && sizeof(T) == 4 && narrow_escapes(si_.sc);
     const bool new_only = a.dense_new_only != 0;
     const int lanecol = lc.ca - 2;
     // odd only for the last column of a grid whose last interval is short
@@ -1078,6 +1079,19 @@ rsym_kernel(RestrictArgs<T> a, int seg_len)
     auto patch = [&](int kk, T *Wt, unsigned escm) {
         if (!SYM || !escm) return;
         const long long *et = esc_tile0;
+        if (sizeof(T) == 4 && narrow) {
+#pragma unroll
+            for (int it = 0; it < kDqItems; it++) {
+                const int u = tid + it * DCW * 32;
+                const int i1 = u / NQ, i2b = (u - i1 * NQ) * 4;
+#pragma unroll
+                for (int e = 0; e < 4; e++)
+                    if ((escm >> (4 * it + e)) & 1u)
+                        Wt[i1 * kWPitch + i2b + e] =
+                            mul_rn((T)*reinterpret_cast<const int *>(&et[i1 * S::EPITCH + i2b + e]), q);
+            }
+            return;
+        }
 #pragma unroll
         for (int it = 0; it < kDqItems; it++) {
             const int u = tid + it * DCW * 32;
@@ -1338,6 +1352,7 @@ expand_kernel(LevelGeom<T> g, const T *vc, const T *coef_in, SymIn symin,
     // copies, one plane ahead of their use; with a register destination a
     // warp would wait on every node at which any lane escapes.
     long long *eslot = reinterpret_cast<long long *>(xsm) + threadIdx.x * 7;   // [2][XTHREADS][7]
+    const bool narrow = SRC == (int)WSrc::SYMBOLS && sizeof(T) == 4 && narrow_escapes(symin.sc);
     bool pend = false;   // escapes of the current plane in flight
     auto issue_esc = [&](const Raw &r, int j0, int b) -> bool {
         if constexpr (SRC == (int)WSrc::SYMBOLS) {
@@ -1366,7 +1381,10 @@ expand_kernel(LevelGeom<T> g, const T *vc, const T *coef_in, SymIn symin,
         if constexpr (SRC == (int)WSrc::STREAM) {
             return wv;
         } else {
-            return wv != 0u ? dequant_code<T>(deq, wv, halfD, q) : mul_rn(escape_value<T>(eslot[(size_t)b * XTHREADS * 7 + j]), q);
+            const long long *e = &eslot[(size_t)b * XTHREADS * 7 + j];
+            if (wv != 0u) return dequant_code<T>(deq, wv, halfD, q);
+            if (sizeof(T) == 4 && narrow) return mul_rn((T)*reinterpret_cast<const int *>(e), q);
+            return mul_rn(escape_value<T>(*e), q);
         }
     };
     auto step = [&](int j0, Raw &cur, const Raw &nxt, int b) {

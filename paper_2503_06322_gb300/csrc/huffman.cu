@@ -915,6 +915,7 @@ __global__ void __launch_bounds__(kTabThreads, 1) dec_tables_kernel(TabArgs a, H
         }
         if (lead && tid == 0) {
             a.sc->n_esc = a.dh ? h.n_esc : a.si.n_esc;
+            a.sc->esc_w = a.dh ? h.esc_w : a.si.esc_w;
             a.sc->total_bits = a.dh ? h.total_bits : a.si.total_bits;
             if (a.dh) *a.dh = h;
         }

@@ -72,6 +72,7 @@ struct ScalarInit {
     double q[kMaxLevels + 1];
     int L;
     unsigned long long n_esc, total_bits;
+    unsigned int esc_w;
 };
 // Canonical tables and look-up tables from the code lengths of the symbols
 // s_lo..s_hi (device bytes; every other symbol absent), decoder side.
