@@ -26,17 +26,18 @@ enum { MP_RT_FINAL = 1, MP_DT_FINAL = 2 };
 //   MP_DT_FINAL: out[p] = coef[rank(p)] + y_f(p)
 // One pass over the fine grid is all it needs from memory (a pass per dimension,
 // through two partial grids, moved 2.6 times the bytes and took 173 us for the
-// finest level of 257^3; this takes 62, bound by instruction issue: 78 with 64-bit offsets
-// and the window's edges tested at every node).  A warp owns coarse row j1 of a tile,
+// finest level of 257^3; this takes 65, bound by instruction issue: 78 with the
+// window's edges tested at every node).  A warp owns coarse row j1 of a tile,
 // lane l coarse column j2, and the CTA marches along the coarse planes of its
 // segment; for each plane a lane forms the dimension-2, then the dimension-1
 // products at its 2 x 2 fine nodes (rows Ra, Ra + 1, columns Ca, Ca + 1) from the
 // four rows and four columns of y around it (cached loads, coalesced per row)
 // and keeps the last three planes' for the dimension-0 products.  Every value
-// sums its taps in a fixed order, so nothing depends on the tiling.
+// sums its taps in a fixed order, so nothing depends on the tiling.  Binary32 keeps
+// to 64 registers, four CTAs an SM (72 without the bound: three).
 constexpr int kMpWarps = 8;
 template <typename T, int MODE>
-__global__ void __launch_bounds__(32 * kMpWarps)
+__global__ void __launch_bounds__(32 * kMpWarps, sizeof(T) == 4 ? 4 : 2)
 prolong_kernel(LevelGeom<T> g, const T *y, const T *gsrc, T *__restrict__ stream, const T *coef, T *__restrict__ out,
                int seg_len)
 {
@@ -54,35 +55,33 @@ prolong_kernel(LevelGeom<T> g, const T *y, const T *gsrc, T *__restrict__ stream
     // taps of the two fine columns and rows; the second ones start at the same
     // coarse index or one later
     T e2[2][3], e1[2][3];
-    const int c2 = d2.efirst[Ca], c1 = d1.efirst[Ra];
+    const int c2 = d2.efirst[Ca], c1 = __shfl_sync(0xffffffffu, d1.efirst[Ra], 0);
     const bool s2 = hb && d2.efirst[Ca + 1] != c2, s1 = hr && d1.efirst[Ra + 1] != c1;
 #pragma unroll
     for (int i = 0; i < 3; i++) {
-        e2[0][i] = d2.etap[Ca * 3 + i];
-        e2[1][i] = hb ? d2.etap[(Ca + 1) * 3 + i] : (T)0;
-        e1[0][i] = d1.etap[Ra * 3 + i];
-        e1[1][i] = hr ? d1.etap[(Ra + 1) * 3 + i] : (T)0;
+        e2[0][i] = d2.etap[Ca * 3ll + i];
+        e2[1][i] = hb ? d2.etap[(Ca + 1) * 3ll + i] : (T)0;
+        e1[0][i] = d1.etap[Ra * 3ll + i];
+        e1[1][i] = hr ? d1.etap[(Ra + 1) * 3ll + i] : (T)0;
     }
     const int nc2 = mc2 - c2, nc1 = mc1 - c1;   // columns and rows from the first on
     // away from the grid's edges the window is whole and the second taps start one later
     const bool inner = __all_sync(0xffffffffu, s2 && s1 && nc2 >= 4 && nc1 >= 4);
     if (!live) return;
     const long long cplane = (long long)mc1 * mc2;
-    // offsets inside a coarse plane, a fine plane, and a kept plane of the stream
-    const unsigned oy = (unsigned)(c1 * mc2 + c2);
-    const unsigned ox0 = (unsigned)(Ra * m2 + Ca), ox1 = ox0 + (unsigned)m2;
-    const unsigned ok0 = (unsigned)(Ra * m2 - kept_before(Ra) * mc2 + (Ca >> 1));
-    const unsigned ok1 = (unsigned)((Ra + 1) * m2 - kept_before(Ra + 1) * mc2 + Ca);
+    // the same in every lane: the plane pointers take the rows once per warp
+    const PlaneRows rows = plane_rows(m2, mc2, Ra);
+    const long long ry = (long long)c1 * mc2;
     struct D4 { T v[2][2]; };
     // dimension-2 and -1 products of coarse plane j at the lane's nodes
     auto plane = [&](int j) -> D4 {
-        const T *p = y + j * cplane;
+        const T *p = y + (j * cplane + ry);   // row c1 of the plane
         T r2[4][2];   // rows c1.., the two columns
         D4 d;
         if (inner) {
 #pragma unroll
             for (int r = 0; r < 4; r++) {
-                const T *q = p + (oy + (unsigned)(r * mc2));
+                const T *q = p + (long long)r * mc2 + (unsigned)c2;
                 const T x0 = q[0], x1 = q[1], x2 = q[2], x3 = q[3];
                 r2[r][0] = fma_rn(e2[0][2], x2, fma_rn(e2[0][1], x1, fma_rn(e2[0][0], x0, (T)0)));
                 r2[r][1] = fma_rn(e2[1][2], x3, fma_rn(e2[1][1], x2, fma_rn(e2[1][0], x1, (T)0)));
@@ -94,12 +93,12 @@ prolong_kernel(LevelGeom<T> g, const T *y, const T *gsrc, T *__restrict__ stream
             }
             return d;
         }
-        p += oy;
 #pragma unroll
         for (int r = 0; r < 4; r++) {
             T x[4];
+            const T *q = p + (long long)r * mc2 + (unsigned)c2;
 #pragma unroll
-            for (int c = 0; c < 4; c++) x[c] = r < nc1 && c < nc2 ? p[r * mc2 + c] : (T)0;
+            for (int c = 0; c < 4; c++) x[c] = r < nc1 && c < nc2 ? q[c] : (T)0;
             T a = (T)0, b = (T)0;
 #pragma unroll
             for (int i = 0; i < 3; i++) {
@@ -129,7 +128,7 @@ prolong_kernel(LevelGeom<T> g, const T *y, const T *gsrc, T *__restrict__ stream
     auto emit = [&](int P, int j) {
         const bool k0 = kept_pos(m0, P);
         const int o = d0.efirst[P] - (j - 1);
-        const T *e = d0.etap + P * 3;
+        const T *e = d0.etap + P * 3ll;
         const T tA = o == 0 ? e[0] : o < 0 ? e[1] : (T)0, tB = o == 0 ? e[1] : o < 0 ? e[2] : e[0];
         const T tC = o == 0 ? e[2] : o < 0 ? (T)0 : e[1];
         const bool useA = j > 0 && o <= 0, useC = j + 1 < mc0 && o >= 0;
@@ -138,9 +137,12 @@ prolong_kernel(LevelGeom<T> g, const T *y, const T *gsrc, T *__restrict__ stream
         for (int r = 0; r < 2; r++) {
             if (r && !hr) continue;
             const bool rownew = !k0 || r;
-            const unsigned f = r ? ox1 : ox0, k = k0 ? (r ? ok1 : ok0) : f;   // of column Ca, or the row's first new one
-            const T *gp = MODE == MP_RT_FINAL ? gsrc + fp + f : coef + sp + k;
-            T *op = MODE == MP_RT_FINAL ? stream + sp + k : out + fp + f;
+            // the grid's row and the stream's; the column, in a kept row of a kept plane
+            // that of the row's new nodes
+            const long long f = fp + rows.x[r], k = sp + (k0 ? rows.k[r] : rows.x[r]);
+            const unsigned col = rownew ? (unsigned)Ca : (unsigned)Ca >> 1;
+            const T *gp = MODE == MP_RT_FINAL ? gsrc + f + (unsigned)Ca : coef + k + col;
+            T *op = MODE == MP_RT_FINAL ? stream + k + col : out + f + (unsigned)Ca;
 #pragma unroll
             for (int c = 0; c < 2; c++) {
                 if ((c && !hb) || (!rownew && !c)) continue;
