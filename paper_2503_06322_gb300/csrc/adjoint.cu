@@ -36,6 +36,22 @@ enum { MP_RT_FINAL = 1, MP_DT_FINAL = 2 };
 // sums its taps in a fixed order, so nothing depends on the tiling.  Binary32 keeps
 // to 64 registers, four CTAs an SM (72 without the bound: three).
 constexpr int kMpWarps = 8;
+// The tiles of a coarse plane run along gridDim.x, columns first: gridDim.y ends at
+// 65535, and a tall field has more row tiles.
+__host__ __device__ inline int tile_cols(int mc2) { return (mc2 + 31) / 32; }
+__host__ __device__ inline long long plane_tiles(int mc1, int mc2)
+{
+    return (long long)tile_cols(mc2) * ((mc1 + kMpWarps - 1) / kMpWarps);
+}
+// first coarse row and column of tile b
+struct PlaneTile {
+    int j1, j2;
+};
+__host__ __device__ inline PlaneTile plane_tile(unsigned b, int mc2)
+{
+    const unsigned cols = (unsigned)tile_cols(mc2), r = b / cols;
+    return {(int)r * kMpWarps, (int)(b - r * cols) * 32};
+}
 template <typename T, int MODE>
 __global__ void __launch_bounds__(32 * kMpWarps, sizeof(T) == 4 ? 4 : 2)
 prolong_kernel(LevelGeom<T> g, const T *y, const T *gsrc, T *__restrict__ stream, const T *coef, T *__restrict__ out,
@@ -44,8 +60,9 @@ prolong_kernel(LevelGeom<T> g, const T *y, const T *gsrc, T *__restrict__ stream
     const DimTables<T> &d0 = g.dim[0], &d1 = g.dim[1], &d2 = g.dim[2];
     const int m0 = d0.m, m1 = d1.m, m2 = d2.m, mc0 = d0.mc, mc1 = d1.mc, mc2 = d2.mc;
     const int lane = threadIdx.x & 31, warp = warp_index();
-    const int j2 = blockIdx.x * 32 + lane, j1 = blockIdx.y * kMpWarps + warp;
-    const int J0a = blockIdx.z * seg_len, J0b = min(J0a + seg_len, mc0);
+    const PlaneTile tile = plane_tile(blockIdx.x, mc2);
+    const int j2 = tile.j2 + lane, j1 = tile.j1 + warp;
+    const int J0a = blockIdx.y * seg_len, J0b = min(J0a + seg_len, mc0);
     next_begin();
     if (J0a >= J0b || j1 >= mc1) return;
     const bool live = j2 < mc2;
@@ -210,12 +227,12 @@ template <typename T, int MODE>
 cudaError_t launch_prolong(const LevelGeom<T> &g, const T *y, T *out, const T *gsrc, T *stream, const T *coef,
                            cudaStream_t s)
 {
-    const int mc0 = g.dim[0].mc, mc1 = g.dim[1].mc, mc2 = g.dim[2].mc;
-    const int gx = (mc2 + 31) / 32, gy = (mc1 + kMpWarps - 1) / kMpWarps;
-    const int seg = choose_segment(mc0, (long long)gx * gy, resident_ctas(prolong_kernel<T, MODE>, 32 * kMpWarps, 0));
+    const int mc0 = g.dim[0].mc;
+    const long long tiles = plane_tiles(g.dim[1].mc, g.dim[2].mc);
+    const int seg = choose_segment(mc0, tiles, resident_ctas(prolong_kernel<T, MODE>, 32 * kMpWarps, 0));
     count_launch();
-    return launch_next(prolong_kernel<T, MODE>, dim3(gx, gy, (mc0 + seg - 1) / seg), 32 * kMpWarps, 0, s, g, y, gsrc, stream,
-                       coef, out, seg);
+    return launch_next(prolong_kernel<T, MODE>, dim3((unsigned)tiles, (mc0 + seg - 1) / seg), 32 * kMpWarps, 0, s, g, y, gsrc,
+                       stream, coef, out, seg);
 }
 
 }  // namespace
