@@ -19,7 +19,8 @@ namespace {
 // low word (its last place is worth 1/2).  That is the floor of the exact
 // p + 1/2; the rounded sum of the definition reaches the next integer only from
 // p = n + 1/2 - ulp(p), whose low 20 bits are all ones (p < 2^30): such p, and
-// larger ones, take the definition as it stands.
+// larger ones, take the definition as it stands.  So does a NaN of either sign (an
+// overflowed coefficient times a rho of zero): its code is refused.
 __device__ __noinline__ long long quant_code_slow(double p)
 {
     const double t = __dadd_rn(p, 0.5);
@@ -32,7 +33,7 @@ __device__ __forceinline__ long long quant_code(T x, double rho)
 {
     const double p = __dmul_rn(fabs((double)x), rho);
     long long k;
-    if (__double2hiint(p) < 0x41D00000 && (__double2loint(p) & 0xFFFFF) != 0xFFFFF)
+    if ((unsigned)__double2hiint(p) < 0x41D00000u && (__double2loint(p) & 0xFFFFF) != 0xFFFFF)
         k = (unsigned)__double2loint(__dadd_rd(p, 2251799813685248.5)) >> 1;
     else
         k = quant_code_slow(p);
