@@ -1727,6 +1727,16 @@ __device__ __forceinline__ void stg32(long long *p, long long a, long long b, lo
 {
     asm volatile("st.global.v4.b64 [%0], {%1, %2, %3, %4};" :: "l"(p), "l"(a), "l"(b), "l"(c), "l"(d) : "memory");
 }
+__device__ __forceinline__ uint32_t lds32(uint32_t addr)
+{
+    uint32_t v;
+    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+    return v;
+}
+__device__ __forceinline__ void sts32(uint32_t addr, uint32_t v)
+{
+    asm volatile("st.shared.u32 [%0], %1;" :: "r"(addr), "r"(v) : "memory");
+}
 // predicated shared load and global store (no branch around them)
 __device__ __forceinline__ void lds_if(uint32_t &v, uint32_t cond, uint32_t addr)
 {
@@ -1741,7 +1751,7 @@ __device__ __forceinline__ void stg_if(long long *dst, uint32_t cond, long long 
 
 // A thread's view of its chunk's words, counted in 32 bits from `base`, the
 // 32-byte sector of memory in which the chunk starts (a chunk has at most 32768
-// symbols of 126 bits).  rc: ring index of the prefetched word `next`, wr: end
+// symbols of 126 bits); no word outside the stream is loaded.  rc: ring index of the prefetched word `next`, wr: end
 // of the words in the ring, pa: the sector after it.  left: words of the stream
 // from base on (words past it read as zero), lvec: the same as far as whole
 // sectors can be loaded (0 for a stream that does not start on 16 bytes).
@@ -1761,18 +1771,12 @@ struct BitQueue {
         return r;
     }
     __device__ __forceinline__ uint32_t addr(unsigned i) const { return ring + (i % kRingWords) * (4 * kDecThreads); }
-    __device__ __forceinline__ uint32_t at(unsigned i) const
-    {
-        uint32_t v;
-        asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr(i)) : "memory");
-        return v;
-    }
+    __device__ __forceinline__ uint32_t at(unsigned i) const { return lds32(addr(i)); }
     __device__ __forceinline__ void append()
     {
         const uint32_t r = addr(wr);   // wr is a multiple of 8: no wrap inside
 #pragma unroll
-        for (unsigned k = 0; k < 8; k++)
-            asm volatile("st.shared.u32 [%0], %1;" :: "r"(r + 4 * kDecThreads * k), "r"(pa.v[k]) : "memory");
+        for (unsigned k = 0; k < 8; k++) sts32(r + 4 * kDecThreads * k, pa.v[k]);
         wr += 8;
         pa = sector(wr);
     }
@@ -1800,7 +1804,8 @@ struct BitQueue {
     __device__ __forceinline__ void start(const uint32_t *w, unsigned long long n, unsigned long long pos, uint32_t &hi,
                                           uint32_t &lo, int &nb)
     {
-        // a stream on 16 bytes may start in the middle of a sector, whose first half is then loaded too
+        // a stream on 16 bytes may start in the middle of a sector: the words before
+        // it are not its own and are not loaded
         const bool vec = (reinterpret_cast<uintptr_t>(w) & 15) == 0;
         const long long lead = vec ? (long long)((reinterpret_cast<uintptr_t>(w) & 31) / 4) : 0;
         const long long wb = (((long long)(pos >> 5) + lead) & ~7LL) - lead, l = (long long)n - wb;
@@ -1808,7 +1813,12 @@ struct BitQueue {
         left = l < 0x7FFFFFFFll ? (unsigned)l : 0x7FFFFFFFu;
         lvec = vec ? left : 0u;
         wr = 0;
-        pa = sector(0);
+        if (wb < 0) {
+#pragma unroll
+            for (int k = 0; k < 8; k++) pa.v[k] = k + wb >= 0 ? ldw(w, (unsigned long long)(k + wb), n) : 0u;
+        } else {
+            pa = sector(0);
+        }
         seek((unsigned)((long long)pos - 32 * wb), hi, lo, nb);
     }
     // bit position of the window, from base
@@ -1888,8 +1898,7 @@ __device__ __forceinline__ bool decode_chunk(const DecodeArgs &a, const HuffScra
     unsigned emask = 0;
     // symbol in the high half
     auto step = [&](unsigned j, uint32_t &zj) -> uint32_t {
-        uint32_t e;
-        asm volatile("ld.shared.u32 %0, [%1];" : "=r"(e) : "r"(lut + 4 * (hi >> (32 - kLutBits))) : "memory");
+        uint32_t e = lds32(lut + 4 * (hi >> (32 - kLutBits)));
         // a codeword of up to 23 bits: its second-level entry, indexed by the
         // bits after the prefix (all within hi, nb >= 32)
         lds_if(e, e & kDecSub, sub + (e >> 16) + 4 * ((hi << kLutBits) >> (e & 31u)));
