@@ -87,7 +87,7 @@ prolong_kernel(LevelGeom<T> g, const T *y, const T *gsrc, T *__restrict__ stream
     if (!live) return;
     const long long cplane = (long long)mc1 * mc2;
     // the same in every lane: the plane pointers take the rows once per warp
-    const PlaneRows rows = plane_rows(m2, mc2, Ra);
+    const PlaneRows<long long> rows = plane_rows(m2, mc2, Ra);
     const long long ry = (long long)c1 * mc2;
     struct D4 { T v[2][2]; };
     // dimension-2 and -1 products of coarse plane j at the lane's nodes

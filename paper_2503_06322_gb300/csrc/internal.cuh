@@ -48,16 +48,18 @@ __host__ __device__ inline int kept_before(int p) { return (p + 1) >> 1; }
 __host__ __device__ inline int cidx_of(int m, int mc, int p) { return (p == m - 1) ? mc - 1 : (p >> 1); }
 // Where the fine rows R and R + 1 start inside a fine plane (x) and, by their new
 // nodes, inside a kept plane of the stream (k); rows of m2 nodes, mc2 of them kept.
-// In 64 bits: a 2-D field is one plane, of any size.
+// A 2-D field is one plane, of any size: Off has 64 bits where planes reach 2^31 nodes.
+template <typename Off>
 struct PlaneRows {
-    long long x[2], k[2];
+    Off x[2], k[2];
 };
-__host__ __device__ inline PlaneRows plane_rows(int m2, int mc2, int R)
+template <typename Off = long long>
+__host__ __device__ inline PlaneRows<Off> plane_rows(int m2, int mc2, int R)
 {
-    PlaneRows w;
+    PlaneRows<Off> w;
     for (int r = 0; r < 2; r++) {
-        w.x[r] = (long long)(R + r) * m2;
-        w.k[r] = w.x[r] - (long long)kept_before(R + r) * mc2;
+        w.x[r] = ((Off)R + r) * m2;
+        w.k[r] = w.x[r] - (Off)kept_before(R + r) * mc2;
     }
     return w;
 }

@@ -43,15 +43,23 @@ class Ops:
         np.add.at(full, self.new + 1, self.wr * v[self.new])
         return full[self.kept]
 
-    def prolong_mass(self, c):                   # M P
-        v = np.zeros(self.kept.size + self.new.size)
-        v[self.kept] = c
+    def prolong(self, c):                        # P
+        v = self.inject(c)
         v[self.new] = self.wl * v[self.new - 1] + self.wr * v[self.new + 1]
+        return v
+
+    def mass(self, v):                           # M
         d, o = self.fine
         r = d * v
         r[1:] += o * v[:-1]
         r[:-1] += o * v[1:]
         return r
+
+    def prolong_mass(self, c):                   # M P
+        return self.mass(self.prolong(c))
+
+    def project(self, v):                        # the coarse values of a decomposition
+        return self.solve(self.restrict(self.mass(v)))
 
     def solve(self, b):                          # the coarse mass matrix
         from scipy.linalg import solveh_banded
@@ -156,3 +164,35 @@ def test_adjoints(n):
         scale = max(scale, ref.abs().max().item())
         err = max(err, (g[r:e] - ref).abs().max().item())
     assert err <= TOL * scale, (err, scale)
+
+
+@pytest.mark.parametrize("n", [129, N])
+def test_transforms(n):
+    from paper_2503_06322_gb300 import hpdr as H
+    x = levels(n)
+    a, b = vectors(n, 3, 2)
+    u = product(a, b, torch.empty(n, n, dtype=torch.float32, device="cuda"))
+    coef = H.hpdr_decompose(u)
+    m, p, q = n, a, b
+    for grid in x[:2]:
+        ops = Ops(grid)
+        check_section(coef[:m * m], [(1.0, p, q), (-1.0, ops.prolong(p[ops.kept]), ops.prolong(q[ops.kept]))], m)
+        m, p, q = (m + 1) // 2, ops.project(p), ops.project(q)
+    back = H.hpdr_recompose(coef, (n, n))
+    del coef
+    err = max((back[r:r + 4096] - u[r:r + 4096]).abs().max().item() for r in range(0, n, 4096))
+    assert err <= TOL * np.abs(a).max() * np.abs(b).max()
+
+
+@pytest.mark.parametrize("n", [129, N])
+def test_containers(n):
+    from paper_2503_06322_gb300 import hpdr as H
+    a, b = vectors(n, 4, 2)
+    u = product(a, b, torch.empty(n, n, dtype=torch.float32, device="cuda"))
+    buf = H.hpdr_compress(u, 1e-2)
+    back = H.hpdr_decompress(buf)
+    del buf
+    err = max((back[r:r + 4096].double() - u[r:r + 4096]).abs().max().item() for r in range(0, n, 4096))
+    del back
+    torch.cuda.empty_cache()
+    assert err <= 1e-2 * u.abs().max().item()
