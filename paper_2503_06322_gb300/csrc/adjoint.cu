@@ -26,15 +26,14 @@ enum { MP_RT_FINAL = 1, MP_DT_FINAL = 2 };
 //   MP_DT_FINAL: out[p] = coef[rank(p)] + y_f(p)
 // One pass over the fine grid is all it needs from memory (a pass per dimension,
 // through two partial grids, moved 2.6 times the bytes and took 173 us for the
-// finest level of 257^3; this takes 65, bound by instruction issue: 78 with the
+// finest level of 257^3; this takes 62, bound by instruction issue: 78 with the
 // window's edges tested at every node).  A warp owns coarse row j1 of a tile,
 // lane l coarse column j2, and the CTA marches along the coarse planes of its
 // segment; for each plane a lane forms the dimension-2, then the dimension-1
 // products at its 2 x 2 fine nodes (rows Ra, Ra + 1, columns Ca, Ca + 1) from the
 // four rows and four columns of y around it (cached loads, coalesced per row)
 // and keeps the last three planes' for the dimension-0 products.  Every value
-// sums its taps in a fixed order, so nothing depends on the tiling.  Binary32 keeps
-// to 64 registers, four CTAs an SM (72 without the bound: three).
+// sums its taps in a fixed order, so nothing depends on the tiling.
 constexpr int kMpWarps = 8;
 // The tiles of a coarse plane run along gridDim.x, columns first: gridDim.y ends at
 // 65535, and a tall field has more row tiles.
@@ -52,8 +51,9 @@ __host__ __device__ inline PlaneTile plane_tile(unsigned b, int mc2)
     const unsigned cols = (unsigned)tile_cols(mc2), r = b / cols;
     return {(int)r * kMpWarps, (int)(b - r * cols) * 32};
 }
-template <typename T, int MODE>
-__global__ void __launch_bounds__(32 * kMpWarps, sizeof(T) == 4 ? 4 : 2)
+// BIG: planes of 2^31 nodes and more, whose offsets take 64 bits
+template <typename T, int MODE, bool BIG>
+__global__ void __launch_bounds__(32 * kMpWarps)
 prolong_kernel(LevelGeom<T> g, const T *y, const T *gsrc, T *__restrict__ stream, const T *coef, T *__restrict__ out,
                int seg_len)
 {
@@ -72,7 +72,7 @@ prolong_kernel(LevelGeom<T> g, const T *y, const T *gsrc, T *__restrict__ stream
     // taps of the two fine columns and rows; the second ones start at the same
     // coarse index or one later
     T e2[2][3], e1[2][3];
-    const int c2 = d2.efirst[Ca], c1 = __shfl_sync(0xffffffffu, d1.efirst[Ra], 0);
+    const int c2 = d2.efirst[Ca], c1 = d1.efirst[Ra];
     const bool s2 = hb && d2.efirst[Ca + 1] != c2, s1 = hr && d1.efirst[Ra + 1] != c1;
 #pragma unroll
     for (int i = 0; i < 3; i++) {
@@ -86,19 +86,21 @@ prolong_kernel(LevelGeom<T> g, const T *y, const T *gsrc, T *__restrict__ stream
     const bool inner = __all_sync(0xffffffffu, s2 && s1 && nc2 >= 4 && nc1 >= 4);
     if (!live) return;
     const long long cplane = (long long)mc1 * mc2;
-    // the same in every lane: the plane pointers take the rows once per warp
-    const PlaneRows<long long> rows = plane_rows(m2, mc2, Ra);
-    const long long ry = (long long)c1 * mc2;
+    // offsets inside a coarse plane, a fine plane, and a kept plane of the stream
+    using Off = typename std::conditional<BIG, unsigned long long, unsigned>::type;
+    const PlaneRows<Off> rows = plane_rows<Off>(m2, mc2, Ra);
+    const Off oy = (Off)c1 * mc2 + c2;
+    const Off ox0 = rows.x[0] + Ca, ox1 = rows.x[1] + Ca, ok0 = rows.k[0] + (Ca >> 1), ok1 = rows.k[1] + Ca;
     struct D4 { T v[2][2]; };
     // dimension-2 and -1 products of coarse plane j at the lane's nodes
     auto plane = [&](int j) -> D4 {
-        const T *p = y + (j * cplane + ry);   // row c1 of the plane
+        const T *p = y + j * cplane;
         T r2[4][2];   // rows c1.., the two columns
         D4 d;
         if (inner) {
 #pragma unroll
             for (int r = 0; r < 4; r++) {
-                const T *q = p + (long long)r * mc2 + (unsigned)c2;
+                const T *q = p + (oy + (Off)r * mc2);
                 const T x0 = q[0], x1 = q[1], x2 = q[2], x3 = q[3];
                 r2[r][0] = fma_rn(e2[0][2], x2, fma_rn(e2[0][1], x1, fma_rn(e2[0][0], x0, (T)0)));
                 r2[r][1] = fma_rn(e2[1][2], x3, fma_rn(e2[1][1], x2, fma_rn(e2[1][0], x1, (T)0)));
@@ -113,7 +115,7 @@ prolong_kernel(LevelGeom<T> g, const T *y, const T *gsrc, T *__restrict__ stream
 #pragma unroll
         for (int r = 0; r < 4; r++) {
             T x[4];
-            const T *q = p + (long long)r * mc2 + (unsigned)c2;
+            const T *q = p + (oy + (Off)r * mc2);
 #pragma unroll
             for (int c = 0; c < 4; c++) x[c] = r < nc1 && c < nc2 ? q[c] : (T)0;
             T a = (T)0, b = (T)0;
@@ -154,12 +156,9 @@ prolong_kernel(LevelGeom<T> g, const T *y, const T *gsrc, T *__restrict__ stream
         for (int r = 0; r < 2; r++) {
             if (r && !hr) continue;
             const bool rownew = !k0 || r;
-            // the grid's row and the stream's; the column, in a kept row of a kept plane
-            // that of the row's new nodes
-            const long long f = fp + rows.x[r], k = sp + (k0 ? rows.k[r] : rows.x[r]);
-            const unsigned col = rownew ? (unsigned)Ca : (unsigned)Ca >> 1;
-            const T *gp = MODE == MP_RT_FINAL ? gsrc + f + (unsigned)Ca : coef + k + col;
-            T *op = MODE == MP_RT_FINAL ? stream + k + col : out + f + (unsigned)Ca;
+            const Off f = r ? ox1 : ox0, k = k0 ? (r ? ok1 : ok0) : f;   // of column Ca, or the row's first new one
+            const T *gp = MODE == MP_RT_FINAL ? gsrc + fp + f : coef + sp + k;
+            T *op = MODE == MP_RT_FINAL ? stream + sp + k : out + fp + f;
 #pragma unroll
             for (int c = 0; c < 2; c++) {
                 if ((c && !hb) || (!rownew && !c)) continue;
@@ -228,10 +227,11 @@ cudaError_t launch_prolong(const LevelGeom<T> &g, const T *y, T *out, const T *g
                            cudaStream_t s)
 {
     const int mc0 = g.dim[0].mc;
+    const auto kern = big_planes(g) ? prolong_kernel<T, MODE, true> : prolong_kernel<T, MODE, false>;
     const long long tiles = plane_tiles(g.dim[1].mc, g.dim[2].mc);
-    const int seg = choose_segment(mc0, tiles, resident_ctas(prolong_kernel<T, MODE>, 32 * kMpWarps, 0));
+    const int seg = choose_segment(mc0, tiles, resident_ctas(kern, 32 * kMpWarps, 0));
     count_launch();
-    return launch_next(prolong_kernel<T, MODE>, dim3((unsigned)tiles, (mc0 + seg - 1) / seg), 32 * kMpWarps, 0, s, g, y, gsrc,
+    return launch_next(kern, dim3((unsigned)tiles, (mc0 + seg - 1) / seg), 32 * kMpWarps, 0, s, g, y, gsrc,
                        stream, coef, out, seg);
 }
 

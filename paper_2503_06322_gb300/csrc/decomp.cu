@@ -422,12 +422,7 @@ __device__ __forceinline__ void sum_rows(const LevelGeom<T> &g, const TileGeom &
     }
 }
 
-// BIG: planes of 2^31 nodes and more (a 2-D field is one plane), whose offsets take
-// 64 bits; with them for every field 513^3 compression took 1448 us instead of 1410
-// and decompression 1463 instead of 1397.
-template <typename T>
-bool big_planes(const LevelGeom<T> &g) { return (long long)g.dim[1].m * g.dim[2].m >= 1ll << 31; }
-
+// BIG: big_planes
 template <typename T, int SINK, bool BIG>
 __global__ void __launch_bounds__((decomp_warps<T>() + 1) * 32, sizeof(T) == 4 ? 2 : 1)
 decomp_kernel(RestrictArgs<T> a, int seg_len)

@@ -303,6 +303,12 @@ __device__ __forceinline__ int first_coarse_at_or_after(const DimTables<T> &d, i
 
 }  // namespace
 
+// Planes whose offsets take 64 bits (a 2-D field is one plane).  With 64 bits for
+// every field 513^3 compression took 1448 us instead of 1410, decompression 1463
+// instead of 1397, a training step at 257^3 647 instead of 641.
+template <typename T>
+bool big_planes(const LevelGeom<T> &g) { return (long long)g.dim[1].m * g.dim[2].m >= 1ll << 31; }
+
 // Coarse planes per CTA (segment) for a grid of `tiles` x segments CTAs.
 int choose_segment(int mc0, long long tiles, int per_sm);
 

@@ -46,7 +46,8 @@ def exe(tmp_path_factory):
     grid = open(os.path.join(CSRC, "internal.cuh")).read()
     a, b = grid.index("__host__ __device__ inline int cpos_of"), grid.index("// Explicitly rounded arithmetic")
     src = open(os.path.join(CSRC, "adjoint.cu")).read()
-    c, d = src.index("constexpr int kMpWarps"), src.index("template <typename T, int MODE>")
+    c = src.index("constexpr int kMpWarps")
+    d = src.rindex("template <typename T", c, src.index("__global__ void", c))
     t = tmp_path_factory.mktemp("rows_host")
     (t / "p.cpp").write_text(PRELUDE + grid[a:b] + src[c:d] + MAIN)
     subprocess.run([cxx, "-O2", "-std=c++17", "-Wall", "-fsanitize=undefined", "-fno-sanitize-recover", "-o", str(t / "p"),
