@@ -29,30 +29,33 @@ enum { MP_RT_FINAL = 1, MP_DT_FINAL = 2 };
 // finest level of 257^3; this takes 62, bound by instruction issue: 78 with the
 // window's edges tested at every node).  A warp owns coarse row j1 of a tile,
 // lane l coarse column j2, and the CTA marches along the coarse planes of its
-// segment; for each plane a lane forms the dimension-2, then the dimension-1
+// segment (on thin grids a warp owns four rows and eight columns); for each plane a lane forms the dimension-2, then the dimension-1
 // products at its 2 x 2 fine nodes (rows Ra, Ra + 1, columns Ca, Ca + 1) from the
 // four rows and four columns of y around it (cached loads, coalesced per row)
 // and keeps the last three planes' for the dimension-0 products.  Every value
 // sums its taps in a fixed order, so nothing depends on the tiling.
 constexpr int kMpWarps = 8;
-// The tiles of a coarse plane run along gridDim.x, columns first: gridDim.y ends at
-// 65535, and a tall field has more row tiles.
-__host__ __device__ inline int tile_cols(int mc2) { return (mc2 + 31) / 32; }
-__host__ __device__ inline long long plane_tiles(int mc1, int mc2)
+// The tiles of a coarse plane, LC columns wide, run along gridDim.x, columns first:
+// gridDim.y ends at 65535, and a tall field has more row tiles.
+__host__ __device__ inline int tile_cols(int mc2, int LC) { return (mc2 + LC - 1) / LC; }
+__host__ __device__ inline int tile_rows(int LC) { return kMpWarps * (32 / LC); }
+__host__ __device__ inline long long plane_tiles(int mc1, int mc2, int LC)
 {
-    return (long long)tile_cols(mc2) * ((mc1 + kMpWarps - 1) / kMpWarps);
+    return (long long)tile_cols(mc2, LC) * ((mc1 + tile_rows(LC) - 1) / tile_rows(LC));
 }
 // first coarse row and column of tile b
 struct PlaneTile {
     int j1, j2;
 };
-__host__ __device__ inline PlaneTile plane_tile(unsigned b, int mc2)
+__host__ __device__ inline PlaneTile plane_tile(unsigned b, int mc2, int LC)
 {
-    const unsigned cols = (unsigned)tile_cols(mc2), r = b / cols;
-    return {(int)r * kMpWarps, (int)(b - r * cols) * 32};
+    const unsigned cols = (unsigned)tile_cols(mc2, LC), r = b / cols;
+    return {(int)r * tile_rows(LC), (int)(b - r * cols) * LC};
 }
-// BIG: planes of 2^31 nodes and more, whose offsets take 64 bits
-template <typename T, int MODE, bool BIG>
+// BIG: planes of 2^31 nodes and more, whose offsets take 64 bits.  LC: a warp takes
+// 32 columns of one coarse row, or 8 of four rows, which leaves fewer lanes without a
+// column on grids that are thin in the last dimension.
+template <typename T, int MODE, int LC, bool BIG>
 __global__ void __launch_bounds__(32 * kMpWarps)
 prolong_kernel(LevelGeom<T> g, const T *y, const T *gsrc, T *__restrict__ stream, const T *coef, T *__restrict__ out,
                int seg_len)
@@ -60,14 +63,14 @@ prolong_kernel(LevelGeom<T> g, const T *y, const T *gsrc, T *__restrict__ stream
     const DimTables<T> &d0 = g.dim[0], &d1 = g.dim[1], &d2 = g.dim[2];
     const int m0 = d0.m, m1 = d1.m, m2 = d2.m, mc0 = d0.mc, mc1 = d1.mc, mc2 = d2.mc;
     const int lane = threadIdx.x & 31, warp = warp_index();
-    const PlaneTile tile = plane_tile(blockIdx.x, mc2);
-    const int j2 = tile.j2 + lane, j1 = tile.j1 + warp;
+    constexpr int RW = 32 / LC;   // rows of a warp
+    const PlaneTile tile = plane_tile(blockIdx.x, mc2, LC);
+    const int w1 = tile.j1 + warp * RW, j2 = tile.j2 + lane % LC, j1 = w1 + (RW > 1 ? lane / LC : 0);
     const int J0a = blockIdx.y * seg_len, J0b = min(J0a + seg_len, mc0);
     next_begin();
-    if (J0a >= J0b || j1 >= mc1) return;
-    const bool live = j2 < mc2;
-    const int jc = live ? j2 : mc2 - 1;
-    const int Ca = cpos_of(m2, mc2, jc), Ra = cpos_of(m1, mc1, j1);
+    if (J0a >= J0b || w1 >= mc1) return;
+    const bool live = j2 < mc2 && (RW == 1 || j1 < mc1);
+    const int Ca = cpos_of(m2, mc2, min(j2, mc2 - 1)), Ra = cpos_of(m1, mc1, RW == 1 ? j1 : min(j1, mc1 - 1));
     const bool hb = Ca + 1 < m2 && !kept_pos(m2, Ca + 1), hr = Ra + 1 < m1 && !kept_pos(m1, Ra + 1);
     // taps of the two fine columns and rows; the second ones start at the same
     // coarse index or one later
@@ -226,13 +229,19 @@ template <typename T, int MODE>
 cudaError_t launch_prolong(const LevelGeom<T> &g, const T *y, T *out, const T *gsrc, T *stream, const T *coef,
                            cudaStream_t s)
 {
-    const int mc0 = g.dim[0].mc;
-    const auto kern = big_planes(g) ? prolong_kernel<T, MODE, true> : prolong_kernel<T, MODE, false>;
-    const long long tiles = plane_tiles(g.dim[1].mc, g.dim[2].mc);
+    const int mc0 = g.dim[0].mc, mc1 = g.dim[1].mc, mc2 = g.dim[2].mc;
+    // Eight columns below 64 and where tiles of 32 have over a quarter more lanes
+    // (recomposition's adjoint, binary64, 32 or 8 columns: 1000x1000x15 2668 or 1639 us,
+    // x63 2840 or 2738, x65 4318 or 3610, x80 4540 or 4185; 200x200x127 460 or 477,
+    // 100x200x400 635 or 644).
+    const bool big = big_planes(g), thin = !big && (mc2 < 64 || 4 * 32 * tile_cols(mc2, 32) > 5 * 8 * tile_cols(mc2, 8));
+    const auto kern = big ? prolong_kernel<T, MODE, 32, true>
+                    : thin ? prolong_kernel<T, MODE, 8, false> : prolong_kernel<T, MODE, 32, false>;
+    const long long tiles = plane_tiles(mc1, mc2, thin ? 8 : 32);
     const int seg = choose_segment(mc0, tiles, resident_ctas(kern, 32 * kMpWarps, 0));
     count_launch();
-    return launch_next(kern, dim3((unsigned)tiles, (mc0 + seg - 1) / seg), 32 * kMpWarps, 0, s, g, y, gsrc,
-                       stream, coef, out, seg);
+    return launch_next(kern, dim3((unsigned)tiles, (mc0 + seg - 1) / seg), 32 * kMpWarps, 0, s, g, y, gsrc, stream, coef, out,
+                       seg);
 }
 
 }  // namespace

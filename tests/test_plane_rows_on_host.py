@@ -20,16 +20,16 @@ PRELUDE = r'''
 MAIN = r'''
 int main(int argc, char **argv)
 {
-    if (argc == 3) {     // every coarse row and column in exactly one tile, all of them in gridDim.x
-        const int mc1 = atoi(argv[1]), mc2 = atoi(argv[2]);
-        const long long n = plane_tiles(mc1, mc2);
+    if (argc == 5) {     // every coarse row and column in exactly one tile, all of them in gridDim.x
+        const int mc1 = atoi(argv[1]), mc2 = atoi(argv[2]), LC = atoi(argv[3]), R = tile_rows(LC);
+        const long long n = plane_tiles(mc1, mc2, LC);
         long long next = 0;
         for (long long b = 0; b < n; b++) {
-            const PlaneTile t = plane_tile((unsigned)b, mc2);
-            if (t.j1 >= mc1 || t.j2 >= mc2 || t.j1 % kMpWarps || t.j2 % 32) return 1;
-            if ((long long)(t.j1 / kMpWarps) * tile_cols(mc2) + t.j2 / 32 != next++) return 2;
+            const PlaneTile t = plane_tile((unsigned)b, mc2, LC);
+            if (t.j1 >= mc1 || t.j2 >= mc2 || t.j1 % R || t.j2 % LC) return 1;
+            if ((long long)(t.j1 / R) * tile_cols(mc2, LC) + t.j2 / LC != next++) return 2;
         }
-        return n * kMpWarps * 32 < (long long)mc1 * mc2 || n > 2147483647ll;
+        return n * R * LC < (long long)mc1 * mc2 || n > 2147483647ll;
     }
     const PlaneRows w = plane_rows(atoi(argv[1]), atoi(argv[2]), atoi(argv[3]));
     printf("%lld %lld %lld %lld\n", w.x[0], w.x[1], w.k[0], w.k[1]);
@@ -66,6 +66,7 @@ def test_row_offsets(exe, m1, m2):
 
 
 @pytest.mark.parametrize("mc1,mc2", [(1, 2), (8, 32), (9, 33), (550001, 3), (1 << 29, 2), (3, 1 << 29), (35001, 35001)])
-def test_tiles(exe, mc1, mc2):
+@pytest.mark.parametrize("cols", [32, 8])
+def test_tiles(exe, mc1, mc2, cols):
     """550001 coarse rows: a field of 1.1 million rows, past 65535 tiles of eight"""
-    assert subprocess.run([exe, str(mc1), str(mc2)]).returncode == 0
+    assert subprocess.run([exe, str(mc1), str(mc2), str(cols), "tiles"]).returncode == 0
