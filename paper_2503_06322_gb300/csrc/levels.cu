@@ -188,125 +188,122 @@ __device__ __forceinline__ void sweep_line(T *p, int st, int n, const T *sub, co
     for (; t >= 0; t--) x = sweep_bwd<1>(p, st, cp, t, x, [&](int q, const T(&v)[1]) { fin(q, v); });
 }
 
+// i / d by a multiply-high: exact for i d < 2^32, so for i and d below 2^16 (the
+// arrays of the coarse block hold at most kCoarseSmem / 2 / sizeof(float) = 25600
+// nodes); mul = 0 for d = 1
+__device__ __forceinline__ unsigned small_div_mul(int d) { return 0xFFFFFFFFu / (unsigned)d + 1u; }
+__device__ __forceinline__ int small_div(int i, unsigned mul)
+{
+    return mul == 0u ? i : (int)__umulhi((unsigned)i, mul);
+}
+
 // a contiguous run of cnt elements between global and shared memory in 16-byte
 // pieces, single elements at its ends; dst and src agree modulo 16 bytes
 __device__ __forceinline__ void cp_async16(void *dst_smem, const void *src)
 {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst_smem)), "l"(src) : "memory");
 }
+template <typename T> struct alignas(16) Four16 {
+    T v[16 / sizeof(T)];
+};
 template <typename T>
 __device__ __forceinline__ int run_head(const T *g, int cnt)
 {
     const int h = (int)((16 - ((uintptr_t)g & 15)) & 15) / (int)sizeof(T);
     return h < cnt ? h : cnt;
 }
+// where element i of a run of lines of n sits in a tile of pitch n, or (pad) in one
+// of pitch n + V, V a 16-byte piece; mul: small_div factor of the n / V pieces of a line
 template <typename T>
-__device__ __forceinline__ void run_load(T *dst, const T *src, int cnt)
+__device__ __forceinline__ int tile_at(int i, bool pad, unsigned mul)
+{
+    constexpr int V = 16 / sizeof(T);
+    return pad ? i + small_div(i / V, mul) * V : i;
+}
+template <typename T>
+__device__ __forceinline__ void run_load(T *dst, const T *src, int cnt, bool pad, unsigned mul)
 {
     constexpr int V = 16 / sizeof(T);
     const int h = run_head(src, cnt), nv = (cnt - h) / V;
-    for (int i = threadIdx.x; i < nv; i += blockDim.x) cp_async16(dst + h + i * V, src + h + i * V);
+    for (int i = threadIdx.x; i < nv; i += blockDim.x)
+        cp_async16(dst + tile_at<T>(h + i * V, pad, mul), src + h + i * V);
     if ((int)threadIdx.x < h) cp_async_elem(dst + threadIdx.x, src + threadIdx.x);
     for (int i = h + nv * V + threadIdx.x; i < cnt; i += blockDim.x) cp_async_elem(dst + i, src + i);
 }
+// the tile src into the run dst: as it is (sign 0), or added to it or subtracted
 template <typename T>
-__device__ __forceinline__ void run_store(T *dst, const T *src, int cnt)
+__device__ __forceinline__ void run_store(T *dst, const T *src, int cnt, bool pad, unsigned mul, int sign)
 {
-    constexpr int V = 16 / sizeof(T);
-    const int h = run_head(dst, cnt), nv = (cnt - h) / V;
-#pragma unroll 4
-    for (int i = threadIdx.x; i < nv; i += blockDim.x)
-        *reinterpret_cast<uint4 *>(dst + h + i * V) = *reinterpret_cast<const uint4 *>(src + h + i * V);
-    if ((int)threadIdx.x < h) dst[threadIdx.x] = src[threadIdx.x];
-    for (int i = h + nv * V + threadIdx.x; i < cnt; i += blockDim.x) dst[i] = src[i];
+    constexpr int V = 16 / sizeof(T), U = 4;
+    const auto take = [&](T old, T x) { return sign == 0 ? x : sign > 0 ? add_rn(old, x) : sub_rn(old, x); };
+    // whole pieces where the tile sits like the run modulo 16 bytes
+    const bool vec = (smem_u32(src) & 15) == ((uintptr_t)dst & 15);
+    const int h = vec ? run_head(dst, cnt) : cnt, nv = (cnt - h) / V;
+    for (int i0 = threadIdx.x; i0 < nv; i0 += U * blockDim.x) {
+        Four16<T> o[U];
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            const int i = i0 + u * (int)blockDim.x;
+            if (sign != 0 && i < nv) o[u] = *reinterpret_cast<const Four16<T> *>(dst + h + i * V);
+        }
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            const int i = i0 + u * (int)blockDim.x;
+            if (i >= nv) break;
+            Four16<T> x = *reinterpret_cast<const Four16<T> *>(src + tile_at<T>(h + i * V, pad, mul));
+#pragma unroll
+            for (int k = 0; k < V; k++) x.v[k] = take(o[u].v[k], x.v[k]);
+            *reinterpret_cast<Four16<T> *>(dst + h + i * V) = x;
+        }
+    }
+    for (int i = threadIdx.x; i < h; i += blockDim.x) dst[i] = take(sign ? dst[i] : (T)0, src[tile_at<T>(i, pad, mul)]);
+    for (int i = h + nv * V + threadIdx.x; i < cnt; i += blockDim.x) dst[i] = take(sign ? dst[i] : (T)0, src[tile_at<T>(i, pad, mul)]);
 }
 
-// Contiguous lines: a tile of up to 32 lines, one lane of a warp each, with the
-// tile of v_c that takes the result beside it.  A tile is one contiguous run of
-// memory, so both tiles arrive by 16-byte asynchronous copies in flight together
-// and leave by 16-byte stores: element-wise copies and a read-modify-write of v_c
-// after the sweeps kept the kernel at 2.4 TB/s.  Lines of 257: 84 -> 60 us at
-// 513^3 (204 MB), lines of 129: 19 -> 10 us.
-// The lines keep the pitch n they have in memory, so the lanes of a warp meet in
-// gcd(n, 32) words of a bank: where n is a multiple of kContigLag, lane i runs i
-// steps behind, which makes the stride between lanes odd (not below that: the
-// lag adds 31 steps with bound checks, and 2- and 4-fold conflicts cost less).
+// Contiguous lines: a tile of up to 32 lines, one lane of a warp each.  A tile is one
+// contiguous run of memory: it arrives by 16-byte asynchronous copies, and leaves by
+// 16-byte stores that add it to v_c.  What counts is how many lines an SM holds at
+// once, so v_c does not sit beside the tile (binary64 lines of 1001, eight in one CTA
+// with their v_c: 896 us at 15x1500x2000, eighteen in two CTAs without: 444;
+// lines of 257 at 513^3, 204 MB: 53 and 42).
+// A line keeps the pitch n that it has in memory, so the lanes of a warp meet in
+// gcd(n, 32) words of a bank; where n is a multiple of kContigPad the lines are a
+// 16-byte piece further apart (binary64 lines of 8 at 2000x2000x15, in memory's pitch
+// with the lanes a step apart: 250 us, like this: 65).
 constexpr int kContigRows = 32;
-constexpr int kContigLag = 8;
+constexpr int kContigPad = 8;
 constexpr int kContigThreads = 128;
 constexpr size_t kContigMaxKb = 220;
 template <typename T>
 __global__ void __launch_bounds__(kContigThreads)
-solve_contig_kernel(T *b, const T *src, int n, long long nlines, int rows, const T *__restrict__ sub, const T *__restrict__ cp,
+solve_contig_kernel(T *b, const T *src, int n, long long nlines, int rows, bool pad, const T *__restrict__ sub, const T *__restrict__ cp,
                     const T *__restrict__ inv_den, T *vc, int sign)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     constexpr int V = 16 / sizeof(T);
     T *csub = reinterpret_cast<T *>(smem_raw), *ccp = csub + n, *cinv = ccp + n;
     T *tile = csub + (3 * n + V - 1) / V * V;
+    const int pitch = pad ? n + V : n;
+    const unsigned mul = pad ? small_div_mul(n / V) : 0u;
     const long long row0 = blockIdx.x * (long long)rows, first = row0 * n;
     const int nr = (int)min((long long)rows, nlines - row0), cnt = nr * n;
     for (int t = threadIdx.x; t < n; t += blockDim.x) { csub[t] = sub[t]; ccp[t] = cp[t]; cinv[t] = inv_den[t]; }
     next_begin();
-    // the right-hand side (b, or an array that is kept) and where it sits modulo
-    // 16 bytes; without v_c the solution takes its place, so b has to agree
+    // the right-hand side (b, or an array that is kept) where it sits modulo 16
+    // bytes; the solution takes its place
     T *B = tile + ((uintptr_t)(src + first) & 15) / sizeof(T);
-    run_load(B, src + first, cnt);
-    T *X = B;
-    if (sign != 0) {
-        X = tile + (rows * n + 2 * V - 1) / V * V + ((uintptr_t)(vc + first) & 15) / sizeof(T);
-        run_load(X, vc + first, cnt);
-    }
+    run_load(B, src + first, cnt, pad, mul);
     cp_async_wait_all();
     __syncthreads();
     if ((int)threadIdx.x < nr) {
-        T *p = B + threadIdx.x * n, *xo = X + threadIdx.x * n;
-        if (n % kContigLag) {
-            sweep_line<T>(p, 1, n, csub, ccp, cinv, [&](int t, const auto &v) {
-                constexpr int U = sizeof(v) / sizeof(T);
-                T old[U];
-                if (sign != 0) {
+        T *p = B + threadIdx.x * pitch;
+        sweep_line<T>(p, 1, n, csub, ccp, cinv, [&](int t, const auto &v) {
 #pragma unroll
-                    for (int u = 0; u < U; u++) old[u] = xo[t - u];
-                }
-#pragma unroll
-                for (int u = 0; u < U; u++)
-                    xo[t - u] = sign == 0 ? v[u] : sign > 0 ? add_rn(old[u], v[u]) : sub_rn(old[u], v[u]);
-            });
-        } else {
-            const int lag = (int)threadIdx.x;
-            constexpr int U = 8;
-            T y = (T)0;
-            for (int k0 = -lag; k0 < n; k0 += U) {
-                T v[U], f[U], g[U];
-#pragma unroll
-                for (int u = 0; u < U; u++) {
-                    const int t = min(max(k0 + u, 0), n - 1);
-                    v[u] = p[t]; f[u] = csub[t]; g[u] = cinv[t];
-                }
-#pragma unroll
-                for (int u = 0; u < U; u++)
-                    if (k0 + u >= 0 && k0 + u < n) { y = mul_rn(fma_rn(-f[u], y, v[u]), g[u]); p[k0 + u] = y; }
-            }
-            T x = (T)0;
-            for (int k0 = n - 1 + lag; k0 >= 0; k0 -= U) {
-                T v[U], f[U], old[U];
-#pragma unroll
-                for (int u = 0; u < U; u++) {
-                    const int t = min(max(k0 - u, 0), n - 1);
-                    v[u] = p[t]; f[u] = ccp[t]; old[u] = xo[t];
-                }
-#pragma unroll
-                for (int u = 0; u < U; u++)
-                    if (k0 - u >= 0 && k0 - u < n) {
-                        x = fma_rn(-f[u], x, v[u]);
-                        xo[k0 - u] = sign == 0 ? x : sign > 0 ? add_rn(old[u], x) : sub_rn(old[u], x);
-                    }
-            }
-        }
+            for (int u = 0; u < (int)(sizeof(v) / sizeof(T)); u++) p[t - u] = v[u];
+        });
     }
     __syncthreads();
-    run_store(sign == 0 ? b + first : vc + first, X, cnt);
+    run_store(sign == 0 ? b + first : vc + first, B, cnt, pad, mul, sign);
 }
 
 // --------------------------------------------------------------------------
@@ -518,14 +515,6 @@ __host__ __device__ inline void coarse_sizes(const LevelGeom<T> &g, long long &n
     nc = c0 * c1 * c2;
     r2 = m0 * m1 * c2;
     r1 = m0 * c1 * c2;
-}
-
-// i / d by a multiply-high: exact for i and d below 2^16 (the block's arrays
-// hold at most kCoarseSmem / 2 / sizeof(float) = 25600 nodes); mul = 0 for d = 1
-__device__ __forceinline__ unsigned small_div_mul(int d) { return 0xFFFFFFFFu / (unsigned)d + 1u; }
-__device__ __forceinline__ int small_div(int i, unsigned mul)
-{
-    return mul == 0u ? i : (int)__umulhi((unsigned)i, mul);
 }
 
 // One dimension of one level.  Tables: wl[m], wr[m], tap[5 mc], sub[mc],
@@ -1147,12 +1136,22 @@ cudaError_t launch_solves(const LevelGeom<T> &g, T *b, T *vc, int sign, cudaStre
         } else {
             int n = d.mc;
             long long nlines = c0 * c1;
-            // one tile of lines (two with v_c) and the three factor tables in 100 KB,
-            // two or three CTAs per SM; long lines take the SM's shared memory
-            const size_t line = (size_t)n * sizeof(T) * (sg ? 2 : 1), fixed = 3 * (size_t)n * sizeof(T) + 96;
-            const auto lines_in = [&](size_t kb) { return kb * 1024 > fixed ? (kb * 1024 - fixed) / line : 0; };
-            size_t rows = std::min<size_t>(kContigRows, lines_in(100));
-            if (rows < 8) rows = std::min<size_t>(8, lines_in(kContigMaxKb));
+            // a tile of lines and the three factor tables in 100 KB, two or three CTAs per
+            // SM; lines of which fewer than eight fit that take the SM's shared memory
+            // where it holds more of them
+            constexpr int V = 16 / sizeof(T);
+            const bool pad = n % kContigPad == 0 && !(((uintptr_t)b | (uintptr_t)src | (uintptr_t)vc) & 15);
+            const size_t line = (size_t)(pad ? n + V : n) * sizeof(T), fixed = 3 * (size_t)n * sizeof(T) + 96;
+            const auto lines_in = [&](size_t kb) {
+                return kb * 1024 > fixed ? std::min<size_t>(kContigRows, (kb * 1024 - fixed) / line) : 0;
+            };
+            size_t rows = lines_in(100);
+            if (rows < 8 && lines_in(kContigMaxKb) > 2 * rows) rows = lines_in(kContigMaxKb);
+            // One or two lines an SM pay a sweep's latency alone (55 ns a step in binary64, 11
+            // in binary32) once per wave; the strided kernel has every line in flight at about
+            // a microsecond a step (9000x9501 binary64: 20.6 ms with tiles of two, 16.7
+            // with the strided kernel on its finest level; 2000x9501 4.6 with tiles).
+            if (rows <= 2 && nlines > (sizeof(T) == 8 ? 8 : 40) * (long long)rows * sm_count()) rows = 0;
             if (rows < 1) {
                 e = launch_next(solve_strided_kernel<T>, (unsigned)((nlines + 255) / 256), 256, 0, s, b, src, n, 1, nlines,
                                 d.sub, d.cp, d.inv_den, vc, sg);
@@ -1164,7 +1163,7 @@ cudaError_t launch_solves(const LevelGeom<T> &g, T *b, T *vc, int sign, cudaStre
                 });
                 if (ea != cudaSuccess) return ea;
                 e = launch_next(solve_contig_kernel<T>, (unsigned)((nlines + rows - 1) / rows), kContigThreads,
-                                fixed + rows * line, s, b, src, n, nlines, (int)rows, d.sub, d.cp, d.inv_den, vc, sg);
+                                fixed + rows * line, s, b, src, n, nlines, (int)rows, pad, d.sub, d.cp, d.inv_den, vc, sg);
             }
         }
         src = b;
