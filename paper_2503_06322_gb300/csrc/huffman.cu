@@ -1686,6 +1686,12 @@ __global__ void __launch_bounds__(kHeaderThreads) header_batch_kernel(const Head
 // 513^3 at 1e-3: 515 -> 335 us; 300x431x517 at 1e-4, where most symbols are
 // escapes: 434 -> 295 us; 64 Mi byte keys: 222 -> 130 us.
 //
+// An escape whose codeword and payload do not fit 32 bits is three such steps where
+// escapes are dense (decode_chunk<3>; out of line, with its code stored alone, as
+// sparse ones still are, the 45 million codes of 15x1500x2000 binary64 at 1e-8 took 2099
+// us where the decoder before had
+// taken 1408; in line 330).
+//
 // Escaped codes: where they are dense (more than one symbol in sixteen) a
 // thread keeps the payloads of eight symbols in registers and writes each half
 // with an escape as one 32-byte sector: single 8-byte stores scattered over the
@@ -1878,7 +1884,8 @@ __device__ __noinline__ SlowOut decode_slow(uint32_t e, unsigned long long pos, 
 }
 
 // One chunk: cnt symbols from symbol beg on, from bit pos0 to bit expect.  EW: 0 no escapes,
-// 1 sparse ones, 2 dense ones.  Returns whether the stream was sound.
+// 1 sparse ones, 2 dense ones, 3 dense ones of which codewords and payloads do not fit
+// 32 bits.  Returns whether the stream was sound.
 template <typename S, int EW>
 __device__ __forceinline__ bool decode_chunk(const DecodeArgs &a, const HuffScratch &hs, const LenTabs *T, unsigned nsym,
                                              uint32_t lut, uint32_t sub, uint32_t ring, unsigned long long pos0,
@@ -1894,39 +1901,13 @@ __device__ __forceinline__ bool decode_chunk(const DecodeArgs &a, const HuffScra
     bool bad = false;
     S *sym = reinterpret_cast<S *>(a.sym) + beg;
     long long *e8 = EW ? a.esc + beg : nullptr;   // escape slots of the current group of eight symbols
-    uint32_t z[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};   // EW 2: payloads of the group, bit j of emask where there is one
+    // EW 2: payloads of the group, bit j of emask where there is one; EW 3: of half a
+    // group, the high words in z[4..7]
+    uint32_t z[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
     unsigned emask = 0;
-    // symbol in the high half
-    auto step = [&](unsigned j, uint32_t &zj) -> uint32_t {
-        uint32_t e = lds32(lut + 4 * (hi >> (32 - kLutBits)));
-        // a codeword of up to 23 bits: its second-level entry, indexed by the
-        // bits after the prefix (all within hi, nb >= 32)
-        lds_if(e, e & kDecSub, sub + (e >> 16) + 4 * ((hi << kLutBits) >> (e & 31u)));
-        if (e & kDecSlow) {
-            long long kv = 0;
-            const SlowOut o = decode_slow(e, q.pos(nb), q.base, q.left, T, hs.sorted_sym, nsym, (int)ew, &kv);
-            if (EW && o.sv == 0) {
-                // at once: its payload may not fit the group's registers
-                e8[j] = kv;
-                if (EW == 2) emask |= 0x100u << j;
-            }
-            bad |= o.bad != 0;
-            q.seek((unsigned)o.pos, hi, lo, nb);
-            return o.sv << 16;
-        }
-        const unsigned L = e & 63u;
-        if (EW) {
-            // folded escape: codeword of L - ew bits, then zigzag(k) in ew < 32 bits
-            const uint32_t y = (hi << ((L - ew) & 31u)) >> ((32u - ew) & 31u);
-            if (EW == 2) {
-                zj = y;
-                emask |= ((e / kDecEsc) & 1u) << j;
-            } else {
-                stg_if(e8 + j, e & kDecEsc, (long long)((int)(y >> 1) ^ -(int)(y & 1u)));
-            }
-        }
-        // drop L <= 32 bits, then refill to at least 32 valid bits (the valid
-        // bits are all in hi then)
+    // drops L <= 32 bits, then refills to at least 32 valid bits (the valid bits are
+    // all in hi then)
+    auto drop = [&](unsigned L) {
         hi = __funnelshift_lc(lo, hi, L);
         lo = __funnelshift_lc(0u, lo, L);
         nb -= (int)L;
@@ -1937,15 +1918,66 @@ __device__ __forceinline__ bool decode_chunk(const DecodeArgs &a, const HuffScra
         nb += need ? 32 : 0;
         q.rc += need ? 1u : 0u;
         lds_if(q.next, need, q.addr(q.rc));
+    };
+    // symbol in the high half
+    auto step = [&](unsigned j, uint32_t &zj, uint32_t &zh) -> uint32_t {
+        uint32_t e = lds32(lut + 4 * (hi >> (32 - kLutBits)));
+        // a codeword of up to 23 bits: its second-level entry, indexed by the
+        // bits after the prefix (all within hi, nb >= 32)
+        lds_if(e, e & kDecSub, sub + (e >> 16) + 4 * ((hi << kLutBits) >> (e & 31u)));
+        if (EW == 3 && (e & kDecOpen)) {
+            // the escape's codeword, then up to 63 bits of payload: three words at most,
+            // and the ring is topped up behind them
+            drop((e >> 16) & 0x3Fu);
+            const unsigned w0 = min(ew, 32u), w1 = ew - w0;
+            const uint32_t p0 = hi >> (32u - w0);
+            drop(w0);
+            const uint32_t p1 = w1 ? hi >> (32u - w1) : 0u;
+            drop(w1);
+            zh = w1 ? p0 >> (32u - w1) : 0u;
+            zj = w1 ? p0 << w1 | p1 : p0;
+            emask |= 1u << j;
+            q.top_up();
+            return 0u;
+        }
+        if (e & kDecSlow) {
+            long long kv = 0;
+            const SlowOut o = decode_slow(e, q.pos(nb), q.base, q.left, T, hs.sorted_sym, nsym, (int)ew, &kv);
+            if (EW && o.sv == 0) {
+                // at once: its payload may not fit the group's registers
+                e8[j] = kv;
+                if (EW >= 2) emask |= 0x100u << j;
+            }
+            bad |= o.bad != 0;
+            q.seek((unsigned)o.pos, hi, lo, nb);
+            return o.sv << 16;
+        }
+        const unsigned L = e & 63u;
+        if (EW) {
+            // folded escape: codeword of L - ew bits, then zigzag(k) in ew < 32 bits
+            const uint32_t y = (hi << ((L - ew) & 31u)) >> ((32u - ew) & 31u);
+            if (EW >= 2) {
+                zj = y;
+                if (EW == 3) zh = 0u;
+                emask |= ((e / kDecEsc) & 1u) << j;
+            } else {
+                stg_if(e8 + j, e & kDecEsc, (long long)((int)(y >> 1) ^ -(int)(y & 1u)));
+            }
+        }
+        drop(L);
         return e;
     };
     // the escaped codes of a group: each half with an escape as one 32-byte
     // store; a code stored by its own step (upper mask) keeps its half from being
     // overwritten: the others of that half go one by one
-    auto flush8 = [&]() {
-        auto code = [&](unsigned j) { return (long long)((int)(z[j] >> 1) ^ -(int)(z[j] & 1u)); };
+    auto code = [&](unsigned j) -> long long {
+        if (EW == 3) return unzigzag((unsigned long long)z[4 + (j & 3u)] << 32 | z[j & 3u]);
+        return (long long)((int)(z[j] >> 1) ^ -(int)(z[j] & 1u));
+    };
+    // (symbols h0..h1 of it)
+    auto flush = [&](unsigned h0, unsigned h1) {
 #pragma unroll
-        for (unsigned h = 0; h < 8; h += 4) {
+        for (unsigned h = h0; h < h1; h += 4) {
             const unsigned m = (emask >> h) & 0xFu;
             if (!m) continue;
             if ((emask >> (8 + h)) & 0xFu) {
@@ -1963,7 +1995,12 @@ __device__ __forceinline__ bool decode_chunk(const DecodeArgs &a, const HuffScra
         q.top_up();
 #pragma unroll
         for (unsigned j = 0; j < 8; j += 2) {
-            const uint32_t v0 = step(j, z[j]), v1 = step(j + 1, z[j + 1]);
+            if (EW == 3 && j == 4) {
+                if (emask) flush(0, 4);
+                q.top_up();
+            }
+            const unsigned i = EW == 3 ? j & 3u : j;
+            const uint32_t v0 = step(j, z[i], z[EW == 3 ? 4 + i : 0]), v1 = step(j + 1, z[i + 1], z[EW == 3 ? 5 + i : 0]);
             o[j / 2] = __byte_perm(v0, v1, sizeof(S) == 2 ? 0x7632 : 0x0062);
         }
         // streaming store: the symbols are written once and read by the next
@@ -1972,15 +2009,17 @@ __device__ __forceinline__ bool decode_chunk(const DecodeArgs &a, const HuffScra
         else __stcs(reinterpret_cast<uint2 *>(sym),
                     make_uint2(__byte_perm(o[0], o[1], 0x5410), __byte_perm(o[2], o[3], 0x5410)));
         sym += 8;
-        if (EW == 2 && emask) flush8();
+        if (EW == 2 && emask) flush(0, 8);
+        if (EW == 3 && emask) flush(4, 8);
         if (EW) e8 += 8;
     }
     // a last group of fewer than eight: its escapes one by one
     q.top_up();
     for (unsigned j = 0; j < cnt % 8; j++) {
-        uint32_t y = 0;
-        sym[j] = (S)(step(j, y) >> 16);
-        if (EW == 2 && ((emask >> j) & 1u)) e8[j] = (long long)((int)(y >> 1) ^ -(int)(y & 1u));
+        uint32_t y = 0, yh = 0;
+        sym[j] = (S)(step(j, y, yh) >> 16);
+        if (EW >= 2 && ((emask >> j) & 1u))
+            e8[j] = EW == 3 ? unzigzag((unsigned long long)yh << 32 | y) : (long long)((int)(y >> 1) ^ -(int)(y & 1u));
     }
     return !bad && q.pos(nb) == expos;
 }
@@ -2011,6 +2050,7 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_kernel(DecodeArgs a_in,
     uint32_t *ring = reinterpret_cast<uint32_t *>(T + 1);                      // [kRingWords][kDecThreads]
     const unsigned nsym = *hs.nsym;
     const unsigned nsub = *hs.nsub < kSubCap ? *hs.nsub : kSubCap;
+    int open = 0;   // whether an escape's codeword and payload do not fit 32 bits
     {
         // escape entries take their payload width into their length when both fit 32 bits
         const unsigned ewc = a.esc ? a.esc_w : 0u;
@@ -2019,7 +2059,11 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_kernel(DecodeArgs a_in,
             const unsigned L = (e >> 16) & 0x3Fu;
             if (e & kLongFlag) return kDecSlow | (L << 16) | (((e >> 24) & 0x3Fu) << 24);
             if (e & kSubFlag) return ((e & 0x3FFFu) << 18) | kDecSub | (32u - ((e >> 16) & 0xFu));
-            if (ewc && (e & 0xFFFFu) == 0) return L + ewc <= 32 ? kDecEsc | (L + ewc) : kDecSlow | kDecOpen | (L << 16);
+            if (ewc && (e & 0xFFFFu) == 0) {
+                if (L + ewc <= 32) return kDecEsc | (L + ewc);
+                open = 1;
+                return kDecSlow | kDecOpen | (L << 16);
+            }
             return (e << 16) | L;
         };
         auto four = [&](uint4 v) { return make_uint4(entry(v.x), entry(v.y), entry(v.z), entry(v.w)); };
@@ -2044,8 +2088,8 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_kernel(DecodeArgs a_in,
         T->start[threadIdx.x] = hs.start[threadIdx.x];
         T->count[threadIdx.x] = hs.count[threadIdx.x];
     }
-    __syncthreads();
-    const int mode = !a.esc || !a.esc_w ? 0 : a.n_esc * 16 > a.N ? 2 : 1;
+    open = __syncthreads_or(open);
+    const int mode = !a.esc || !a.esc_w ? 0 : a.n_esc * 16 > a.N ? (open ? 3 : 2) : 1;
     const uint32_t lut_a = smem_u32(lut), sub_a = smem_u32(sub), ring_a = smem_u32(ring + threadIdx.x);
     // chunks interleave over the blocks so that every SM gets a share
     for (unsigned long long c = blockIdx.x + (unsigned long long)gridDim.x * threadIdx.x; c < nch;
@@ -2060,6 +2104,7 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_kernel(DecodeArgs a_in,
         if (ok) {
             if (sizeof(S) == 1 || mode == 0) ok = decode_chunk<S, 0>(a, hs, T, nsym, lut_a, sub_a, ring_a, pos0, expect, beg, cnt);
             else if (mode == 1) ok = decode_chunk<S, 1>(a, hs, T, nsym, lut_a, sub_a, ring_a, pos0, expect, beg, cnt);
+            else if (mode == 3) ok = decode_chunk<S, 3>(a, hs, T, nsym, lut_a, sub_a, ring_a, pos0, expect, beg, cnt);
             else ok = decode_chunk<S, 2>(a, hs, T, nsym, lut_a, sub_a, ring_a, pos0, expect, beg, cnt);
         }
         if (!ok) atomicExch(hs.status, (unsigned)DS_FORMAT);
