@@ -453,29 +453,31 @@ __global__ void __launch_bounds__(kZfpThreads) zfp_encode_kernel(const T *__rest
         w[r] = ((UI)q[ord.p[r]] + (UI)Z::M) ^ (UI)Z::M;
         any |= w[r];
     }
-    uint32_t pl[B == 64 ? P : 1][2];   // planes of a block of 64
-    if constexpr (B == 64) {
-#pragma unroll
-        for (int h = 0; h < 2; h++)
-#pragma unroll
-            for (int c = 0; c < P / 32; c++) {
-                uint32_t a[32];
-#pragma unroll
-                for (int r = 0; r < 32; r++) a[r] = (uint32_t)(w[32 * h + r] >> (32 * c));
-                transpose32(a);
-#pragma unroll
-                for (int k = 0; k < 32; k++) pl[32 * c + k][h] = a[k];
-            }
-    }
     // the planes above the highest one set: a 0 test each
     int k = P - 1;
     while (k >= 0 && !((any >> k) & 1)) k--;
     bw.zeros(P - 1 - k);
     int n = 0;
-    for (; k >= 0 && !bw.full(); k--) {
+    uint32_t pl[B == 64 ? 32 : 1][2];   // 32 planes of a block of 64
+#pragma unroll
+    for (int c = P / 32 - 1; c >= 0; c--) {
+    if (P > 32 && (k < 32 * c || bw.full())) continue;   // binary64 at a low rate ends in its upper planes
+    if constexpr (B == 64) {
+#pragma unroll
+        for (int h = 0; h < 2; h++) {
+            uint32_t a[32];
+#pragma unroll
+            for (int r = 0; r < 32; r++) a[r] = (uint32_t)(w[32 * h + r] >> (32 * c));
+            transpose32(a);
+#pragma unroll
+            for (int i = 0; i < 32; i++) pl[i][h] = a[i];
+        }
+    }
+    for (; k >= 32 * c && !bw.full(); k--) {
         unsigned long long mask = 0;
         if constexpr (B == 64) {
-            mask = (unsigned long long)pl[k][1] << 32 | pl[k][0];
+            const int i = P > 32 ? k & 31 : k;
+            mask = (unsigned long long)pl[i][1] << 32 | pl[i][0];
         } else {
 #pragma unroll
             for (int r = 0; r < B; r++) mask |= (unsigned long long)((w[r] >> k) & 1) << r;
@@ -504,6 +506,7 @@ __global__ void __launch_bounds__(kZfpThreads) zfp_encode_kernel(const T *__rest
             n += j + 1;
             rest = rest >> j >> 1;
         }
+    }
     }
     bw.finish();
 }
@@ -540,8 +543,8 @@ __global__ void __launch_bounds__(kZfpThreads) zfp_decode_kernel(const uint32_t 
 #pragma unroll
                 for (int k = 0; k < P; k++) pl[k][0] = pl[k][1] = 0u;
             }
-            int n = 0;
-            for (int k = P - 1; k >= 0 && !br.done(); k--) {
+            int n = 0, k = P - 1;
+            for (; k >= 0 && !br.done(); k--) {
                 unsigned long long mask = 0;
                 // verbatim bits of coefficients 0..n-1
                 if (n > 32) {
@@ -593,9 +596,10 @@ __global__ void __launch_bounds__(kZfpThreads) zfp_decode_kernel(const uint32_t 
                 for (int h = 0; h < 2; h++)
 #pragma unroll
                     for (int c = 0; c < P / 32; c++) {
+                        if (P > 32 && c == 0 && k >= 31) continue;   // none of the lower planes was reached
                         uint32_t a[32];
 #pragma unroll
-                        for (int k = 0; k < 32; k++) a[k] = pl[32 * c + k][h];
+                        for (int i = 0; i < 32; i++) a[i] = pl[32 * c + i][h];
                         transpose32(a);
 #pragma unroll
                         for (int r = 0; r < 32; r++) w[32 * h + r] |= (UI)a[r] << (32 * c);
