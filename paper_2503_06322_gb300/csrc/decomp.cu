@@ -1482,12 +1482,6 @@ cudaError_t launch_decomp(Sink sink, const RestrictArgs<T> &a0, cudaStream_t s)
 }
 
 template <typename T>
-cudaError_t launch_restrict_symbols(const RestrictArgs<T> &a0, cudaStream_t s)
-{
-    return launch_restrict_planes<T>(WSrc::SYMBOLS, a0, s);
-}
-
-template <typename T>
 cudaError_t launch_restrict_planes(WSrc src, const RestrictArgs<T> &a0, cudaStream_t s)
 {
     RestrictArgs<T> a = a0;
@@ -1541,8 +1535,6 @@ cudaError_t launch_expand_planes(WSrc src, const LevelGeom<T> &g, const T *vc, c
 
 template cudaError_t launch_decomp<float>(Sink, const RestrictArgs<float> &, cudaStream_t);
 template cudaError_t launch_decomp<double>(Sink, const RestrictArgs<double> &, cudaStream_t);
-template cudaError_t launch_restrict_symbols<float>(const RestrictArgs<float> &, cudaStream_t);
-template cudaError_t launch_restrict_symbols<double>(const RestrictArgs<double> &, cudaStream_t);
 template cudaError_t launch_restrict_planes<float>(WSrc, const RestrictArgs<float> &, cudaStream_t);
 template cudaError_t launch_restrict_planes<double>(WSrc, const RestrictArgs<double> &, cudaStream_t);
 template cudaError_t launch_expand_planes<float>(WSrc, const LevelGeom<float> &, const float *, const float *,

@@ -30,12 +30,10 @@ __device__ __forceinline__ unsigned long long warp_sum64(unsigned long long v)
     return v;
 }
 
-// keys of the present symbols, in increasing symbol order:
-//   from a histogram: (frequency << 16) | s   (frequency > 0)
-//   from lengths:     (length << 16) | s      (length > 0)
+// keys (frequency << 16) | s of the present symbols, in increasing symbol order
 __global__ void __launch_bounds__(1024)
-compact_kernel(const unsigned long long *hist, const uint8_t *len, unsigned D,
-               unsigned long long *keys, unsigned *nsym, unsigned *s_lo, unsigned *s_hi)
+compact_kernel(const unsigned long long *hist, unsigned D, unsigned long long *keys, unsigned *nsym, unsigned *s_lo,
+               unsigned *s_hi)
 {
     __shared__ unsigned wcnt[32], wpre[32];
     __shared__ unsigned base, lo, hi;
@@ -45,7 +43,7 @@ compact_kernel(const unsigned long long *hist, const uint8_t *len, unsigned D,
     for (unsigned t0 = 0; t0 < D; t0 += 1024) {
         unsigned s = t0 + threadIdx.x;
         unsigned long long f = 0;
-        if (s < D) f = hist ? hist[s] : (unsigned long long)len[s];
+        if (s < D) f = hist[s];
         bool p = f != 0;
         unsigned ball = __ballot_sync(0xffffffffu, p);
         if (lane == 0) wcnt[w] = __popc(ball);
@@ -70,7 +68,8 @@ compact_kernel(const unsigned long long *hist, const uint8_t *len, unsigned D,
     }
     if (threadIdx.x == 0) {
         *nsym = base;
-        if (s_lo) { *s_lo = base ? lo : 0; *s_hi = base ? hi : 0; }
+        *s_lo = base ? lo : 0;
+        *s_hi = base ? hi : 0;
     }
 }
 
@@ -2350,7 +2349,7 @@ cudaError_t launch_codebook(const unsigned long long *hist, unsigned int D, cons
         count_launch();
         return launch_next(codebook_kernel, 1, 1024, kCodebookSmem, s, hist, D, hs);
     }
-    compact_kernel<<<1, 1024, 0, s>>>(hist, nullptr, D, hs.keys, hs.nsym, hs.s_lo, hs.s_hi);
+    compact_kernel<<<1, 1024, 0, s>>>(hist, D, hs.keys, hs.nsym, hs.s_lo, hs.s_hi);
     rank_kernel<<<kRankBlocks, 256, kSmemKeys * 8, s>>>(hs.keys, hs.nsym, hs.sorted, nullptr);
     merge_kernel<<<1, 1024, kSmemKeys * 16, s>>>(hs, D);
     rank_kernel<<<kRankBlocks, 256, kSmemKeys * 8, s>>>(hs.keys2, hs.nsym, nullptr, hs.rank);

@@ -38,7 +38,7 @@ struct HuffScratch {
     unsigned int *start;          // [64]
     uint8_t *len;                 // [D]
     unsigned long long *code;     // [D]
-    uint32_t *pack;               // [D] encoder: codeword << 8 | length, short codewords (pack_code)
+    uint32_t *pack;               // [D] encoder: codeword << 6 | length, codewords of at most 26 bits (pack_code)
     uint16_t *sorted_sym;         // [D]
     uint32_t *lut1;               // [1 << kLutBits] first-level decoder table of every 13-bit prefix
     uint32_t *lut_sub;            // [kSubCap] second-level entries of longer codewords
@@ -112,7 +112,7 @@ struct EncodeArgs {
                                       // escape and esc[i] its code k (payload after the codeword,
                                       // in sc->esc_w bits)
     unsigned long long *chunk_bits;   // ws [nch+1] totals then offsets
-    unsigned long long *bsum;         // ws [kEncBlocks] per-block sums, then offsets
+    unsigned long long *bsum;         // ws [kEncBlocks] per-block sums
     Scalars *sc;
     // destination
     uint8_t *container;               // if non-null: chunk table and bits go into the container

@@ -137,20 +137,8 @@ __device__ __forceinline__ void mbar_arrive_expect_tx(unsigned long long *bar, u
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes)
                  : "memory");
 }
-__device__ __forceinline__ bool mbar_try_wait(unsigned long long *bar, uint32_t parity)
-{
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(smem_u32(bar)), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-// As mbar_try_wait, but a thread whose phase is not complete is suspended in
-// hardware until the phase completes or about `ns` nanoseconds pass, so a
+// Whether the phase with the given parity is complete.  A thread whose phase is not
+// is suspended in hardware until it completes or about `ns` nanoseconds pass, so a
 // waiting warp issues no instructions.
 __device__ __forceinline__ bool mbar_try_wait_sleep(unsigned long long *bar, uint32_t parity, uint32_t ns)
 {
@@ -163,13 +151,6 @@ __device__ __forceinline__ bool mbar_try_wait_sleep(unsigned long long *bar, uin
         : "r"(smem_u32(bar)), "r"(parity), "r"(ns)
         : "memory");
     return ok != 0;
-}
-// Waits for the phase with the given parity; gives up after `limit` polls.
-__device__ __forceinline__ bool mbar_wait_bounded(unsigned long long *bar, uint32_t parity, int limit)
-{
-    for (int i = 0; i < limit; i++)
-        if (mbar_try_wait(bar, parity)) return true;
-    return false;
 }
 // 16-byte aligned source, destination and size.
 __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t bytes, unsigned long long *bar)

@@ -315,7 +315,7 @@ __global__ void level0_kernel(const T *v0, long long N0, T *coef_out, QuantOut q
     if (i >= N0) return;
     T x = v0[i];
     if (SINK == (int)Sink::STREAM) { coef_out[i] = x; return; }
-    quant_emit(qo, nullptr, false, i, x, rho64_of(qo.sc, 0));
+    quant_emit(qo, i, x, rho64_of(qo.sc, 0));
 }
 
 template <typename T, int SRC>

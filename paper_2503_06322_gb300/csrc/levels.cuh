@@ -59,9 +59,7 @@ cudaError_t launch_restrict(WSrc src, Sink sink, const RestrictArgs<T> &a, cudaS
 // (SYMBOLS source), warp-specialised plane pipelines.
 template <typename T>
 cudaError_t launch_decomp(Sink sink, const RestrictArgs<T> &a, cudaStream_t s);
-template <typename T>
-cudaError_t launch_restrict_symbols(const RestrictArgs<T> &a, cudaStream_t s);
-// the same plane pipeline over any decompression-side source: SYMBOLS,
+// the plane pipeline over any decompression-side source: SYMBOLS,
 // STREAM (a coefficient stream) or DENSE (a level-l grid, all or new nodes)
 template <typename T>
 cudaError_t launch_restrict_planes(WSrc src, const RestrictArgs<T> &a, cudaStream_t s);

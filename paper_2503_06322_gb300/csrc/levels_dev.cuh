@@ -69,20 +69,6 @@ template <typename T> __device__ __forceinline__ T q_of(const Scalars *sc, int l
 template <> __device__ __forceinline__ float q_of<float>(const Scalars *sc, int l) { return sc->q_f[l]; }
 template <> __device__ __forceinline__ double q_of<double>(const Scalars *sc, int l) { return sc->q[l]; }
 
-template <typename T>
-__device__ __forceinline__ long long stream_rank(const LevelGeom<T> &g, int p0, int p1, int p2)
-{
-    const long long m1 = g.dim[1].m, m2 = g.dim[2].m;
-    const long long mc1 = g.dim[1].mc, mc2 = g.dim[2].mc;
-    long long flat = ((long long)p0 * m1 + p1) * m2 + p2;
-    long long cr = (long long)kept_before(p0) * mc1 * mc2;
-    if (kept_pos(g.dim[0].m, p0)) {
-        cr += (long long)kept_before(p1) * mc2;
-        if (kept_pos((int)m1, p1)) cr += kept_before(p2);
-    }
-    return g.Nprev + flat - cr;
-}
-
 // Stream index of the new nodes of row (p0, p1) of level l:
 //   every node new (p0 or p1 new):        base + p2
 //   p0 and p1 kept (only odd p2 new):     base + (p2 - 1) / 2
@@ -156,10 +142,9 @@ __device__ __noinline__ unsigned quant_far_f32(const QuantOut &qo, long long si,
     return escape_f32(qo, si, w, rho_hi, rho_lo, rho) << 16;
 }
 
-// quantize one coefficient into the symbol stream (+ block histogram / escapes)
+// quantize one coefficient into the symbol stream, the global histogram and the escapes
 template <typename T>
-__device__ __forceinline__ void quant_emit(const QuantOut &qo, unsigned int *hs, bool smem_hist,
-                                           long long si, T w, double rho)
+__device__ __forceinline__ void quant_emit(const QuantOut &qo, long long si, T w, double rho)
 {
     long long k = quant_code(w, rho);
     long long s = k + (long long)(qo.D / 2);
@@ -171,8 +156,7 @@ __device__ __forceinline__ void quant_emit(const QuantOut &qo, unsigned int *hs,
         atomicMax(&qo.sc->esc_w, escape_store(qo, si, k));
     }
     qo.sym[si] = (uint16_t)sym;
-    if (smem_hist) atomicAdd(&hs[sym], 1u);
-    else atomicAdd(&qo.hist[sym], 1ULL);
+    atomicAdd(&qo.hist[sym], 1ULL);
 }
 
 // The binary64 decision of a binary32 coefficient without binary64 arithmetic
