@@ -643,8 +643,10 @@ decomp_kernel(RestrictArgs<T> a, int seg_len)
         }
         // Away from a short last interval the mass rows have taps at the kept
         // nodes of the window only (offsets -2, 0 and 2): a fused multiply-add
-        // with a zero tap changes no bit, and binary64, bound by the FP64 pipe,
-        // skips it (in binary32 the test costs what the products do).
+        // with a zero tap changes no bit of a finite sum, and binary64, bound by the
+        // FP64 pipe, skips it (in binary32 the test costs what the products do).  An
+        // infinity or NaN under such a tap enters b through the restriction's taps,
+        // none of which is zero.
         const bool even2 = sizeof(T) == 8 && __all_sync(0xffffffffu, lc.m2t[1] == (T)0 && lc.m2t[3] == (T)0);
         const bool even1 = sizeof(T) == 8 && wr.ma[1] == (T)0 && wr.ma[3] == (T)0 && wr.mb[1] == (T)0 && wr.mb[3] == (T)0;
         T acc[2][3];

@@ -1702,13 +1702,12 @@ __global__ void __launch_bounds__(kHeaderThreads) header_batch_kernel(const Head
 //     predicated (as branches they cost the warp both sides at nearly every
 //     step); only the out-of-line cases branch.
 // 513^3 at 1e-3: 515 -> 335 us; 300x431x517 at 1e-4, where most symbols are
-// escapes: 434 -> 295 us; 64 Mi byte keys: 222 -> 130 us.
+// escapes: 434 -> 295 us; 64 Mi byte keys: 222 -> 114 us.
 //
 // An escape whose codeword and payload do not fit 32 bits is three such steps where
 // escapes are dense (decode_chunk<3>; out of line, with its code stored alone, as
-// sparse ones still are, the 45 million codes of 15x1500x2000 binary64 at 1e-8 took 2099
-// us where the decoder before had
-// taken 1408; in line 330).
+// sparse ones still are, the 45 million codes of 15x1500x2000 binary64 at 1e-8 took
+// 2099 us; in line 303).
 //
 // Escaped codes: where they are dense (more than one symbol in sixteen) a
 // thread keeps the payloads of eight symbols in registers and writes each half
