@@ -26,15 +26,15 @@ enum { MP_RT_FINAL = 1, MP_DT_FINAL = 2 };
 //   MP_DT_FINAL: out[p] = coef[rank(p)] + y_f(p)
 // One pass over the fine grid is all it needs from memory (a pass per dimension,
 // through two partial grids, moved 2.6 times the bytes and took 173 us for the
-// finest level of 257^3; this takes 62, bound by instruction issue: 78 with the
-// window's edges tested at every node).  A warp owns coarse row j1 of a tile and lane l
-// coarse column j2 (or, on thin grids, four rows and eight columns), and the CTA
-// marches along the coarse planes of its segment; for each plane a lane forms the
-// dimension-2, then the dimension-1 products at its 2 x 2 fine nodes (rows Ra, Ra + 1,
-// columns Ca, Ca + 1) from the four rows and four columns of y around it (cached
-// loads, coalesced per row) and keeps the last three planes' for the dimension-0
-// products.  Every value sums its taps in a fixed order, so nothing depends on the
-// tiling.
+// finest level of 257^3; this takes 62, bound by the latency of its sixteen cached
+// loads a plane at 42% of the issue slots: 78 with the window's edges tested at every
+// node).  A warp owns coarse row j1 of a tile and lane l coarse column j2 (or, on thin
+// grids, four rows and eight columns), and the CTA marches along the coarse planes of
+// its segment; for each plane a lane forms the dimension-2, then the dimension-1
+// products at its 2 x 2 fine nodes (rows Ra, Ra + 1, columns Ca, Ca + 1) from the four
+// rows and four columns of y around it (cached loads, coalesced per row) and keeps the
+// last three planes' for the dimension-0 products.  Every value sums its taps in a
+// fixed order, so nothing depends on the tiling.
 constexpr int kMpWarps = 8;
 // The tiles of a coarse plane, LC columns wide, run along gridDim.x, columns first:
 // gridDim.y ends at 65535, and a tall field has more row tiles.
