@@ -613,6 +613,15 @@ __global__ void __launch_bounds__(kZfpThreads) zfp_decode_kernel(const uint32_t 
         }
     }
 #ifdef __CUDA_ARCH__
+    // binary64 rows of fewer dimensions are whole sectors as they are
+    if constexpr (sizeof(T) == 8 && D < 3) {
+        if (live) {
+#pragma unroll
+            for (int i = 0; i < B; i++)
+                if (value_inside<D>(bp, i)) u[bp.base + value_offset<D>(bp, i)] = val[i];
+        }
+        return;
+    }
     // A warp's blocks lie side by side along the last dimension: their rows of
     // four values meet in shared memory and leave as whole lines.  Value t = 32 it +
     // lane of a row of the warp belongs to lane t / 4 and sits at position t & 3.
